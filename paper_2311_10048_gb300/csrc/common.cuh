@@ -148,7 +148,7 @@ struct TcProb {
   void* out;        // output of this problem: [N][ldo] (transposed) or [M][ldo] (row-major)
 };
 
-// Output layout of a row-major (RM) float32 contraction launch.
+// Output layout of a row-major float32 contraction launch (tc_pair.cu).
 //   kOutRows:  out[m][n], pitch ldo.
 //   kOutYTile: mixed-spin Y, rows m = b nvt + C, columns a, stored as 16^3
 //              tiles (b/16, C/16, a/16), tile index (B nbt + C') nbs + A; in a
@@ -175,23 +175,35 @@ constexpr int kTile = 4096;   // floats of one 16^3 tile
 struct TcDiag {
   long long wait_cycles;
   int starve;
-  // mixed spin: Y and Z' stored as 16^3 tiles (kOutYTile / kOutZTile, strides
-  // in floats per triplet above); selects the TMA-staged kernel
-  int tiled;
 };
 
 // tc_gemm.cu: grouped sliced contraction.  mA: maps with 128-row boxes,
-// mB: maps with BN-row boxes; instances (S, BN, OutT, TF, RM) are listed there
-// (RM: row-major output out[m][n], else the transposed out[n][m]).
-template <int S, int BN, typename OutT, bool TF = false, bool RM = false>
+// mB: maps with BN-row boxes; transposed output out[n][m].  The instances
+// (S, BN, OutT, TF) are listed there.
+template <int S, int BN, typename OutT, bool TF = false>
 cudaError_t launch_tc_gemm(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs_dev,
                            int nprob, int M, int N, int ldo, double scale, int* flag,
-                           unsigned long long* amax, int nsm, cudaStream_t st, TcDiag diag,
-                           TcOut lay = TcOut{kOutRows, 0, 0, 0});
+                           unsigned long long* amax, int nsm, cudaStream_t st, TcDiag diag);
 long long tc_default_wait_cycles();
 inline TcDiag tc_normal() { return TcDiag{tc_default_wait_cycles(), 0}; }
 int make_operand_map(CUtensorMap* map, const void* base, int64_t Kp, int64_t rows, int S,
-                     int64_t slice_stride, int box_rows, int esz = 2);
+                     int64_t slice_stride, int box_rows, int esz = 2, int box_slices = 1);
+
+// tc_pair.cu: the W contractions on CTA pairs, float32 row-major output
+// out[m][n] in the layout `lay`.  Slice formats (the instruction descriptor's
+// codes); tile of a launch (pair_tile).
+constexpr int kFmtBF16 = 1, kFmtTF32 = 2;
+struct PairTile {
+  int w;        // columns of one n-tile (multiple of 16)
+  int nN;       // n-tiles
+  int nbuf;     // accumulator sets in TMEM (2 when 2 S w <= 512)
+  int stages;   // k blocks in flight in shared memory
+};
+PairTile pair_tile(int S, int N, int cap);
+template <int S, int FMT>
+cudaError_t launch_tc_pair(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs_dev,
+                           int nprob, int M, int N, int ldo, double scale, int* flag, int nsm,
+                           cudaStream_t st, TcDiag diag, TcOut lay, PairTile tile);
 int sliced_product_bn(int S);
 cudaError_t launch_sliced_product(int S, const CUtensorMap* mA, const CUtensorMap* mB,
                                   const TcProb* dp, int M, int N, double scale, int* flag,

@@ -251,54 +251,40 @@ struct Operand {
   int esz = 2;                   // bytes per slice element
   int S = 0;
   int64_t slice_stride = 0;
-  CUtensorMap map128, map256, map96, map64;  // TMA maps with boxes of 128 (A role, B of BN 128), 256, 96, 64 rows
+  CUtensorMap map128, map64;  // TMA maps of one slice, boxes of 128 and 64 rows (tc_gemm.cu)
   int64_t total_rows() const { return (int64_t)nslot * rows; }
-};
-
-// Tile width of the W contraction for S slices: the tuned value when it is
-// one the build has (S * BN <= 512 TMEM columns), else the default.
-int contract_bn(int S, int bn) {
-  switch (S) {
-    case 2: return bn == 128 ? 128 : 256;
-    case 3: return bn == 64 ? 64 : 128;
-    case 4: return bn == 64 ? 64 : bn == 96 ? 96 : 128;
-    default: return 64;
+  // TMA map of the pair kernel: boxes of box_rows rows x all slices
+  int pair_map(CUtensorMap* m, int box_rows) const {
+    return make_operand_map(m, esz == 4 ? (const void*)f32 : (const void*)bf, Kp,
+                            std::max<int64_t>(total_rows(), 1), S, slice_stride, box_rows, esz, S);
   }
-}
-
-const CUtensorMap& map_for(const Operand& op, int box) {
-  return box == 256 ? op.map256 : box == 96 ? op.map96 : box == 64 ? op.map64 : op.map128;
-}
+};
 
 // One grouped W-contraction launch with float32 output XT[n][m] (pitch ldo)
 // = sum_seg A_seg[m] . B_seg[n], m < M the virtual index of the A operands, n
 // < N the (pair) rows of the B operands.  The kernel runs it row-major with
-// the roles exchanged: its 128-row tiles run over the N rows (a long
-// dimension, so they are full) and its n-tiles over the M rows, the last one
-// only as wide as needed (M rounded up to 16).  seg_tc stores the segments
-// with the roles already exchanged.
-cudaError_t launch_contract(int S, bool tf, int bn_req, const Operand& A0, const Operand& A1,
+// the roles exchanged: its row tiles run over the N rows (a long dimension, so
+// they are full) and its n-tiles over the M rows.  seg_tc stores the segments
+// with the roles already exchanged.  bn > 0 caps the tile width.
+cudaError_t launch_contract(int S, bool tf, int bn, const Operand& A0, const Operand& A1,
                             const Operand& B0, const Operand& B1, const TcProb* dpt, int nprob,
                             int M, int N, int ldo, double scale, int* flag, int nsm,
                             cudaStream_t st, TcOut lay) {
-  const int bn = contract_bn(S, bn_req);
-  CUtensorMap mA[2] = {B0.map128, B1.map128};
-  CUtensorMap mB[2] = {map_for(A0, bn), map_for(A1, bn)};
-  const TcDiag dg = tc_normal();
   std::swap(M, N);
-#define LNO_CALL(SS, BB)                                                                      \
-  launch_tc_gemm<SS, BB, float, false, true>(mA, mB, dpt, nprob, M, N, ldo, scale, flag, nullptr, \
-                                             nsm, st, dg, lay)
-  if (tf)
-    return bn == 128
-               ? launch_tc_gemm<2, 128, float, true, true>(mA, mB, dpt, nprob, M, N, ldo, scale,
-                                                           flag, nullptr, nsm, st, dg, lay)
-               : launch_tc_gemm<2, 256, float, true, true>(mA, mB, dpt, nprob, M, N, ldo, scale,
-                                                           flag, nullptr, nsm, st, dg, lay);
-  if (S == 2) return bn == 128 ? LNO_CALL(2, 128) : LNO_CALL(2, 256);
-  if (S == 3) return bn == 64 ? LNO_CALL(3, 64) : LNO_CALL(3, 128);
-  if (S == 4) return bn == 64 ? LNO_CALL(4, 64) : bn == 96 ? LNO_CALL(4, 96) : LNO_CALL(4, 128);
-  return LNO_CALL(5, 64);
+  const PairTile t = pair_tile(S, N, bn);
+  CUtensorMap mA[2], mB[2];
+  if (B0.pair_map(&mA[0], 128) || B1.pair_map(&mA[1], 128) || A0.pair_map(&mB[0], t.w / 2) ||
+      A1.pair_map(&mB[1], t.w / 2))
+    return cudaErrorInvalidValue;
+#define LNO_CALL(SS, FF) \
+  launch_tc_pair<SS, FF>(mA, mB, dpt, nprob, M, N, ldo, scale, flag, nsm, st, tc_normal(), lay, t)
+  if (tf) return LNO_CALL(2, kFmtTF32);
+  switch (S) {
+    case 2: return LNO_CALL(2, kFmtBF16);
+    case 3: return LNO_CALL(3, kFmtBF16);
+    case 4: return LNO_CALL(4, kFmtBF16);
+    default: return LNO_CALL(5, kFmtBF16);
+  }
 #undef LNO_CALL
 }
 
@@ -373,7 +359,9 @@ struct Run {
     op.nslot = nslot;
     op.rows = rows;
     op.K = K;
-    op.Kp = (int)round_up(std::max(K, 1), 8);
+    // sliced rows start on 64-byte boundaries: the contractions' 64-byte box
+    // rows then are two sectors of L2 (1.3x fewer bytes than at 16-byte pitches)
+    op.Kp = (int)round_up(std::max(K, 1), f64 ? 8 : tf ? 16 : 32);
     op.S = f64 ? 0 : S_;
     const int64_t n = std::max<int64_t>((int64_t)nslot * rows * op.Kp, 8);
     if (f64) {
@@ -392,9 +380,7 @@ struct Run {
       }
       const int64_t rows_ = std::max<int64_t>(op.total_rows(), 1);
       TRY(make_operand_map(&op.map128, base, op.Kp, rows_, op.S, op.slice_stride, 128, op.esz));
-      TRY(make_operand_map(&op.map256, base, op.Kp, rows_, op.S, op.slice_stride, 256, op.esz));
       TRY(make_operand_map(&op.map64, base, op.Kp, rows_, op.S, op.slice_stride, 64, op.esz));
-      TRY(make_operand_map(&op.map96, base, op.Kp, rows_, op.S, op.slice_stride, 96, op.esz));
     }
     return LNO_OT_OK;
   }
@@ -624,7 +610,7 @@ struct SpinPass {
   std::vector<int> slotAT, slotBT, slotA1, slotBG, slotBF, slotAT2;  // -1 = unused
   std::vector<int2> listAT, listA1, listAT2;
   std::vector<int> listBT, listBG, listBF;
-  int bn = 0;                // contraction tile width of the current case (0 = default)
+  int bn = 0;                // widest contraction tile of the current case (0 = default)
   int group_cap = 64;        // triplets per group (upper bound)
   double* t2st = nullptr;    // [os][ot][vs][vt]
   const double* t2ss = nullptr;
@@ -1878,7 +1864,7 @@ int tc_matmul(Run& R, Arena& A, int M, int N, int K, View a, View b, double* C, 
   TcProb* dp;
   TRY(A.get(&dp, (size_t)nsp));
   CU(cudaMemcpyAsync(dp, pv.data(), nsp * sizeof(TcProb), cudaMemcpyHostToDevice, st));
-  CU((launch_tc_gemm<4, 128, double, false, false>(mA, mB, dp, nsp, N, M,
+  CU((launch_tc_gemm<4, 128, double, false>(mA, mB, dp, nsp, N, M,
                                                    nsp == 1 ? (int)ldc : N, scale,
                                                    R.ctx->d_flag, nullptr, R.ctx->nsm, st,
                                                    tc_normal())));
@@ -2651,6 +2637,18 @@ int lno_ot_selftest_timeout(int device, long long wait_cycles, int* code, void* 
   int hflag = 0;
   CU(cudaMemcpyAsync(&hflag, flag, 4, cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));
+  if (hflag) {   // the same of the pair kernel: one tile, one pair
+    const PairTile t = pair_tile(S, N, 0);
+    TRY(make_operand_map(&mA[0], a16, K, M, S, (int64_t)M * K, 128, 2, S));
+    TRY(make_operand_map(&mB[0], b16, K, N, S, (int64_t)N * K, t.w / 2, 2, S));
+    mA[1] = mA[0];
+    mB[1] = mB[0];
+    CU(cudaMemsetAsync(flag, 0, 4, st));
+    CU((launch_tc_pair<S, kFmtBF16>(mA, mB, dp, 1, M, N, N, 1.0, flag, 2, st,
+                                    TcDiag{wait_cycles, 1}, TcOut{kOutRows, 0, 0, 0}, t)));
+    CU(cudaMemcpyAsync(&hflag, flag, 4, cudaMemcpyDeviceToHost, st));
+    CU(cudaStreamSynchronize(st));
+  }
   if (code) *code = hflag;
   return hflag ? LNO_OT_ETIMEOUT : LNO_OT_OK;
 }

@@ -188,59 +188,6 @@ __device__ __forceinline__ uint32_t idesc_mma(int neg, int n) {
          ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 
-// 16 consecutive floats of one output row; `left` columns remain in the row
-// (the rest of the 16 are not written).  16-byte aligned when left >= 16.
-__device__ __forceinline__ void store_row16(float* p, const uint32_t (&v)[16], int left) {
-  if (left >= 16) {
-    float4* p4 = reinterpret_cast<float4*>(p);
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      p4[q] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
-                          __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
-  } else {
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-      if (j < left) p[j] = __uint_as_float(v[j]);
-  }
-}
-
-// One 16-float row chunk (columns n0 .. n0+15 of output row m) of a
-// row-major launch, in the launch's output layout; `left` = columns remaining
-// in the row (only those are written).
-__device__ __forceinline__ void store_out16(float* out, const TcOut& lay, int ldo, int m, int n0,
-                                            const uint32_t (&v)[16], int left) {
-  if (lay.mode == kOutRows) {
-    store_row16(out + (int64_t)m * ldo + n0, v, left);
-  } else if (lay.mode == kOutYTile) {
-    const int b = m / lay.nvt, c = m - b * lay.nvt;
-    const int r = ((b & 15) << 4) | (c & 15), sw = (r >> 1) & 3;
-    float* row = out + ((int64_t)((b >> 4) * lay.nbt + (c >> 4)) * lay.nbs + (n0 >> 4)) * kTile +
-                 r * 16;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      float* d = row + ((q ^ sw) << 2);
-      if (left >= 4 * q + 4) {
-        *reinterpret_cast<float4*>(d) =
-            make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
-                        __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
-      } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (4 * q + j < left) d[j] = __uint_as_float(v[4 * q + j]);
-      }
-    }
-  } else {   // kOutZTile: m = pair(a, b) = b (b - 1) / 2 + a
-    int b = (int)((1.0 + sqrt(1.0 + 8.0 * (double)m)) * 0.5);
-    while ((int64_t)b * (b - 1) / 2 > m) --b;
-    while ((int64_t)(b + 1) * b / 2 <= m) ++b;
-    const int a = m - (int)((int64_t)b * (b - 1) / 2);
-    const int A = a >> 4, B = b >> 4;
-    const int r = ((a & 15) << 4) | (b & 15), slot = r ^ ((r >> 1) & 1);
-    store_row16(out + ((int64_t)(B * (B + 1) / 2 + A) * lay.nbt + (n0 >> 4)) * kTile + slot * 16,
-                v, left);
-  }
-}
-
 template <int S, int BN>
 struct Cfg {
   static constexpr int kABytes = BM * BK * 2;          // one slice of A
@@ -261,16 +208,14 @@ struct Cfg {
 // TF: TF32 slices (32-bit elements, 16 per 64-byte row, K 8 per MMA) instead
 // of BF16 ones (32 per row, K 16 per MMA); the shared-memory layout, the
 // descriptors and the MMAs per row are the same in bytes.
-// RM: row-major output out[m][n] (pitch ldo), n-tiles fastest; otherwise the
-// transposed out[n][m], m-tiles fastest.  The last n-tile's MMAs are only as
-// wide as its columns (rounded up to 16), so a narrow n costs little.
-template <int S, int BN, typename OutT, bool TF, bool RM>
+// Transposed output out[n][m], m-tiles fastest.  The last n-tile's MMAs are only
+// as wide as its columns (rounded up to 16), so a narrow n costs little.
+template <int S, int BN, typename OutT, bool TF>
 __global__ void __launch_bounds__(192, 1)
 tc_gemm_sliced(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
                const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
                const TcProb* __restrict__ probs, int nprob, int M, int N, int ldo, double scale,
-               int* __restrict__ flag, unsigned long long* __restrict__ amax, TcDiag diag,
-               TcOut lay) {
+               int* __restrict__ flag, unsigned long long* __restrict__ amax, TcDiag diag) {
   using C = Cfg<S, BN>;
   constexpr int BKE = TF ? BK / 2 : BK;   // elements per 64-byte row
   constexpr int KM = TF ? 8 : 16;         // K of one MMA
@@ -294,21 +239,13 @@ tc_gemm_sliced(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
   auto b_addr = [&](int st, int sl) {
     return smem_u32(smem + st * C::kStage + S * C::kABytes + sl * C::kBBytes);
   };
-  // unit -> (problem, m-tile, n-tile): m fastest (transposed output: the
-  // concurrent CTAs share one n-tile of B), n fastest for RM (they share one
-  // m-tile of A)
+  // unit -> (problem, m-tile, n-tile), m fastest (the concurrent CTAs share one
+  // n-tile of B)
   auto decode = [&](long long u, int& mt, int& nt, long long& pr) {
-    if constexpr (RM) {
-      nt = (int)(u % nN);
-      const long long r = u / nN;
-      mt = (int)(r % nM);
-      pr = r / nM;
-    } else {
-      mt = (int)(u % nM);
-      const long long r = u / nM;
-      nt = (int)(r % nN);
-      pr = r / nN;
-    }
+    mt = (int)(u % nM);
+    const long long r = u / nM;
+    nt = (int)(r % nN);
+    pr = r / nN;
   };
   // MMA width of n-tile nt: its columns rounded up to 16
   auto ntile_w = [&](int nt) { return min(BN, (N - nt * BN + 15) & ~15); };
@@ -486,53 +423,12 @@ tc_gemm_sliced(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
           tmem_ld16(spare + c * 16, v);
           tmem_ld_wait();
           const int n0 = nt * BN + c * 16;
-          if constexpr (RM) {
-            if (mok) store_out16(reinterpret_cast<float*>(out), lay, ldo, m, n0, v, N - n0);
-          } else {
-            OutT* op = out + (int64_t)n0 * ldo + m;
+          OutT* op = out + (int64_t)n0 * ldo + m;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const float x = __uint_as_float(v[j]);
-              if (mok && n0 + j < N) op[(int64_t)j * ldo] = x;
-              if (amax != nullptr && m < M && n0 + j < N) lmax = fmaxf(lmax, fabsf(x));
-            }
-          }
-        }
-      } else if constexpr (RM && BN <= 128) {
-        // the class accumulators fill TMEM: combine the whole row into
-        // registers, free TMEM for the next tile's MMAs, then store
-        static_assert(sizeof(OutT) == 4, "row-major output is float32");
-        const int nch = ntile_w(nt) / 16;
-        uint32_t v[BN];
-#pragma unroll
-        for (int c = 0; c < BN / 16; ++c) {
-          if (c < nch) {
-            uint32_t acc[S][16];
-#pragma unroll
-            for (int g = 0; g < S; ++g) tmem_ld16(tbase + g * BN + c * 16, acc[g]);
-            tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              float lo = 0.f;
-#pragma unroll
-              for (int g = S - 1; g >= 1; --g) lo = __fadd_rn(lo, __uint_as_float(acc[g][j]));
-              v[c * 16 + j] =
-                  __float_as_uint(__fmul_rn(__fadd_rn(__uint_as_float(acc[0][j]), lo), fscale));
-            }
-          }
-        }
-        tc_fence_before();
-        mbar_arrive(tempty);
-        if (mok) {
-#pragma unroll
-          for (int c = 0; c < BN / 16; ++c) {
-            if (c < nch) {
-              uint32_t w[16];
-#pragma unroll
-              for (int j = 0; j < 16; ++j) w[j] = v[c * 16 + j];
-              const int n0 = nt * BN + c * 16;
-              store_out16(reinterpret_cast<float*>(out), lay, ldo, m, n0, w, N - n0);
-            }
+          for (int j = 0; j < 16; ++j) {
+            const float x = __uint_as_float(v[j]);
+            if (mok && n0 + j < N) op[(int64_t)j * ldo] = x;
+            if (amax != nullptr && m < M && n0 + j < N) lmax = fmaxf(lmax, fabsf(x));
           }
         }
       } else {
@@ -544,19 +440,6 @@ tc_gemm_sliced(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
           for (int g = 0; g < S; ++g) tmem_ld16(tbase + g * BN + c * 16, acc[g]);
           tmem_ld_wait();
           const int n0 = nt * BN + c * 16;
-          if constexpr (RM) {
-            static_assert(sizeof(OutT) == 4, "row-major output is float32");
-            uint32_t v[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              float lo = 0.f;
-#pragma unroll
-              for (int g = S - 1; g >= 1; --g) lo = __fadd_rn(lo, __uint_as_float(acc[g][j]));
-              v[j] = __float_as_uint(__fmul_rn(__fadd_rn(__uint_as_float(acc[0][j]), lo), fscale));
-            }
-            if (mok) store_out16(reinterpret_cast<float*>(out), lay, ldo, m, n0, v, N - n0);
-            continue;
-          }
           OutT* op = out + (int64_t)n0 * ldo + m;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
@@ -629,9 +512,9 @@ static EncodeTiledFn get_encode() {
 
 // 3-D map over a sliced operand tensor: (k < Kp, row < rows, slice < S) of
 // esz-byte elements (2: BF16, 4: TF32 values stored as float).
-// Box: one 64-byte row of k x box_rows rows x 1 slice, 64-byte swizzle, zero fill.
+// Box: one 64-byte row of k x box_rows rows x box_slices slices, 64-byte swizzle, zero fill.
 int make_operand_map(CUtensorMap* map, const void* base, int64_t Kp, int64_t rows, int S,
-                     int64_t slice_stride, int box_rows, int esz) {
+                     int64_t slice_stride, int box_rows, int esz, int box_slices) {
   EncodeTiledFn enc = get_encode();
   if (!enc) return LNO_OT_ECUDA;
   if ((esz != 2 && esz != 4) || Kp % 8 || slice_stride % 8 ||
@@ -639,7 +522,7 @@ int make_operand_map(CUtensorMap* map, const void* base, int64_t Kp, int64_t row
     return LNO_OT_EINVAL;
   cuuint64_t dims[3] = {(cuuint64_t)Kp, (cuuint64_t)rows, (cuuint64_t)S};
   cuuint64_t strides[2] = {(cuuint64_t)(Kp * esz), (cuuint64_t)(slice_stride * esz)};
-  cuuint32_t box[3] = {(cuuint32_t)(64 / esz), (cuuint32_t)box_rows, 1};
+  cuuint32_t box[3] = {(cuuint32_t)(64 / esz), (cuuint32_t)box_rows, (cuuint32_t)box_slices};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = enc(map, esz == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                    3, const_cast<void*>(base), dims, strides, box, es,
@@ -649,25 +532,19 @@ int make_operand_map(CUtensorMap* map, const void* base, int64_t Kp, int64_t row
 }
 
 // mB must be maps with boxes of BN rows; mA boxes of 128 rows.
-template <int S, int BN, typename OutT, bool TF, bool RM>
+template <int S, int BN, typename OutT, bool TF>
 cudaError_t launch_tc_gemm(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs_dev,
                            int nprob, int M, int N, int ldo, double scale, int* flag,
-                           unsigned long long* amax, int nsm, cudaStream_t st, TcDiag diag,
-                           TcOut lay) {
+                           unsigned long long* amax, int nsm, cudaStream_t st, TcDiag diag) {
   using C = Cfg<S, BN>;
   if (nprob <= 0 || M <= 0 || N <= 0) return cudaSuccess;
-  if (RM && lay.mode == kOutRows && (ldo % 4 != 0 || ldo < ((N + 15) & ~15)))
-    return cudaErrorInvalidValue;
-  if (lay.mode != kOutRows &&
-      (!RM || lay.nbs < 1 || lay.nbt < 1 || (lay.mode == kOutYTile && lay.nvt < 1)))
-    return cudaErrorInvalidValue;
-  auto k = tc_gemm_sliced<S, BN, OutT, TF, RM>;
+  auto k = tc_gemm_sliced<S, BN, OutT, TF>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
   if (e != cudaSuccess) return e;
   const long long ntiles = (long long)nprob * ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
   const int grid = (int)(ntiles < nsm ? ntiles : nsm);
   k<<<grid, 192, C::kSmem, st>>>(mA[0], mA[1], mB[0], mB[1], probs_dev, nprob, M, N, ldo, scale,
-                                 flag, amax, diag, lay);
+                                 flag, amax, diag);
   return cudaGetLastError();
 }
 
@@ -682,38 +559,26 @@ cudaError_t launch_sliced_product(int S, const CUtensorMap* mA, const CUtensorMa
                                   const TcProb* dp, int M, int N, double scale, int* flag,
                                   int nsm, cudaStream_t st, TcDiag dg) {
   switch (S) {
-    case 1: return launch_tc_gemm<1, 256, double, false, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
-    case 2: return launch_tc_gemm<2, 256, double, false, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
-    case 3: return launch_tc_gemm<3, 128, double, false, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
-    case 4: return launch_tc_gemm<4, 128, double, false, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
-    case 5: return launch_tc_gemm<5, 64, double, false, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
+    case 1: return launch_tc_gemm<1, 256, double, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
+    case 2: return launch_tc_gemm<2, 256, double, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
+    case 3: return launch_tc_gemm<3, 128, double, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
+    case 4: return launch_tc_gemm<4, 128, double, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
+    case 5: return launch_tc_gemm<5, 64, double, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
     default: return cudaErrorInvalidValue;
   }
 }
 long long tc_default_wait_cycles() { return kWaitCycles; }
 
-#define LNO_TC_INST(S, BN, T, TF, RM)                                                        \
-  template cudaError_t launch_tc_gemm<S, BN, T, TF, RM>(                                     \
+#define LNO_TC_INST(S, BN, T, TF)                                                            \
+  template cudaError_t launch_tc_gemm<S, BN, T, TF>(                                         \
       const CUtensorMap*, const CUtensorMap*, const TcProb*, int, int, int, int, double, int*, \
-      unsigned long long*, int, cudaStream_t, TcDiag, TcOut);
-// W contractions (float32 row-major output): slices x tile width
-LNO_TC_INST(2, 256, float, false, true)
-LNO_TC_INST(2, 128, float, false, true)
-LNO_TC_INST(3, 128, float, false, true)
-LNO_TC_INST(3, 64, float, false, true)
-LNO_TC_INST(4, 128, float, false, true)
-LNO_TC_INST(4, 96, float, false, true)
-LNO_TC_INST(4, 64, float, false, true)
-LNO_TC_INST(5, 64, float, false, true)
-// TF32 W contractions (2 TF32 slices, 3 products)
-LNO_TC_INST(2, 256, float, true, true)
-LNO_TC_INST(2, 128, float, true, true)
+      unsigned long long*, int, cudaStream_t, TcDiag);
 // DF assembly and the diagnostics (float64 transposed output)
-LNO_TC_INST(1, 256, double, false, false)
-LNO_TC_INST(2, 256, double, false, false)
-LNO_TC_INST(3, 128, double, false, false)
-LNO_TC_INST(4, 128, double, false, false)
-LNO_TC_INST(5, 64, double, false, false)
+LNO_TC_INST(1, 256, double, false)
+LNO_TC_INST(2, 256, double, false)
+LNO_TC_INST(3, 128, double, false)
+LNO_TC_INST(4, 128, double, false)
+LNO_TC_INST(5, 64, double, false)
 #undef LNO_TC_INST
 
 }  // namespace lno

@@ -1,0 +1,61 @@
+"""W contraction on CTA pairs (csrc/tc_pair.cu) at the edges of its tiles.
+
+Per-triplet energies of a few triplets per case against the float64 path of
+the library (itself pinned to the oracle elsewhere), for virtual counts around
+one and two n-tiles of each slice count, row counts around 256-row tiles, k
+lengths around the 32-element blocks, and tuned tile caps.
+
+Tolerances: the slices of a precision with S slices of 8 bits leave 2^(-8 S)
+of the largest operand product per term, and the float32 rounding of the W
+intermediates and of the energy sums leaves ~1e-9 of a triplet's energy for
+the smallest virtual spaces here; 16 (S = 2), 24 (S = 3) and >= 32 bits give
+1e-3, 1e-6 and 2e-8 relative to the largest triplet energy with a margin of at
+least 4 over the worst per-triplet errors the larger suites see."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2311_10048_gb300 import lno_ot
+from paper_2311_10048_gb300.synth import make_domain
+
+pytestmark = pytest.mark.gpu
+TOL = {"bf16x3": 1e-3, "tf32": 1e-3, "bf16x6": 1e-6, "bf16x10": 2e-8, "bf16x15": 2e-8}
+
+
+def e_trips(prec, dd, sel, tune=None):
+    ctx = lno_ot.Context(0, prec, tune_cache=tune)
+    et = [torch.zeros(max(x.size, 1), dtype=torch.float64, device="cuda") for x in sel]
+    ctx.energy(dd, e_trip=et, trip_sel=sel)
+    ctx.close()
+    return np.concatenate([e[:x.size].cpu().numpy() for e, x in zip(et, sel)])
+
+
+def sample(na, nb):
+    n = [na * (na - 1) * (na - 2) // 6, na * (na - 1) // 2 * nb, nb * (nb - 1) // 2 * na,
+         nb * (nb - 1) * (nb - 2) // 6]
+    return [np.unique(np.array([0, x // 2, x - 1]) if x else np.zeros(0)).astype(np.int64)
+            for x in n]
+
+
+@pytest.mark.parametrize("v,na,nb", [(15, 4, 3), (16, 4, 4), (23, 5, 4), (33, 3, 3), (65, 4, 3),
+                                     (80, 3, 3), (81, 4, 3), (97, 5, 3), (128, 4, 3),
+                                     (129, 3, 3), (160, 4, 4), (161, 3, 3), (257, 3, 3)])
+def test_tile_edges(v, na, nb):
+    d = make_domain(v + na, (na, nb), naux=v + na + 5, L=(v + na) / 3, seed=100 + v, t1_sd=0.02)
+    dd = lno_ot.to_device(d)
+    sel = sample(na, nb)
+    ref = e_trips("fp64", dd, sel)
+    for prec, tol in TOL.items():
+        got = e_trips(prec, dd, sel)
+        assert np.abs(got - ref).max() <= tol * np.abs(ref).max(), prec
+
+
+@pytest.mark.parametrize("cap", [16, 48, 80])
+def test_tile_caps_are_bitwise_equal(tmp_path, cap):
+    d = make_domain(101, (4, 3), naux=90, L=30.0, seed=9, t1_sd=0.02)
+    dd = lno_ot.to_device(d)
+    sel = sample(4, 3)
+    p = tmp_path / "t.txt"
+    p.write_text(f"100000 {cap} 3\n")
+    for prec in ("bf16x3", "bf16x6", "bf16x10", "bf16x15"):
+        assert np.array_equal(e_trips(prec, dd, sel, str(p)), e_trips(prec, dd, sel)), prec
