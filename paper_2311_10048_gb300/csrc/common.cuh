@@ -204,6 +204,10 @@ template <int S, int FMT>
 cudaError_t launch_tc_pair(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs_dev,
                            int nprob, int M, int N, int ldo, double scale, int* flag, int nsm,
                            cudaStream_t st, TcDiag diag, TcOut lay, PairTile tile);
+template <int S, int FMT>
+cudaError_t launch_tc_pair_f64(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb& p,
+                               int M, int N, int ldo, double scale, int* flag,
+                               unsigned long long* amax, int nsm, cudaStream_t st, PairTile tile);
 int sliced_product_bn(int S);
 cudaError_t launch_sliced_product(int S, const CUtensorMap* mA, const CUtensorMap* mB,
                                   const TcProb* dp, int M, int N, double scale, int* flag,
@@ -230,52 +234,126 @@ int laplace_quadrature(double xmin, double xmax, double tol, int nmax, double* s
 
 // Operand stores used by the layout kernels.  `part` says whether the value
 // is an amplitude (0) or an integral (1): the two have separate scales.
+// store16 writes 16 consecutive elements (idx a multiple of 16, rows starting
+// on 32-byte boundaries); bit j of `parts` is the part of element j.
 struct StoreF64 {
   double* p;
   __device__ __forceinline__ void operator()(int64_t idx, double v, int) const { p[idx] = v; }
+  __device__ __forceinline__ void store16(int64_t idx, const double (&v)[16], uint32_t) const {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) p[idx + j] = v[j];
+  }
 };
 
-// Exact BF16 slices: value = scale 2^-7 (s_0 + ... + s_{S-1}), s_0 an integer
-// in [-128,128], s_q a multiple of 2^(-8q) with |s_q| <= 2^(-8q+7), every
-// step rounded to nearest (ties to even) in float64.
+// round(v 2^e2) to nearest (ties to even) from the bits of v, in integer
+// arithmetic (this GPU's float64 rate is 1/64 of its float32 rate); |v 2^e2|
+// must stay below 2^62, v finite.
+__device__ __forceinline__ int64_t round_scaled(double v, int e2) {
+  const uint64_t b = (uint64_t)__double_as_longlong(v);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  uint64_t m = b & ((1ull << 52) - 1);
+  if (ex != 0) m |= 1ull << 52;
+  const int sh = (ex == 0 ? 1 : ex) - 1075 + e2;   // |v| 2^e2 = m 2^sh
+  uint64_t q;
+  if (m == 0) {
+    q = 0;
+  } else if (sh >= 0) {
+    q = m << sh;
+  } else if (-sh > 54) {
+    q = 0;                                        // m 2^sh < 1/2
+  } else {
+    const int r = -sh;
+    const uint64_t rem = m & ((1ull << r) - 1), half = 1ull << (r - 1);
+    q = m >> r;
+    if (rem > half || (rem == half && (q & 1))) ++q;
+  }
+  return (b >> 63) ? -(int64_t)q : (int64_t)q;
+}
+
+// Exact slices of S digits of BITS bits: value = 2^-e (s_0 + ... + s_{S-1}),
+// s_q an integer multiple of 2^(-BITS q), |s_0| <= 2^(BITS - 1) (2^BITS / 2, the
+// scale's choice), |s_q| 2^(BITS q) <= 2^(BITS - 1) below it, each digit the
+// nearest one to what is left.  Integer arithmetic throughout: the value is
+// rounded once, 16 bits below the last digit, and cut into digits from the top
+// (float64 rounding steps of every digit made the layout kernels 10-20x slower
+// than their memory traffic).  A value that is not finite, or too large for the
+// scale, becomes NaN.
+template <int S, int BITS>
+__device__ __forceinline__ void slice_digits(double v, int e, float (&f)[S]) {
+  constexpr int kX = 16;
+  const int ex = (int)(((uint64_t)__double_as_longlong(v) >> 52) & 0x7ff);
+  if (ex == 0x7ff || ex - 1023 + e > 60 - (BITS * (S - 1) + kX)) {
+    f[0] = __int_as_float(0x7fc00000);
+#pragma unroll
+    for (int q = 1; q < S; ++q) f[q] = 0.f;
+    return;
+  }
+  int64_t R = round_scaled(v, e + BITS * (S - 1) + kX);
+  float w = 1.0f;
+#pragma unroll
+  for (int q = 0; q < S; ++q) {
+    const int sh = BITS * (S - 1 - q) + kX;
+    const int64_t d = (R + (1ll << (sh - 1))) >> sh;
+    R -= d << sh;
+    f[q] = (float)(int)d * w;   // exact
+    w *= 1.0f / (float)(1 << BITS);
+  }
+}
+
+// BF16 slices: value = scale 2^-7 (s_0 + ... + s_{S-1}), s_0 an integer in
+// [-128,128], s_q a multiple of 2^(-8q).
 template <int S>
 struct StoreSlices {
   __nv_bfloat16* p;
   int64_t slice_stride;  // elements between slices
-  double inv_t;          // 2^7 / amplitude scale
-  double inv_i;          // 2^7 / integral scale
+  int e_t, e_i;          // log2(2^7 / scale) of amplitudes and of integrals
   __device__ __forceinline__ void operator()(int64_t idx, double v, int part) const {
-    double x = v * (part ? inv_i : inv_t);
-    double w = 1.0;
+    float f[S];
+    slice_digits<S, 8>(v, part ? e_i : e_t, f);
+#pragma unroll
+    for (int s = 0; s < S; ++s) p[s * slice_stride + idx] = __float2bfloat16_rn(f[s]);
+  }
+  __device__ __forceinline__ void store16(int64_t idx, const double (&v)[16],
+                                          uint32_t parts) const {
+    uint32_t w[S][8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float a[S], b[S];
+      slice_digits<S, 8>(v[2 * j], (parts >> (2 * j)) & 1 ? e_i : e_t, a);
+      slice_digits<S, 8>(v[2 * j + 1], (parts >> (2 * j + 1)) & 1 ? e_i : e_t, b);
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        const __nv_bfloat162 x = __floats2bfloat162_rn(a[s], b[s]);
+        w[s][j] = *reinterpret_cast<const uint32_t*>(&x);
+      }
+    }
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      double q = rint(x * w) / w;   // w = 2^(8s): exact scaling
-      x -= q;                        // exact
-      p[s * slice_stride + idx] = __double2bfloat16(q);
-      w *= 256.0;
+      uint4* d = reinterpret_cast<uint4*>(p + s * slice_stride + idx);
+      d[0] = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+      d[1] = make_uint4(w[s][4], w[s][5], w[s][6], w[s][7]);
     }
   }
 };
 
-// Exact TF32 slices (stored as float): value = scale 2^-10 (s_0 + ... +
-// s_{S-1}), s_0 an integer in [-1024, 1024], s_q a multiple of 2^(-11q): 11
-// significant bits each, what one TF32 operand holds.
+// TF32 slices (stored as float): value = scale 2^-10 (s_0 + ... + s_{S-1}), s_0
+// an integer in [-1024, 1024], s_q a multiple of 2^(-11q): 11 significant bits
+// each, what one TF32 operand holds.
 template <int S>
 struct StoreTF32 {
   float* p;
   int64_t slice_stride;
-  double inv_t;          // 2^10 / amplitude scale
-  double inv_i;          // 2^10 / integral scale
+  int e_t, e_i;          // log2(2^10 / scale) of amplitudes and of integrals
   __device__ __forceinline__ void operator()(int64_t idx, double v, int part) const {
-    double x = v * (part ? inv_i : inv_t);
-    double w = 1.0;
+    float f[S];
+    slice_digits<S, 11>(v, part ? e_i : e_t, f);
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      double q = rint(x * w) / w;   // w = 2^(11s): exact scaling
-      x -= q;
-      p[s * slice_stride + idx] = (float)q;
-      w *= 2048.0;
-    }
+    for (int s = 0; s < S; ++s) p[s * slice_stride + idx] = f[s];
+  }
+  __device__ __forceinline__ void store16(int64_t idx, const double (&v)[16],
+                                          uint32_t parts) const {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) (*this)(idx + j, v[j], (parts >> j) & 1);
   }
 };
 

@@ -53,17 +53,17 @@ template <class St>
 cudaError_t launch_pack_at_same(const int2*, int, int, int, int, int, const double*, const double*,
                                 St, cudaStream_t);
 template <class St>
-cudaError_t launch_pack_bt_same(int, int, int, int, int, int, const double*, const double*, St,
-                                cudaStream_t);
+cudaError_t launch_pack_bt_same(int, int, int, int, int, int, int, const double*, const double*,
+                                St, cudaStream_t);
 template <class St>
 cudaError_t launch_pack_a1(const int2*, int, int, int, int, int, int, int, const double*,
                            const double*, St, cudaStream_t);
 template <class St>
-cudaError_t launch_pack_bg(int, int, int, int, int, int, int, int, const double*, const double*,
-                           St, cudaStream_t);
+cudaError_t launch_pack_bg(int, int, int, int, int, int, int, int, int, const double*,
+                           const double*, St, cudaStream_t);
 template <class St>
-cudaError_t launch_pack_bf(int, int, int, int, int, int, int, int, const double*, const double*,
-                           St, cudaStream_t);
+cudaError_t launch_pack_bf(int, int, int, int, int, int, int, int, int, const double*,
+                           const double*, St, cudaStream_t);
 template <class St>
 cudaError_t launch_pack_at2(const int2*, int, int, int, int, int, int, int, const double*,
                             const double*, St, cudaStream_t);
@@ -162,12 +162,14 @@ struct lno_ot_ctx {
       if (v <= r.vmax) return &r;
     return tune.empty() ? nullptr : &tune.back();
   }
-  int* d_flag = nullptr;               // device error flag (bounded waits)
-  unsigned long long* d_amax = nullptr;
-  double* d_sums = nullptr;            // [8]
+  // one device block (CallState), read back in one copy at the end of a call
+  double* d_sums = nullptr;                 // [4] per-case sums
+  unsigned long long* d_amax = nullptr;     // [4] magnitudes (bits of doubles)
+  int* d_flag = nullptr;                    // error flag (bounded waits)
   lno_ot_stats stats{};
   std::vector<cudaEvent_t> ev_pool;
   size_t ev_used = 0;
+  bool exact_measure = false;          // integral scale from every slice (measure_sigI)
   // prepared operands of the last domain (options.keep_operands)
   bool keep = false;
   struct DomainCache* cache = nullptr;
@@ -176,6 +178,16 @@ struct lno_ot_ctx {
 void destroy_cache(DomainCache* c);
 
 namespace {
+
+// Device state of a call: per-case sums, magnitudes (0, 1 scratch, 2 the largest
+// DF integral assembled with the current scale), error flag.
+struct CallState {
+  double sums[4];
+  unsigned long long amax[4];
+  int flag;
+};
+
+constexpr int kRescale = 1;   // internal: the call has to run again (scale_too_small)
 
 #define TRY(expr)                       \
   do {                                  \
@@ -251,12 +263,13 @@ struct Operand {
   int esz = 2;                   // bytes per slice element
   int S = 0;
   int64_t slice_stride = 0;
-  CUtensorMap map128, map64;  // TMA maps of one slice, boxes of 128 and 64 rows (tc_gemm.cu)
   int64_t total_rows() const { return (int64_t)nslot * rows; }
-  // TMA map of the pair kernel: boxes of box_rows rows x all slices
-  int pair_map(CUtensorMap* m, int box_rows) const {
+  // TMA map of the pair kernel: boxes of box_rows rows x the first ns slices
+  // (0: all)
+  int pair_map(CUtensorMap* m, int box_rows, int ns = 0) const {
     return make_operand_map(m, esz == 4 ? (const void*)f32 : (const void*)bf, Kp,
-                            std::max<int64_t>(total_rows(), 1), S, slice_stride, box_rows, esz, S);
+                            std::max<int64_t>(total_rows(), 1), S, slice_stride, box_rows, esz,
+                            ns > 0 ? ns : S);
   }
 };
 
@@ -320,7 +333,8 @@ struct Run {
   int Sdf = 4;        // slices of the DF factors
   double sigT = 1, sigI = 1, sigB = 1;
   bool amax_pass = false;  // true while measuring integral magnitudes
-  double amax_int = 0.0;
+  bool amax_exact = false; // ... with every slice of the factors
+  bool track_amax = false; // while building the operands: their largest integral
   int nbas, naux, no[2], nv[2];
   // orbitals per spin: nbas, or nbas + P for a spin that carries P central
   // pseudo-orbitals (set before stage(); 0 = nbas)
@@ -361,26 +375,20 @@ struct Run {
     op.K = K;
     // sliced rows start on 64-byte boundaries: the contractions' 64-byte box
     // rows then are two sectors of L2 (1.3x fewer bytes than at 16-byte pitches)
-    op.Kp = (int)round_up(std::max(K, 1), f64 ? 8 : tf ? 16 : 32);
+    op.Kp = (int)round_up(std::max(K, 1), f64 || tf ? 16 : 32);
     op.S = f64 ? 0 : S_;
     const int64_t n = std::max<int64_t>((int64_t)nslot * rows * op.Kp, 8);
     if (f64) {
       TRY(ar.get(&op.f64, (size_t)n));
     } else {
       op.slice_stride = round_up(n, 8);
-      void* base;
       if (tf) {
         op.esz = 4;
         TRY(ar.get(&op.f32, (size_t)(op.slice_stride * op.S)));
-        base = op.f32;
       } else {
         op.esz = 2;
         TRY(ar.get(&op.bf, (size_t)(op.slice_stride * op.S)));
-        base = op.bf;
       }
-      const int64_t rows_ = std::max<int64_t>(op.total_rows(), 1);
-      TRY(make_operand_map(&op.map128, base, op.Kp, rows_, op.S, op.slice_stride, 128, op.esz));
-      TRY(make_operand_map(&op.map64, base, op.Kp, rows_, op.S, op.slice_stride, 64, op.esz));
     }
     return LNO_OT_OK;
   }
@@ -388,10 +396,10 @@ struct Run {
   // Store functor for an operand (amplitude scale sigT, integral scale sigI).
   template <int SS>
   StoreSlices<SS> slices(const Operand& op) const {
-    return StoreSlices<SS>{op.bf, op.slice_stride, 128.0 / sigT, 128.0 / sigI};
+    return StoreSlices<SS>{op.bf, op.slice_stride, 7 - std::ilogb(sigT), 7 - std::ilogb(sigI)};
   }
   StoreTF32<2> tf32_slices(const Operand& op) const {
-    return StoreTF32<2>{op.f32, op.slice_stride, 1024.0 / sigT, 1024.0 / sigI};
+    return StoreTF32<2>{op.f32, op.slice_stride, 10 - std::ilogb(sigT), 10 - std::ilogb(sigI)};
   }
 
   // ---- DF integrals: out[n][m] = sum_Q L[m][Q] R[n][Q] (float64) ------------
@@ -418,20 +426,24 @@ struct Run {
     p.nseg = 1;
     p.seg[0] = TcSeg{0, 0, (int)l0, (int)r0, naux, 0};
     p.out = amax_pass ? nullptr : out;
-    TcProb* dp;
-    TRY(arena.get(&dp, 1));
-    CU(cudaMemcpyAsync(dp, &p, sizeof p, cudaMemcpyHostToDevice, st));
     const double scale = sigB * sigB * std::ldexp(1.0, -14);
-    unsigned long long* am = amax_pass ? ctx->d_amax : nullptr;
-    if (Sdf == 5) {
-      CUtensorMap mA[2] = {Lo.map128, Lo.map128}, mB[2] = {Ro.map64, Ro.map64};
-      CU(launch_tc_gemm<5, 64, double>(mA, mB, dp, 1, M, N, ldo, scale, ctx->d_flag, am,
-                                       ctx->nsm, st, tc_normal()));
-    } else {
-      CUtensorMap mA[2] = {Lo.map128, Lo.map128}, mB[2] = {Ro.map128, Ro.map128};
-      CU(launch_tc_gemm<4, 128, double>(mA, mB, dp, 1, M, N, ldo, scale, ctx->d_flag, am,
-                                        ctx->nsm, st, tc_normal()));
-    }
+    // the measuring pass takes the two leading slices of each factor (3 of the 10
+    // products) unless that leaves the scale open (measure_sigI)
+    const int ns = amax_pass && !amax_exact ? 2 : Sdf;
+    unsigned long long* am = amax_pass ? ctx->d_amax : track_amax ? ctx->d_amax + 2 : nullptr;
+    const PairTile t = pair_tile(ns, N, 128);
+    CUtensorMap mA[2], mB[2];
+    TRY(Lo.pair_map(&mA[0], 128, ns));
+    TRY(Ro.pair_map(&mB[0], t.w / 2, ns));
+    mA[1] = mA[0];
+    mB[1] = mB[0];
+#define LNO_DF(SS)                                                                            \
+  CU((launch_tc_pair_f64<SS, kFmtBF16>(mA, mB, p, M, N, ldo, scale, ctx->d_flag,               \
+                                       am, ctx->nsm, st, t)))
+    if (ns == 2) LNO_DF(2);
+    else if (ns == 5) LNO_DF(5);
+    else LNO_DF(4);
+#undef LNO_DF
     return LNO_OT_OK;
   }
 
@@ -487,6 +499,7 @@ struct Run {
         Operand* op;
         int p0, np, q0, nq;
       } blks[3] = {{&Boo[s], 0, oi, 0, o}, {&Bov[s], 0, o, o, v}, {&Bvv[s], o, v, o, v}};
+      const int eB = 7 - std::ilogb(sigB);
       for (auto& b : blks) {
         stats->other_launches++;
         if (f64)
@@ -495,11 +508,11 @@ struct Run {
         else if (Sdf == 5)
           CU(launch_transpose_block(
               dom->B[s], naux, nbs[s], b.p0, b.np, b.q0, b.nq, b.op->Kp,
-              StoreSlices<5>{b.op->bf, b.op->slice_stride, 128.0 / sigB, 128.0 / sigB}, st));
+              StoreSlices<5>{b.op->bf, b.op->slice_stride, eB, eB}, st));
         else
           CU(launch_transpose_block(
               dom->B[s], naux, nbs[s], b.p0, b.np, b.q0, b.nq, b.op->Kp,
-              StoreSlices<4>{b.op->bf, b.op->slice_stride, 128.0 / sigB, 128.0 / sigB}, st));
+              StoreSlices<4>{b.op->bf, b.op->slice_stride, eB, eB}, st));
       }
     }
     return LNO_OT_OK;
@@ -686,94 +699,120 @@ struct SpinPass {
     }
   }
 
+  // Runs of consecutive orbitals in a slot list: slots [q, q + n) hold orbitals
+  // x, x + 1, ...; the DF blocks of a run come from one launch (their rows are
+  // consecutive) and are laid out by one.  A run's float64 blocks stay within
+  // kRunBytes, except a single block that is larger.
+  struct OrbRun {
+    int q, x, n;
+  };
+  static constexpr int64_t kRunBytes = (int64_t)512 << 20;
+  static std::vector<OrbRun> orb_runs(const std::vector<int>& list, int64_t block_elems) {
+    const int cap = (int)std::max<int64_t>(
+        1, std::min<int64_t>(65535, kRunBytes / 8 / std::max<int64_t>(block_elems, 1)));
+    std::vector<OrbRun> runs;
+    for (size_t q = 0; q < list.size(); ++q) {
+      if (!runs.empty() && runs.back().n < cap && runs.back().x + runs.back().n == list[q])
+        runs.back().n++;
+      else
+        runs.push_back({(int)q, list[q], 1});
+    }
+    return runs;
+  }
+  static int longest(const std::vector<OrbRun>& runs) {
+    int n = 0;
+    for (const OrbRun& r : runs) n = std::max(n, r.n);
+    return n;
+  }
+
   template <class St>
   int pack_all(St stAT, St stBT, St stA1, St stBG, St stBF, St stAT2) {
     Arena& A = own;
     cudaStream_t st = R.st;
+    const bool meas = R.amax_pass;   // magnitudes only: no blocks, no layout
+    R.track_amax = !meas;
+    auto block = [&](double** p, int64_t n) -> int {
+      *p = nullptr;
+      return meas ? LNO_OT_OK : A.get(p, (size_t)n);
+    };
+    auto drop = [&](double* p) {
+      if (p) A.drop(p);
+    };
+    // pair operands: one DF block, one layout launch
+    auto upload_pairs = [&](const std::vector<int2>& l, int2** dl) -> int {
+      TRY(A.get(dl, l.size()));
+      CU(cudaMemcpyAsync(*dl, l.data(), l.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
+      R.stats->other_launches++;
+      return LNO_OT_OK;
+    };
+    // per-orbital operands: the blocks (L rows x [x][r_rows]) of a run at a time
+    auto per_orbital = [&](const std::vector<int>& list, const Operand& L, int64_t l_rows,
+                           const Operand& Ro, int r_rows, auto&& pack) -> int {
+      const auto runs = orb_runs(list, l_rows * r_rows);
+      double* buf;
+      TRY(block(&buf, l_rows * r_rows * longest(runs)));
+      for (const OrbRun& r : runs) {
+        TRY(R.df(L, 0, (int)l_rows, Ro, (int64_t)r.x * r_rows, r.n * r_rows, buf, (int)l_rows));
+        if (!meas) {
+          R.stats->other_launches++;
+          CU(pack(r, buf));
+        }
+      }
+      drop(buf);
+      return LNO_OT_OK;
+    };
     // ---- same-spin operands -------------------------------------------------
     if (!listAT.empty()) {
       double* oovoT;
-      TRY(A.get(&oovoT, (size_t)o * v * oi * o));
+      TRY(block(&oovoT, (int64_t)o * v * oi * o));
       TRY(R.df(R.Boo[s], 0, oi * o, R.Bov[s], 0, o * v, oovoT, oi * o));
-      if (!R.amax_pass) {
+      if (!meas) {
         int2* dl;
-        TRY(A.get(&dl, listAT.size()));
-        CU(cudaMemcpyAsync(dl, listAT.data(), listAT.size() * sizeof(int2),
-                           cudaMemcpyHostToDevice, st));
-        R.stats->other_launches++;
+        TRY(upload_pairs(listAT, &dl));
         CU(launch_pack_at_same(dl, (int)listAT.size(), o, oi, v, AT.Kp, t2ss, oovoT, stAT, st));
       }
-      A.drop(oovoT);
+      drop(oovoT);
     }
-    if (!listBT.empty()) {
-      double* vvovT;
-      TRY(A.get(&vvovT, (size_t)v * v * v));
-      for (size_t q = 0; q < listBT.size(); ++q) {
-        const int x = listBT[q];
-        TRY(R.df(R.Bvv[s], 0, v * v, R.Bov[s], (int64_t)x * v, v, vvovT, v * v));
-        if (!R.amax_pass) {
-          R.stats->other_launches++;
-          CU(launch_pack_bt_same((int)q, x, o, oi, v, BT.Kp, vvovT, t2ss, stBT, st));
-        }
-      }
-      A.drop(vvovT);
-    }
+    TRY(per_orbital(listBT, R.Bvv[s], (int64_t)v * v, R.Bov[s], v,
+                    [&](const OrbRun& r, const double* b) {
+                      return launch_pack_bt_same(r.q, r.x, r.n, o, oi, v, BT.Kp, b, t2ss, stBT,
+                                                 st);
+                    }));
     // ---- mixed operands -----------------------------------------------------
     if (!listA1.empty()) {
       double* jT;
-      TRY(A.get(&jT, (size_t)o * v * oti * ot));
+      TRY(block(&jT, (int64_t)o * v * oti * ot));
       TRY(R.df(R.Bov[s], 0, o * v, R.Boo[t], 0, oti * ot, jT, o * v));
-      if (!R.amax_pass) {
+      if (!meas) {
         int2* dl;
-        TRY(A.get(&dl, listA1.size()));
-        CU(cudaMemcpyAsync(dl, listA1.data(), listA1.size() * sizeof(int2),
-                           cudaMemcpyHostToDevice, st));
-        R.stats->other_launches++;
+        TRY(upload_pairs(listA1, &dl));
         CU(launch_pack_a1(dl, (int)listA1.size(), o, v, ot, oti, vt, A1.Kp, t2st, jT, stA1, st));
       }
-      A.drop(jT);
+      drop(jT);
     }
-    if (!listBG.empty()) {
-      double* gT;
-      TRY(A.get(&gT, (size_t)v * vt * vt));
-      for (size_t q = 0; q < listBG.size(); ++q) {
-        const int x = listBG[q];
-        TRY(R.df(R.Bvv[t], 0, vt * vt, R.Bov[s], (int64_t)x * v, v, gT, vt * vt));
-        if (!R.amax_pass) {
-          R.stats->other_launches++;
-          CU(launch_pack_bg((int)q, x, o, v, ot, oti, vt, BG.Kp, gT, t2st, stBG, st));
-        }
-      }
-      A.drop(gT);
-    }
-    if (!listBF.empty()) {
-      double* fT;
-      TRY(A.get(&fT, (size_t)vt * v * v));
-      for (size_t q = 0; q < listBF.size(); ++q) {
-        const int K = listBF[q];
-        TRY(R.df(R.Bvv[s], 0, v * v, R.Bov[t], (int64_t)K * vt, vt, fT, v * v));
-        if (!R.amax_pass) {
-          R.stats->other_launches++;
-          CU(launch_pack_bf((int)q, K, o, oi, v, ot, vt, BF.Kp, fT, t2st, stBF, st));
-        }
-      }
-      A.drop(fT);
-    }
+    TRY(per_orbital(listBG, R.Bvv[t], (int64_t)vt * vt, R.Bov[s], v,
+                    [&](const OrbRun& r, const double* b) {
+                      return launch_pack_bg(r.q, r.x, r.n, o, v, ot, oti, vt, BG.Kp, b, t2st,
+                                            stBG, st);
+                    }));
+    TRY(per_orbital(listBF, R.Bvv[s], (int64_t)v * v, R.Bov[t], vt,
+                    [&](const OrbRun& r, const double* b) {
+                      return launch_pack_bf(r.q, r.x, r.n, o, oi, v, ot, vt, BF.Kp, b, t2st, stBF,
+                                            st);
+                    }));
     if (!listAT2.empty()) {
       double* lT;
-      TRY(A.get(&lT, (size_t)ot * vt * oi * o));
+      TRY(block(&lT, (int64_t)ot * vt * oi * o));
       TRY(R.df(R.Boo[s], 0, oi * o, R.Bov[t], 0, ot * vt, lT, oi * o));
-      if (!R.amax_pass) {
+      if (!meas) {
         int2* dl;
-        TRY(A.get(&dl, listAT2.size()));
-        CU(cudaMemcpyAsync(dl, listAT2.data(), listAT2.size() * sizeof(int2),
-                           cudaMemcpyHostToDevice, st));
-        R.stats->other_launches++;
+        TRY(upload_pairs(listAT2, &dl));
         CU(launch_pack_at2(dl, (int)listAT2.size(), o, oi, v, ot, vt, AT2.Kp, t2st, lT, stAT2,
                            st));
       }
-      A.drop(lT);
+      drop(lT);
     }
+    R.track_amax = false;
     return LNO_OT_OK;
   }
 
@@ -939,8 +978,8 @@ struct SpinPass {
     char *X = nullptr, *Z = nullptr;
     TRY(A.get(&X, (size_t)(G * xs * esz) + 64));
     if (is_mixed) TRY(A.get(&Z, (size_t)(G * zs * esz) + 64));
-    CU(cudaMemsetAsync(X, 0, (size_t)(G * xs * esz), R.st));
-    if (is_mixed) CU(cudaMemsetAsync(Z, 0, (size_t)(G * zs * esz), R.st));
+    // (the pads of rows and tiles stay unwritten: the energy kernels select the
+    // restricted elements, so no pad reaches a sum)
     // cube tiles
     std::vector<int3> blocks;
     if (!is_mixed) {
@@ -1224,10 +1263,20 @@ int validate(const lno_ot_ctx* ctx, const lno_ot_domain* d) {
   return LNO_OT_OK;
 }
 
+// Whether the blocks built with this scale hold larger integrals than it
+// allows (d_amax[2], collected by the assembly; its rounding to float32 is the
+// measuring pass's).
+bool scale_too_small(const Run& R, unsigned long long built) {
+  if (R.f64) return false;
+  double m;
+  std::memcpy(&m, &built, 8);
+  return std::isfinite(m) && 2.0 * m > R.sigI;
+}
+
 // Per-case sums, per-triplet and orbital outputs, results and stats of one
 // call (after the spin passes have filled e_int).
 int finish_call(lno_ot_ctx* ctx, Run& R, Arena& A, const lno_ot_domain* dom, const CaseSel* cs,
-                double* const* e_int, bool thirds, cudaEvent_t t0, cudaEvent_t t1,
+                double* const* e_int, bool thirds, bool kept, cudaEvent_t t0, cudaEvent_t t1,
                 cudaEvent_t t2, lno_ot_result* out) {
   // per-case sums
   for (int c = 0; c < 4; ++c) {
@@ -1262,13 +1311,13 @@ int finish_call(lno_ot_ctx* ctx, Run& R, Arena& A, const lno_ot_domain* dom, con
     CU(launch_orbital_partition(oa, R.st));
     R.stats->other_launches++;
   }
-  double hs[4];
-  CU(cudaMemcpyAsync(hs, ctx->d_sums, sizeof hs, cudaMemcpyDeviceToHost, R.st));
+  CallState h;
+  CU(cudaMemcpyAsync(&h, ctx->d_sums, sizeof h, cudaMemcpyDeviceToHost, R.st));
   if (t2) cudaEventRecord(t2, R.st);
   CU(cudaStreamSynchronize(R.st));
-  int flag = 0;
-  CU(cudaMemcpy(&flag, ctx->d_flag, sizeof flag, cudaMemcpyDeviceToHost));
-  if (flag) return LNO_OT_ETIMEOUT;
+  if (h.flag) return LNO_OT_ETIMEOUT;
+  if (!kept && scale_too_small(R, h.amax[2])) return kRescale;
+  const double* hs = h.sums;
   // stats
   float ms = 0;
   if (t0 && t2 && cudaEventElapsedTime(&ms, t0, t2) == cudaSuccess) ctx->stats.ms_total = ms;
@@ -1355,15 +1404,26 @@ int measure_sigI(lno_ot_ctx* ctx, Run& R, SpinPass* pa, SpinPass* pb) {
   if (pb) pb->plan();
   if (pa) TRY(pa->prepare_inputs());
   if (pb) TRY(pb->prepare_inputs());
-  CU(cudaMemsetAsync(ctx->d_amax, 0, sizeof(unsigned long long), R.st));
-  if (pa) TRY(pa->measure());
-  if (pb) TRY(pb->measure());
-  unsigned long long h;
-  CU(cudaMemcpyAsync(&h, ctx->d_amax, sizeof h, cudaMemcpyDeviceToHost, R.st));
-  CU(cudaStreamSynchronize(R.st));
-  double m;
-  std::memcpy(&m, &h, 8);
-  R.sigI = pow2_scale(2.0 * m);  // antisymmetrised combinations are <= 2 max
+  // Two of the four or five slices of each factor (3 products instead of 10 or
+  // 15) give the largest integral to ~1e-4, and the scale is a power of two: it
+  // is settled unless the maximum lies within 1% of one.  Then, or when the
+  // blocks as built turn out larger than this measure said (finish_call), every
+  // slice is taken.
+  for (int pass = ctx->exact_measure ? 1 : 0; pass < 2; ++pass) {
+    CU(cudaMemsetAsync(ctx->d_amax, 0, 4 * sizeof(unsigned long long), R.st));
+    R.amax_exact = pass == 1;
+    if (pa) TRY(pa->measure());
+    if (pb) TRY(pb->measure());
+    unsigned long long h;
+    CU(cudaMemcpyAsync(&h, ctx->d_amax, sizeof h, cudaMemcpyDeviceToHost, R.st));
+    CU(cudaStreamSynchronize(R.st));
+    double m;
+    std::memcpy(&m, &h, 8);
+    R.sigI = pow2_scale(2.0 * m);  // antisymmetrised combinations are <= 2 max
+    int ex;
+    const double f = std::frexp(2.0 * m, &ex);
+    if (f > 0.505 && f < 0.99) break;
+  }
   return LNO_OT_OK;
 }
 
@@ -1392,7 +1452,16 @@ int build_cache(lno_ot_ctx* ctx, const lno_ot_domain* dom) {
   TRY(measure_sigI(ctx, R, C->has_a ? C->pa.get() : nullptr, C->has_b ? C->pb.get() : nullptr));
   if (C->has_a) TRY(C->pa->prepare());
   if (C->has_b) TRY(C->pb->prepare());
+  unsigned long long built;
+  CU(cudaMemcpyAsync(&built, ctx->d_amax + 2, sizeof built, cudaMemcpyDeviceToHost, R.st));
   CU(cudaStreamSynchronize(R.st));
+  if (scale_too_small(R, built) && !ctx->exact_measure) {   // once more, measured in full
+    C.reset();
+    ctx->exact_measure = true;
+    const int rc = build_cache(ctx, dom);
+    ctx->exact_measure = false;
+    return rc;
+  }
   ctx->cache = C.release();
   return LNO_OT_OK;
 }
@@ -1451,7 +1520,7 @@ int cached_energy(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out)
   C->pb->e_mixed = e_int[2];
   if (C->has_a) TRY(C->pa->compute());
   if (C->has_b) TRY(C->pb->compute());
-  return finish_call(ctx, R, A, dom, C->cs, e_int, false, t0, t1, t2, out);
+  return finish_call(ctx, R, A, dom, C->cs, e_int, false, true, t0, t1, t2, out);
 }
 
 bool flip_candidate(const lno_ot_domain* dom) {
@@ -1462,8 +1531,8 @@ bool flip_candidate(const lno_ot_domain* dom) {
   return flip;
 }
 
-int energy_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
-                const PassSpec* spec = nullptr) {
+int energy_once(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
+                const PassSpec* spec) {
   if (!spec) TRY(validate(ctx, dom));
   CU(cudaSetDevice(ctx->device));
   if (!spec && ctx->keep && !flip_candidate(dom)) {
@@ -1541,7 +1610,19 @@ int energy_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
                            cudaMemcpyDeviceToDevice, R.st));
     }
   }
-  return finish_call(ctx, R, R.arena, dom, cs, e_int, spec != nullptr, t0, t1, t2, out);
+  return finish_call(ctx, R, R.arena, dom, cs, e_int, spec != nullptr, false, t0, t1, t2, out);
+}
+
+int energy_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
+                const PassSpec* spec = nullptr) {
+  int rc = energy_once(ctx, dom, out, spec);
+  if (rc == kRescale) {
+    ctx->exact_measure = true;
+    rc = energy_once(ctx, dom, out, spec);
+    ctx->exact_measure = false;
+    if (rc == kRescale) rc = LNO_OT_EINVAL;   // not reached: the measure is the assembly's own
+  }
+  return rc;
 }
 
 // ---------------------------------------------------------------------------
@@ -2409,12 +2490,14 @@ int lno_ot_init(lno_ot_ctx** ctx, const lno_ot_options* opt) {
     uint64_t thr = UINT64_MAX;
     cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
   }
-  if (cudaMalloc(&c->d_flag, 256) != cudaSuccess || cudaMalloc(&c->d_amax, 256) != cudaSuccess ||
-      cudaMalloc(&c->d_sums, 256) != cudaSuccess) {
+  if (cudaMalloc(&c->d_sums, sizeof(CallState)) != cudaSuccess) {
+    c->d_sums = nullptr;
     cudaGetLastError();
     lno_ot_destroy(c);
     return LNO_OT_ENOMEM;
   }
+  c->d_amax = reinterpret_cast<unsigned long long*>(c->d_sums + 4);
+  c->d_flag = reinterpret_cast<int*>(c->d_amax + 4);
   *ctx = c;
   return LNO_OT_OK;
 }
@@ -2427,8 +2510,6 @@ void lno_ot_destroy(lno_ot_ctx* c) {
   c->cache = nullptr;
   if (c->stream) cudaStreamSynchronize(c->stream);
   for (auto e : c->ev_pool) cudaEventDestroy(e);
-  cudaFree(c->d_flag);
-  cudaFree(c->d_amax);
   cudaFree(c->d_sums);
   if (c->own_stream) cudaStreamDestroy(c->stream);
   delete c;

@@ -25,6 +25,8 @@
 #include <mutex>
 #include <string>
 
+#include <cmath>
+
 #include "common.cuh"
 
 namespace lno {
@@ -127,7 +129,7 @@ cudaError_t launch_slices(const double* in, int rows, int K, int Kp, __nv_bfloat
   const int64_t n = (int64_t)rows * Kp;
   const int64_t b = (n + 255) / 256;
   const int grid = (int)(b < 4864 ? (b < 1 ? 1 : b) : 4864);
-  slice_rows<S><<<grid, 256, 0, st>>>(in, rows, K, Kp, StoreSlices<S>{out, stride, inv, inv});
+  slice_rows<S><<<grid, 256, 0, st>>>(in, rows, K, Kp, StoreSlices<S>{out, stride, std::ilogb(inv), std::ilogb(inv)});
   return cudaGetLastError();
 }
 

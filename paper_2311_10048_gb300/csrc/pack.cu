@@ -89,32 +89,54 @@ __global__ void pack_at_same(const int2* __restrict__ pairs, int nslot, int o, i
   }
 }
 
-// BT[slot][pair(b<c)][kk] for occupied x; vvovT[c][(e*v+b)] = (eb|xc)
+// The large operands BT, BG, BF are written in runs of 16 consecutive k per
+// thread (32 bytes per slice: whole sectors), read so that a warp's loads run
+// along the DF block's contiguous index; blockIdx.z is the occupied orbital x0 +
+// z, slot slot0 + z, whose DF block follows the previous one.  Bound by the
+// float64 reads and the slice writes plus ~50 integer operations per element.
+
+// BT[slot][pair(b<c)][kk] for occupied x; vvovT[c][(e*v+b)] = (eb|xc).
+// A CTA owns a 16 x 16 block of (b, c), b-block <= c-block, and 16 k: thread
+// (c, b) keeps (eb|xc) of its row (read along b) and takes (ec|xb), read along c
+// by the transposed thread, from shared memory.
 template <class St>
-__global__ void pack_bt_same(int slot, int x, int o, int oi, int v, int Kp,
-                             const double* __restrict__ vvovT, const double* __restrict__ t2ss,
-                             St st) {
-  const int64_t np = npairs(v);
-  const int64_t total = np * Kp;
-  const int64_t base = (int64_t)slot * np * Kp;
+__global__ void __launch_bounds__(256)
+pack_bt_same(int slot0, int x0, int o, int oi, int v, int Kp, const double* __restrict__ vvovT,
+             const double* __restrict__ t2ss, St st) {
+  __shared__ double tr[16][16][17];
+  const int slot = slot0 + (int)blockIdx.z, x = x0 + (int)blockIdx.z;
+  // block pair (B <= C): index C (C + 1) / 2 + B
+  int C = (int)((sqrtf(8.0f * (float)blockIdx.x + 1.0f) - 1.0f) * 0.5f);
+  while (C * (C + 1) / 2 > (int)blockIdx.x) --C;
+  while ((C + 1) * (C + 2) / 2 <= (int)blockIdx.x) ++C;
+  const int B = (int)blockIdx.x - C * (C + 1) / 2;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int k0 = blockIdx.y * 16;
   const int64_t vv = (int64_t)v * v;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int kk = (int)(idx % Kp);
-    const int64_t pr = idx / Kp;
-    // decode pair index pr = c(c-1)/2 + b
-    int c = (int)((1.0 + sqrt(1.0 + 8.0 * (double)pr)) * 0.5);
-    while ((int64_t)c * (c - 1) / 2 > pr) --c;
-    while ((int64_t)(c + 1) * c / 2 <= pr) ++c;
-    const int b = (int)(pr - (int64_t)c * (c - 1) / 2);
-    double val = 0.0;
+  const double* src = vvovT + (int64_t)blockIdx.z * v * vv;
+  const int b = B * 16 + tx, c = C * 16 + ty;      // this thread's row
+  const int b2 = B * 16 + ty, c2 = C * 16 + tx;    // what it fetches for the others
+  double val[16];
+  uint32_t parts = 0;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const int kk = k0 + j;
+    double own = 0.0, other = 0.0;
     if (kk < v) {
-      val = vvovT[(int64_t)c * vv + (int64_t)kk * v + b] - vvovT[(int64_t)b * vv + (int64_t)kk * v + c];
-    } else if (kk < v + oi) {
-      const int m = kk - v;
-      val = t2ss[(((int64_t)x * o + m) * v + b) * v + c];
+      if (b < v && c < v) own = src[(int64_t)c * vv + (int64_t)kk * v + b];
+      if (b2 < v && c2 < v) other = src[(int64_t)b2 * vv + (int64_t)kk * v + c2];
+      parts |= 1u << j;
+    } else if (kk < v + oi && b2 < v && c2 < v) {
+      other = -t2ss[(((int64_t)x * o + (kk - v)) * v + b2) * v + c2];
     }
-    st(base + idx, val, kk < v);
+    val[j] = own;
+    tr[j][ty][tx] = other;
+  }
+  __syncthreads();
+  if (b < c && c < v) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) val[j] -= tr[j][tx][ty];
+    st.store16(((int64_t)slot * npairs(v) + pair_index(b, c)) * Kp + k0, val, parts);
   }
 }
 
@@ -142,52 +164,62 @@ __global__ void pack_a1(const int2* __restrict__ pk, int nslot, int os, int vs, 
   }
 }
 
-// BG[slot][(b*vt+C)][kk] for occupied x (spin s); gT[b][(E*vt+C)] = (xb|EC)
+// BG[slot][(b*vt+C)][kk] for occupied x (spin s); gT[b][(E*vt+C)] = (xb|EC):
+// thread = row, reads along C
 template <class St>
-__global__ void pack_bg(int slot, int x, int os, int vs, int ot, int oti, int vt, int Kp,
-                        const double* __restrict__ gT, const double* __restrict__ t2st, St st) {
-  const int64_t rows = (int64_t)vs * vt;
-  const int64_t total = rows * Kp;
-  const int64_t base = (int64_t)slot * total;
-  const int64_t vv = (int64_t)vt * vt;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int kk = (int)(idx % Kp);
-    const int64_t r = idx / Kp;
-    const int b = (int)(r / vt), C = (int)(r % vt);
-    double val = 0.0;
+__global__ void __launch_bounds__(256)
+pack_bg(int slot0, int x0, int os, int vs, int ot, int oti, int vt, int Kp,
+        const double* __restrict__ gT, const double* __restrict__ t2st, St st) {
+  const int slot = slot0 + (int)blockIdx.z, x = x0 + (int)blockIdx.z;
+  const int64_t rows = (int64_t)vs * vt, vv = (int64_t)vt * vt;
+  const int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (r >= rows) return;
+  const int k0 = blockIdx.y * 16;
+  const int b = (int)(r / vt), C = (int)(r - (int64_t)b * vt);
+  const double* src = gT + ((int64_t)blockIdx.z * vs + b) * vv + C;
+  double val[16];
+  uint32_t parts = 0;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const int kk = k0 + j;
+    val[j] = 0.0;
     if (kk < vt) {
-      val = gT[(int64_t)b * vv + (int64_t)kk * vt + C];
+      val[j] = src[(int64_t)kk * vt];
+      parts |= 1u << j;
     } else if (kk < vt + oti) {
-      const int M = kk - vt;
-      val = t2st[(((int64_t)x * ot + M) * vs + b) * vt + C];
+      val[j] = t2st[(((int64_t)x * ot + (kk - vt)) * vs + b) * vt + C];
     }
-    st(base + idx, val, kk < vt);
   }
+  st.store16(((int64_t)slot * rows + r) * Kp + k0, val, parts);
 }
 
-// BF[slot][(b*vt+C)][kk] for occupied K (spin t); fT[C][(b*vs+e)] = (be|KC)
+// BF[slot][(b*vt+C)][kk] for occupied K (spin t); fT[C][(b*vs+e)] = (be|KC):
+// thread = row, reads its 16 e (one 128-byte line)
 template <class St>
-__global__ void pack_bf(int slot, int K, int os, int osi, int vs, int ot, int vt, int Kp,
-                        const double* __restrict__ fT, const double* __restrict__ t2st, St st) {
-  const int64_t rows = (int64_t)vs * vt;
-  const int64_t total = rows * Kp;
-  const int64_t base = (int64_t)slot * total;
-  const int64_t vv = (int64_t)vs * vs;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int kk = (int)(idx % Kp);
-    const int64_t r = idx / Kp;
-    const int b = (int)(r / vt), C = (int)(r % vt);
-    double val = 0.0;
+__global__ void __launch_bounds__(256)
+pack_bf(int slot0, int K0, int os, int osi, int vs, int ot, int vt, int Kp,
+        const double* __restrict__ fT, const double* __restrict__ t2st, St st) {
+  const int slot = slot0 + (int)blockIdx.z, K = K0 + (int)blockIdx.z;
+  const int64_t rows = (int64_t)vs * vt, vv = (int64_t)vs * vs;
+  const int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (r >= rows) return;
+  const int k0 = blockIdx.y * 16;
+  const int b = (int)(r / vt), C = (int)(r - (int64_t)b * vt);
+  const double* src = fT + ((int64_t)blockIdx.z * vt + C) * vv + (int64_t)b * vs;
+  double val[16];
+  uint32_t parts = 0;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const int kk = k0 + j;
+    val[j] = 0.0;
     if (kk < vs) {
-      val = fT[(int64_t)C * vv + (int64_t)b * vs + kk];
+      val[j] = src[kk];
+      parts |= 1u << j;
     } else if (kk < vs + osi) {
-      const int m = kk - vs;
-      val = -t2st[(((int64_t)m * ot + K) * vs + b) * vt + C];
+      val[j] = -t2st[(((int64_t)(kk - vs) * ot + K) * vs + b) * vt + C];
     }
-    st(base + idx, val, kk < vs);
   }
+  st.store16(((int64_t)slot * rows + r) * Kp + k0, val, parts);
 }
 
 // AT2[slot][C][kk] for (p,K) = pk[slot]; lT[(K*vt+C)][(m*os+p)] = (mp|KC)
@@ -256,31 +288,6 @@ __global__ void view_absmax(const double* __restrict__ in, int64_t rs, int64_t k
   }
   for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
   if ((tx & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
-}
-
-// round(v 2^e2) to nearest (ties to even) from the bits of v, in integer
-// arithmetic (this GPU's float64 rate is 1/64 of its float32 rate); |v 2^e2|
-// must stay below 2^62, v finite.
-__device__ __forceinline__ int64_t round_scaled(double v, int e2) {
-  const uint64_t b = (uint64_t)__double_as_longlong(v);
-  const int ex = (int)((b >> 52) & 0x7ff);
-  uint64_t m = b & ((1ull << 52) - 1);
-  if (ex != 0) m |= 1ull << 52;
-  const int sh = (ex == 0 ? 1 : ex) - 1075 + e2;   // |v| 2^e2 = m 2^sh
-  uint64_t q;
-  if (m == 0) {
-    q = 0;
-  } else if (sh >= 0) {
-    q = m << sh;
-  } else if (-sh > 54) {
-    q = 0;                                        // m 2^sh < 1/2
-  } else {
-    const int r = -sh;
-    const uint64_t rem = m & ((1ull << r) - 1), half = 1ull << (r - 1);
-    q = m >> r;
-    if (rem > half || (rem == half && (q & 1))) ++q;
-  }
-  return (b >> 63) ? -(int64_t)q : (int64_t)q;
 }
 
 // The same exact slices as StoreSlices, from one rounding of the scaled value
@@ -429,11 +436,12 @@ cudaError_t launch_pack_at_same(const int2* pairs, int nslot, int o, int oi, int
 }
 
 template <class St>
-cudaError_t launch_pack_bt_same(int slot, int x, int o, int oi, int v, int Kp,
+cudaError_t launch_pack_bt_same(int slot0, int x0, int nx, int o, int oi, int v, int Kp,
                                 const double* vvovT, const double* t2ss, St st, cudaStream_t s) {
-  int64_t n = npairs(v) * Kp;
-  if (n == 0) return cudaSuccess;
-  pack_bt_same<<<grid_for(n), 256, 0, s>>>(slot, x, o, oi, v, Kp, vvovT, t2ss, st);
+  if (npairs(v) * Kp * nx == 0) return cudaSuccess;
+  const int nb = (v + 15) / 16;
+  pack_bt_same<<<dim3(nb * (nb + 1) / 2, (Kp + 15) / 16, nx), 256, 0, s>>>(slot0, x0, o, oi, v, Kp,
+                                                                         vvovT, t2ss, st);
   return cudaGetLastError();
 }
 
@@ -447,20 +455,20 @@ cudaError_t launch_pack_a1(const int2* pk, int nslot, int os, int vs, int ot, in
 }
 
 template <class St>
-cudaError_t launch_pack_bg(int slot, int x, int os, int vs, int ot, int oti, int vt, int Kp,
-                           const double* gT, const double* t2st, St st, cudaStream_t s) {
-  int64_t n = (int64_t)vs * vt * Kp;
-  if (n == 0) return cudaSuccess;
-  pack_bg<<<grid_for(n), 256, 0, s>>>(slot, x, os, vs, ot, oti, vt, Kp, gT, t2st, st);
+cudaError_t launch_pack_bg(int slot0, int x0, int nx, int os, int vs, int ot, int oti, int vt,
+                           int Kp, const double* gT, const double* t2st, St st, cudaStream_t s) {
+  if ((int64_t)vs * vt * Kp * nx == 0) return cudaSuccess;
+  const dim3 grid(ceil_div((int64_t)vs * vt, 256), (Kp + 15) / 16, nx);
+  pack_bg<<<grid, 256, 0, s>>>(slot0, x0, os, vs, ot, oti, vt, Kp, gT, t2st, st);
   return cudaGetLastError();
 }
 
 template <class St>
-cudaError_t launch_pack_bf(int slot, int K, int os, int osi, int vs, int ot, int vt, int Kp,
-                           const double* fT, const double* t2st, St st, cudaStream_t s) {
-  int64_t n = (int64_t)vs * vt * Kp;
-  if (n == 0) return cudaSuccess;
-  pack_bf<<<grid_for(n), 256, 0, s>>>(slot, K, os, osi, vs, ot, vt, Kp, fT, t2st, st);
+cudaError_t launch_pack_bf(int slot0, int K0, int nx, int os, int osi, int vs, int ot, int vt,
+                           int Kp, const double* fT, const double* t2st, St st, cudaStream_t s) {
+  if ((int64_t)vs * vt * Kp * nx == 0) return cudaSuccess;
+  const dim3 grid(ceil_div((int64_t)vs * vt, 256), (Kp + 15) / 16, nx);
+  pack_bf<<<grid, 256, 0, s>>>(slot0, K0, os, osi, vs, ot, vt, Kp, fT, t2st, st);
   return cudaGetLastError();
 }
 
@@ -557,13 +565,13 @@ template cudaError_t launch_view_slices<5>(const double*, int64_t, int64_t, int,
                                                   int, St, cudaStream_t);                       \
   template cudaError_t launch_pack_at_same<St>(const int2*, int, int, int, int, int,           \
                                                const double*, const double*, St, cudaStream_t); \
-  template cudaError_t launch_pack_bt_same<St>(int, int, int, int, int, int, const double*,     \
-                                               const double*, St, cudaStream_t);               \
+  template cudaError_t launch_pack_bt_same<St>(int, int, int, int, int, int, int,               \
+                                               const double*, const double*, St, cudaStream_t); \
   template cudaError_t launch_pack_a1<St>(const int2*, int, int, int, int, int, int, int,      \
                                           const double*, const double*, St, cudaStream_t);     \
-  template cudaError_t launch_pack_bg<St>(int, int, int, int, int, int, int, int,               \
+  template cudaError_t launch_pack_bg<St>(int, int, int, int, int, int, int, int, int,          \
                                           const double*, const double*, St, cudaStream_t);     \
-  template cudaError_t launch_pack_bf<St>(int, int, int, int, int, int, int, int,               \
+  template cudaError_t launch_pack_bf<St>(int, int, int, int, int, int, int, int, int,          \
                                           const double*, const double*, St, cudaStream_t);     \
   template cudaError_t launch_pack_at2<St>(const int2*, int, int, int, int, int, int, int,     \
                                            const double*, const double*, St, cudaStream_t);

@@ -1,6 +1,7 @@
 // Tensor-core contraction on CTA pairs for sm_103a: tcgen05.mma.cta_group::2
 // (256 x w tiles, FP32 accumulators in TMEM) fed by TMA, on exactly sliced
-// float64 operands.  Runs the W contractions.  The slicing, the weight-class
+// float64 operands.  Runs the W contractions (float32 row-major output) and the
+// DF assembly (float64 output out[n][m], or only its largest magnitude).  The slicing, the weight-class
 // accumulators and the segment sums are those of tc_gemm.cu: one TMEM
 // accumulator per weight class g = p + q of the slice products, so every class
 // sum is exact, added smallest class first in float32.
@@ -31,6 +32,7 @@
 // Every wait is bounded; on a timeout the kernel records an error code, lets
 // its copies and MMAs finish, frees TMEM and returns.
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "ptx.cuh"
@@ -45,8 +47,17 @@ constexpr long long kWaitCycles = 4000000000LL;
 constexpr int kSmemBytes = 227 * 1024;
 constexpr int kMaxStages = 16;
 constexpr int kBarBytes = 512;
-constexpr int kEpiWarps = 8;
-constexpr int kThreads = 64 + 32 * kEpiWarps;
+// Epilogue warps: float32 output 8 (up to 80 columns of results a thread);
+// float64 output 16 (its integer conversions need the lanes, and 32 columns of
+// results are 64 registers)
+template <typename OutT>
+constexpr int epi_warps() {
+  return sizeof(OutT) == 4 ? 8 : 16;
+}
+template <typename OutT>
+constexpr int pair_threads() {
+  return 64 + 32 * epi_warps<OutT>();
+}
 
 __device__ __noinline__ bool pair_wait(uint32_t bar, uint32_t parity, int* flag, int code,
                                        bool abortable, long long limit = kWaitCycles) {
@@ -179,6 +190,13 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7])
+      : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -264,22 +282,59 @@ __device__ __forceinline__ void store_chunk(const RowOut& ro, int chunk, const f
   }
 }
 
-template <int S>
-constexpr int pair_max_width() {   // columns of one tile: S accumulators in TMEM, N <= 256
-  return std::min(256, 512 / S / 16 * 16);
+// Columns of one tile: S accumulators in TMEM, N <= 256; 128 for float64 output
+// (32 results a thread).
+template <int S, typename OutT>
+constexpr int pair_max_width() {
+  return std::min(sizeof(OutT) == 4 ? 256 : 128, 512 / S / 16 * 16);
+}
+
+// I 2^e as a float64, |I| < 2^53 and the result a normal number (integer
+// operations only: a float64 add or conversion of every element would cost
+// more than the tile's MMAs, at 1/64 of the float32 rate).
+__device__ __forceinline__ double fixed_to_double(int64_t I, int e) {
+  const uint64_t a = (uint64_t)(I < 0 ? -I : I);
+  if (a == 0) return 0.0;
+  const int lz = __clzll((long long)a);
+  const uint64_t m = (a << (lz - 11)) & ((1ull << 52) - 1);
+  const uint64_t bits = ((uint64_t)(I < 0) << 63) | ((uint64_t)(1023 + 63 - lz + e) << 52) | m;
+  return __longlong_as_double((long long)bits);
+}
+
+// Float64 value of one element's class sums: the exact sum of the classes times
+// 2^e.  Class g is an integer multiple of 2^(-BITS g); sums too large for the
+// integers (or not finite) become NaN, as the operands' slices say.
+template <int S, int BITS>
+__device__ __forceinline__ double class_sum(const float (&c)[S], int e) {
+  int64_t I = 0;
+  float w = 1.0f, big = 0.0f;
+#pragma unroll
+  for (int g = 0; g < S; ++g) {
+    const float x = c[g] * w;   // integer (exact: a power of two)
+    big = fmaxf(big, fabsf(x));
+    if (isnan(x)) big = INFINITY;
+    I = I * (1 << BITS) + (int64_t)__float2int_rn(x);
+    w *= (float)(1 << BITS);
+  }
+  if (!(big < 1073741824.0f)) return __longlong_as_double(0x7ff8000000000000ll);
+  e -= BITS * (S - 1);
+  if (e < -960 || e > 960) return ldexp((double)I, e);   // extreme scales only
+  return fixed_to_double(I, e);
 }
 
 // TF32: 32-bit elements, 16 per 64-byte row, K 8 per MMA; the 16-bit formats
 // have 32 per row, K 16.  diag is the bounded-wait test hook of tc_gemm.cu.
-template <int S, int FMT>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+template <int S, int FMT, typename OutT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<OutT>(), 1)
 tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
              const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
-             const TcProb* __restrict__ probs, int nprob, int M, int N, int ldo, float scale,
-             int* __restrict__ flag, TcDiag diag, TcOut lay, PairTile tile) {
+             const TcProb* __restrict__ probs, const __grid_constant__ TcProb one, int nprob, int M,
+             int N, int ldo, float scale, int escale, int* __restrict__ flag,
+             unsigned long long* __restrict__ amax, TcDiag diag, TcOut lay, PairTile tile) {
   constexpr int BKE = FMT == kFmtTF32 ? BK / 2 : BK;   // elements per 64-byte row
   constexpr int KM = FMT == kFmtTF32 ? 8 : 16;         // K of one MMA
   constexpr int kABytes = BM * 64;                     // one slice of this CTA's A rows
+  constexpr int kEpiWarps = epi_warps<OutT>();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -349,7 +404,7 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
         int mt, nt;
         long long pr;
         decode(u, mt, nt, pr);
-        const TcProb& P = probs[pr];
+        const TcProb& P = probs ? probs[pr] : one;
         const int ar = mt * 2 * BM + (int)rank * BM;
         const int br = nt * tile.w + (int)rank * (ntile_w(nt) >> 1);
         for (int sg = 0; sg < P.nseg && ok; ++sg) {
@@ -408,7 +463,7 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
         int mt, nt;
         long long pr;
         decode(u, mt, nt, pr);
-        const TcProb& P = probs[pr];
+        const TcProb& P = probs ? probs[pr] : one;
         const int buf = nbuf == 2 ? (int)(it & 1u) : 0;
         const uint32_t use = nbuf == 2 ? it >> 1 : it;   // how often this buffer was used
         const int nseg = P.nseg, nw = ntile_w(nt);
@@ -471,10 +526,10 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
     }
   } else {
     // ------------------------------- epilogue ---------------------------------
-    constexpr int CH = (pair_max_width<S>() / 16 + 1) / 2;   // chunks of one warp
-    const int q = warp & 3, half = (warp - 2) >> 2;
+    const int q = warp & 3, part = (warp - 2) >> 2;   // TMEM quarter, column share
     const int row = (int)rank * BM + q * 32 + lane;
     uint32_t it = 0;
+    float lmax = 0.f;
     for (long long u = u0; u < nunits; u += ustep, ++it) {
       int mt, nt;
       long long pr;
@@ -482,43 +537,94 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
       const int buf = nbuf == 2 ? (int)(it & 1u) : 0;
       const uint32_t use = nbuf == 2 ? it >> 1 : it;
       const int m = mt * 2 * BM + row;
-      float* out = reinterpret_cast<float*>(probs[pr].out);
+      void* outp = probs ? probs[pr].out : one.out;
       const bool mok = m < M;
-      const RowOut ro = mok ? row_out(out, lay, ldo, m) : RowOut{nullptr, 0, 0};
-      if (!pair_wait(tfull(buf), use & 1u, flag, 6, true, wlim)) break;
-      tc_fence_after();
+      const int n0 = nt * tile.w;
       const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * S * tile.w);
-      const int nch = ntile_w(nt) / 16;
-      float v[CH * 16];
+      if constexpr (sizeof(OutT) == 4) {
+        constexpr int CH = (pair_max_width<S, OutT>() / 16 + 1) / 2;   // chunks of one warp
+        const RowOut ro = mok ? row_out(reinterpret_cast<float*>(outp), lay, ldo, m)
+                              : RowOut{nullptr, 0, 0};
+        if (!pair_wait(tfull(buf), use & 1u, flag, 6, true, wlim)) break;
+        tc_fence_after();
+        const int nch = ntile_w(nt) / 16;
+        float v[CH * 16];
 #pragma unroll
-      for (int c = 0; c < CH; ++c) {
-        const int chunk = 2 * c + half;
-        if (chunk < nch) {
-          uint32_t acc[S][16];
+        for (int c = 0; c < CH; ++c) {
+          const int chunk = 2 * c + part;
+          if (chunk < nch) {
+            uint32_t acc[S][16];
 #pragma unroll
-          for (int g = 0; g < S; ++g) tmem_ld16(tb + g * tile.w + chunk * 16, acc[g]);
-          tmem_ld_wait();
+            for (int g = 0; g < S; ++g) tmem_ld16(tb + g * tile.w + chunk * 16, acc[g]);
+            tmem_ld_wait();
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            float lo = 0.f;
+            for (int j = 0; j < 16; ++j) {
+              float lo = 0.f;
 #pragma unroll
-            for (int g = S - 1; g >= 1; --g) lo = __fadd_rn(lo, __uint_as_float(acc[g][j]));
-            v[c * 16 + j] = __fmul_rn(__fadd_rn(__uint_as_float(acc[0][j]), lo), scale);
+              for (int g = S - 1; g >= 1; --g) lo = __fadd_rn(lo, __uint_as_float(acc[g][j]));
+              v[c * 16 + j] = __fmul_rn(__fadd_rn(__uint_as_float(acc[0][j]), lo), scale);
+            }
+          }
+        }
+        // TMEM is read: the leader may start the next tile in this buffer
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive_cluster(map_rank(tempty(buf), 0));
+        if (mok) {
+#pragma unroll
+          for (int c = 0; c < CH; ++c) {
+            const int chunk = 2 * c + part;
+            if (chunk < nch) store_chunk(ro, (n0 >> 4) + chunk, v + c * 16, N - n0 - chunk * 16);
+          }
+        }
+      } else {
+        constexpr int CH = pair_max_width<S, OutT>() / 32;   // 8-column chunks of one warp
+        constexpr int BITS = FMT == kFmtTF32 ? 11 : 8;
+        if (!pair_wait(tfull(buf), use & 1u, flag, 6, true, wlim)) break;
+        tc_fence_after();
+        const int nch = ntile_w(nt) / 8;
+        double v[CH * 8];
+#pragma unroll
+        for (int c = 0; c < CH; ++c) {
+          const int chunk = 4 * c + part;
+          if (chunk < nch) {
+            uint32_t acc[S][8];
+#pragma unroll
+            for (int g = 0; g < S; ++g) tmem_ld8(tb + g * tile.w + chunk * 8, acc[g]);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              float x[S], lo = 0.f;
+#pragma unroll
+              for (int g = S - 1; g >= 0; --g) {
+                x[g] = __uint_as_float(acc[g][j]);
+                if (g > 0) lo = __fadd_rn(lo, x[g]);
+              }
+              if (amax != nullptr && mok && n0 + chunk * 8 + j < N)
+                lmax = fmaxf(lmax, fabsf(__fmul_rn(__fadd_rn(x[0], lo), scale)));
+              if (outp != nullptr) v[c * 8 + j] = class_sum<S, BITS>(x, escale);
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive_cluster(map_rank(tempty(buf), 0));
+        if (mok && outp != nullptr) {
+          double* out = reinterpret_cast<double*>(outp) + m;
+#pragma unroll
+          for (int c = 0; c < CH; ++c) {
+            const int n = n0 + (4 * c + part) * 8;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              if (4 * c + part < nch && n + j < N) out[(int64_t)(n + j) * ldo] = v[c * 8 + j];
           }
         }
       }
-      // TMEM is read: the leader may start the next tile in this buffer
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) arrive_cluster(map_rank(tempty(buf), 0));
-      if (mok) {
-        const int n0 = nt * tile.w;
-#pragma unroll
-        for (int c = 0; c < CH; ++c) {
-          const int chunk = 2 * c + half;
-          if (chunk < nch) store_chunk(ro, (n0 >> 4) + chunk, v + c * 16, N - n0 - chunk * 16);
-        }
-      }
+    }
+    if (sizeof(OutT) == 8 && amax != nullptr) {
+      for (int off = 16; off > 0; off >>= 1)
+        lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, off));
+      if (lane == 0) atomicMax(amax, (unsigned long long)__double_as_longlong((double)lmax));
     }
   }
   __syncwarp();
@@ -533,13 +639,13 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
 
 // Pairs that fit the device at once (queried once; the persistent loop deals
 // its tiles over them, so none may wait for a slot).
-template <int S, int FMT>
+template <int S, int FMT, typename OutT>
 int pair_clusters(int nsm) {
   static const int n = [] {
-    auto k = tc_pair_gemm<S, FMT>;
+    auto k = tc_pair_gemm<S, FMT, OutT>;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(pair_threads<OutT>());
     cfg.dynamicSmemBytes = kSmemBytes;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -557,11 +663,34 @@ int pair_clusters(int nsm) {
   return std::max(1, n > 0 ? std::min(n, nsm / 2) : nsm / 2);
 }
 
+template <int S, int FMT, typename OutT>
+cudaError_t launch_pair(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs,
+                        const TcProb& one, int nprob, int M, int N, int ldo, double scale,
+                        int* flag, unsigned long long* amax, int nsm, cudaStream_t st,
+                        TcDiag diag, TcOut lay, PairTile tile) {
+  if (nprob <= 0 || M <= 0 || N <= 0) return cudaSuccess;
+  if (tile.w < 16 || tile.w % 16 || tile.w > pair_max_width<S, OutT>() || tile.stages < 2 ||
+      tile.stages > kMaxStages || (tile.nbuf == 2 && 2 * S * tile.w > 512) ||
+      (int64_t)tile.nN * tile.w < N || (int64_t)(tile.nN - 1) * tile.w >= N)
+    return cudaErrorInvalidValue;
+  int ex;
+  if (std::frexp(scale, &ex) != 0.5) return cudaErrorInvalidValue;   // scale = 2^(ex - 1)
+  auto k = tc_pair_gemm<S, FMT, OutT>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+  if (e != cudaSuccess) return e;
+  const long long units = (long long)nprob * ((M + 2 * BM - 1) / (2 * BM)) * tile.nN;
+  const int pairs = (int)std::min<long long>(units, pair_clusters<S, FMT, OutT>(nsm));
+  k<<<2 * pairs, pair_threads<OutT>(), kSmemBytes, st>>>(mA[0], mA[1], mB[0], mB[1], probs, one,
+                                                         nprob, M, N, ldo, (float)scale, ex - 1,
+                                                         flag, amax, diag, lay, tile);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
-// Tile of a row-major pair launch with N columns: the fewest n-tiles the
-// widest tile allows (cap > 0: no wider than cap), equal up to 16 columns; two
-// accumulator sets where they fit; as many stages as shared memory holds.
+// Tile of a pair launch with N columns: the fewest n-tiles the widest tile
+// allows (cap > 0: no wider than cap), equal up to 16 columns; two accumulator
+// sets where they fit; as many stages as shared memory holds.
 PairTile pair_tile(int S, int N, int cap) {
   const int wmax = std::min(256, 512 / S / 16 * 16);
   const int lim = cap > 0 ? std::max(16, std::min(wmax, cap / 16 * 16)) : wmax;
@@ -580,22 +709,23 @@ template <int S, int FMT>
 cudaError_t launch_tc_pair(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs_dev,
                            int nprob, int M, int N, int ldo, double scale, int* flag, int nsm,
                            cudaStream_t st, TcDiag diag, TcOut lay, PairTile tile) {
-  if (nprob <= 0 || M <= 0 || N <= 0) return cudaSuccess;
-  if (tile.w < 16 || tile.w % 16 || tile.w > pair_max_width<S>() || tile.stages < 2 ||
-      tile.stages > kMaxStages || (tile.nbuf == 2 && 2 * S * tile.w > 512) ||
-      (int64_t)tile.nN * tile.w < N || (int64_t)(tile.nN - 1) * tile.w >= N)
-    return cudaErrorInvalidValue;
   if (lay.mode == kOutRows ? (ldo % 4 != 0 || ldo < ((N + 15) & ~15))
                            : (lay.nbs < 1 || lay.nbt < 1 || (lay.mode == kOutYTile && lay.nvt < 1)))
     return cudaErrorInvalidValue;
-  auto k = tc_pair_gemm<S, FMT>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-  if (e != cudaSuccess) return e;
-  const long long units = (long long)nprob * ((M + 2 * BM - 1) / (2 * BM)) * tile.nN;
-  const int pairs = (int)std::min<long long>(units, pair_clusters<S, FMT>(nsm));
-  k<<<2 * pairs, kThreads, kSmemBytes, st>>>(mA[0], mA[1], mB[0], mB[1], probs_dev, nprob, M, N,
-                                             ldo, (float)scale, flag, diag, lay, tile);
-  return cudaGetLastError();
+  if (probs_dev == nullptr) return cudaErrorInvalidValue;
+  return launch_pair<S, FMT, float>(mA, mB, probs_dev, TcProb{}, nprob, M, N, ldo, scale, flag,
+                                    nullptr, nsm, st, diag, lay, tile);
+}
+
+// One product with float64 output: p.out[n][m] (pitch ldo) = scale 2^14 units of
+// the class sums of segment p.seg[0], and / or its largest magnitude in *amax
+// (p.out NULL: only that).  Tile from pair_tile(S, N, 128).
+template <int S, int FMT>
+cudaError_t launch_tc_pair_f64(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb& p,
+                               int M, int N, int ldo, double scale, int* flag,
+                               unsigned long long* amax, int nsm, cudaStream_t st, PairTile tile) {
+  return launch_pair<S, FMT, double>(mA, mB, nullptr, p, 1, M, N, ldo, scale, flag, amax, nsm, st,
+                                     tc_normal(), TcOut{kOutRows, 0, 0, 0}, tile);
 }
 
 #define LNO_PAIR_INST(S, F)                                                                   \
@@ -608,5 +738,13 @@ LNO_PAIR_INST(4, kFmtBF16)
 LNO_PAIR_INST(5, kFmtBF16)
 LNO_PAIR_INST(2, kFmtTF32)
 #undef LNO_PAIR_INST
+#define LNO_PAIR_F64(S, F)                                                                      \
+  template cudaError_t launch_tc_pair_f64<S, F>(const CUtensorMap*, const CUtensorMap*,          \
+                                                const TcProb&, int, int, int, double, int*,     \
+                                                unsigned long long*, int, cudaStream_t, PairTile);
+LNO_PAIR_F64(2, kFmtBF16)
+LNO_PAIR_F64(4, kFmtBF16)
+LNO_PAIR_F64(5, kFmtBF16)
+#undef LNO_PAIR_F64
 
 }  // namespace lno

@@ -59,3 +59,36 @@ def test_tile_caps_are_bitwise_equal(tmp_path, cap):
     p.write_text(f"100000 {cap} 3\n")
     for prec in ("bf16x3", "bf16x6", "bf16x10", "bf16x15"):
         assert np.array_equal(e_trips(prec, dd, sel, str(p)), e_trips(prec, dd, sel)), prec
+
+
+@pytest.mark.parametrize("off", [0.0, 2e-3, -2e-3, 0.02, -0.02])
+def test_integral_scale_near_a_power_of_two(off):
+    """The integral scale is measured on two slices of the DF factors and settled
+    in full when the largest integral is within 1% of a power of two."""
+    d = make_domain(26, (4, 3), naux=40, L=14.0, seed=31, t1_sd=0.02)
+    va, vb = 22, 23
+    m = 0.0
+    for s, o in ((0, 4), (1, 3)):
+        for t, p in ((0, 4), (1, 3)):
+            g = np.einsum("Qab,Qic->abic", d["B"][s][:, o:, o:], d["B"][t][:, :p, p:])
+            h = np.einsum("Qij,Qka->ijka", d["B"][s][:, :o, :o], d["B"][t][:, :p, p:])
+            m = max(m, np.abs(g).max(), np.abs(h).max())
+    f = np.sqrt(2.0 ** np.ceil(np.log2(2 * m)) * (1 + off) / (2 * m))
+    d["B"] = [b * f for b in d["B"]]
+    dd = lno_ot.to_device(d)
+    sel = sample(4, 3)
+    ref = e_trips("fp64", dd, sel)
+    for prec in ("bf16x10", "bf16x15", "bf16x6"):
+        assert np.abs(e_trips(prec, dd, sel) - ref).max() <= TOL[prec] * np.abs(ref).max(), prec
+
+
+@pytest.mark.parametrize("key", ["B", "t2aa", "t2ab"])
+def test_nan_reaches_the_energy(key):
+    d = make_domain(20, (4, 3), naux=30, L=10.0, seed=8)
+    dd = lno_ot.to_device(d)
+    x = dd["B"][0] if key == "B" else dd[key]
+    x.view(-1)[x.numel() // 2 + 3] = float("nan")
+    for prec in ("fp64", "bf16x6", "bf16x10"):
+        ctx = lno_ot.Context(0, prec)
+        assert np.isnan(ctx.energy(dd)["total"]), prec
+        ctx.close()
