@@ -3,6 +3,7 @@
 
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -192,7 +193,9 @@ int make_operand_map(CUtensorMap* map, const void* base, int64_t Kp, int64_t row
 // tc_pair.cu: the W contractions on CTA pairs, float32 row-major output
 // out[m][n] in the layout `lay`.  Slice formats (the instruction descriptor's
 // codes); tile of a launch (pair_tile).
-constexpr int kFmtBF16 = 1, kFmtTF32 = 2;
+// BF16 and TF32 slices carry their weights 2^(-8q), 2^(-11q); FP16 slices are
+// the integer digits (weights 2^(-11q) applied to the class sums).
+constexpr int kFmtF16 = 0, kFmtBF16 = 1, kFmtTF32 = 2;
 struct PairTile {
   int w;        // columns of one n-tile (multiple of 16)
   int nN;       // n-tiles
@@ -274,13 +277,14 @@ __device__ __forceinline__ int64_t round_scaled(double v, int e2) {
 // s_q an integer multiple of 2^(-BITS q), |s_0| <= 2^(BITS - 1) (2^BITS / 2, the
 // scale's choice), |s_q| 2^(BITS q) <= 2^(BITS - 1) below it, each digit the
 // nearest one to what is left.  Integer arithmetic throughout: the value is
-// rounded once, 16 bits below the last digit, and cut into digits from the top
+// rounded once, to 54 - BITS bits after the point (beyond what a float64 near the
+// scale holds, so the digits are those of the value itself), and cut from the top
 // (float64 rounding steps of every digit made the layout kernels 10-20x slower
 // than their memory traffic).  A value that is not finite, or too large for the
 // scale, becomes NaN.
-template <int S, int BITS>
+template <int S, int BITS, bool INTS = false>   // INTS: f[q] = s_q 2^(BITS q)
 __device__ __forceinline__ void slice_digits(double v, int e, float (&f)[S]) {
-  constexpr int kX = 16;
+  constexpr int kX = 54 - BITS * S;   // bits kept below the last digit
   const int ex = (int)(((uint64_t)__double_as_longlong(v) >> 52) & 0x7ff);
   if (ex == 0x7ff || ex - 1023 + e > 60 - (BITS * (S - 1) + kX)) {
     f[0] = __int_as_float(0x7fc00000);
@@ -293,25 +297,51 @@ __device__ __forceinline__ void slice_digits(double v, int e, float (&f)[S]) {
 #pragma unroll
   for (int q = 0; q < S; ++q) {
     const int sh = BITS * (S - 1 - q) + kX;
-    const int64_t d = (R + (1ll << (sh - 1))) >> sh;
+    // nearest, ties to even (integrals lie on a grid of their own, so ties are common)
+    const int64_t d = (R + ((1ll << (sh - 1)) - 1) + ((R >> sh) & 1)) >> sh;
     R -= d << sh;
     f[q] = (float)(int)d * w;   // exact
-    w *= 1.0f / (float)(1 << BITS);
+    if (!INTS) w *= 1.0f / (float)(1 << BITS);
   }
 }
 
-// BF16 slices: value = scale 2^-7 (s_0 + ... + s_{S-1}), s_0 an integer in
-// [-128,128], s_q a multiple of 2^(-8q).
-template <int S>
+// 16-bit slices.  BF16: value = scale 2^-7 (s_0 + ... + s_{S-1}), s_0 an integer
+// in [-128,128], s_q a multiple of 2^(-8q).  FP16: value = scale 2^-10 (d_0 +
+// 2^-11 d_1 + 2^-22 d_2), integers of [-1024, 1024] (11 bits, exact in FP16).
+template <typename T>
+struct SliceFmt;
+template <>
+struct SliceFmt<__nv_bfloat16> {
+  static constexpr int bits = 8;
+  static constexpr bool ints = false;
+  static __device__ __forceinline__ __nv_bfloat16 one(float x) { return __float2bfloat16_rn(x); }
+  static __device__ __forceinline__ uint32_t two(float a, float b) {
+    const __nv_bfloat162 x = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&x);
+  }
+};
+template <>
+struct SliceFmt<__half> {
+  static constexpr int bits = 11;
+  static constexpr bool ints = true;
+  static __device__ __forceinline__ __half one(float x) { return __float2half_rn(x); }
+  static __device__ __forceinline__ uint32_t two(float a, float b) {
+    const __half2 x = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&x);
+  }
+};
+
+template <int S, typename T = __nv_bfloat16>
 struct StoreSlices {
-  __nv_bfloat16* p;
+  using F = SliceFmt<T>;
+  T* p;
   int64_t slice_stride;  // elements between slices
-  int e_t, e_i;          // log2(2^7 / scale) of amplitudes and of integrals
+  int e_t, e_i;          // log2(2^7 or 2^10 / scale) of amplitudes and of integrals
   __device__ __forceinline__ void operator()(int64_t idx, double v, int part) const {
     float f[S];
-    slice_digits<S, 8>(v, part ? e_i : e_t, f);
+    slice_digits<S, F::bits, F::ints>(v, part ? e_i : e_t, f);
 #pragma unroll
-    for (int s = 0; s < S; ++s) p[s * slice_stride + idx] = __float2bfloat16_rn(f[s]);
+    for (int s = 0; s < S; ++s) p[s * slice_stride + idx] = F::one(f[s]);
   }
   __device__ __forceinline__ void store16(int64_t idx, const double (&v)[16],
                                           uint32_t parts) const {
@@ -319,13 +349,10 @@ struct StoreSlices {
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       float a[S], b[S];
-      slice_digits<S, 8>(v[2 * j], (parts >> (2 * j)) & 1 ? e_i : e_t, a);
-      slice_digits<S, 8>(v[2 * j + 1], (parts >> (2 * j + 1)) & 1 ? e_i : e_t, b);
+      slice_digits<S, F::bits, F::ints>(v[2 * j], (parts >> (2 * j)) & 1 ? e_i : e_t, a);
+      slice_digits<S, F::bits, F::ints>(v[2 * j + 1], (parts >> (2 * j + 1)) & 1 ? e_i : e_t, b);
 #pragma unroll
-      for (int s = 0; s < S; ++s) {
-        const __nv_bfloat162 x = __floats2bfloat162_rn(a[s], b[s]);
-        w[s][j] = *reinterpret_cast<const uint32_t*>(&x);
-      }
+      for (int s = 0; s < S; ++s) w[s][j] = F::two(a[s], b[s]);
     }
 #pragma unroll
     for (int s = 0; s < S; ++s) {

@@ -69,6 +69,8 @@ cudaError_t launch_pack_at2(const int2*, int, int, int, int, int, int, int, cons
                             const double*, St, cudaStream_t);
 cudaError_t launch_transpose_t2ab(const double*, int, int, int, int, double*, cudaStream_t);
 cudaError_t launch_absmax(const double*, int64_t, unsigned long long*, cudaStream_t);
+cudaError_t launch_row_norm2(const void* p, int64_t rows, int Kp, unsigned long long* out,
+                             cudaStream_t s);
 cudaError_t launch_view_absmax(const double* in, int64_t rs, int64_t ks, int rows, int K,
                                unsigned long long* out, cudaStream_t s);
 cudaError_t launch_sum_partials(const double* part, int nsp, int M, int N, double* C,
@@ -164,12 +166,13 @@ struct lno_ot_ctx {
   }
   // one device block (CallState), read back in one copy at the end of a call
   double* d_sums = nullptr;                 // [4] per-case sums
-  unsigned long long* d_amax = nullptr;     // [4] magnitudes (bits of doubles)
+  unsigned long long* d_amax = nullptr;     // magnitudes (bits of doubles)
   int* d_flag = nullptr;                    // error flag (bounded waits)
   lno_ot_stats stats{};
   std::vector<cudaEvent_t> ev_pool;
   size_t ev_used = 0;
   bool exact_measure = false;          // integral scale from every slice (measure_sigI)
+  bool no_f16 = false;                 // BF16X10 on its BF16 slices only (kNoF16)
   // prepared operands of the last domain (options.keep_operands)
   bool keep = false;
   struct DomainCache* cache = nullptr;
@@ -180,14 +183,43 @@ void destroy_cache(DomainCache* c);
 namespace {
 
 // Device state of a call: per-case sums, magnitudes (0, 1 scratch, 2 the largest
-// DF integral assembled with the current scale), error flag.
+// DF integral assembled with the current scale; squared row norms of FP16
+// operands: of the DF blocks per spin, of AT, BT, A1, BG, BF, AT2), error flag.
+constexpr int kNormB = 4, kNormW = 8, kAmaxSlots = 16;
 struct CallState {
   double sums[4];
-  unsigned long long amax[4];
+  unsigned long long amax[kAmaxSlots];
   int flag;
 };
 
-constexpr int kRescale = 1;   // internal: the call has to run again (scale_too_small)
+// Internal codes, the call has to run again: with the integral scale measured in
+// full (scale_too_small), or without FP16 slices (class 0 not provably exact).
+constexpr int kRescale = 1, kNoF16 = 2;
+
+// Precision BF16X10 runs on three FP16 slices of 11 bits (6 slice products
+// instead of 10) for domains of at least
+// kF16MinVirtuals virtual orbitals per spin and kF16MinOccupied occupied ones, or
+// of kF16WideVirtuals virtuals whatever they occupy.  200/20/18 domain: whole
+// call 600 -> 436 ms, error against float64 slightly smaller.  Where the line
+// lies: the two slicings' triplet energies differ by the coarser one's error,
+// ~1e-9 (100 / v)^1.5 of a triplet's energy (measured 1.0e-9 at 100 virtuals,
+// 4.2e-10 at 180, 1.6e-10 at 360), and a precision keeps its results: the rule
+// holds that to half of 1e-9 for cases of many triplets and to a quarter for
+// single ones.  Smaller domains spend little of a call in the contraction.
+// Amplitudes use 10 bits of their leading slice: 32 bits of each operand's
+// largest magnitude for them and 33 for integrals (BF16: 32 and 32), dropped slice
+// products of at most 2 x 2^-32 of the largest product (BF16: 3 x 2^-32), and
+// leading sums half as large (kExactSum).
+constexpr int kF16MinVirtuals = 160, kF16MinOccupied = 8, kF16WideVirtuals = 256;
+bool f16_sizes(const int* nvir, const int* nocc) {
+  const int v = std::min(nvir[0], nvir[1]);
+  return v >= kF16WideVirtuals ||
+         (v >= kF16MinVirtuals && std::min(nocc[0], nocc[1]) >= kF16MinOccupied);
+}
+// FP32 sums of integers are exact while no partial sum exceeds 2^24: by
+// Cauchy-Schwarz the product of the row norms bounds every one (the BF16 slices
+// are exact for any data only to K = 1024).  0.999: the norms' own rounding.
+constexpr double kExactSum = 16777216.0 * 0.999;
 
 #define TRY(expr)                       \
   do {                                  \
@@ -279,7 +311,7 @@ struct Operand {
 // the roles exchanged: its row tiles run over the N rows (a long dimension, so
 // they are full) and its n-tiles over the M rows.  seg_tc stores the segments
 // with the roles already exchanged.  bn > 0 caps the tile width.
-cudaError_t launch_contract(int S, bool tf, int bn, const Operand& A0, const Operand& A1,
+cudaError_t launch_contract(int S, int fmt, int bn, const Operand& A0, const Operand& A1,
                             const Operand& B0, const Operand& B1, const TcProb* dpt, int nprob,
                             int M, int N, int ldo, double scale, int* flag, int nsm,
                             cudaStream_t st, TcOut lay) {
@@ -291,7 +323,8 @@ cudaError_t launch_contract(int S, bool tf, int bn, const Operand& A0, const Ope
     return cudaErrorInvalidValue;
 #define LNO_CALL(SS, FF) \
   launch_tc_pair<SS, FF>(mA, mB, dpt, nprob, M, N, ldo, scale, flag, nsm, st, tc_normal(), lay, t)
-  if (tf) return LNO_CALL(2, kFmtTF32);
+  if (fmt == kFmtTF32) return LNO_CALL(2, kFmtTF32);
+  if (fmt == kFmtF16) return LNO_CALL(3, kFmtF16);
   switch (S) {
     case 2: return LNO_CALL(2, kFmtBF16);
     case 3: return LNO_CALL(3, kFmtBF16);
@@ -328,6 +361,7 @@ struct Run {
   Arena arena;
   bool f64;
   bool tf32 = false;  // W contraction operands as TF32 slices (precision TF32)
+  bool f16 = false;   // precision BF16X10 on three FP16 slices (choose_f16)
   bool tc_adjoint = false;  // adjoint: its contractions on the tensor cores (tc_matmul)
   int S = 0;          // slices of the W contraction operands
   int Sdf = 4;        // slices of the DF factors
@@ -401,6 +435,18 @@ struct Run {
   StoreTF32<2> tf32_slices(const Operand& op) const {
     return StoreTF32<2>{op.f32, op.slice_stride, 10 - std::ilogb(sigT), 10 - std::ilogb(sigI)};
   }
+  StoreSlices<3, __half> f16_slices(const Operand& op) const {
+    return StoreSlices<3, __half>{reinterpret_cast<__half*>(op.bf), op.slice_stride,
+                                  9 - std::ilogb(sigT), 10 - std::ilogb(sigI)};
+  }
+  int fmt() const { return tf32 ? kFmtTF32 : f16 ? kFmtF16 : kFmtBF16; }
+
+  // Largest squared row norm of the leading (integer) slice of an FP16 operand.
+  int row_norm2(const Operand& op, int slot) {
+    stats->other_launches++;
+    CU(launch_row_norm2(op.bf, op.total_rows(), op.Kp, ctx->d_amax + slot, st));
+    return LNO_OT_OK;
+  }
 
   // ---- DF integrals: out[n][m] = sum_Q L[m][Q] R[n][Q] (float64) ------------
   // L rows [l0, l0+M) of operand Lo, R rows [r0, r0+N) of Ro.
@@ -426,7 +472,7 @@ struct Run {
     p.nseg = 1;
     p.seg[0] = TcSeg{0, 0, (int)l0, (int)r0, naux, 0};
     p.out = amax_pass ? nullptr : out;
-    const double scale = sigB * sigB * std::ldexp(1.0, -14);
+    const double scale = sigB * sigB * std::ldexp(1.0, f16 ? -20 : -14);
     // the measuring pass takes the two leading slices of each factor (3 of the 10
     // products) unless that leaves the scale open (measure_sigI)
     const int ns = amax_pass && !amax_exact ? 2 : Sdf;
@@ -437,12 +483,18 @@ struct Run {
     TRY(Ro.pair_map(&mB[0], t.w / 2, ns));
     mA[1] = mA[0];
     mB[1] = mB[0];
-#define LNO_DF(SS)                                                                            \
-  CU((launch_tc_pair_f64<SS, kFmtBF16>(mA, mB, p, M, N, ldo, scale, ctx->d_flag,               \
-                                       am, ctx->nsm, st, t)))
-    if (ns == 2) LNO_DF(2);
-    else if (ns == 5) LNO_DF(5);
-    else LNO_DF(4);
+#define LNO_DF(SS, FF)                                                                        \
+  CU((launch_tc_pair_f64<SS, FF>(mA, mB, p, M, N, ldo, scale, ctx->d_flag, am, ctx->nsm, st, t)))
+    if (f16) {
+      if (ns == 2) LNO_DF(2, kFmtF16);
+      else LNO_DF(3, kFmtF16);
+    } else if (ns == 2) {
+      LNO_DF(2, kFmtBF16);
+    } else if (ns == 5) {
+      LNO_DF(5, kFmtBF16);
+    } else {
+      LNO_DF(4, kFmtBF16);
+    }
 #undef LNO_DF
     return LNO_OT_OK;
   }
@@ -505,6 +557,11 @@ struct Run {
         if (f64)
           CU(launch_transpose_block(dom->B[s], naux, nbs[s], b.p0, b.np, b.q0, b.nq, b.op->Kp,
                                     StoreF64{b.op->f64}, st));
+        else if (f16)
+          CU(launch_transpose_block(
+              dom->B[s], naux, nbs[s], b.p0, b.np, b.q0, b.nq, b.op->Kp,
+              StoreSlices<3, __half>{reinterpret_cast<__half*>(b.op->bf), b.op->slice_stride,
+                                     eB + 3, eB + 3}, st));
         else if (Sdf == 5)
           CU(launch_transpose_block(
               dom->B[s], naux, nbs[s], b.p0, b.np, b.q0, b.nq, b.op->Kp,
@@ -513,6 +570,10 @@ struct Run {
           CU(launch_transpose_block(
               dom->B[s], naux, nbs[s], b.p0, b.np, b.q0, b.nq, b.op->Kp,
               StoreSlices<4>{b.op->bf, b.op->slice_stride, eB, eB}, st));
+      }
+      if (f16) {
+        CU(cudaMemsetAsync(ctx->d_amax + kNormB + s, 0, sizeof(unsigned long long), st));
+        for (const Operand* op : {&Boo[s], &Bov[s], &Bvv[s]}) TRY(row_norm2(*op, kNormB + s));
       }
     }
     return LNO_OT_OK;
@@ -890,6 +951,9 @@ struct SpinPass {
     if (tf)
       return pack_all(R.tf32_slices(AT), R.tf32_slices(BT), R.tf32_slices(A1),
                       R.tf32_slices(BG), R.tf32_slices(BF), R.tf32_slices(AT2));
+    if (R.f16)
+      return pack_all(R.f16_slices(AT), R.f16_slices(BT), R.f16_slices(A1), R.f16_slices(BG),
+                      R.f16_slices(BF), R.f16_slices(AT2));
     if (R.S == 2)
       return pack_all(R.slices<2>(AT), R.slices<2>(BT), R.slices<2>(A1), R.slices<2>(BG),
                       R.slices<2>(BF), R.slices<2>(AT2));
@@ -915,8 +979,8 @@ struct SpinPass {
       CU(launch_gemm_f64(dpf, nprob, M, N, ldo, R.st));
     } else {
       CU(cudaMemcpyAsync(dpt, pt.data(), nprob * sizeof(TcProb), cudaMemcpyHostToDevice, R.st));
-      const double scale = R.sigT * R.sigI * std::ldexp(1.0, R.tf32 ? -20 : -14);
-      CU(launch_contract(R.S, R.tf32, bn, opA0, opA1, opB0, opB1, dpt, nprob, M, N, ldo, scale,
+      const double scale = R.sigT * R.sigI * std::ldexp(1.0, R.f16 ? -19 : R.tf32 ? -20 : -14);
+      CU(launch_contract(R.S, R.fmt(), bn, opA0, opA1, opB0, opB1, dpt, nprob, M, N, ldo, scale,
                          R.ctx->d_flag, R.ctx->nsm, R.st, lay));
     }
     if (e1) cudaEventRecord(e1, R.st);
@@ -1212,7 +1276,22 @@ struct SpinPass {
     TRY(prepare_inputs());
     TRY(build_v_blocks());
     TRY(build());
-    return LNO_OT_OK;
+    return R.f16 ? check_exact() : LNO_OT_OK;
+  }
+  // FP16 slices: the class-0 sums of every contraction are exact (kExactSum)
+  int check_exact() {
+    unsigned long long* slot = R.ctx->d_amax + kNormW;
+    CU(cudaMemsetAsync(slot, 0, 6 * sizeof(unsigned long long), R.st));
+    const Operand* ops[6] = {&AT, &BT, &A1, &BG, &BF, &AT2};
+    for (int q = 0; q < 6; ++q) TRY(R.row_norm2(*ops[q], kNormW + q));
+    unsigned long long h[6];
+    CU(cudaMemcpyAsync(h, slot, sizeof h, cudaMemcpyDeviceToHost, R.st));
+    CU(cudaStreamSynchronize(R.st));
+    double n[6];
+    std::memcpy(n, h, sizeof h);
+    for (double& x : n) x = std::sqrt(x);
+    const double x = 3 * n[0] * n[1], y = 2 * n[2] * n[3] + n[0] * n[4], z = 2 * n[5] * n[1];
+    return std::max({x, y, z}) <= kExactSum ? LNO_OT_OK : kNoF16;
   }
   int compute() {
     TRY(run_case(false));
@@ -1386,14 +1465,15 @@ struct PassSpec {
   double lap_s, lap_w;
 };
 
-void set_precision(Run& R, int prec) {
+void set_precision(Run& R, int prec, const int* nvir, const int* nocc, bool no_f16) {
+  R.f16 = prec == LNO_OT_BF16X10 && !no_f16 && f16_sizes(nvir, nocc);
   R.f64 = prec == LNO_OT_FP64;
   R.tf32 = prec == LNO_OT_TF32;
-  R.S = prec == LNO_OT_BF16X6    ? 3
+  R.S = prec == LNO_OT_BF16X6 || R.f16 ? 3
         : prec == LNO_OT_BF16X10 ? 4
         : prec == LNO_OT_BF16X15 ? 5
                                  : 2;
-  R.Sdf = prec == LNO_OT_BF16X15 ? 5 : 4;
+  R.Sdf = prec == LNO_OT_BF16X15 ? 5 : R.f16 ? 3 : 4;
 }
 
 // Integral scale of the sliced path: one pass over every DF block the two
@@ -1414,11 +1494,13 @@ int measure_sigI(lno_ot_ctx* ctx, Run& R, SpinPass* pa, SpinPass* pb) {
     R.amax_exact = pass == 1;
     if (pa) TRY(pa->measure());
     if (pb) TRY(pb->measure());
-    unsigned long long h;
-    CU(cudaMemcpyAsync(&h, ctx->d_amax, sizeof h, cudaMemcpyDeviceToHost, R.st));
+    unsigned long long h[kNormB + 2];
+    CU(cudaMemcpyAsync(h, ctx->d_amax, sizeof h, cudaMemcpyDeviceToHost, R.st));
     CU(cudaStreamSynchronize(R.st));
-    double m;
+    double m, nB[2];
     std::memcpy(&m, &h, 8);
+    std::memcpy(nB, h + kNormB, sizeof nB);
+    if (R.f16 && !(std::max(nB[0], nB[1]) <= kExactSum)) return kNoF16;
     R.sigI = pow2_scale(2.0 * m);  // antisymmetrised combinations are <= 2 max
     int ex;
     const double f = std::frexp(2.0 * m, &ex);
@@ -1442,7 +1524,8 @@ int build_cache(lno_ot_ctx* ctx, const lno_ot_domain* dom) {
   C->prec = ctx->prec;
   C->R.reset(new Run(ctx, &C->key));
   Run& R = *C->R;
-  set_precision(R, ctx->prec);
+  const int nvir[2] = {dom->nbas - dom->nocc[0], dom->nbas - dom->nocc[1]};
+  set_precision(R, ctx->prec, nvir, dom->nocc, ctx->no_f16);
   for (int c = 0; c < 4; ++c) TRY(select_case(&C->key, c, C->cs[c]));
   TRY(R.stage());
   C->has_a = !C->cs[0].trips.empty() || !C->cs[1].trips.empty();
@@ -1455,13 +1538,7 @@ int build_cache(lno_ot_ctx* ctx, const lno_ot_domain* dom) {
   unsigned long long built;
   CU(cudaMemcpyAsync(&built, ctx->d_amax + 2, sizeof built, cudaMemcpyDeviceToHost, R.st));
   CU(cudaStreamSynchronize(R.st));
-  if (scale_too_small(R, built) && !ctx->exact_measure) {   // once more, measured in full
-    C.reset();
-    ctx->exact_measure = true;
-    const int rc = build_cache(ctx, dom);
-    ctx->exact_measure = false;
-    return rc;
-  }
+  if (scale_too_small(R, built) && !ctx->exact_measure) return kRescale;
   ctx->cache = C.release();
   return LNO_OT_OK;
 }
@@ -1550,7 +1627,9 @@ int energy_once(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
     R.lap_s = spec->lap_s;
     R.lap_w = spec->lap_w;
   }
-  set_precision(R, ctx->prec);
+  const int nvir[2] = {(spec ? spec->nbs[0] : dom->nbas) - dom->nocc[0],
+                       (spec ? spec->nbs[1] : dom->nbas) - dom->nocc[1]};
+  set_precision(R, ctx->prec, nvir, dom->nocc, ctx->no_f16);
   CU(cudaMemsetAsync(ctx->d_flag, 0, sizeof(int), ctx->stream));
   cudaEvent_t t0 = R.event(), t1 = R.event(), t2 = R.event();
   if (t0) cudaEventRecord(t0, R.st);
@@ -1616,13 +1695,12 @@ int energy_once(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
 int energy_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
                 const PassSpec* spec = nullptr) {
   int rc = energy_once(ctx, dom, out, spec);
-  if (rc == kRescale) {
-    ctx->exact_measure = true;
+  for (int tries = 0; rc > 0 && tries < 2; ++tries) {
+    (rc == kRescale ? ctx->exact_measure : ctx->no_f16) = true;
     rc = energy_once(ctx, dom, out, spec);
-    ctx->exact_measure = false;
-    if (rc == kRescale) rc = LNO_OT_EINVAL;   // not reached: the measure is the assembly's own
   }
-  return rc;
+  ctx->exact_measure = ctx->no_f16 = false;
+  return rc > 0 ? LNO_OT_EINVAL : rc;   // not reached: neither can come twice
 }
 
 // ---------------------------------------------------------------------------
@@ -2497,7 +2575,7 @@ int lno_ot_init(lno_ot_ctx** ctx, const lno_ot_options* opt) {
     return LNO_OT_ENOMEM;
   }
   c->d_amax = reinterpret_cast<unsigned long long*>(c->d_sums + 4);
-  c->d_flag = reinterpret_cast<int*>(c->d_amax + 4);
+  c->d_flag = reinterpret_cast<int*>(c->d_amax + kAmaxSlots);
   *ctx = c;
   return LNO_OT_OK;
 }

@@ -387,6 +387,31 @@ __global__ void scatter_add_rows_kernel(const double* __restrict__ src, double* 
   }
 }
 
+// Largest sum of squares of one row of an operand's leading FP16 slice (the
+// integers d_0), as the bits of a double in *out (atomicMax): a warp per row.
+__global__ void __launch_bounds__(256)
+row_norm2(const uint4* __restrict__ p, int64_t rows, int row16, unsigned long long* out) {
+  const int lane = threadIdx.x & 31;
+  float best = 0.f;
+  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < rows;
+       r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    float ss = 0.f;
+    for (int w = lane; w < row16; w += 32) {
+      const uint4 u = p[r * row16 + w];
+      const uint32_t h[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h[q]));
+        ss += f.x * f.x + f.y * f.y;
+      }
+    }
+    for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+    best = isnan(ss) ? INFINITY : fmaxf(best, ss);
+  }
+  if (lane == 0 && best > 0.f)
+    atomicMax(out, (unsigned long long)__double_as_longlong((double)best));
+}
+
 // Number of elements with |t2ab[i][J][a][B] - t2ab[J][i][B][a]| > tol (n
 // occupied and v virtual of each spin); zero means the mixed amplitudes are
 // spin-flip symmetric to within tol.
@@ -520,6 +545,14 @@ cudaError_t launch_t2ab_flip_mismatch(const double* t2ab, int n, int v, double t
   return cudaGetLastError();
 }
 
+cudaError_t launch_row_norm2(const void* p, int64_t rows, int Kp, unsigned long long* out,
+                             cudaStream_t s) {
+  if (rows <= 0) return cudaSuccess;
+  if (Kp % 8 || reinterpret_cast<uintptr_t>(p) % 16) return cudaErrorInvalidValue;
+  row_norm2<<<grid_for(rows * 32), 256, 0, s>>>(static_cast<const uint4*>(p), rows, Kp / 8, out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_absmax(const double* x, int64_t n, unsigned long long* out, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   absmax_kernel<<<grid_for(n), 256, 0, s>>>(x, n, out);
@@ -582,6 +615,8 @@ LNO_INST(StoreSlices<3>)
 LNO_INST(StoreSlices<4>)
 LNO_INST(StoreSlices<5>)
 LNO_INST(StoreTF32<2>)
+using StoreF16x3 = StoreSlices<3, __half>;
+LNO_INST(StoreF16x3)
 #undef LNO_INST
 
 }  // namespace lno

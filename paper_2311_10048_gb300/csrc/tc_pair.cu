@@ -302,9 +302,9 @@ __device__ __forceinline__ double fixed_to_double(int64_t I, int e) {
 }
 
 // Float64 value of one element's class sums: the exact sum of the classes times
-// 2^e.  Class g is an integer multiple of 2^(-BITS g); sums too large for the
+// 2^e.  Class g is an integer multiple of 2^(-BITS g), or (INTS) that integer; sums too large for the
 // integers (or not finite) become NaN, as the operands' slices say.
-template <int S, int BITS>
+template <int S, int BITS, bool INTS>
 __device__ __forceinline__ double class_sum(const float (&c)[S], int e) {
   int64_t I = 0;
   float w = 1.0f, big = 0.0f;
@@ -314,7 +314,7 @@ __device__ __forceinline__ double class_sum(const float (&c)[S], int e) {
     big = fmaxf(big, fabsf(x));
     if (isnan(x)) big = INFINITY;
     I = I * (1 << BITS) + (int64_t)__float2int_rn(x);
-    w *= (float)(1 << BITS);
+    if (!INTS) w *= (float)(1 << BITS);
   }
   if (!(big < 1073741824.0f)) return __longlong_as_double(0x7ff8000000000000ll);
   e -= BITS * (S - 1);
@@ -335,6 +335,7 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
   constexpr int KM = FMT == kFmtTF32 ? 8 : 16;         // K of one MMA
   constexpr int kABytes = BM * 64;                     // one slice of this CTA's A rows
   constexpr int kEpiWarps = epi_warps<OutT>();
+  constexpr float kW = 1.0f / 2048.0f;                 // weight step of FP16 classes
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -559,10 +560,16 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
             tmem_ld_wait();
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
+              // lower classes first (each exact), then one rounding against class 0
               float lo = 0.f;
 #pragma unroll
-              for (int g = S - 1; g >= 1; --g) lo = __fadd_rn(lo, __uint_as_float(acc[g][j]));
-              v[c * 16 + j] = __fmul_rn(__fadd_rn(__uint_as_float(acc[0][j]), lo), scale);
+              for (int g = S - 1; g >= 1; --g)
+                lo = FMT == kFmtF16 ? __fmaf_rn(lo, kW, __uint_as_float(acc[g][j]))
+                                    : __fadd_rn(lo, __uint_as_float(acc[g][j]));
+              v[c * 16 + j] =
+                  __fmul_rn(FMT == kFmtF16 ? __fmaf_rn(lo, kW, __uint_as_float(acc[0][j]))
+                                           : __fadd_rn(__uint_as_float(acc[0][j]), lo),
+                            scale);
             }
           }
         }
@@ -579,7 +586,7 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
         }
       } else {
         constexpr int CH = pair_max_width<S, OutT>() / 32;   // 8-column chunks of one warp
-        constexpr int BITS = FMT == kFmtTF32 ? 11 : 8;
+        constexpr int BITS = FMT == kFmtBF16 ? 8 : 11;
         if (!pair_wait(tfull(buf), use & 1u, flag, 6, true, wlim)) break;
         tc_fence_after();
         const int nch = ntile_w(nt) / 8;
@@ -598,11 +605,12 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
 #pragma unroll
               for (int g = S - 1; g >= 0; --g) {
                 x[g] = __uint_as_float(acc[g][j]);
-                if (g > 0) lo = __fadd_rn(lo, x[g]);
+                lo = FMT == kFmtF16 ? __fmaf_rn(lo, kW, x[g]) : __fadd_rn(lo, x[g]);
               }
               if (amax != nullptr && mok && n0 + chunk * 8 + j < N)
-                lmax = fmaxf(lmax, fabsf(__fmul_rn(__fadd_rn(x[0], lo), scale)));
-              if (outp != nullptr) v[c * 8 + j] = class_sum<S, BITS>(x, escale);
+                lmax = fmaxf(lmax, fabsf(__fmul_rn(lo, scale)));
+              if (outp != nullptr)
+                v[c * 8 + j] = class_sum<S, BITS, FMT == kFmtF16>(x, escale);
             }
           }
         }
@@ -737,6 +745,7 @@ LNO_PAIR_INST(3, kFmtBF16)
 LNO_PAIR_INST(4, kFmtBF16)
 LNO_PAIR_INST(5, kFmtBF16)
 LNO_PAIR_INST(2, kFmtTF32)
+LNO_PAIR_INST(3, kFmtF16)
 #undef LNO_PAIR_INST
 #define LNO_PAIR_F64(S, F)                                                                      \
   template cudaError_t launch_tc_pair_f64<S, F>(const CUtensorMap*, const CUtensorMap*,          \
@@ -745,6 +754,8 @@ LNO_PAIR_INST(2, kFmtTF32)
 LNO_PAIR_F64(2, kFmtBF16)
 LNO_PAIR_F64(4, kFmtBF16)
 LNO_PAIR_F64(5, kFmtBF16)
+LNO_PAIR_F64(2, kFmtF16)
+LNO_PAIR_F64(3, kFmtF16)
 #undef LNO_PAIR_F64
 
 }  // namespace lno

@@ -92,3 +92,29 @@ def test_nan_reaches_the_energy(key):
         ctx = lno_ot.Context(0, prec)
         assert np.isnan(ctx.energy(dd)["total"]), prec
         ctx.close()
+
+
+@pytest.mark.parametrize("kind", ["plain", "B", "t2", "occupied"])
+def test_fp16_slices_and_their_fallback(kind):
+    """BF16X10 on FP16 slices (256 virtuals, or 160 with 8 occupied), and the data
+    for which their leading sums are not provably exact: DF factors (or doubles)
+    all near the largest magnitude, which run on the BF16 slices."""
+    v, na, nb = (160, 8, 8) if kind == "occupied" else (256, 3, 3)
+    d = make_domain(v + na, (na, nb), naux=150, L=50.0, seed=77, t1_sd=0.02)
+    rng = np.random.default_rng(1)
+    if kind == "B":
+        d["B"] = [np.where(b < 0, -1.0, 1.0) * rng.uniform(0.09, 0.1) for b in d["B"]]
+    if kind == "t2":
+        for k in ("t2aa", "t2bb", "t2ab"):
+            d[k] = np.sign(d[k]) * 0.03
+    dd = lno_ot.to_device(d)
+    sel = sample(na, nb)
+    ref = e_trips("fp64", dd, sel)
+    assert np.abs(e_trips("bf16x10", dd, sel) - ref).max() <= TOL["bf16x10"] * np.abs(ref).max()
+    ctx = lno_ot.Context(0, "bf16x10", keep_operands=True)
+    for _ in range(2):
+        et = [torch.zeros(max(x.size, 1), dtype=torch.float64, device="cuda") for x in sel]
+        ctx.energy(dd, e_trip=et, trip_sel=sel)
+        got = np.concatenate([e[:x.size].cpu().numpy() for e, x in zip(et, sel)])
+        assert np.abs(got - ref).max() <= TOL["bf16x10"] * np.abs(ref).max()
+    ctx.close()
