@@ -9,7 +9,8 @@
 // Each X entry with distinct virtual labels belongs to exactly one
 // restricted element, so dX is written with plain stores (the caller zeroes
 // it first).  Per-tile sums of dT1, deps and the V-integral gradients are
-// reduced in shared memory and added to global memory with atomics.
+// formed without atomics, in three passes over the tile's g_V and g_D in shared
+// memory, one per pair of indices, and added to global memory with atomics.
 //
 // Contraction adjoint (grouped strided GEMM, atomically accumulated):
 //   X^T[n][m] = sum_seg s A[m][:] . B[n][:]  ->  dA += s dX.B,  dB += s dX^T.A
@@ -94,6 +95,24 @@ __global__ void __launch_bounds__(256) gemm_f64_strided(const GemmS* __restrict_
 // FM (a.vmode 1, the f_ov part sum W V_f / D): dX is added to, dt1s/dt1t are
 // the f_ov gradients and dov_ss/dov_ts the raw T2 gradients (t2ss / t2st
 // layouts), since the planes are then the amplitudes themselves.
+//
+// Per 16^3 tile: pass 1, thread (b, c), runs over a, stores g_V and g_D of every
+// element in shared memory and sums what belongs to (b, c), b and c; pass 2,
+// thread (a, c), sums over b what belongs to (a, c) and a; pass 3, thread (a,
+// b), sums over c.  Sums along a thread index are 16-lane shuffles.  Bound by
+// its ~50 float64 operations per element (one division).  60/7/5 domain, all
+// triplets: 9.8 ms with shared-memory atomics (256 threads on one address for
+// every a), 1.0 ms so.
+constexpr int kGvPitch = TB + 1;
+constexpr int kGvTile = TB * TB * kGvPitch;   // doubles of one padded tile [a][b][c]
+constexpr size_t kBackwardSmem = 2 * kGvTile * sizeof(double);
+
+__device__ __forceinline__ double sum16(double x) {   // over the 16 lanes that share r1
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
 template <bool MIXED, bool FM>
 __global__ void __launch_bounds__(256)
 energy_backward(EnergyArgs a, const double* __restrict__ X, const double* __restrict__ Z,
@@ -101,11 +120,18 @@ energy_backward(EnergyArgs a, const double* __restrict__ X, const double* __rest
                 double* __restrict__ dt1t, double* __restrict__ dov_ss,
                 double* __restrict__ dov_ts, double* __restrict__ deps_s,
                 double* __restrict__ deps_t, double gscale) {
-  __shared__ double vt[9][TB][TB];   // V integral tables (as in the forward)
-  __shared__ double gvt[9][TB][TB];  // their gradients
-  __shared__ double t1s[9][TB], gt1[9][TB];
-  __shared__ double ev[3][TB], gev[3][TB];
-  __shared__ double gocc;
+  constexpr int NO = MIXED ? 2 : 3;        // planes (and T1 rows) of the (b, c) and (a, c) passes
+  constexpr int NC = MIXED ? 1 : 3;        // ... of the (a, b) pass
+  constexpr int AC = MIXED ? 2 : 3, AB = MIXED ? 4 : 6;   // first (a, c) and (a, b) plane
+  extern __shared__ double dyn[];
+  double* const gvs = dyn;                 // g_V [a][b][c]
+  double* const gds = dyn + kGvTile;       // g_D
+  __shared__ double vt[9][TB][TB];         // V integral tables (as in the forward)
+  __shared__ double t1s[9][TB];
+  __shared__ double ev[3][TB];
+  __shared__ double ga[4][TB], gb[4][TB];  // sums of a and of b: T1 rows, then energies
+  __shared__ double gc[8][4][TB];          // sums of c, per warp
+  __shared__ double gocc[8];
   const int g = blockIdx.y;
   const Trip tr = a.trips[g];
   const double* Xg = X + (int64_t)g * a.x_stride;
@@ -113,47 +139,56 @@ energy_backward(EnergyArgs a, const double* __restrict__ X, const double* __rest
   double* dXg = dX + (int64_t)g * a.x_stride;
   double* dZg = MIXED ? dZ + (int64_t)g * a.z_stride : nullptr;
   const int tid = threadIdx.x, r1 = tid / TB, r2 = tid % TB;
+  const int lane = tid & 31, warp = tid >> 5;
   const int nvs = a.nvs, nvt = a.nvt, nos = a.nos;
   const double eocc = MIXED ? a.eps_s[tr.i] + a.eps_s[tr.j] + a.eps_t[tr.k]
                             : a.eps_s[tr.i] + a.eps_s[tr.j] + a.eps_s[tr.k];
-  if (tid == 0) gocc = 0.0;
+  const int occ3[3][2] = {{tr.j, tr.k}, {tr.k, tr.i}, {tr.i, tr.j}};
+  // gradient of plane o of the pair (x, y): same spin K^{pr}_{xy} (pair of
+  // occupied o), mixed (px|KC) with p = j, i for the first two, <ij||xy> last
+  auto add_ss = [&](int p, int r, int x, int y, double gk) {
+    if (gk == 0.0) return;
+    if (FM) {
+      atomicAdd(&dov_ss[(((int64_t)p * nos + r) * nvs + x) * nvs + y], gk);
+    } else {
+      atomicAdd(&dov_ss[ovss_idx(a, p, x, r, y)], gk);
+      atomicAdd(&dov_ss[ovss_idx(a, p, y, r, x)], -gk);
+    }
+  };
+  auto add_ts = [&](int p, int x, int y, double gk) {
+    if (gk == 0.0) return;
+    if (FM)
+      atomicAdd(&dov_ts[(((int64_t)p * a.not_ + tr.k) * nvs + x) * nvt + y], gk);
+    else
+      atomicAdd(&dov_ts[ovts_idx(a, tr.k, y, p, x)], gk);
+  };
+  double occ_acc = 0.0;
   for (int q = blockIdx.x; q < a.nblocks; q += gridDim.x) {
     const int3 blk = a.blocks[q];
     const int a0 = blk.x * TB, b0 = blk.y * TB, c0 = blk.z * TB;
     // ---- V tables and t1 / eps of the tile (as in the forward) -------------
     if (!MIXED) {
-      const int occ3[3][2] = {{tr.j, tr.k}, {tr.k, tr.i}, {tr.i, tr.j}};
       const int offs[3][2] = {{b0, c0}, {a0, c0}, {a0, b0}};
       for (int pl = 0; pl < 3; ++pl) {
         const int x = offs[pl][0] + r1, y = offs[pl][1] + r2;
-        for (int o = 0; o < 3; ++o) {
-          double v = 0.0;
-          if (x < nvs && y < nvs) v = vplane_ss(a, occ3[o][0], x, occ3[o][1], y);
-          vt[pl * 3 + o][r1][r2] = v;
-          gvt[pl * 3 + o][r1][r2] = 0.0;
-        }
+        for (int o = 0; o < 3; ++o)
+          vt[pl * 3 + o][r1][r2] =
+              x < nvs && y < nvs ? vplane_ss(a, occ3[o][0], x, occ3[o][1], y) : 0.0;
       }
     } else {
       const int offs[2] = {b0, a0};
       for (int pl = 0; pl < 2; ++pl) {
         const int x = offs[pl] + r1, y = c0 + r2;
-        for (int o = 0; o < 2; ++o) {
-          double v = 0.0;
-          if (x < nvs && y < nvt) v = vplane_ts(a, tr.k, y, o == 0 ? tr.j : tr.i, x);
-          vt[pl * 2 + o][r1][r2] = v;
-          gvt[pl * 2 + o][r1][r2] = 0.0;
-        }
+        for (int o = 0; o < 2; ++o)
+          vt[pl * 2 + o][r1][r2] =
+              x < nvs && y < nvt ? vplane_ts(a, tr.k, y, o == 0 ? tr.j : tr.i, x) : 0.0;
       }
       const int x = a0 + r1, y = b0 + r2;
-      double v = 0.0;
-      if (x < nvs && y < nvs) v = vplane_ss(a, tr.i, x, tr.j, y);
-      vt[4][r1][r2] = v;
-      gvt[4][r1][r2] = 0.0;
+      vt[4][r1][r2] = x < nvs && y < nvs ? vplane_ss(a, tr.i, x, tr.j, y) : 0.0;
     }
     if (tid < 3 * TB) {
       const int bl = tid / TB, l = tid % TB;
-      const int base = bl == 0 ? a0 : (bl == 1 ? b0 : c0);
-      const int x = base + l;
+      const int x = (bl == 0 ? a0 : (bl == 1 ? b0 : c0)) + l;
       const bool tblock = MIXED && bl == 2;
       const int nv = tblock ? nvt : nvs;
       if (!MIXED) {
@@ -163,28 +198,25 @@ energy_backward(EnergyArgs a, const double* __restrict__ X, const double* __rest
       } else if (!tblock) {
         t1s[bl * 3 + 0][l] = x < nvs ? a.t1s[(int64_t)tr.i * nvs + x] : 0.0;
         t1s[bl * 3 + 1][l] = x < nvs ? a.t1s[(int64_t)tr.j * nvs + x] : 0.0;
-        t1s[bl * 3 + 2][l] = 0.0;
       } else {
-        t1s[bl * 3 + 0][l] = x < nvt ? a.t1t[(int64_t)tr.k * nvt + x] : 0.0;
-        t1s[bl * 3 + 1][l] = t1s[bl * 3 + 2][l] = 0.0;
+        t1s[bl * 3][l] = x < nvt ? a.t1t[(int64_t)tr.k * nvt + x] : 0.0;
       }
-      for (int o = 0; o < 3; ++o) gt1[bl * 3 + o][l] = 0.0;
       const double* e = tblock ? a.eps_t : a.eps_s;
       const int no = tblock ? a.not_ : a.nos;
       ev[bl][l] = x < nv ? e[no + x] : 0.0;
-      gev[bl][l] = 0.0;
     }
     __syncthreads();
-    // ---- elements: thread (b, c), loop over a ------------------------------
+    // ---- pass 1: thread (b, c), every a -------------------------------------
     {
       const int bl = r1, cl = r2;
       const int b = b0 + bl, c = c0 + cl;
       const bool rowok = MIXED ? (b < nvs && c < nvt) : (b < c && c < nvs);
-      if (rowok) {
-        const int na = min(b, a0 + TB) - a0;
-        double gb_e = 0.0, gc_e = 0.0, gocc_t = 0.0;
-        double gk_bc[3] = {0.0, 0.0, 0.0}, gtb[3] = {0.0, 0.0, 0.0}, gtc[3] = {0.0, 0.0, 0.0};
-        for (int al = 0; al < na; ++al) {
+      const int na = rowok ? min(b, a0 + TB) - a0 : 0;
+      double ge = 0.0, gk[NO] = {}, gtb[NO] = {}, gtc[NC] = {};
+#pragma unroll 2
+      for (int al = 0; al < TB; ++al) {
+        double gv = 0.0, gd = 0.0;
+        if (al < na) {
           const int aa = a0 + al;
           int64_t i1, i2, i3;
           double x1, x2, x3;
@@ -216,131 +248,151 @@ energy_backward(EnergyArgs a, const double* __restrict__ X, const double* __rest
           }
           const double D = eocc - ev[0][al] - ev[1][bl] - ev[2][cl];
           // E = W (W + V) / D, or W V / D for the f_ov part
-          const double gw = gscale * (FM ? v : 2.0 * w + v) / D;
-          const double gv = gscale * w / D;
-          const double gd = -gscale * w * (FM ? v : w + v) / (D * D);
+          const double s = gscale / D;
+          const double gw = s * (FM ? v : 2.0 * w + v);
+          gv = s * w;
+          gd = -gv * (FM ? v : w + v) / D;
+          double* d3 = MIXED ? dZg : dXg;
+          if (FM) {
+            dXg[i1] += gw; dXg[i2] -= gw; d3[i3] += gw;
+          } else {
+            dXg[i1] = gw; dXg[i2] = -gw; d3[i3] = gw;
+          }
           if (!MIXED) {
-            if (FM) {
-              dXg[i1] += gw; dXg[i2] -= gw; dXg[i3] += gw;
-            } else {
-              dXg[i1] = gw; dXg[i2] = -gw; dXg[i3] = gw;
-            }
+#pragma unroll
             for (int o = 0; o < 3; ++o) {
-              gk_bc[o] += gv * t1s[o][al];
-              atomicAdd(&gt1[o][al], gv * vt[o][bl][cl]);
+              gk[o] += gv * t1s[o][al];
               gtb[o] -= gv * vt[3 + o][al][cl];
-              atomicAdd(&gvt[3 + o][al][cl], -gv * t1s[3 + o][bl]);
-              gtc[o] += gv * vt[6 + o][al][bl];
-              atomicAdd(&gvt[6 + o][al][bl], gv * t1s[6 + o][cl]);
+              gtc[o % NC] += gv * vt[6 + o][al][bl];
             }
           } else {
-            if (FM) {
-              dXg[i1] += gw; dXg[i2] -= gw; dZg[i3] += gw;
-            } else {
-              dXg[i1] = gw; dXg[i2] = -gw; dZg[i3] = gw;
-            }
-            gk_bc[0] += gv * t1s[0][al];             // (jb|KC)
-            gk_bc[1] -= gv * t1s[1][al];             // (ib|KC)
-            atomicAdd(&gt1[0][al], gv * vt[0][bl][cl]);
-            atomicAdd(&gt1[1][al], -gv * vt[1][bl][cl]);
-            gtb[0] -= gv * vt[2][al][cl];            // t^b_i
-            gtb[1] += gv * vt[3][al][cl];            // t^b_j
-            atomicAdd(&gvt[2][al][cl], -gv * t1s[3][bl]);
-            atomicAdd(&gvt[3][al][cl], gv * t1s[4][bl]);
-            gtc[0] += gv * vt[4][al][bl];            // t^C_K
-            atomicAdd(&gvt[4][al][bl], gv * t1s[6][cl]);
+            gk[0] += gv * t1s[0][al];             // (jb|KC)
+            gk[1] -= gv * t1s[1][al];             // (ib|KC)
+            gtb[0] -= gv * vt[2][al][cl];         // t^b_i
+            gtb[1] += gv * vt[3][al][cl];         // t^b_j
+            gtc[0] += gv * vt[4][al][bl];         // t^C_K
           }
-          gocc_t += gd;
-          atomicAdd(&gev[0][al], -gd);
-          gb_e -= gd;
-          gc_e -= gd;
+          ge += gd;
         }
-        const int nk = MIXED ? 2 : 3;
-        for (int o = 0; o < nk; ++o) atomicAdd(&gvt[o][bl][cl], gk_bc[o]);
-        for (int o = 0; o < 3; ++o) {
-          atomicAdd(&gt1[3 + o][bl], gtb[o]);
-          atomicAdd(&gt1[6 + o][cl], gtc[o]);
+        gvs[(al * TB + bl) * kGvPitch + cl] = gv;
+        gds[(al * TB + bl) * kGvPitch + cl] = gd;
+      }
+      if (rowok) {
+#pragma unroll
+        for (int o = 0; o < NO; ++o) {
+          if (MIXED)
+            add_ts(o == 0 ? tr.j : tr.i, b, c, gk[o]);
+          else
+            add_ss(occ3[o][0], occ3[o][1], b, c, gk[o]);
         }
-        atomicAdd(&gev[1][bl], gb_e);
-        atomicAdd(&gev[2][cl], gc_e);
-        atomicAdd(&gocc, gocc_t);
+      }
+      // sums over c (the 16 lanes of one b), over b (the two of a warp, then warps)
+#pragma unroll
+      for (int o = 0; o < NO; ++o) {
+        const double x = sum16(gtb[o]);
+        if (cl == 0) gb[o][bl] = x;
+      }
+      const double eb = sum16(ge);
+      if (cl == 0) gb[3][bl] = -eb;
+#pragma unroll
+      for (int o = 0; o < NC; ++o) {
+        const double x = gtc[o] + __shfl_xor_sync(0xffffffffu, gtc[o], 16);
+        if (lane < 16) gc[warp][o][cl] = x;
+      }
+      const double ec = ge + __shfl_xor_sync(0xffffffffu, ge, 16);
+      if (lane < 16) gc[warp][3][cl] = -ec;
+      occ_acc += ge;
+    }
+    __syncthreads();
+    // ---- pass 2: thread (a, c), every b --------------------------------------
+    {
+      const int al = r1, cl = r2;
+      double gk[NO] = {}, gta[NO] = {}, ge = 0.0;
+#pragma unroll 4
+      for (int bl = 0; bl < TB; ++bl) {
+        const double gv = gvs[(al * TB + bl) * kGvPitch + cl];
+        ge += gds[(al * TB + bl) * kGvPitch + cl];
+#pragma unroll
+        for (int o = 0; o < NO; ++o) {
+          const double sg = MIXED && o == 1 ? -gv : gv;   // signs of planes (a,c) and t^a
+          gk[o] -= sg * t1s[3 + o][bl];
+          gta[o] += sg * vt[o][bl][cl];
+        }
+      }
+      const int x = a0 + al, y = c0 + cl;
+      if (x < nvs && y < (MIXED ? nvt : nvs)) {
+#pragma unroll
+        for (int o = 0; o < NO; ++o) {
+          if (MIXED)
+            add_ts(o == 0 ? tr.j : tr.i, x, y, gk[o]);
+          else
+            add_ss(occ3[o][0], occ3[o][1], x, y, gk[o]);
+        }
+      }
+#pragma unroll
+      for (int o = 0; o < NO; ++o) {
+        const double t = sum16(gta[o]);
+        if (cl == 0) ga[o][al] = t;
+      }
+      ge = sum16(ge);
+      if (cl == 0) ga[3][al] = -ge;
+    }
+    // ---- pass 3: thread (a, b), every c --------------------------------------
+    {
+      const int al = r1, bl = r2;
+      double gk[NC] = {};
+#pragma unroll 4
+      for (int cl = 0; cl < TB; ++cl) {
+        const double gv = gvs[(al * TB + bl) * kGvPitch + cl];
+#pragma unroll
+        for (int o = 0; o < NC; ++o) gk[o] += gv * t1s[6 + o][cl];
+      }
+      const int x = a0 + al, y = b0 + bl;
+      if (x < nvs && y < nvs) {
+#pragma unroll
+        for (int o = 0; o < NC; ++o)
+          add_ss(MIXED ? tr.i : occ3[o][0], MIXED ? tr.j : occ3[o][1], x, y, gk[o]);
       }
     }
     __syncthreads();
-    // ---- flush tile gradients ----------------------------------------------
-    if (!MIXED) {
-      const int occ3[3][2] = {{tr.j, tr.k}, {tr.k, tr.i}, {tr.i, tr.j}};
-      const int offs[3][2] = {{b0, c0}, {a0, c0}, {a0, b0}};
-      for (int pl = 0; pl < 3; ++pl) {
-        const int x = offs[pl][0] + r1, y = offs[pl][1] + r2;
-        if (x >= nvs || y >= nvs) continue;
-        for (int o = 0; o < 3; ++o) {
-          const double gk = gvt[pl * 3 + o][r1][r2];
-          if (gk == 0.0) continue;
-          const int p = occ3[o][0], r = occ3[o][1];
-          if (FM) {
-            atomicAdd(&dov_ss[(((int64_t)p * nos + r) * nvs + x) * nvs + y], gk);
-          } else {
-            atomicAdd(&dov_ss[ovss_idx(a, p, x, r, y)], gk);
-            atomicAdd(&dov_ss[ovss_idx(a, p, y, r, x)], -gk);
-          }
-        }
-      }
-    } else {
-      const int offs[2] = {b0, a0};
-      for (int pl = 0; pl < 2; ++pl) {
-        const int x = offs[pl] + r1, y = c0 + r2;
-        if (x >= nvs || y >= nvt) continue;
-        for (int o = 0; o < 2; ++o) {
-          const double gk = gvt[pl * 2 + o][r1][r2];
-          if (gk == 0.0) continue;
-          const int p = o == 0 ? tr.j : tr.i;
-          if (FM)
-            atomicAdd(&dov_ts[(((int64_t)p * a.not_ + tr.k) * nvs + x) * nvt + y], gk);
-          else
-            atomicAdd(&dov_ts[ovts_idx(a, tr.k, y, p, x)], gk);
-        }
-      }
-      const int x = a0 + r1, y = b0 + r2;
-      const double gk = gvt[4][r1][r2];
-      if (x < nvs && y < nvs && gk != 0.0) {
-        if (FM) {
-          atomicAdd(&dov_ss[(((int64_t)tr.i * nos + tr.j) * nvs + x) * nvs + y], gk);
-        } else {
-          atomicAdd(&dov_ss[ovss_idx(a, tr.i, x, tr.j, y)], gk);
-          atomicAdd(&dov_ss[ovss_idx(a, tr.i, y, tr.j, x)], -gk);
-        }
-      }
-    }
+    // ---- T1 and energy gradients of the tile ----------------------------------
     if (tid < 3 * TB) {
       const int bl = tid / TB, l = tid % TB;
-      const int base = bl == 0 ? a0 : (bl == 1 ? b0 : c0);
-      const int x = base + l;
+      const int x = (bl == 0 ? a0 : (bl == 1 ? b0 : c0)) + l;
       const bool tblock = MIXED && bl == 2;
       const int nv = tblock ? nvt : nvs;
       if (x < nv) {
-        if (!MIXED) {
-          const int occ[3] = {tr.i, tr.j, tr.k};
-          for (int o = 0; o < 3; ++o)
-            if (gt1[bl * 3 + o][l] != 0.0)
-              atomicAdd(&dt1s[(int64_t)occ[o] * nvs + x], gt1[bl * 3 + o][l]);
-        } else if (!tblock) {
-          atomicAdd(&dt1s[(int64_t)tr.i * nvs + x], gt1[bl * 3 + 0][l]);
-          atomicAdd(&dt1s[(int64_t)tr.j * nvs + x], gt1[bl * 3 + 1][l]);
-        } else {
-          atomicAdd(&dt1t[(int64_t)tr.k * nvt + x], gt1[bl * 3 + 0][l]);
+        const int occ[3] = {tr.i, tr.j, tr.k};
+        const int nrow = bl == 2 ? NC : NO;
+        for (int o = 0; o < 4; ++o) {
+          if (o >= nrow && o < 3) continue;
+          double t = 0.0;
+          if (bl == 2) {
+            for (int w = 0; w < 8; ++w) t += gc[w][o][l];
+          } else {
+            t = bl == 0 ? ga[o][l] : gb[o][l];
+          }
+          if (t == 0.0) continue;
+          if (o == 3)
+            atomicAdd(&(tblock ? deps_t : deps_s)[(tblock ? a.not_ : a.nos) + x], t);
+          else if (tblock)
+            atomicAdd(&dt1t[(int64_t)tr.k * nvt + x], t);
+          else
+            atomicAdd(&dt1s[(int64_t)occ[o] * nvs + x], t);
         }
-        double* de = tblock ? deps_t : deps_s;
-        const int no = tblock ? a.not_ : a.nos;
-        if (gev[bl][l] != 0.0) atomicAdd(&de[no + x], gev[bl][l]);
       }
     }
     __syncthreads();
   }
+  for (int o = 16; o > 0; o >>= 1) occ_acc += __shfl_xor_sync(0xffffffffu, occ_acc, o);
+  if (lane == 0) gocc[warp] = occ_acc;
+  __syncthreads();
   if (tid == 0) {
-    atomicAdd(&deps_s[tr.i], gocc);
-    atomicAdd(&deps_s[tr.j], gocc);
-    atomicAdd(MIXED ? &deps_t[tr.k] : &deps_s[tr.k], gocc);
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += gocc[w];
+    atomicAdd(&deps_s[tr.i], t);
+    atomicAdd(&deps_s[tr.j], t);
+    atomicAdd(MIXED ? &deps_t[tr.k] : &deps_s[tr.k], t);
   }
 }
 
@@ -621,23 +673,15 @@ cudaError_t launch_energy_backward(const EnergyArgs& a, const double* X, const d
                                    double* deps_t, double gscale, int ntrip, int nchunks,
                                    cudaStream_t st) {
   if (ntrip <= 0) return cudaSuccess;
-  dim3 grid(nchunks, ntrip);
-  const bool fm = a.vmode != 0;
-  if (a.kind == SAME) {
-    if (fm)
-      energy_backward<false, true><<<grid, 256, 0, st>>>(a, X, Z, dX, dZ, dt1s, dt1t, dov_ss,
-                                                         dov_ts, deps_s, deps_t, gscale);
-    else
-      energy_backward<false, false><<<grid, 256, 0, st>>>(a, X, Z, dX, dZ, dt1s, dt1t, dov_ss,
-                                                          dov_ts, deps_s, deps_t, gscale);
-  } else {
-    if (fm)
-      energy_backward<true, true><<<grid, 256, 0, st>>>(a, X, Z, dX, dZ, dt1s, dt1t, dov_ss,
-                                                        dov_ts, deps_s, deps_t, gscale);
-    else
-      energy_backward<true, false><<<grid, 256, 0, st>>>(a, X, Z, dX, dZ, dt1s, dt1t, dov_ss,
-                                                         dov_ts, deps_s, deps_t, gscale);
-  }
+  const dim3 grid(nchunks, ntrip);
+  auto k = a.kind == SAME
+               ? (a.vmode != 0 ? energy_backward<false, true> : energy_backward<false, false>)
+               : (a.vmode != 0 ? energy_backward<true, true> : energy_backward<true, false>);
+  const cudaError_t e =
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBackwardSmem);
+  if (e != cudaSuccess) return e;
+  k<<<grid, 256, kBackwardSmem, st>>>(a, X, Z, dX, dZ, dt1s, dt1t, dov_ss, dov_ts, deps_s, deps_t,
+                                      gscale);
   return cudaGetLastError();
 }
 

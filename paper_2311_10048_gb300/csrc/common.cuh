@@ -133,20 +133,23 @@ struct TcSeg {
   int a_row, b_row; // first row of the A / B operand block in its tensor
   int K;            // contraction length (k < K is real data)
   int neg;          // 1: subtract this segment
+  int k0;           // first k (multiple of 32), tc_pair.cu only
 };
 
 // TcProb.flags: kTcAccum adds the result to out instead of storing it;
 // kTcFloatRest forms the float64 result as HI + the float32 sum of the lower
-// weight classes, scaled in float32 (the scale must be a power of two): two
-// float64 operations per element instead of six, ~2^-32 relative instead of
-// the exact class sums (used by the adjoint's products)
-constexpr int kTcAccum = 1, kTcFloatRest = 2;
+// weight classes instead of the exact sum of all (the adjoint's products)
+// kTcAtomic (tc_pair.cu) adds with atomics: problems of one launch share an output
+constexpr int kTcAccum = 1, kTcFloatRest = 2, kTcAtomic = 4;
 
 struct TcProb {
   TcSeg seg[kMaxSeg];
   int nseg;
-  int flags;        // float64 transposed output only: kTcAccum, kTcFloatRest
+  int flags;        // float64 transposed output only: kTcAccum, kTcFloatRest, kTcAtomic
   void* out;        // output of this problem: [N][ldo] (transposed) or [M][ldo] (row-major)
+  // float64 output of tc_pair.cu: exponents of the operands' scales on the
+  // device (scale 2^(*ea + *eb - 14)); NULL: the launch's scale
+  const int *ea, *eb;
 };
 
 // Output layout of a row-major float32 contraction launch (tc_pair.cu).
@@ -161,7 +164,8 @@ struct TcProb {
 //              tile.
 // The energy kernel reads each 16^3 sub-cube of the tiled layouts with one
 // 16 KB bulk copy, in the shared-memory layout its element loops index.
-constexpr int kOutRows = 0, kOutYTile = 1, kOutZTile = 2;
+// Float64 output (tc_pair.cu): kOutRows out[n][m], kOutF64Rows out[m][n].
+constexpr int kOutRows = 0, kOutYTile = 1, kOutZTile = 2, kOutF64Rows = 3;
 struct TcOut {
   int mode;
   int nvt;    // kOutYTile: C count per b
@@ -211,6 +215,11 @@ template <int S, int FMT>
 cudaError_t launch_tc_pair_f64(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb& p,
                                int M, int N, int ldo, double scale, int* flag,
                                unsigned long long* amax, int nsm, cudaStream_t st, PairTile tile);
+template <int S, int FMT>
+cudaError_t launch_tc_pair_f64_group(const CUtensorMap* mA, const CUtensorMap* mB,
+                                     const TcProb* probs_dev, int nprob, int M, int N, int ldo,
+                                     double scale, int* flag, int nsm, cudaStream_t st,
+                                     int mode, PairTile tile);
 int sliced_product_bn(int S);
 cudaError_t launch_sliced_product(int S, const CUtensorMap* mA, const CUtensorMap* mB,
                                   const TcProb* dp, int M, int N, double scale, int* flag,

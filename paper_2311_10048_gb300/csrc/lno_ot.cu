@@ -79,6 +79,10 @@ template <int S>
 cudaError_t launch_view_slices(const double* in, int64_t rs, int64_t ks, int rows, int K,
                                int Kp, __nv_bfloat16* out, int64_t slice_stride, double inv,
                                cudaStream_t s);
+cudaError_t launch_batch_slices(const double* src, int64_t src_stride, int count, int rows,
+                                int cols, int ld, unsigned long long* amax, int* e, int* flag,
+                                __nv_bfloat16* dn, int Kd, int64_t stride_n, __nv_bfloat16* dt,
+                                int Nd, int64_t stride_t, cudaStream_t s);
 cudaError_t launch_t2ab_flip_mismatch(const double* t2ab, int n, int v, double tol,
                                      unsigned int* count, cudaStream_t s);
 cudaError_t launch_gather_rows(const void* src, void* dst, const int* list, int nlist,
@@ -595,6 +599,89 @@ struct Run {
   }
 };
 
+// ---- grouped products of the adjoint -----------------------------------------
+// A batch of float64 matrices [rows][cols] as 4 BF16 slices in one or both
+// layouts (launch_batch_slices), each matrix with its own power-of-two scale kept
+// on the device: nothing waits for the host.
+struct SlicedBatch {
+  int count = 0, rows = 0, cols = 0, Kd = 0, Nd = 0;
+  __nv_bfloat16 *n = nullptr, *t = nullptr;
+  int64_t sn = 0, st = 0;
+  int* e = nullptr;
+  unsigned long long* amax = nullptr;
+  static int64_t bytes(int64_t count, int64_t rows, int64_t cols, bool both) {
+    return 8 * count * ((both ? rows * round_up(cols, 32) : 0) + cols * round_up(rows, 32));
+  }
+  int alloc(Arena& A, int count_, int rows_, int cols_, bool want_n, bool want_t) {
+    count = count_;
+    rows = rows_;
+    cols = cols_;
+    Kd = (int)round_up(cols, 32);
+    Nd = (int)round_up(rows, 32);
+    sn = (int64_t)count * rows * Kd;
+    st = (int64_t)count * cols * Nd;
+    if (want_n) TRY(A.get(&n, (size_t)(4 * sn)));
+    if (want_t) TRY(A.get(&t, (size_t)(4 * st)));
+    TRY(A.get(&e, (size_t)std::max(count, 1)));
+    TRY(A.get(&amax, (size_t)std::max(count, 1)));
+    return LNO_OT_OK;
+  }
+  int fill(Run& R, const double* src, int64_t stride, int ld, int ncount) {
+    R.stats->other_launches += 3;
+    CU(launch_batch_slices(src, stride, ncount, rows, cols, ld, amax, e, R.ctx->d_flag, n, Kd, sn,
+                           t, Nd, st, R.st));
+    return LNO_OT_OK;
+  }
+  int map(CUtensorMap* m, bool tr, int box) const {
+    return tr ? make_operand_map(m, t, Nd, std::max<int64_t>((int64_t)count * cols, 1), 4, st, box,
+                                 2, 4)
+              : make_operand_map(m, n, Kd, std::max<int64_t>((int64_t)count * rows, 1), 4, sn, box,
+                                 2, 4);
+  }
+};
+
+// One launch of products 2^(ea + eb - 14) sum_k a[m][k] b[n][k], m < M, n < N, into
+// out[n][m] (mode kOutRows) or out[m][n] (kOutF64Rows), over slices of two batches
+// (ta, tb: their transposed layouts).  a takes the longer side: row tiles are 256.
+int grouped_products(Run& R, Arena& A, const std::vector<TcProb>& pr, const SlicedBatch& a,
+                     bool ta, const SlicedBatch& b, bool tb, int M, int N, int ldo, int mode) {
+  if (pr.empty() || M <= 0 || N <= 0) return LNO_OT_OK;
+  const PairTile t = pair_tile(4, N, 128);
+  CUtensorMap mA[2], mB[2];
+  TRY(a.map(&mA[0], ta, 128));
+  TRY(b.map(&mB[0], tb, t.w / 2));
+  mA[1] = mA[0];
+  mB[1] = mB[0];
+  TcProb* dp;
+  TRY(A.get(&dp, pr.size()));
+  cudaEvent_t e0 = R.event(), e1 = R.event();
+  if (e0) cudaEventRecord(e0, R.st);
+  CU(cudaMemcpyAsync(dp, pr.data(), pr.size() * sizeof(TcProb), cudaMemcpyHostToDevice, R.st));
+  CU((launch_tc_pair_f64_group<4, kFmtBF16>(mA, mB, dp, (int)pr.size(), M, N, ldo, 1.0,
+                                            R.ctx->d_flag, R.ctx->nsm, R.st, mode, t)));
+  if (e1) cudaEventRecord(e1, R.st);
+  if (e0 && e1) R.contract_ev.push_back({e0, e1});
+  R.stats->contract_launches++;
+  A.drop(dp);
+  return LNO_OT_OK;
+}
+
+// Problems of one product, its k range in chunks of at most `chunk` (enough
+// problems for the device, and class sums within what FP32 holds exactly).
+void add_chunks(std::vector<TcProb>& out, int a_row, int b_row, int K, bool neg, double* dst,
+                int flags, const int* ea, const int* eb, int chunk = 4096) {
+  for (int k = 0; k < K; k += chunk) {
+    TcProb p{};
+    p.nseg = 1;
+    p.seg[0] = TcSeg{0, 0, a_row, b_row, std::min(chunk, K - k), neg ? 1 : 0, k};
+    p.flags = flags | kTcFloatRest;
+    p.out = dst;
+    p.ea = ea;
+    p.eb = eb;
+    out.push_back(p);
+  }
+}
+
 // Spin-case triplet selection.
 struct CaseSel {
   std::vector<Trip> trips;   // triplets to compute, in output order
@@ -812,14 +899,38 @@ struct SpinPass {
       const auto runs = orb_runs(list, l_rows * r_rows);
       double* buf;
       TRY(block(&buf, l_rows * r_rows * longest(runs)));
+      // adjoint on the tensor cores: one launch per run as well, each orbital's rows
+      // with their own scale
+      SlicedBatch sL, sR;
+      const bool sliced = R.tc_adjoint && !runs.empty() && l_rows > 0 && r_rows > 0;
+      if (sliced) {
+        const int norb = (int)(Ro.total_rows() / r_rows);
+        TRY(sL.alloc(A, 1, (int)l_rows, R.naux, true, false));
+        TRY(sL.fill(R, L.f64, 0, L.Kp, 1));
+        TRY(sR.alloc(A, norb, r_rows, R.naux, true, false));
+        TRY(sR.fill(R, Ro.f64, (int64_t)r_rows * Ro.Kp, Ro.Kp, norb));
+      }
       for (const OrbRun& r : runs) {
-        TRY(R.df(L, 0, (int)l_rows, Ro, (int64_t)r.x * r_rows, r.n * r_rows, buf, (int)l_rows));
+        if (sliced) {
+          std::vector<TcProb> pr;
+          for (int i = 0; i < r.n; ++i)
+            add_chunks(pr, 0, (r.x + i) * r_rows, R.naux, false, buf + i * l_rows * r_rows, 0,
+                       sL.e, sR.e + r.x + i, R.naux);
+          TRY(grouped_products(R, A, pr, sL, false, sR, false, (int)l_rows, r_rows, (int)l_rows,
+                               kOutRows));
+        } else {
+          TRY(R.df(L, 0, (int)l_rows, Ro, (int64_t)r.x * r_rows, r.n * r_rows, buf, (int)l_rows));
+        }
         if (!meas) {
           R.stats->other_launches++;
           CU(pack(r, buf));
         }
       }
       drop(buf);
+      if (sliced)
+        for (void* q : {(void*)sL.n, (void*)sL.e, (void*)sL.amax, (void*)sR.n, (void*)sR.e,
+                        (void*)sR.amax})
+          A.drop(q);
       return LNO_OT_OK;
     };
     // ---- same-spin operands -------------------------------------------------
@@ -969,16 +1080,13 @@ struct SpinPass {
 
   // ---- contraction launches -------------------------------------------------
   int contract(int nprob, int M, int N, int ldo, const Operand& opA0, const Operand& opA1,
-               const Operand& opB0, const Operand& opB1, const std::vector<ProbF64>& pf,
-               const std::vector<TcProb>& pt, ProbF64* dpf, TcProb* dpt,
-               TcOut lay = TcOut{kOutRows, 0, 0, 0}) {
+               const Operand& opB0, const Operand& opB1, const ProbF64* dpf, const TcProb* dpt,
+               TcOut lay) {
     cudaEvent_t e0 = R.event(), e1 = R.event();
     if (e0) cudaEventRecord(e0, R.st);
     if (R.f64) {
-      CU(cudaMemcpyAsync(dpf, pf.data(), nprob * sizeof(ProbF64), cudaMemcpyHostToDevice, R.st));
       CU(launch_gemm_f64(dpf, nprob, M, N, ldo, R.st));
     } else {
-      CU(cudaMemcpyAsync(dpt, pt.data(), nprob * sizeof(TcProb), cudaMemcpyHostToDevice, R.st));
       const double scale = R.sigT * R.sigI * std::ldexp(1.0, R.f16 ? -19 : R.tf32 ? -20 : -14);
       CU(launch_contract(R.S, R.fmt(), bn, opA0, opA1, opB0, opB1, dpt, nprob, M, N, ldo, scale,
                          R.ctx->d_flag, R.ctx->nsm, R.st, lay));
@@ -986,6 +1094,14 @@ struct SpinPass {
     if (e1) cudaEventRecord(e1, R.st);
     if (e0 && e1) R.contract_ev.push_back({e0, e1});
     R.stats->contract_launches++;
+    return LNO_OT_OK;
+  }
+
+  template <typename T>
+  int upload(Arena& A, const std::vector<T>& h, T** d) {
+    if (h.empty()) return LNO_OT_OK;
+    TRY(A.get(d, h.size()));
+    CU(cudaMemcpyAsync(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, R.st));
     return LNO_OT_OK;
   }
 
@@ -1086,15 +1202,6 @@ struct SpinPass {
     const bool fuse = fov && !f64 && is_mixed;
     float* vtab = nullptr;
     if (!f64) TRY(A.get(&vtab, (size_t)(G * vt_stride * (fuse ? 2 : 1))));
-    ProbF64* dpf = nullptr;
-    TcProb* dpt = nullptr;
-    if (f64) {
-      TRY(A.get(&dpf, (size_t)G));
-    } else {
-      TRY(A.get(&dpt, (size_t)G));
-    }
-    std::vector<ProbF64> pf(G), pf2(G);
-    std::vector<TcProb> pt(G), pt2(G);
     double* eout = is_mixed ? e_mixed : e_same;
 
     EnergyArgs ea{};
@@ -1138,86 +1245,89 @@ struct SpinPass {
     R.stats->elements += (int64_t)ntrip *
                          (is_mixed ? npairs(v) * vt : (int64_t)v * (v - 1) * (v - 2) / 6);
 
+    // Contraction problems of every triplet, uploaded once: a copy from pageable
+    // memory waits for the stream, so one per group kept the launches from running
+    // ahead of the device
+    std::vector<ProbF64> pf(f64 ? ntrip : 0), pf2(f64 && is_mixed ? ntrip : 0);
+    std::vector<TcProb> pt(f64 ? 0 : ntrip), pt2(!f64 && is_mixed ? ntrip : 0);
+    for (int q = 0; q < ntrip; ++q) {
+      const Trip tr = cs.trips[q];
+      const int g = q % G;   // its place in its group
+      const int i = tr.i, j = tr.j, k = tr.k;
+      char* Xg = X + (size_t)g * xs * esz;
+      if (!is_mixed) {
+        const int64_t r_jk = (int64_t)slotAT[(size_t)j * o + k] * v;
+        const int64_t r_ki = (int64_t)slotAT[(size_t)k * o + i] * v;
+        const int64_t r_ij = (int64_t)slotAT[(size_t)i * o + j] * v;
+        const int64_t b_i = slotBT[i] * npairs(v), b_j = slotBT[j] * npairs(v),
+                      b_k = slotBT[k] * npairs(v);
+        if (f64) {
+          ProbF64& p = pf[q];
+          p.nseg = 3;
+          seg_f64(p.seg[0], AT, r_jk, BT, b_i, 1.0);
+          seg_f64(p.seg[1], AT, r_ki, BT, b_j, 1.0);
+          seg_f64(p.seg[2], AT, r_ij, BT, b_k, 1.0);
+          p.XT = reinterpret_cast<double*>(Xg);
+        } else {
+          TcProb& p = pt[q];
+          p.nseg = 3;
+          seg_tc(p.seg[0], 0, AT, r_jk, 0, BT, b_i, 0);
+          seg_tc(p.seg[1], 0, AT, r_ki, 0, BT, b_j, 0);
+          seg_tc(p.seg[2], 0, AT, r_ij, 0, BT, b_k, 0);
+          p.out = Xg;
+        }
+      } else {
+        const int K = k;
+        const int64_t a1_jK = (int64_t)slotA1[(size_t)j * ot + K] * v;
+        const int64_t a1_iK = (int64_t)slotA1[(size_t)i * ot + K] * v;
+        const int64_t at_ij = (int64_t)slotAT[(size_t)i * o + j] * v;
+        const int64_t bg_i = (int64_t)slotBG[i] * v * vt, bg_j = (int64_t)slotBG[j] * v * vt;
+        const int64_t bf_K = (int64_t)slotBF[K] * v * vt;
+        const int64_t a2_jK = (int64_t)slotAT2[(size_t)j * ot + K] * vt;
+        const int64_t a2_iK = (int64_t)slotAT2[(size_t)i * ot + K] * vt;
+        const int64_t bt_i = slotBT[i] * npairs(v), bt_j = slotBT[j] * npairs(v);
+        char* Zg = Z + (size_t)g * zs * esz;
+        if (f64) {
+          ProbF64& p = pf[q];
+          p.nseg = 3;
+          seg_f64(p.seg[0], A1, a1_jK, BG, bg_i, 1.0);
+          seg_f64(p.seg[1], A1, a1_iK, BG, bg_j, -1.0);
+          seg_f64(p.seg[2], AT, at_ij, BF, bf_K, 1.0);
+          p.XT = reinterpret_cast<double*>(Xg);
+          ProbF64& p2 = pf2[q];
+          p2.nseg = 2;
+          seg_f64(p2.seg[0], AT2, a2_jK, BT, bt_i, -1.0);
+          seg_f64(p2.seg[1], AT2, a2_iK, BT, bt_j, 1.0);
+          p2.XT = reinterpret_cast<double*>(Zg);
+        } else {
+          TcProb& p = pt[q];
+          p.nseg = 3;
+          seg_tc(p.seg[0], 0, A1, a1_jK, 0, BG, bg_i, 0);
+          seg_tc(p.seg[1], 0, A1, a1_iK, 0, BG, bg_j, 1);
+          seg_tc(p.seg[2], 1, AT, at_ij, 1, BF, bf_K, 0);
+          p.out = Xg;
+          TcProb& p2 = pt2[q];
+          p2.nseg = 2;
+          seg_tc(p2.seg[0], 0, AT2, a2_jK, 0, BT, bt_i, 1);
+          seg_tc(p2.seg[1], 0, AT2, a2_iK, 0, BT, bt_j, 0);
+          p2.out = Zg;
+        }
+      }
+    }
+    ProbF64 *dpf = nullptr, *dpf2 = nullptr;
+    TcProb *dpt = nullptr, *dpt2 = nullptr;
+    TRY(upload(A, pf, &dpf));
+    TRY(upload(A, pf2, &dpf2));
+    TRY(upload(A, pt, &dpt));
+    TRY(upload(A, pt2, &dpt2));
+
     for (int g0 = 0; g0 < ntrip; g0 += G) {
       const int ng = std::min(G, ntrip - g0);
-      for (int g = 0; g < ng; ++g) {
-        const Trip tr = cs.trips[g0 + g];
-        const int i = tr.i, j = tr.j, k = tr.k;
-        char* Xg = X + (size_t)g * xs * esz;
-        if (!is_mixed) {
-          const int64_t r_jk = (int64_t)slotAT[(size_t)j * o + k] * v;
-          const int64_t r_ki = (int64_t)slotAT[(size_t)k * o + i] * v;
-          const int64_t r_ij = (int64_t)slotAT[(size_t)i * o + j] * v;
-          const int64_t b_i = slotBT[i] * npairs(v), b_j = slotBT[j] * npairs(v),
-                        b_k = slotBT[k] * npairs(v);
-          if (f64) {
-            ProbF64& p = pf[g];
-            p.nseg = 3;
-            seg_f64(p.seg[0], AT, r_jk, BT, b_i, 1.0);
-            seg_f64(p.seg[1], AT, r_ki, BT, b_j, 1.0);
-            seg_f64(p.seg[2], AT, r_ij, BT, b_k, 1.0);
-            p.XT = reinterpret_cast<double*>(Xg);
-          } else {
-            TcProb& p = pt[g];
-            p.nseg = 3;
-            seg_tc(p.seg[0], 0, AT, r_jk, 0, BT, b_i, 0);
-            seg_tc(p.seg[1], 0, AT, r_ki, 0, BT, b_j, 0);
-            seg_tc(p.seg[2], 0, AT, r_ij, 0, BT, b_k, 0);
-            p.out = Xg;
-          }
-        } else {
-          const int K = k;
-          const int64_t a1_jK = (int64_t)slotA1[(size_t)j * ot + K] * v;
-          const int64_t a1_iK = (int64_t)slotA1[(size_t)i * ot + K] * v;
-          const int64_t at_ij = (int64_t)slotAT[(size_t)i * o + j] * v;
-          const int64_t bg_i = (int64_t)slotBG[i] * v * vt, bg_j = (int64_t)slotBG[j] * v * vt;
-          const int64_t bf_K = (int64_t)slotBF[K] * v * vt;
-          const int64_t a2_jK = (int64_t)slotAT2[(size_t)j * ot + K] * vt;
-          const int64_t a2_iK = (int64_t)slotAT2[(size_t)i * ot + K] * vt;
-          const int64_t bt_i = slotBT[i] * npairs(v), bt_j = slotBT[j] * npairs(v);
-          char* Zg = Z + (size_t)g * zs * esz;
-          if (f64) {
-            ProbF64& p = pf[g];
-            p.nseg = 3;
-            seg_f64(p.seg[0], A1, a1_jK, BG, bg_i, 1.0);
-            seg_f64(p.seg[1], A1, a1_iK, BG, bg_j, -1.0);
-            seg_f64(p.seg[2], AT, at_ij, BF, bf_K, 1.0);
-            p.XT = reinterpret_cast<double*>(Xg);
-            ProbF64& q = pf2[g];
-            q.nseg = 2;
-            seg_f64(q.seg[0], AT2, a2_jK, BT, bt_i, -1.0);
-            seg_f64(q.seg[1], AT2, a2_iK, BT, bt_j, 1.0);
-            q.XT = reinterpret_cast<double*>(Zg);
-          } else {
-            TcProb& p = pt[g];
-            p.nseg = 3;
-            seg_tc(p.seg[0], 0, A1, a1_jK, 0, BG, bg_i, 0);
-            seg_tc(p.seg[1], 0, A1, a1_iK, 0, BG, bg_j, 1);
-            seg_tc(p.seg[2], 1, AT, at_ij, 1, BF, bf_K, 0);
-            p.out = Xg;
-            TcProb& q = pt2[g];
-            q.nseg = 2;
-            seg_tc(q.seg[0], 0, AT2, a2_jK, 0, BT, bt_i, 1);
-            seg_tc(q.seg[1], 0, AT2, a2_iK, 0, BT, bt_j, 0);
-            q.out = Zg;
-          }
-        }
-      }
-      if (!is_mixed) {
-        TRY(contract(ng, M1, (int)N1, P1, AT, AT, BT, BT, pf, pt, dpf, dpt));
-      } else {
-        TRY(contract(ng, M1, (int)N1, P1, A1, AT, BG, BF, pf, pt, dpf, dpt, lay1));
-        ProbF64* dpf2 = nullptr;
-        TcProb* dpt2 = nullptr;
-        // second problem list uses its own device array (the first may still be read)
-        if (f64) {
-          TRY(A.get(&dpf2, (size_t)ng));
-        } else {
-          TRY(A.get(&dpt2, (size_t)ng));
-        }
-        TRY(contract(ng, M2, (int)N2, P2, AT2, AT2, BT, BT, pf2, pt2, dpf2, dpt2, lay2));
-        A.drop(f64 ? (void*)dpf2 : (void*)dpt2);
-      }
+      TRY(contract(ng, M1, (int)N1, P1, is_mixed ? A1 : AT, AT, is_mixed ? BG : BT,
+                   is_mixed ? BF : BT, f64 ? dpf + g0 : nullptr, f64 ? nullptr : dpt + g0, lay1));
+      if (is_mixed)
+        TRY(contract(ng, M2, (int)N2, P2, AT2, AT2, BT, BT, f64 ? dpf2 + g0 : nullptr,
+                     f64 ? nullptr : dpt2 + g0, lay2));
       // energy
       ea.trips = dtrips + g0;
       ea.partial = partial;
@@ -1263,9 +1373,6 @@ struct SpinPass {
       if (e1) cudaEventRecord(e1, R.st);
       if (e0 && e1) R.energy_ev.push_back({e0, e1});
       R.stats->energy_launches += 2;
-      // no host sync: the next group's descriptors overwrite pf/pt only after
-      // cudaMemcpyAsync has staged this group's (pageable source), and the
-      // device array is reused in stream order after this group's kernels
     }
     return LNO_OT_OK;
   }
@@ -1948,7 +2055,7 @@ int tc_matmul(Run& R, Arena& A, int M, int N, int K, View a, View b, double* C, 
                                                        K / 2048, kMaxSplit}));
   const int Kc = (int)round_up(ceil_div(K, nsp), 32);
   nsp = ceil_div(K, Kc);
-  const int64_t Kp = round_up(Kc, 8);
+  const int64_t Kp = round_up(Kc, 32);
   // a read-only B view sliced before with the same chunking
   const SliceCacheEntry* hit = nullptr;
   if (b_const)
@@ -1999,34 +2106,32 @@ int tc_matmul(Run& R, Arena& A, int M, int N, int K, View a, View b, double* C, 
   // the kernel writes its output transposed: its rows (A role) are n, its
   // columns (B role) m, so out[m ldc + n]
   CUtensorMap mA[2], mB[2];
-  TRY(make_operand_map(&mA[0], qb, Kp, (int64_t)nsp * N, S, (int64_t)nsp * N * Kp, 128));
-  TRY(make_operand_map(&mB[0], qa, Kp, (int64_t)nsp * M, S, (int64_t)nsp * M * Kp, 128));
+  const PairTile tile = pair_tile(S, M, 128);
+  TRY(make_operand_map(&mA[0], qb, Kp, (int64_t)nsp * N, S, (int64_t)nsp * N * Kp, 128, 2, S));
+  TRY(make_operand_map(&mB[0], qa, Kp, (int64_t)nsp * M, S, (int64_t)nsp * M * Kp, tile.w / 2, 2,
+                       S));
   mA[1] = mA[0];
   mB[1] = mB[0];
   double* part = nullptr;
   if (nsp > 1) TRY(A.get(&part, (size_t)nsp * M * N));
-  // the float32 rest scales in float32: |alpha| must be a power of two (the
+  // the output is formed with a power-of-two scale: |alpha| must be one (the
   // adjoint's products use +-1)
   int ex;
   if (std::frexp(std::fabs(alpha), &ex) != 0.5) return LNO_OT_EINVAL;
   const double scale = sa * sb * std::ldexp(1.0, -14) * std::fabs(alpha);
-  // products of the class sums with the scale stay normal floats
-  const bool float_rest = scale >= std::ldexp(1.0, -100) && scale <= std::ldexp(1.0, 100);
   std::vector<TcProb> pv(nsp);
   for (int c = 0; c < nsp; ++c) {
     TcProb& p = pv[c];
     p.nseg = 1;
     p.seg[0] = TcSeg{0, 0, c * N, c * M, std::min(Kc, K - c * Kc), alpha < 0 ? 1 : 0};
-    p.flags = (float_rest ? kTcFloatRest : 0) | (nsp == 1 && accum ? kTcAccum : 0);
+    p.flags = kTcFloatRest | (nsp == 1 && accum ? kTcAccum : 0);
     p.out = nsp == 1 ? C : part + (int64_t)c * M * N;
   }
   TcProb* dp;
   TRY(A.get(&dp, (size_t)nsp));
   CU(cudaMemcpyAsync(dp, pv.data(), nsp * sizeof(TcProb), cudaMemcpyHostToDevice, st));
-  CU((launch_tc_gemm<4, 128, double, false>(mA, mB, dp, nsp, N, M,
-                                                   nsp == 1 ? (int)ldc : N, scale,
-                                                   R.ctx->d_flag, nullptr, R.ctx->nsm, st,
-                                                   tc_normal())));
+  CU((launch_tc_pair_f64_group<S, kFmtBF16>(mA, mB, dp, nsp, N, M, nsp == 1 ? (int)ldc : N, scale,
+                                            R.ctx->d_flag, R.ctx->nsm, st, kOutRows, tile)));
   if (nsp > 1) CU(launch_sum_partials(part, nsp, M, N, C, ldc, accum, st));
   if (e1) cudaEventRecord(e1, st);
   if (e0 && e1) R.contract_ev.push_back({e0, e1});
@@ -2068,6 +2173,11 @@ int df_adjoint(Run& R, Arena& A, const Operand& Lo, Operand& dL, int64_t l0, int
   return LNO_OT_OK;
 }
 
+// Operands of the adjoint in the batched form: slices of every slot in both
+// layouts, kept while they are within kBatchBytes; otherwise the products run one
+// by one (tc_matmul), slicing what they need.
+constexpr int64_t kBatchBytes = (int64_t)8 << 30;
+
 int backward_spin(SpinPass& P, GradAcc& G, double gE) {
   Run& R = P.R;
   cudaStream_t st = R.st;
@@ -2090,6 +2200,31 @@ int backward_spin(SpinPass& P, GradAcc& G, double gE) {
   double* dt2ss = s == 0 ? G.dt2aa : G.dt2bb;
   double* dt2st = G.dt2ab;
   if (s == 1 && !P.mixed.trips.empty()) TRY(zeros(A, &dt2st, (int64_t)o * ot * v * vt, st));
+
+  // slices of all operand slots (batched form)
+  const Operand* ops[6] = {&P.AT, &P.BT, &P.A1, &P.BG, &P.BF, &P.AT2};
+  SlicedBatch sl[6];
+  bool batched = R.tc_adjoint;
+  if (batched) {
+    int64_t bytes = 0;
+    for (const Operand* op : ops) {
+      if (op->nslot * op->rows == 0) continue;
+      bytes += SlicedBatch::bytes(op->nslot, op->rows, op->K, true);
+      batched = batched && op->nslot <= 65535 && op->rows <= (1 << 20);
+    }
+    batched = batched && bytes <= kBatchBytes;
+  }
+  if (batched)
+    for (int q = 0; q < 6; ++q) {
+      if (ops[q]->nslot * ops[q]->rows == 0) continue;
+      TRY(sl[q].alloc(A, ops[q]->nslot, (int)ops[q]->rows, ops[q]->K, true, true));
+      TRY(sl[q].fill(R, ops[q]->f64, ops[q]->rows * ops[q]->Kp, ops[q]->Kp, ops[q]->nslot));
+    }
+  auto sliced = [&](const Operand* op) -> const SlicedBatch& {
+    for (int q = 0; q < 6; ++q)
+      if (ops[q] == op) return sl[q];
+    return sl[0];
+  };
 
   // ---- per case: recompute, energy adjoint, contraction adjoint ------------
   for (int im = 0; im < 2; ++im) {
@@ -2132,6 +2267,11 @@ int backward_spin(SpinPass& P, GradAcc& G, double gE) {
     CU(cudaMemcpyAsync(dtrips, cs.trips.data(), ntrip * sizeof(Trip), cudaMemcpyHostToDevice,
                        st));
     const int Pch = std::max(1, std::min((int)blocks.size(), R.ctx->nsm * 4 / Gn + 1));
+    SlicedBatch sx, sz;   // slices of a group's dX and dZ'
+    if (batched) {
+      TRY(sx.alloc(A, Gn, (int)N1, M1, true, true));
+      if (is_mixed) TRY(sz.alloc(A, Gn, (int)N2, M2, true, true));
+    }
     EnergyArgs ea{};
     ea.kind = is_mixed ? MIXED : SAME;
     ea.nvs = v;
@@ -2197,7 +2337,34 @@ int backward_spin(SpinPass& P, GradAcc& G, double gE) {
         if (is_mixed) fill(pf2[g], segs2[g], Z + (size_t)g * N2 * P2);
       }
       // recompute X (and Z')
-      if (R.tc_adjoint) {
+      if (batched) {
+        // XT[n][m] = sum_seg sign A[arow+m][:] . B[brow+n][:]: segment q of all the
+        // group's triplets in one launch, the later ones added
+        auto recompute = [&](const std::vector<std::vector<SegRef>>& segs, double* Xb, int64_t Nn,
+                             int Mm, int ldo) -> int {
+          for (size_t q = 0; q < segs[0].size(); ++q) {
+            std::vector<TcProb> pr;
+            const SegRef& r0 = segs[0][q];
+            const SlicedBatch &a = sliced(r0.A), &b = sliced(r0.B);
+            for (int g = 0; g < ng; ++g) {
+              const SegRef& r = segs[g][q];
+              const int ia = (int)(r.arow / a.rows), ib = (int)(r.brow / b.rows);
+              TcProb p{};
+              p.nseg = 1;
+              p.seg[0] = TcSeg{0, 0, (int)r.brow, (int)r.arow, r.A->K, r.sign < 0 ? 1 : 0, 0};
+              p.flags = kTcFloatRest | (q > 0 ? kTcAccum : 0);
+              p.out = Xb + (size_t)g * Nn * ldo;
+              p.ea = b.e + ib;
+              p.eb = a.e + ia;
+              pr.push_back(p);
+            }
+            TRY(grouped_products(R, A, pr, b, false, a, false, (int)Nn, Mm, ldo, kOutF64Rows));
+          }
+          return LNO_OT_OK;
+        };
+        TRY(recompute(segs1, X, N1, M1, P1));
+        if (is_mixed) TRY(recompute(segs2, Z, N2, M2, P2));
+      } else if (R.tc_adjoint) {
         // XT[n][m] = sum_seg sign A[arow+m][:] . B[brow+n][:], one tensor-core
         // product per segment, the later ones added
         auto recompute = [&](const std::vector<std::vector<SegRef>>& segs, double* Xb, int64_t Nn,
@@ -2242,6 +2409,45 @@ int backward_spin(SpinPass& P, GradAcc& G, double gE) {
         CU(launch_energy_backward(ef, X, Z, dX, dZ, G.dfov[s], G.dfov[is_mixed ? t : s], dt2ss,
                                   dt2st, G.deps[s], G.deps[is_mixed ? t : s], gE, ng, Pch, st));
         R.stats->energy_launches += 1;
+      }
+      // contraction adjoint, batched: per operand pair (A, B) one launch of
+      // dA[arow+m][k] += s sum_n dX[n][m] B[brow+n][k] over all triplets and
+      // segments, one of dB[brow+n][k] += s sum_m dX[n][m] A[arow+m][k]
+      auto adj_batched = [&](const std::vector<std::vector<SegRef>>& segs, const SlicedBatch& dx,
+                             int64_t Nn, int Mm) -> int {
+        std::vector<bool> done(segs[0].size(), false);
+        for (size_t q0 = 0; q0 < segs[0].size(); ++q0) {
+          if (done[q0]) continue;
+          const SegRef& r0 = segs[0][q0];
+          const SlicedBatch &a = sliced(r0.A), &b = sliced(r0.B);
+          std::vector<TcProb> pa, pb;
+          for (size_t q = q0; q < segs[0].size(); ++q) {
+            if (segs[0][q].A != r0.A || segs[0][q].B != r0.B) continue;
+            done[q] = true;
+            for (int g = 0; g < ng; ++g) {
+              const SegRef& r = segs[g][q];
+              const int ia = (int)(r.arow / a.rows), ib = (int)(r.brow / b.rows);
+              add_chunks(pa, ib * b.cols, g * Mm, (int)Nn, r.sign < 0,
+                         r.dA->f64 + r.arow * r.A->Kp, kTcAtomic, b.e + ib, dx.e + g);
+              add_chunks(pb, (int)(g * Nn), ia * a.cols, Mm, r.sign < 0,
+                         r.dB->f64 + r.brow * r.B->Kp, kTcAtomic, dx.e + g, a.e + ia);
+            }
+          }
+          TRY(grouped_products(R, A, pa, b, true, dx, true, r0.A->K, Mm, r0.A->Kp, kOutRows));
+          TRY(grouped_products(R, A, pb, dx, false, a, true, (int)Nn, r0.A->K, r0.B->Kp,
+                               kOutF64Rows));
+        }
+        return LNO_OT_OK;
+      };
+      if (batched) {
+        TRY(sx.fill(R, dX, N1 * P1, P1, ng));
+        TRY(adj_batched(segs1, sx, N1, M1));
+        if (is_mixed) {
+          TRY(sz.fill(R, dZ, N2 * P2, P2, ng));
+          TRY(adj_batched(segs2, sz, N2, M2));
+        }
+        R.stats->energy_launches += 1;
+        continue;
       }
       // contraction adjoint: dA += sign dX.B, dB += sign dX^T.A
       auto adj = [&](const std::vector<std::vector<SegRef>>& segs, const double* dXb, int64_t Nn,
@@ -2312,7 +2518,70 @@ int backward_spin(SpinPass& P, GradAcc& G, double gE) {
                    o * o));
     A.drop(doovoT);
   }
-  if (!P.listBT.empty()) {
+  // Per-orbital DF blocks, batched: a run of orbitals x, x + 1, ... at a time,
+  // dout[x][n][m] (n < r_rows, m < l_rows): dL[m][Q] += sum_n dout R[x r_rows + n][Q],
+  // dR[x r_rows + n][Q] += sum_m dout L[m][Q].
+  auto per_orbital = [&](const std::vector<int>& list, const Operand& L, Operand& dL,
+                         int64_t l_rows, const Operand& Ro, Operand& dR, int r_rows,
+                         auto&& layout) -> int {
+    const auto runs = SpinPass::orb_runs(list, l_rows * r_rows);
+    const int nmax = SpinPass::longest(runs);
+    if (nmax == 0 || l_rows == 0 || r_rows == 0) return LNO_OT_OK;
+    const int64_t blk = l_rows * r_rows;
+    const int norb = (int)(Ro.total_rows() / r_rows);
+    double* dout;
+    TRY(A.get(&dout, (size_t)(blk * nmax)));
+    SlicedBatch sL, sR, sd;
+    TRY(sL.alloc(A, 1, (int)l_rows, R.naux, false, true));
+    TRY(sL.fill(R, L.f64, 0, L.Kp, 1));
+    TRY(sR.alloc(A, norb, r_rows, R.naux, false, true));
+    TRY(sR.fill(R, Ro.f64, (int64_t)r_rows * Ro.Kp, Ro.Kp, norb));
+    TRY(sd.alloc(A, nmax, r_rows, (int)l_rows, true, true));
+    for (const auto& r : runs) {
+      CU(cudaMemsetAsync(dout, 0, (size_t)(blk * r.n) * sizeof(double), st));
+      for (int i = 0; i < r.n; ++i) CU(layout(r.q + i, r.x + i, dout + i * blk));
+      TRY(sd.fill(R, dout, blk, (int)l_rows, r.n));
+      std::vector<TcProb> pl, pr;
+      for (int i = 0; i < r.n; ++i) {
+        const int x = r.x + i;
+        add_chunks(pl, (int)(i * l_rows), x * R.naux, r_rows, false, dL.f64, kTcAtomic, sd.e + i,
+                   sR.e + x);
+        add_chunks(pr, 0, i * r_rows, (int)l_rows, false, dR.f64 + (int64_t)x * r_rows * dR.Kp,
+                   kTcAtomic, sL.e, sd.e + i);
+      }
+      TRY(grouped_products(R, A, pl, sd, true, sR, true, (int)l_rows, R.naux, dL.Kp,
+                           kOutF64Rows));
+      TRY(grouped_products(R, A, pr, sL, true, sd, false, R.naux, r_rows, dR.Kp, kOutRows));
+    }
+    A.drop(dout);
+    for (SlicedBatch* b : {&sL, &sR, &sd}) {
+      if (b->n) A.drop(b->n);
+      A.drop(b->t);
+      A.drop(b->e);
+      A.drop(b->amax);
+    }
+    return LNO_OT_OK;
+  };
+  // within the run and slice budgets (one orbital's block may not be)
+  const bool batched_df = batched && 24 * (int64_t)v * v * std::max(v, vt) <= kBatchBytes &&
+                          24 * (int64_t)vt * vt * v <= kBatchBytes &&
+                          SlicedBatch::bytes(1, (int64_t)std::max(v, vt) * std::max(v, vt), R.naux,
+                                             false) <= kBatchBytes;
+  if (batched_df) {
+    TRY(per_orbital(P.listBT, R.Bvv[s], G.dBvv[s], (int64_t)v * v, R.Bov[s], G.dBov[s], v,
+                    [&](int q, int x, double* d) {
+                      return launch_adj_bt_same(q, x, o, v, dBT.Kp, dBT.f64, d, dt2ss, st);
+                    }));
+    TRY(per_orbital(P.listBG, R.Bvv[t], G.dBvv[t], (int64_t)vt * vt, R.Bov[s], G.dBov[s], v,
+                    [&](int q, int x, double* d) {
+                      return launch_adj_bg(q, x, o, v, ot, vt, dBG.Kp, dBG.f64, d, dt2st, st);
+                    }));
+    TRY(per_orbital(P.listBF, R.Bvv[s], G.dBvv[s], (int64_t)v * v, R.Bov[t], G.dBov[t], vt,
+                    [&](int q, int x, double* d) {
+                      return launch_adj_bf(q, x, o, v, ot, vt, dBF.Kp, dBF.f64, d, dt2st, st);
+                    }));
+  }
+  if (!batched_df && !P.listBT.empty()) {
     double* dvv;
     TRY(A.get(&dvv, (size_t)v * v * v));
     for (size_t q = 0; q < P.listBT.size(); ++q) {
@@ -2334,7 +2603,7 @@ int backward_spin(SpinPass& P, GradAcc& G, double gE) {
                    o * v));
     A.drop(djT);
   }
-  if (!P.listBG.empty()) {
+  if (!batched_df && !P.listBG.empty()) {
     double* dgT;
     TRY(A.get(&dgT, (size_t)v * vt * vt));
     for (size_t q = 0; q < P.listBG.size(); ++q) {
@@ -2346,7 +2615,7 @@ int backward_spin(SpinPass& P, GradAcc& G, double gE) {
     }
     A.drop(dgT);
   }
-  if (!P.listBF.empty()) {
+  if (!batched_df && !P.listBF.empty()) {
     double* dfT;
     TRY(A.get(&dfT, (size_t)vt * v * v));
     for (size_t q = 0; q < P.listBF.size(); ++q) {
@@ -2498,6 +2767,7 @@ int backward_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, double gE, lno_ot_g
   CU(cudaStreamSynchronize(R.st));
   int flag = 0;
   CU(cudaMemcpy(&flag, ctx->d_flag, sizeof flag, cudaMemcpyDeviceToHost));
+  if (flag == 9) return LNO_OT_EINVAL;   // an infinite operand (slice_exponents)
   if (flag) return LNO_OT_ETIMEOUT;
   // stats of the adjoint: ms_total wall clock, ms_stage the staging plus the
   // operand and V-block builds (their DF assembly), ms_contract the event time

@@ -300,6 +300,12 @@ struct StoreSlicesInt {
   int64_t slice_stride;
   int e2;   // log2(2^7 / scale) + 8 (S - 1)
   __device__ __forceinline__ void operator()(int64_t idx, double v) const {
+    if (isnan(v)) {   // NaN in the leading slice reaches the product
+      p[idx] = __float2bfloat16_rn(__int_as_float(0x7fc00000));
+#pragma unroll
+      for (int q = 1; q < S; ++q) p[q * slice_stride + idx] = __float2bfloat16_rn(0.f);
+      return;
+    }
     int64_t R = round_scaled(v, e2);
 #pragma unroll
     for (int q = 0; q < S; ++q) {
@@ -310,6 +316,69 @@ struct StoreSlicesInt {
     }
   }
 };
+
+// Matrices of a batch, each rows x cols float64 at src + z src_stride (row pitch
+// ld), sliced in both layouts for the adjoint's grouped products: n [z][r][Kd] (k
+// = column) and t [z][c][Nd] (k = row), Kd and Nd multiples of 32, zero in the
+// pads.  Each matrix has its own scale 2^e[z] (slice_exponents).
+__global__ void batch_absmax(const double* __restrict__ src, int64_t src_stride, int rows,
+                             int cols, int ld, unsigned long long* __restrict__ amax) {
+  const double* p = src + (int64_t)blockIdx.y * src_stride;
+  const int64_t n = (int64_t)rows * cols;
+  double m = 0.0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = i / cols;
+    m = fmax(m, fabs(p[r * ld + (i - r * cols)]));
+  }
+  for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
+  if ((threadIdx.x & 31) == 0 && m > 0.0)
+    atomicMax(amax + blockIdx.y, (unsigned long long)__double_as_longlong(m));
+}
+
+// e = smallest exponent with 2^e >= max (0 for a zero matrix); an infinite
+// maximum raises the error flag (code 9: invalid input).
+__global__ void slice_exponents(const unsigned long long* __restrict__ amax, int n,
+                                int* __restrict__ e, int* __restrict__ flag) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double m = __longlong_as_double((long long)amax[i]);
+    int ex = 0;
+    if (isinf(m)) {
+      atomicCAS(flag, 0, 9);
+    } else if (m > 0.0) {
+      const double f = frexp(m, &ex);
+      if (f == 0.5) --ex;
+    }
+    e[i] = ex;
+  }
+}
+
+template <int S>
+__global__ void batch_slices(const double* __restrict__ src, int64_t src_stride, int rows,
+                             int cols, int ld, const int* __restrict__ e,
+                             __nv_bfloat16* __restrict__ dn, int Kd, int64_t stride_n,
+                             __nv_bfloat16* __restrict__ dt, int Nd, int64_t stride_t) {
+  __shared__ double t[32][33];   // [r][c]
+  const int tx = threadIdx.x, ty = threadIdx.y, z = blockIdx.z;
+  const double* p = src + (int64_t)z * src_stride;
+  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+  for (int i = ty; i < 32; i += 8) {
+    const int r = r0 + i, c = c0 + tx;
+    t[i][tx] = r < rows && c < cols ? p[(int64_t)r * ld + c] : 0.0;
+  }
+  __syncthreads();
+  const int e2 = 7 - e[z] + 8 * (S - 1);
+  if (dn != nullptr) {
+    const StoreSlicesInt<S> st{dn, stride_n, e2};
+    for (int i = ty; i < 32; i += 8)
+      if (r0 + i < rows) st(((int64_t)z * rows + r0 + i) * Kd + c0 + tx, t[i][tx]);
+  }
+  if (dt != nullptr) {
+    const StoreSlicesInt<S> st{dt, stride_t, e2};
+    for (int i = ty; i < 32; i += 8)
+      if (c0 + i < cols) st(((int64_t)z * cols + c0 + i) * Nd + r0 + tx, t[tx][i]);
+  }
+}
 
 // view -> S BF16 slices [s][r][Kp] (k-contiguous rows, zero for k >= K)
 template <int S>
@@ -572,6 +641,24 @@ cudaError_t launch_view_absmax(const double* in, int64_t rs, int64_t ks, int row
   if (rows <= 0 || K <= 0) return cudaSuccess;
   const dim3 grid((unsigned)((K + 31) / 32), (unsigned)std::min((rows + 31) / 32, 4096));
   view_absmax<<<grid, dim3(32, 8), 0, s>>>(in, rs, ks, rows, K, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_slices(const double* src, int64_t src_stride, int count, int rows,
+                                int cols, int ld, unsigned long long* amax, int* e, int* flag,
+                                __nv_bfloat16* dn, int Kd, int64_t stride_n, __nv_bfloat16* dt,
+                                int Nd, int64_t stride_t, cudaStream_t s) {
+  if (count <= 0 || rows <= 0 || cols <= 0) return cudaSuccess;
+  if (count > 65535 || Kd % 32 || Nd % 32) return cudaErrorInvalidValue;
+  cudaError_t rc = cudaMemsetAsync(amax, 0, (size_t)count * sizeof(unsigned long long), s);
+  if (rc != cudaSuccess) return rc;
+  const int bx = (int)std::min<int64_t>(((int64_t)rows * cols + 1023) / 1024, 512);
+  batch_absmax<<<dim3(bx, count), 256, 0, s>>>(src, src_stride, rows, cols, ld, amax);
+  slice_exponents<<<ceil_div(count, 256), 256, 0, s>>>(amax, count, e, flag);
+  const dim3 grid(Kd / 32, Nd / 32, count);
+  if (grid.y > 65535) return cudaErrorInvalidValue;
+  batch_slices<4><<<grid, dim3(32, 8), 0, s>>>(src, src_stride, rows, cols, ld, e, dn, Kd,
+                                               stride_n, dt, Nd, stride_t);
   return cudaGetLastError();
 }
 

@@ -304,8 +304,9 @@ __device__ __forceinline__ double fixed_to_double(int64_t I, int e) {
 // Float64 value of one element's class sums: the exact sum of the classes times
 // 2^e.  Class g is an integer multiple of 2^(-BITS g), or (INTS) that integer; sums too large for the
 // integers (or not finite) become NaN, as the operands' slices say.
+// rest: class 0 plus the float32 sum of the others (BF16, kTcFloatRest).
 template <int S, int BITS, bool INTS>
-__device__ __forceinline__ double class_sum(const float (&c)[S], int e) {
+__device__ __forceinline__ double class_sum(const float (&c)[S], int e, bool rest) {
   int64_t I = 0;
   float w = 1.0f, big = 0.0f;
 #pragma unroll
@@ -317,6 +318,13 @@ __device__ __forceinline__ double class_sum(const float (&c)[S], int e) {
     if (!INTS) w *= (float)(1 << BITS);
   }
   if (!(big < 1073741824.0f)) return __longlong_as_double(0x7ff8000000000000ll);
+  if (!INTS && rest) {
+    float lo = 0.f;
+#pragma unroll
+    for (int g = S - 1; g >= 1; --g) lo = __fadd_rn(lo, c[g]);
+    constexpr float top = (float)(1ll << (BITS * (S - 1)));
+    I = ((int64_t)__float2int_rn(c[0]) << (BITS * (S - 1))) + __float2ll_rn(lo * top);
+  }
   e -= BITS * (S - 1);
   if (e < -960 || e > 960) return ldexp((double)I, e);   // extreme scales only
   return fixed_to_double(I, e);
@@ -421,8 +429,8 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
             if (rank == 0) mbar_expect_tx(full_bar(stage), 2u * (uint32_t)stage_bytes);
             const uint32_t bar = map_rank(full_bar(stage), 0);
             const uint32_t dst = base + (uint32_t)(stage * stage_bytes);
-            tma_load_3d_pair(dst, ma, bar, k0, seg.a_row + ar, 0);
-            tma_load_3d_pair(dst + S * kABytes, mb, bar, k0, seg.b_row + br, 0);
+            tma_load_3d_pair(dst, ma, bar, seg.k0 + k0, seg.a_row + ar, 0);
+            tma_load_3d_pair(dst + S * kABytes, mb, bar, seg.k0 + k0, seg.b_row + br, 0);
             used |= 1u << stage;
             last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
             if (++stage == nst) {
@@ -538,7 +546,8 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
       const int buf = nbuf == 2 ? (int)(it & 1u) : 0;
       const uint32_t use = nbuf == 2 ? it >> 1 : it;
       const int m = mt * 2 * BM + row;
-      void* outp = probs ? probs[pr].out : one.out;
+      const TcProb& P = probs ? probs[pr] : one;
+      void* outp = P.out;
       const bool mok = m < M;
       const int n0 = nt * tile.w;
       const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * S * tile.w);
@@ -587,6 +596,7 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
       } else {
         constexpr int CH = pair_max_width<S, OutT>() / 32;   // 8-column chunks of one warp
         constexpr int BITS = FMT == kFmtBF16 ? 8 : 11;
+        const int es = P.ea ? *P.ea + *P.eb - 14 : escale, fl = P.flags;
         if (!pair_wait(tfull(buf), use & 1u, flag, 6, true, wlim)) break;
         tc_fence_after();
         const int nch = ntile_w(nt) / 8;
@@ -610,7 +620,7 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
               if (amax != nullptr && mok && n0 + chunk * 8 + j < N)
                 lmax = fmaxf(lmax, fabsf(__fmul_rn(lo, scale)));
               if (outp != nullptr)
-                v[c * 8 + j] = class_sum<S, BITS, FMT == kFmtF16>(x, escale);
+                v[c * 8 + j] = class_sum<S, BITS, FMT == kFmtF16>(x, es, fl & kTcFloatRest);
             }
           }
         }
@@ -618,13 +628,21 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
         __syncwarp();
         if (lane == 0) arrive_cluster(map_rank(tempty(buf), 0));
         if (mok && outp != nullptr) {
-          double* out = reinterpret_cast<double*>(outp) + m;
+          const bool rows = lay.mode == kOutF64Rows;   // out[m][n], else out[n][m]
+          double* out = reinterpret_cast<double*>(outp) + (rows ? (int64_t)m * ldo : m);
+          const int64_t step = rows ? 1 : ldo;
 #pragma unroll
           for (int c = 0; c < CH; ++c) {
             const int n = n0 + (4 * c + part) * 8;
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-              if (4 * c + part < nch && n + j < N) out[(int64_t)(n + j) * ldo] = v[c * 8 + j];
+              if (4 * c + part < nch && n + j < N) {
+                double* o = out + (n + j) * step;
+                if (fl & kTcAtomic)
+                  atomicAdd(o, v[c * 8 + j]);
+                else
+                  *o = fl & kTcAccum ? *o + v[c * 8 + j] : v[c * 8 + j];
+              }
           }
         }
       }
@@ -735,6 +753,22 @@ cudaError_t launch_tc_pair_f64(const CUtensorMap* mA, const CUtensorMap* mB, con
   return launch_pair<S, FMT, double>(mA, mB, nullptr, p, 1, M, N, ldo, scale, flag, amax, nsm, st,
                                      tc_normal(), TcOut{kOutRows, 0, 0, 0}, tile);
 }
+
+// A group of such products, each with its own flags and, where TcProb.ea and eb
+// are given, its own scale.
+template <int S, int FMT>
+cudaError_t launch_tc_pair_f64_group(const CUtensorMap* mA, const CUtensorMap* mB,
+                                     const TcProb* probs_dev, int nprob, int M, int N, int ldo,
+                                     double scale, int* flag, int nsm, cudaStream_t st,
+                                     int mode, PairTile tile) {
+  if (nprob > 0 && probs_dev == nullptr) return cudaErrorInvalidValue;
+  return launch_pair<S, FMT, double>(mA, mB, probs_dev, TcProb{}, nprob, M, N, ldo, scale, flag,
+                                     nullptr, nsm, st, tc_normal(), TcOut{mode, 0, 0, 0}, tile);
+}
+template cudaError_t launch_tc_pair_f64_group<4, kFmtBF16>(const CUtensorMap*, const CUtensorMap*,
+                                                           const TcProb*, int, int, int, int,
+                                                           double, int*, int, cudaStream_t, int,
+                                                           PairTile);
 
 #define LNO_PAIR_INST(S, F)                                                                   \
   template cudaError_t launch_tc_pair<S, F>(const CUtensorMap*, const CUtensorMap*,            \

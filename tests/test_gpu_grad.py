@@ -302,3 +302,16 @@ def test_fov_gradient_at_zero_block(ctx64, lib):
     fd = (E(+1) - E(-1)) / (2 * h)
     an = sum(float((gA["dfov"][s].cpu() * torch.as_tensor(x[s])).sum()) for s in (0, 1))
     assert abs(fd - an) <= 1e-6 * max(abs(an), 1e-3), (fd, an)
+
+
+def test_infinite_operand_is_refused_by_the_tensor_core_adjoint(ctx10):
+    d = make_domain(12, (4, 3), naux=24, L=6.0, seed=5, t1_sd=0.05)
+    dd = lno_ot.to_device(d)
+    dd["t2aa"][0, 1, 0, 1] = float("inf")
+    with pytest.raises(lno_ot.LnoError) as e:
+        ctx10.backward(dd, 1.0, dict(dt2ab=torch.empty_like(dd["t2ab"])))
+    assert e.value.code == lno_ot.EINVAL
+    # the context stays usable
+    g_ref, e_ref = oracle_grad(d)
+    g, e = gpu_grad(ctx10, d, gE=1.0)
+    compare(g, g_ref)
