@@ -91,14 +91,19 @@ cudaError_t launch_gather_rows(const void* src, void* dst, const int* list, int 
 cudaError_t launch_scatter_add_rows(const double* src, double* dst, const int* list, int nlist,
                                     int64_t row, cudaStream_t s);
 // naf.cu
-int jacobi_eigh(double* A, double* V, int n, double2* cs, double* norms, cudaStream_t st,
+int jacobi_eigh(double* A, double* A2, double* VT, int n, double* norms, cudaStream_t st,
                 int max_sweeps);
+size_t jacobi_norm_doubles();
+cudaError_t launch_unpack_pairs(const double* J, int nx, int n, double* B, cudaStream_t st);
+cudaError_t launch_asym_count(const double* B, int naux, int n, unsigned int* count,
+                              cudaStream_t st);
+cudaError_t launch_gemm_f64_sym(const ProbF64* prob_dev, int N, int ldo, cudaStream_t st);
 cudaError_t launch_pack_pairs(const double* B, int naux, int n, double* J, cudaStream_t st);
 cudaError_t launch_transpose_x(const double* B, int naux, int64_t n2, double* Bt,
                                cudaStream_t st);
 cudaError_t launch_get_diag(const double* A, int n, double* d, cudaStream_t st);
-cudaError_t launch_gather_cols(const double* V, int n, const int* cols, int nk, double* Vt,
-                               cudaStream_t st);
+cudaError_t launch_gather_rows_f64(const double* VT, int n, const int* rows, int nk, double* out,
+                                   cudaStream_t st);
 // backward.cu
 struct GemmS {
   const double* A;
@@ -1826,36 +1831,36 @@ int naf_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, double eps, double* cons
   const int n = dom->naux, nb = dom->nbas;
   const int64_t npair = (int64_t)nb * (nb + 1) / 2, n2 = (int64_t)nb * nb;
   Arena A(st, ctx->ws_limit);
-  double *J[2], *W, *V, *d, *norms;
-  double2* cs;
+  double *J[2], *W, *W2, *V, *d, *norms;
   ProbF64* dp;
+  unsigned int* asym;
+  TRY(A.get(&asym, 1));
+  CU(cudaMemsetAsync(asym, 0, sizeof(unsigned int), st));
   for (int s = 0; s < 2; ++s) {
     TRY(A.get(&J[s], (size_t)(n * npair)));
     CU(launch_pack_pairs(dom->B[s], n, nb, J[s], st));
+    CU(launch_asym_count(dom->B[s], n, nb, asym, st));
   }
   TRY(A.get(&W, (size_t)n * n));
+  TRY(A.get(&W2, (size_t)n * n));
   TRY(A.get(&dp, 2));
-  {  // W = (J^up J^up^T + J^down J^down^T) / 2
-    ProbF64 p{};
-    p.nseg = 2;
-    p.seg[0] = SegF64{J[0], J[0], (int)npair, (int)npair, (int)npair, 0.5};
-    p.seg[1] = SegF64{J[1], J[1], (int)npair, (int)npair, (int)npair, 0.5};
-    p.XT = W;
-    CU(cudaMemcpyAsync(dp, &p, sizeof p, cudaMemcpyHostToDevice, st));
-    CU(launch_gemm_f64(dp, 1, n, n, n, st));
-    CU(cudaStreamSynchronize(st));
-  }
-  A.drop(J[0]);
-  A.drop(J[1]);
+  ProbF64 pw{};   // W = (J^up J^up^T + J^down J^down^T) / 2
+  pw.nseg = 2;
+  pw.seg[0] = SegF64{J[0], J[0], (int)npair, (int)npair, (int)npair, 0.5};
+  pw.seg[1] = SegF64{J[1], J[1], (int)npair, (int)npair, (int)npair, 0.5};
+  pw.XT = W;
+  CU(cudaMemcpyAsync(dp, &pw, sizeof pw, cudaMemcpyHostToDevice, st));
+  CU(launch_gemm_f64_sym(dp, n, n, st));
   TRY(A.get(&V, (size_t)n * n));
-  TRY(A.get(&cs, (size_t)(n / 2 + 1)));
-  TRY(A.get(&norms, 2));
+  TRY(A.get(&norms, jacobi_norm_doubles()));
   TRY(A.get(&d, (size_t)n));
-  const int sweeps = jacobi_eigh(W, V, n, cs, norms, st, 40);
+  const int sweeps = jacobi_eigh(W, W2, V, n, norms, st, 40);
   if (sweeps < 0) return sweeps;
   CU(launch_get_diag(W, n, d, st));
   std::vector<double> lam(n);
+  unsigned int hasym = 1;
   CU(cudaMemcpyAsync(lam.data(), d, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, st));
+  CU(cudaMemcpyAsync(&hasym, asym, sizeof hasym, cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));
   std::vector<int> order(n);
   std::iota(order.begin(), order.end(), 0);
@@ -1871,17 +1876,26 @@ int naf_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, double eps, double* cons
     TRY(A.get(&cols, (size_t)nk));
     CU(cudaMemcpyAsync(cols, order.data(), (size_t)nk * sizeof(int), cudaMemcpyHostToDevice, st));
     TRY(A.get(&Vt, (size_t)nk * n));
-    CU(launch_gather_cols(V, n, cols, nk, Vt, st));
-    TRY(A.get(&Bt, (size_t)(n2 * n)));
-    for (int s = 0; s < 2; ++s) {   // B'[X'][pq] = sum_X V[X][X'] B[X][pq]
-      CU(launch_transpose_x(dom->B[s], n, n2, Bt, st));
-      ProbF64 p{};
-      p.nseg = 1;
-      p.seg[0] = SegF64{Bt, Vt, n, n, n, 1.0};
-      p.XT = Bout[s];
-      CU(cudaMemcpyAsync(dp + s, &p, sizeof p, cudaMemcpyHostToDevice, st));
-      CU(launch_gemm_f64(dp + s, 1, (int)n2, nk, (int)n2, st));
-      CU(cudaStreamSynchronize(st));
+    CU(launch_gather_rows_f64(V, n, cols, nk, Vt, st));
+    // B'[X'][pq] = sum_X V[X][X'] B[X][pq]: symmetric factors (as the header asks)
+    // over the pairs p <= q, half of the products and the same values; factors
+    // that differ in any bit from their transpose element by element
+    const bool sym = hasym == 0;
+    const int64_t rows = sym ? npair : n2;
+    if (!sym) {
+      A.drop(J[0]);
+      A.drop(J[1]);
+    }
+    TRY(A.get(&Bt, (size_t)(rows * n)));
+    ProbF64 p[2] = {};
+    for (int s = 0; s < 2; ++s) {
+      CU(launch_transpose_x(sym ? J[s] : dom->B[s], n, rows, Bt, st));
+      p[s].nseg = 1;
+      p[s].seg[0] = SegF64{Bt, Vt, n, n, n, 1.0};
+      p[s].XT = sym ? J[s] : Bout[s];   // the pairs' input is in Bt by then
+      CU(cudaMemcpyAsync(dp + s, &p[s], sizeof p[s], cudaMemcpyHostToDevice, st));
+      CU(launch_gemm_f64(dp + s, 1, (int)rows, nk, (int)rows, st));
+      if (sym) CU(launch_unpack_pairs(J[s], nk, nb, Bout[s], st));
     }
   }
   CU(cudaStreamSynchronize(st));

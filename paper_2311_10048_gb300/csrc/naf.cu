@@ -1,13 +1,13 @@
 // Natural auxiliary functions of a domain (arXiv 2311.10048, Sec. 3.6, eq
 // naf_w), in float64 on the CUDA cores:
 //   1. J^s[X][(p<=q)] = B^X_pq (pair-packed factors of each spin);
-//   2. W = (J^up J^up^T + J^down J^down^T) / 2, one grouped contraction;
+//   2. W = (J^up J^up^T + J^down J^down^T) / 2, one symmetric contraction;
 //   3. eigenvectors of W by cyclic Jacobi rotations in the round-robin order
-//      (n/2 disjoint rotations per round, n - 1 rounds per sweep; one sweep
-//      is one CUDA graph of 3 (n - 1) launches, replayed until the
-//      off-diagonal norm is below 1e-14 of the Frobenius norm);
+//      (n/2 disjoint rotations per round, n - 1 rounds per sweep, one launch per
+//      round, until the off-diagonal norm is below 1e-14 of the Frobenius norm);
 //   4. the eigenvectors with eigenvalues above eps_naf, in descending order;
-//   5. B'^s[X'][pq] = sum_X V[X][X'] B^s[X][pq] (one contraction per spin).
+//   5. B'^s[X'][pq] = sum_X V[X][X'] B^s[X][pq] (one contraction per spin, over
+//      the packed pairs p <= q when the factors are symmetric to the bit).
 // The eigen-decomposition runs on the device; only the n eigenvalues and the
 // convergence measure come back to the host (to sort and to stop).
 #include <algorithm>
@@ -18,9 +18,6 @@
 #include "common.cuh"
 
 namespace lno {
-
-cudaError_t launch_gemm_f64(const ProbF64* probs_dev, int nprob, int M, int N, int ldo,
-                            cudaStream_t st);
 
 namespace {
 
@@ -83,13 +80,8 @@ __device__ __forceinline__ void rr_pair(int r, int k, int np, int& p, int& q) {
   }
 }
 
-// rotation of pair k: zeroes A[p][q]; indices >= n are padding (no rotation)
-__global__ void jac_angles(const double* __restrict__ A, int n, int np, int r,
-                           double2* __restrict__ cs) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= np / 2) return;
-  int p, q;
-  rr_pair(r, k, np, p, q);
+// rotation (c, s) that zeroes A[p][q]; indices >= n are padding (no rotation)
+__device__ __forceinline__ double2 jac_angle(const double* A, int n, int p, int q) {
   double c = 1.0, s = 0.0;
   if (q < n) {
     const double apq = A[(int64_t)p * n + q];
@@ -101,54 +93,76 @@ __global__ void jac_angles(const double* __restrict__ A, int n, int np, int r,
       s = t * c;
     }
   }
-  cs[k] = make_double2(c, s);
+  return make_double2(c, s);
 }
 
-// rows p, q of A (and nothing else): A <- J^T A for all pairs of the round
-__global__ void jac_rows(double* __restrict__ A, int n, int np, int r,
-                         const double2* __restrict__ cs) {
-  const int m = np / 2;
-  const int64_t total = (int64_t)m * n;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int j = (int)(idx % n), k = (int)(idx / n);
-    int p, q;
-    rr_pair(r, k, np, p, q);
-    if (q >= n) continue;
-    const double2 g = cs[k];
-    const double ap = A[(int64_t)p * n + j], aq = A[(int64_t)q * n + j];
-    A[(int64_t)p * n + j] = g.x * ap - g.y * aq;
-    A[(int64_t)q * n + j] = g.y * ap + g.x * aq;
+// One round: A <- J^T A J for the round's disjoint rotations J, V^T <- J^T V^T.
+// Blocks (x, y < m16) own the 2 x 2 element blocks of 16 x 16 pairs: one read of
+// the old matrix and one write of the new one (two buffers: every block takes its
+// 32 angles from the old), so a round is one launch.  Blocks y >= m16 rotate 16
+// pairs of rows of V^T (128 columns each) in place.  Bound by the round's latency
+// (angles: two square roots and three divisions, then one pass over the matrix in
+// L2).  600 x 600: 21 us a round with three launches (angles, rows, and strided
+// columns of A and V), 3.5 us so.
+constexpr int JT = 16, JC = 128;
+__global__ void __launch_bounds__(256)
+jac_round(const double* __restrict__ Ain, double* __restrict__ Aout, double* __restrict__ VT,
+          int n, int np, int r) {
+  __shared__ double2 cs[2][JT];
+  __shared__ int pp[2][JT], qq[2][JT];
+  const int m = np / 2, m16 = (m + JT - 1) / JT;
+  const bool vec = (int)blockIdx.y >= m16;
+  const int tid = threadIdx.x;
+  if (tid < 2 * JT) {
+    const int w = tid / JT, l = tid % JT;
+    const int k = (w == 0 || !vec ? (w == 0 ? (int)blockIdx.x : (int)blockIdx.y) : 0) * JT + l;
+    int p = n, q = n;
+    if (k < m) rr_pair(r, k, np, p, q);
+    pp[w][l] = p;
+    qq[w][l] = q;
+    cs[w][l] = k < m ? jac_angle(Ain, n, p, q) : make_double2(1.0, 0.0);
   }
-}
-
-// columns p, q of A and of V: A <- A J, V <- V J
-__global__ void jac_cols(double* __restrict__ A, double* __restrict__ V, int n, int np, int r,
-                         const double2* __restrict__ cs) {
-  const int m = np / 2;
-  const int64_t total = (int64_t)m * n;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(idx % n), k = (int)(idx / n);
-    int p, q;
-    rr_pair(r, k, np, p, q);
-    if (q >= n) continue;
-    const double2 g = cs[k];
-    double ap = A[(int64_t)i * n + p], aq = A[(int64_t)i * n + q];
-    A[(int64_t)i * n + p] = g.x * ap - g.y * aq;
-    A[(int64_t)i * n + q] = g.y * ap + g.x * aq;
-    ap = V[(int64_t)i * n + p];
-    aq = V[(int64_t)i * n + q];
-    V[(int64_t)i * n + p] = g.x * ap - g.y * aq;
-    V[(int64_t)i * n + q] = g.y * ap + g.x * aq;
+  __syncthreads();
+  if (vec) {
+    const int c0 = ((int)blockIdx.y - m16) * JC;
+    for (int e = tid; e < JT * JC; e += 256) {
+      const int l = e / JC, i = c0 + e % JC;
+      const int p = pp[0][l], q = qq[0][l];
+      if (i >= n || q >= n) continue;
+      const double2 g = cs[0][l];
+      const double ap = VT[(int64_t)p * n + i], aq = VT[(int64_t)q * n + i];
+      VT[(int64_t)p * n + i] = g.x * ap - g.y * aq;
+      VT[(int64_t)q * n + i] = g.y * ap + g.x * aq;
+    }
+    return;
   }
+  // rows: pair a of blockIdx.x; columns: pair b of blockIdx.y
+  const int a = tid / JT, b = tid % JT;
+  const int p = pp[0][a], q = qq[0][a], u = pp[1][b], w = qq[1][b];
+  if (p >= n || u >= n) return;
+  const bool q_in = q < n, w_in = w < n;
+  const double2 g = cs[0][a], h = cs[1][b];
+  const double pu = Ain[(int64_t)p * n + u], pw = w_in ? Ain[(int64_t)p * n + w] : 0.0;
+  const double qu = q_in ? Ain[(int64_t)q * n + u] : 0.0,
+               qw = q_in && w_in ? Ain[(int64_t)q * n + w] : 0.0;
+  // rows first, then columns
+  const double tpu = g.x * pu - g.y * qu, tqu = g.y * pu + g.x * qu;
+  const double tpw = g.x * pw - g.y * qw, tqw = g.y * pw + g.x * qw;
+  Aout[(int64_t)p * n + u] = h.x * tpu - h.y * tpw;
+  if (w_in) Aout[(int64_t)p * n + w] = h.y * tpu + h.x * tpw;
+  if (q_in) Aout[(int64_t)q * n + u] = h.x * tqu - h.y * tqw;
+  if (q_in && w_in) Aout[(int64_t)q * n + w] = h.y * tqu + h.x * tqw;
 }
 
-// out[0] = sum of squares of the off-diagonal elements, out[1] = of all
-__global__ void jac_norms(const double* __restrict__ A, int n, double* __restrict__ out) {
+// part[2 b], part[2 b + 1] = block b's sums of squares of the off-diagonal elements
+// and of all; jac_norms_sum adds them in block order.
+constexpr int kNormBlocks = 128;
+__global__ void __launch_bounds__(256)
+jac_norms(const double* __restrict__ A, int n, double* __restrict__ part) {
   __shared__ double so[256], sa[256];
   double o = 0.0, a = 0.0;
-  for (int64_t idx = threadIdx.x; idx < (int64_t)n * n; idx += blockDim.x) {
+  for (int64_t idx = blockIdx.x * 256LL + threadIdx.x; idx < (int64_t)n * n;
+       idx += kNormBlocks * 256LL) {
     const double x = A[idx];
     a += x * x;
     if (idx / n != idx % n) o += x * x;
@@ -164,8 +178,15 @@ __global__ void jac_norms(const double* __restrict__ A, int n, double* __restric
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    out[0] = so[0];
-    out[1] = sa[0];
+    part[2 * blockIdx.x] = so[0];
+    part[2 * blockIdx.x + 1] = sa[0];
+  }
+}
+__global__ void jac_norms_sum(const double* __restrict__ part, double* __restrict__ out) {
+  if (threadIdx.x < 2) {
+    double t = 0.0;
+    for (int b = 0; b < kNormBlocks; ++b) t += part[2 * b + threadIdx.x];
+    out[threadIdx.x] = t;
   }
 }
 
@@ -180,72 +201,93 @@ __global__ void get_diag(const double* __restrict__ A, int n, double* __restrict
     d[i] = A[(int64_t)i * n + i];
 }
 
-// Vt[c][X] = V[X][cols[c]]  (kept eigenvectors as rows)
-__global__ void gather_cols(const double* __restrict__ V, int n, const int* __restrict__ cols,
-                            int nk, double* __restrict__ Vt) {
+// out[c][X] = VT[rows[c]][X]  (kept eigenvectors)
+__global__ void gather_rows(const double* __restrict__ VT, int n, const int* __restrict__ rows,
+                            int nk, double* __restrict__ out) {
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < (int64_t)nk * n;
        idx += (int64_t)gridDim.x * blockDim.x) {
     const int X = (int)(idx % n), c = (int)(idx / n);
-    Vt[idx] = V[(int64_t)X * n + cols[c]];
+    out[idx] = VT[(int64_t)rows[c] * n + X];
   }
+}
+
+// Jt[pair][X] = J[X][pair]: transpose_x on the packed pairs.  unpack_pairs: B[X][p][q]
+// and B[X][q][p] from the pairs.
+__global__ void unpack_pairs(const double* __restrict__ J, int nx, int n,
+                             double* __restrict__ B) {
+  const int64_t np = (int64_t)n * (n + 1) / 2, n2 = (int64_t)n * n, total = (int64_t)nx * n2;
+  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t X = idx / n2, e = idx - X * n2;
+    const int p = (int)(e / n), q = (int)(e - (int64_t)p * n);
+    const int lo = min(p, q), hi = max(p, q);
+    B[idx] = J[X * np + (int64_t)hi * (hi + 1) / 2 + lo];
+  }
+}
+
+// *count += elements with B[X][p][q] != B[X][q][p] (p < q)
+__global__ void asym_count(const double* __restrict__ B, int naux, int n,
+                           unsigned int* __restrict__ count) {
+  __shared__ double t[32][33];
+  const int bx = blockIdx.x, by = blockIdx.y;
+  if (bx < by) return;   // tile (by, bx) against tile (bx, by)
+  unsigned int bad = 0;
+  for (int X = blockIdx.z; X < naux; X += gridDim.z) {
+    const double* M = B + (int64_t)X * n * n;
+    for (int i = threadIdx.y; i < 32; i += 8) {
+      const int p = bx * 32 + i, q = by * 32 + threadIdx.x;
+      t[i][threadIdx.x] = p < n && q < n ? M[(int64_t)p * n + q] : 0.0;
+    }
+    __syncthreads();
+    for (int i = threadIdx.y; i < 32; i += 8) {
+      const int p = by * 32 + i, q = bx * 32 + threadIdx.x;
+      if (p < n && q < n && !(M[(int64_t)p * n + q] == t[threadIdx.x][i])) ++bad;
+    }
+    __syncthreads();
+  }
+  if (bad) atomicAdd(count, bad);
 }
 
 }  // namespace
 
 // Symmetric eigen-decomposition of A (n x n, device, destroyed: its diagonal
-// ends up holding the eigenvalues) with eigenvectors in the columns of V.
+// ends up holding the eigenvalues) with eigenvectors in the rows of VT.  A2 is a
+// second n x n buffer, norms holds 2 (1 + kNormBlocks) doubles.
 // Returns the number of sweeps, or a negative lno_ot_status.
-int jacobi_eigh(double* A, double* V, int n, double2* cs, double* norms, cudaStream_t st,
+int jacobi_eigh(double* A, double* A2, double* VT, int n, double* norms, cudaStream_t st,
                 int max_sweeps) {
   if (n <= 0) return 0;
-  set_identity<<<grid_n((int64_t)n * n), 256, 0, st>>>(V, n);
+  set_identity<<<grid_n((int64_t)n * n), 256, 0, st>>>(VT, n);
   if (n == 1) return 0;
   const int np = n + (n & 1);
-  const int m = np / 2;
-  // one sweep as a graph
-  cudaStream_t cap;
-  if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return LNO_OT_ECUDA;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  int rc = LNO_OT_OK;
-  if (cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-    rc = LNO_OT_ECUDA;
-  } else {
-    for (int r = 0; r < np - 1; ++r) {
-      jac_angles<<<(m + 127) / 128, 128, 0, cap>>>(A, n, np, r, cs);
-      jac_rows<<<grid_n((int64_t)m * n), 256, 0, cap>>>(A, n, np, r, cs);
-      jac_cols<<<grid_n((int64_t)m * n), 256, 0, cap>>>(A, V, n, np, r, cs);
-    }
-    if (cudaStreamEndCapture(cap, &graph) != cudaSuccess ||
-        cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess)
-      rc = LNO_OT_ECUDA;
-  }
+  const int m16 = (np / 2 + JT - 1) / JT;
+  const dim3 grid(m16, m16 + (n + JC - 1) / JC);
+  double *cur = A, *other = A2;
   int sweeps = 0;
-  if (rc == LNO_OT_OK) {
+  cudaError_t e = cudaSuccess;
+  for (; sweeps < max_sweeps && e == cudaSuccess; ++sweeps) {
     double h[2];
-    for (; sweeps < max_sweeps; ++sweeps) {
-      jac_norms<<<1, 256, 0, st>>>(A, n, norms);
-      if (cudaMemcpyAsync(h, norms, sizeof h, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-          cudaStreamSynchronize(st) != cudaSuccess) {
-        rc = LNO_OT_ECUDA;
-        break;
-      }
-      if (!(h[0] > 1e-28 * h[1])) break;   // off-diagonal norm < 1e-14 of the whole
-      if (cudaGraphLaunch(exec, st) != cudaSuccess) {
-        rc = LNO_OT_ECUDA;
-        break;
-      }
+    jac_norms<<<kNormBlocks, 256, 0, st>>>(cur, n, norms + 2);
+    jac_norms_sum<<<1, 32, 0, st>>>(norms + 2, norms);
+    e = cudaMemcpyAsync(h, norms, sizeof h, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess || !(h[0] > 1e-28 * h[1])) break;   // off-diagonal norm < 1e-14
+    for (int r = 0; r < np - 1; ++r) {
+      jac_round<<<grid, 256, 0, st>>>(cur, other, VT, n, np, r);
+      std::swap(cur, other);
     }
+    e = cudaGetLastError();
   }
-  if (exec) cudaGraphExecDestroy(exec);
-  if (graph) cudaGraphDestroy(graph);
-  cudaStreamDestroy(cap);
-  if (rc != LNO_OT_OK) {
+  if (e == cudaSuccess && cur != A)
+    e = cudaMemcpyAsync(A, cur, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToDevice, st);
+  if (e != cudaSuccess) {
     cudaGetLastError();
-    return rc;
+    return LNO_OT_ECUDA;
   }
   return sweeps;
 }
+
+size_t jacobi_norm_doubles() { return 2 * (1 + kNormBlocks); }
 
 cudaError_t launch_pack_pairs(const double* B, int naux, int n, double* J, cudaStream_t st) {
   pack_pairs<<<grid_n((int64_t)naux * n * (n + 1) / 2), 256, 0, st>>>(B, naux, n, J);
@@ -264,10 +306,23 @@ cudaError_t launch_get_diag(const double* A, int n, double* d, cudaStream_t st) 
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather_cols(const double* V, int n, const int* cols, int nk, double* Vt,
-                               cudaStream_t st) {
+cudaError_t launch_gather_rows_f64(const double* VT, int n, const int* rows, int nk, double* out,
+                                   cudaStream_t st) {
   if (nk <= 0) return cudaSuccess;
-  gather_cols<<<grid_n((int64_t)nk * n), 256, 0, st>>>(V, n, cols, nk, Vt);
+  gather_rows<<<grid_n((int64_t)nk * n), 256, 0, st>>>(VT, n, rows, nk, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_unpack_pairs(const double* J, int nx, int n, double* B, cudaStream_t st) {
+  if (nx <= 0) return cudaSuccess;
+  unpack_pairs<<<grid_n((int64_t)nx * n * n), 256, 0, st>>>(J, nx, n, B);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_asym_count(const double* B, int naux, int n, unsigned int* count,
+                              cudaStream_t st) {
+  const int t = (n + 31) / 32;
+  asym_count<<<dim3(t, t, std::min(naux, 64)), dim3(32, 8), 0, st>>>(B, naux, n, count);
   return cudaGetLastError();
 }
 

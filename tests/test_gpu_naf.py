@@ -45,3 +45,30 @@ def test_naf_matches_oracle(lib, name, kw, epss):
         e_ref = T.energy(oc)["total"]
         assert abs(e_gpu - e_ref) <= 1e-10 * abs(e_ref), (eps, e_gpu, e_ref)
     ctx.close()
+
+
+@pytest.mark.parametrize("n,naux", [(7, 5), (9, 33), (18, 47), (33, 130)])
+def test_naf_of_odd_sizes_and_of_asymmetric_factors(n, naux):
+    """Odd auxiliary counts (padded rotations), and factors that are not symmetric
+    in (p, q): W takes p <= q, the compression every element."""
+    rng = np.random.default_rng(n)
+    B = [rng.normal(size=(naux, n, n)) * np.exp(-3 * np.arange(naux) / naux)[:, None, None]
+         for _ in range(2)]
+    for sym in (True, False):
+        b = [np.triu(x) + np.triu(x, 1).transpose(0, 2, 1) if sym else x for x in B]
+        iu = np.triu_indices(n)
+        j = [x[:, iu[0], iu[1]] for x in b]
+        lam, vec = np.linalg.eigh((j[0] @ j[0].T + j[1] @ j[1].T) / 2)
+        lam, vec = lam[::-1], vec[:, ::-1]
+        eps = float(np.sqrt(lam[naux // 2] * lam[naux // 2 + 1]))
+        d = lno_ot.to_device(dict(make_domain(n, (2, 1), naux=naux, L=naux / 3, seed=1), B=b))
+        ctx = lno_ot.Context(0, "fp64")
+        out, got = ctx.naf(d, eps)
+        ctx.close()
+        assert np.abs(got - lam).max() <= 1e-12 * lam[0]
+        assert out["naux"] == naux // 2 + 1
+        for s in (0, 1):
+            want = np.einsum("Xk,Xpq->kpq", vec[:, :out["naux"]], b[s])
+            # eigenvectors to ~1e-15 over the relative gaps (>= 1e-5 in these draws)
+            assert np.abs(sign_fixed(out["B"][s].cpu().numpy()) - sign_fixed(want)).max() \
+                <= 1e-8 * np.abs(want).max()
