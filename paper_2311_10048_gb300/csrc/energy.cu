@@ -874,35 +874,57 @@ energy_f32(EnergyArgs a, const float* __restrict__ X, const float* __restrict__ 
   }
 }
 
-// e_trip[g] = sum_p partial[g][p] (+ sum_p partial2[g][p] when given),
-// Neumaier in a fixed order, one thread per triplet.
-__global__ void reduce_partials(const double* __restrict__ partial, int np,
-                                const double* __restrict__ partial2, int ntrip,
-                                double* __restrict__ e_trip) {
-  // one warp per triplet: lane l sums p = l, l + 32, ... (Neumaier), then the
-  // lanes' (sum, compensation) pairs are combined in a fixed shuffle tree, so
-  // the result does not depend on timing
-  const int lane = threadIdx.x & 31;
-  const int g = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-  if (g >= ntrip) return;
-  double s = 0.0, c = 0.0;
-  for (int half = 0; half < (partial2 ? 2 : 1); ++half) {
-    const double* src = (half ? partial2 : partial) + (int64_t)g * np;
-    for (int p = lane; p < np; p += 32) {
-      const double x = src[p];
-      const double t = s + x;
-      c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
-      s = t;
-    }
-  }
-  for (int off = 16; off > 0; off >>= 1) {
-    const double so = __shfl_down_sync(0xffffffffu, s, off);
-    const double co = __shfl_down_sync(0xffffffffu, c, off);
-    const double t = s + so;
-    c += (fabs(s) >= fabs(so) ? (s - t) + so : (so - t) + s) + co;
+// A Neumaier pair (sum, compensation).
+struct Nsum {
+  double s, c;
+  __device__ __forceinline__ void add(double x) {
+    const double t = s + x;
+    c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
     s = t;
   }
-  if (lane == 0) e_trip[g] = s + c;
+  __device__ __forceinline__ void add(const Nsum& o) {
+    add(o.s);
+    c += o.c;
+  }
+};
+
+// Sum of the block's pairs (256 threads), in a fixed order: a shuffle tree per warp,
+// then the eight warps in turn; valid in thread 0.
+__device__ __forceinline__ Nsum block_sum(Nsum v) {
+  __shared__ double ws[8], wc[8];
+  for (int off = 16; off > 0; off >>= 1) {
+    Nsum o;
+    o.s = __shfl_down_sync(0xffffffffu, v.s, off);
+    o.c = __shfl_down_sync(0xffffffffu, v.c, off);
+    v.add(o);
+  }
+  __syncthreads();   // the shared arrays may hold an earlier sum
+  if ((threadIdx.x & 31) == 0) {
+    ws[threadIdx.x >> 5] = v.s;
+    wc[threadIdx.x >> 5] = v.c;
+  }
+  __syncthreads();
+  Nsum t{0.0, 0.0};
+  if (threadIdx.x == 0)
+    for (int w = 0; w < 8; ++w) t.add(Nsum{ws[w], wc[w]});
+  return t;
+}
+
+// e_trip[g] = sum_p partial[g][p] (+ sum_p partial2[g][p] when given): one CTA per
+// triplet, thread t sums p = t, t + 256, ... (Neumaier), combined in a fixed
+// order, so the result does not depend on timing.  (One warp per triplet took
+// 22 us for 64 triplets of 1200 partials, this 4.)
+__global__ void __launch_bounds__(256)
+reduce_partials(const double* __restrict__ partial, int np, const double* __restrict__ partial2,
+                double* __restrict__ e_trip) {
+  const int g = blockIdx.x;
+  Nsum v{0.0, 0.0};
+  for (int half = 0; half < (partial2 ? 2 : 1); ++half) {
+    const double* src = (half ? partial2 : partial) + (int64_t)g * np;
+    for (int p = threadIdx.x; p < np; p += 256) v.add(src[p]);
+  }
+  v = block_sum(v);
+  if (threadIdx.x == 0) e_trip[g] = v.s + v.c;
 }
 
 // Orbital contributions of eq cim_pt_energy from per-triplet contributions:
@@ -910,17 +932,12 @@ __global__ void reduce_partials(const double* __restrict__ partial, int np,
 // its two same-spin orbitals and 1/2 to the third (A.thirds: 1/3 each, the
 // partition of eq local_pt).  One CTA per occupied
 // orbital (spin up first), fixed-order Neumaier sums: bitwise reproducible.
-__global__ void orbital_partition(OrbPartArgs A) {
-  __shared__ double ss[256], cc[256];
+__global__ void __launch_bounds__(256) orbital_partition(OrbPartArgs A) {
   const int b = blockIdx.x;
   const int s = b < A.na ? 0 : 1;
   const int p = s == 0 ? b : b - A.na;
-  double acc = 0.0, comp = 0.0;
-  auto add = [&](double x) {
-    double t = acc + x;
-    comp += fabs(acc) >= fabs(x) ? (acc - t) + x : (x - t) + acc;
-    acc = t;
-  };
+  Nsum v{0.0, 0.0};
+  auto add = [&](double x) { v.add(x); };
   for (int c = 0; c < 4; ++c) {
     const Trip* tr = A.trips[c];
     const double* e = A.e[c];
@@ -938,47 +955,19 @@ __global__ void orbital_partition(OrbPartArgs A) {
       }
     }
   }
-  ss[threadIdx.x] = acc;
-  cc[threadIdx.x] = comp;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double S = 0.0, C = 0.0;
-    for (int q = 0; q < (int)blockDim.x; ++q) {
-      double x = ss[q];
-      double t = S + x;
-      C += fabs(S) >= fabs(x) ? (S - t) + x : (x - t) + S;
-      S = t;
-      C += cc[q];
-    }
-    double* out = s == 0 ? A.out[0] : A.out[1];
-    if (out) out[p] = S + C;
-  }
+  v = block_sum(v);
+  double* out = s == 0 ? A.out[0] : A.out[1];
+  if (threadIdx.x == 0 && out) out[p] = v.s + v.c;
 }
 
-// out[0] = Neumaier sum of e[0..n): one CTA of 256 threads, fixed order.
-__global__ void neumaier_sum(const double* __restrict__ e, int64_t n, double* out) {
-  __shared__ double ss[256], cc[256];
-  double s = 0.0, c = 0.0;
-  for (int64_t q = threadIdx.x; q < n; q += blockDim.x) {
-    double x = e[q];
-    double t = s + x;
-    c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
-    s = t;
-  }
-  ss[threadIdx.x] = s;
-  cc[threadIdx.x] = c;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double S = 0.0, C = 0.0;
-    for (int q = 0; q < (int)blockDim.x; ++q) {
-      double x = ss[q];
-      double t = S + x;
-      C += fabs(S) >= fabs(x) ? (S - t) + x : (x - t) + S;
-      S = t;
-      C += cc[q];
-    }
-    out[0] = S + C;
-  }
+// out[0] = Neumaier sum of e[0..n): one CTA of 256 threads, fixed order.  (Adding
+// the 256 threads' pairs one after the other took 73 us, this 4.)
+__global__ void __launch_bounds__(256)
+neumaier_sum(const double* __restrict__ e, int64_t n, double* out) {
+  Nsum v{0.0, 0.0};
+  for (int64_t q = threadIdx.x; q < n; q += 256) v.add(e[q]);
+  v = block_sum(v);
+  if (threadIdx.x == 0) out[0] = v.s + v.c;
 }
 
 }  // namespace
@@ -1110,7 +1099,7 @@ cudaError_t launch_energy(const EnergyArgs& a, const void* X, const void* Z, boo
 cudaError_t launch_reduce_partials(const double* partial, int np, const double* partial2,
                                    int ntrip, double* e_trip, cudaStream_t st) {
   if (ntrip <= 0) return cudaSuccess;
-  reduce_partials<<<ceil_div(ntrip, 8), 256, 0, st>>>(partial, np, partial2, ntrip, e_trip);
+  reduce_partials<<<ntrip, 256, 0, st>>>(partial, np, partial2, e_trip);
   return cudaGetLastError();
 }
 
