@@ -766,6 +766,11 @@ double flops_alg_mixed(double vs, double vt, double os, double ot) {
 }
 double kpad16(double k) { return std::ceil(k / 16.0) * 16.0; }
 
+// Triplets per group where the tuning table says nothing: enough that launch gaps
+// and each launch's last round of tiles are a few percent for virtual spaces of
+// ~100 (larger ones reach the group's memory budget first).
+constexpr int kGroupCap = 256;
+
 // ----------------------------------------------------------------------------
 // Per spin s: same-spin case (sss) and the mixed case with two s orbitals.
 struct SpinPass {
@@ -783,7 +788,7 @@ struct SpinPass {
   std::vector<int2> listAT, listA1, listAT2;
   std::vector<int> listBT, listBG, listBF;
   int bn = 0;                // widest contraction tile of the current case (0 = default)
-  int group_cap = 64;        // triplets per group (upper bound)
+  int group_cap = kGroupCap; // triplets per group (upper bound)
   double* t2st = nullptr;    // [os][ot][vs][vt]
   const double* t2ss = nullptr;
   // V-term integrals over the occupied orbitals in use: spin-s slots are those
@@ -1154,7 +1159,7 @@ struct SpinPass {
     const int64_t per_trip = (xs + zs) * (int64_t)esz;
     const int64_t budget = (int64_t)6 << 30;
     bn = 0;
-    group_cap = 64;
+    group_cap = kGroupCap;
     if (const auto* row = R.ctx->tune_for(v)) {
       bn = row->bn;
       group_cap = std::max(1, row->group_cap);
