@@ -766,10 +766,12 @@ double flops_alg_mixed(double vs, double vt, double os, double ot) {
 }
 double kpad16(double k) { return std::ceil(k / 16.0) * 16.0; }
 
-// Triplets per group where the tuning table says nothing: enough that launch gaps
-// and each launch's last round of tiles are a few percent for virtual spaces of
-// ~100 (larger ones reach the group's memory budget first).
-constexpr int kGroupCap = 256;
+// Triplets per group where the tuning table says nothing: virtual spaces of ~100
+// then reach the group's memory budget or have a case in a few launches.  At 64,
+// launch gaps, each launch's last round of tiles and the energy kernel's items of
+// one or two tiles (their number per triplet falls as the group grows) cost 20%:
+// 121/14/11 domain 28.8 ms at 64, 24.6 at 256, 23.4 at 1024.
+constexpr int kGroupCap = 1024;
 
 // ----------------------------------------------------------------------------
 // Per spin s: same-spin case (sss) and the mixed case with two s orbitals.
@@ -2261,8 +2263,11 @@ int backward_spin(SpinPass& P, GradAcc& G, double gE) {
     const int M2 = vt;
     const int64_t N2 = is_mixed ? npairs(v) : 0;
     const int P2 = (int)round_up(std::max(M2, 1), 16);
-    const int64_t per = (N1 * P1 + N2 * P2) * 8 * 2;
-    int Gn = (int)std::max<int64_t>(1, std::min<int64_t>(32, ((int64_t)4 << 30) / std::max<int64_t>(per, 1)));
+    // X, dX and, in the batched form, the slices of dX in two layouts; there a group
+    // is one launch per product, so it is as large as the budget allows
+    const int64_t per = (N1 * P1 + N2 * P2) * 8 * (batched ? 4 : 2);
+    int Gn = (int)std::max<int64_t>(
+        1, std::min<int64_t>(batched ? 1024 : 32, ((int64_t)4 << 30) / std::max<int64_t>(per, 1)));
     Gn = std::min(Gn, ntrip);
     double *X, *Z = nullptr, *dX, *dZ = nullptr;
     TRY(A.get(&X, (size_t)(Gn * N1 * P1) + 8));
