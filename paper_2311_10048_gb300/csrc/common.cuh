@@ -207,6 +207,7 @@ struct PairTile {
   int stages;   // k blocks in flight in shared memory
 };
 PairTile pair_tile(int S, int N, int cap);
+PairTile pair_tile_f64(int S, int nprob, int M, int N);
 template <int S, int FMT>
 cudaError_t launch_tc_pair(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs_dev,
                            int nprob, int M, int N, int ldo, double scale, int* flag, int nsm,

@@ -492,7 +492,7 @@ struct Run {
     // products) unless that leaves the scale open (measure_sigI)
     const int ns = amax_pass && !amax_exact ? 2 : Sdf;
     unsigned long long* am = amax_pass ? ctx->d_amax : track_amax ? ctx->d_amax + 2 : nullptr;
-    const PairTile t = pair_tile(ns, N, 128);
+    const PairTile t = pair_tile_f64(ns, 1, M, N);
     CUtensorMap mA[2], mB[2];
     TRY(Lo.pair_map(&mA[0], 128, ns));
     TRY(Ro.pair_map(&mB[0], t.w / 2, ns));
@@ -657,7 +657,7 @@ struct SlicedBatch {
 int grouped_products(Run& R, Arena& A, const std::vector<TcProb>& pr, const SlicedBatch& a,
                      bool ta, const SlicedBatch& b, bool tb, int M, int N, int ldo, int mode) {
   if (pr.empty() || M <= 0 || N <= 0) return LNO_OT_OK;
-  const PairTile t = pair_tile(4, N, 128);
+  const PairTile t = pair_tile_f64(4, (int)pr.size(), M, N);
   CUtensorMap mA[2], mB[2];
   TRY(a.map(&mA[0], ta, 128));
   TRY(b.map(&mB[0], tb, t.w / 2));
@@ -2130,7 +2130,7 @@ int tc_matmul(Run& R, Arena& A, int M, int N, int K, View a, View b, double* C, 
   // the kernel writes its output transposed: its rows (A role) are n, its
   // columns (B role) m, so out[m ldc + n]
   CUtensorMap mA[2], mB[2];
-  const PairTile tile = pair_tile(S, M, 128);
+  const PairTile tile = pair_tile_f64(S, nsp, N, M);
   TRY(make_operand_map(&mA[0], qb, Kp, (int64_t)nsp * N, S, (int64_t)nsp * N * Kp, 128, 2, S));
   TRY(make_operand_map(&mB[0], qa, Kp, (int64_t)nsp * M, S, (int64_t)nsp * M * Kp, tile.w / 2, 2,
                        S));

@@ -46,10 +46,10 @@ constexpr int BK = 32;                     // 16-bit elements per 64-byte row, S
 constexpr long long kWaitCycles = 4000000000LL;
 constexpr int kSmemBytes = 227 * 1024;
 constexpr int kMaxStages = 16;
+constexpr int kF64Width = 64;              // widest tile of a float64-output launch
 constexpr int kBarBytes = 512;
 // Epilogue warps: float32 output 8 (up to 80 columns of results a thread);
-// float64 output 16 (its integer conversions need the lanes, and 32 columns of
-// results are 64 registers)
+// float64 output 16, for its integer conversions
 template <typename OutT>
 constexpr int epi_warps() {
   return sizeof(OutT) == 4 ? 8 : 16;
@@ -282,11 +282,15 @@ __device__ __forceinline__ void store_chunk(const RowOut& ro, int chunk, const f
   }
 }
 
-// Columns of one tile: S accumulators in TMEM, N <= 256; 128 for float64 output
-// (32 results a thread).
+// Columns of one tile: S accumulators in TMEM, N <= 256.  Float64 output: 64, and
+// two accumulator sets (2 S w <= 512), so its long epilogue (~100 instructions an
+// element) runs beside the next tile's MMAs, converting and storing 8 columns at a
+// time (holding a 128-column tile's results to free TMEM first spilled, and a K =
+// 60 product of 2809 x 53 outputs took 5.5 us an output tile instead of 1.5).
 template <int S, typename OutT>
 constexpr int pair_max_width() {
-  return std::min(sizeof(OutT) == 4 ? 256 : 128, 512 / S / 16 * 16);
+  return sizeof(OutT) == 4 ? std::min(256, 512 / S / 16 * 16)
+                           : std::min(kF64Width, 256 / S / 16 * 16);
 }
 
 // I 2^e as a float64, |I| < 2^53 and the result a normal number (integer
@@ -302,28 +306,30 @@ __device__ __forceinline__ double fixed_to_double(int64_t I, int e) {
 }
 
 // Float64 value of one element's class sums: the exact sum of the classes times
-// 2^e.  Class g is an integer multiple of 2^(-BITS g), or (INTS) that integer; sums too large for the
-// integers (or not finite) become NaN, as the operands' slices say.
-// rest: class 0 plus the float32 sum of the others (BF16, kTcFloatRest).
+// 2^e.  Class g is an integer multiple of 2^(-BITS g), or (INTS) that integer.  A
+// class 0 too large for the integers or not finite becomes NaN (a NaN operand has
+// it in its leading slice, so in class 0).  rest: class 0 plus the float32 sum of
+// the others (BF16, kTcFloatRest).
 template <int S, int BITS, bool INTS>
 __device__ __forceinline__ double class_sum(const float (&c)[S], int e, bool rest) {
-  int64_t I = 0;
-  float w = 1.0f, big = 0.0f;
-#pragma unroll
-  for (int g = 0; g < S; ++g) {
-    const float x = c[g] * w;   // integer (exact: a power of two)
-    big = fmaxf(big, fabsf(x));
-    if (isnan(x)) big = INFINITY;
-    I = I * (1 << BITS) + (int64_t)__float2int_rn(x);
-    if (!INTS) w *= (float)(1 << BITS);
-  }
-  if (!(big < 1073741824.0f)) return __longlong_as_double(0x7ff8000000000000ll);
-  if (!INTS && rest) {
+  if (!(fabsf(c[0]) < 1073741824.0f)) return __longlong_as_double(0x7ff8000000000000ll);
+  int64_t I = __float2int_rn(c[0]);
+  if (!INTS && S > 1 && rest) {
     float lo = 0.f;
 #pragma unroll
     for (int g = S - 1; g >= 1; --g) lo = __fadd_rn(lo, c[g]);
-    constexpr float top = (float)(1ll << (BITS * (S - 1)));
-    I = ((int64_t)__float2int_rn(c[0]) << (BITS * (S - 1))) + __float2ll_rn(lo * top);
+    constexpr int sh = BITS * (S - 1);      // <= 32
+    const float l1 = rintf(lo);             // lo = l1 + l0, both exact
+    const float l0 = __fmul_rn(__fsub_rn(lo, l1), (float)(1ll << (sh < 24 ? sh : 24)));
+    I = ((I + __float2int_rn(l1)) << sh) +
+        ((int64_t)__float2int_rn(l0) << (sh < 24 ? 0 : sh - 24));
+  } else {
+    float w = 1.0f;
+#pragma unroll
+    for (int g = 1; g < S; ++g) {
+      w *= (float)(1 << BITS);
+      I = (I << BITS) + __float2int_rn(INTS ? c[g] : c[g] * w);   // exact: a power of two
+    }
   }
   e -= BITS * (S - 1);
   if (e < -960 || e > 960) return ldexp((double)I, e);   // extreme scales only
@@ -594,57 +600,44 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
           }
         }
       } else {
-        constexpr int CH = pair_max_width<S, OutT>() / 32;   // 8-column chunks of one warp
         constexpr int BITS = FMT == kFmtBF16 ? 8 : 11;
         const int es = P.ea ? *P.ea + *P.eb - 14 : escale, fl = P.flags;
+        const bool rows = lay.mode == kOutF64Rows;   // out[m][n], else out[n][m]
+        double* out = reinterpret_cast<double*>(outp) + (rows ? (int64_t)m * ldo : m);
+        const int64_t step = rows ? 1 : ldo;
         if (!pair_wait(tfull(buf), use & 1u, flag, 6, true, wlim)) break;
         tc_fence_after();
-        const int nch = ntile_w(nt) / 8;
-        double v[CH * 8];
+        const int nch = ntile_w(nt) / 8;   // 8-column chunks, dealt over the four warps
+#pragma unroll 1
+        for (int chunk = part; chunk < nch; chunk += 4) {
+          uint32_t acc[S][8];
 #pragma unroll
-        for (int c = 0; c < CH; ++c) {
-          const int chunk = 4 * c + part;
-          if (chunk < nch) {
-            uint32_t acc[S][8];
+          for (int g = 0; g < S; ++g) tmem_ld8(tb + g * tile.w + chunk * 8, acc[g]);
+          tmem_ld_wait();
+          const int n = n0 + chunk * 8;
 #pragma unroll
-            for (int g = 0; g < S; ++g) tmem_ld8(tb + g * tile.w + chunk * 8, acc[g]);
-            tmem_ld_wait();
+          for (int j = 0; j < 8; ++j) {
+            float x[S], lo = 0.f;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              float x[S], lo = 0.f;
-#pragma unroll
-              for (int g = S - 1; g >= 0; --g) {
-                x[g] = __uint_as_float(acc[g][j]);
-                lo = FMT == kFmtF16 ? __fmaf_rn(lo, kW, x[g]) : __fadd_rn(lo, x[g]);
-              }
-              if (amax != nullptr && mok && n0 + chunk * 8 + j < N)
-                lmax = fmaxf(lmax, fabsf(__fmul_rn(lo, scale)));
-              if (outp != nullptr)
-                v[c * 8 + j] = class_sum<S, BITS, FMT == kFmtF16>(x, es, fl & kTcFloatRest);
+            for (int g = S - 1; g >= 0; --g) {
+              x[g] = __uint_as_float(acc[g][j]);
+              lo = FMT == kFmtF16 ? __fmaf_rn(lo, kW, x[g]) : __fadd_rn(lo, x[g]);
+            }
+            if (!mok || n + j >= N) continue;
+            if (amax != nullptr) lmax = fmaxf(lmax, fabsf(__fmul_rn(lo, scale)));
+            if (outp != nullptr) {
+              const double v = class_sum<S, BITS, FMT == kFmtF16>(x, es, fl & kTcFloatRest);
+              double* o = out + (n + j) * step;
+              if (fl & kTcAtomic)
+                atomicAdd(o, v);
+              else
+                *o = fl & kTcAccum ? *o + v : v;
             }
           }
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) arrive_cluster(map_rank(tempty(buf), 0));
-        if (mok && outp != nullptr) {
-          const bool rows = lay.mode == kOutF64Rows;   // out[m][n], else out[n][m]
-          double* out = reinterpret_cast<double*>(outp) + (rows ? (int64_t)m * ldo : m);
-          const int64_t step = rows ? 1 : ldo;
-#pragma unroll
-          for (int c = 0; c < CH; ++c) {
-            const int n = n0 + (4 * c + part) * 8;
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-              if (4 * c + part < nch && n + j < N) {
-                double* o = out + (n + j) * step;
-                if (fl & kTcAtomic)
-                  atomicAdd(o, v[c * 8 + j]);
-                else
-                  *o = fl & kTcAccum ? *o + v[c * 8 + j] : v[c * 8 + j];
-              }
-          }
-        }
       }
     }
     if (sizeof(OutT) == 8 && amax != nullptr) {
@@ -699,6 +692,7 @@ cudaError_t launch_pair(const CUtensorMap* mA, const CUtensorMap* mB, const TcPr
       tile.stages > kMaxStages || (tile.nbuf == 2 && 2 * S * tile.w > 512) ||
       (int64_t)tile.nN * tile.w < N || (int64_t)(tile.nN - 1) * tile.w >= N)
     return cudaErrorInvalidValue;
+  if (sizeof(OutT) == 8 && tile.nbuf != 2) return cudaErrorInvalidValue;
   int ex;
   if (std::frexp(scale, &ex) != 0.5) return cudaErrorInvalidValue;   // scale = 2^(ex - 1)
   auto k = tc_pair_gemm<S, FMT, OutT>;
@@ -730,6 +724,16 @@ PairTile pair_tile(int S, int N, int cap) {
   return t;
 }
 
+// Tile of a float64-output launch: 64 columns at most, fewer (32, 16) while the
+// launch has fewer tiles than the device has pairs.
+PairTile pair_tile_f64(int S, int nprob, int M, int N) {
+  const int wide = std::min(kF64Width, 256 / S / 16 * 16);
+  int cap = wide;
+  const long long mt = (long long)nprob * ((M + 2 * BM - 1) / (2 * BM));
+  while (cap > 16 && mt * ((N + cap - 1) / cap) < 76) cap = cap > 32 ? 32 : 16;
+  return pair_tile(S, N, cap);
+}
+
 // mA: maps with boxes of 128 rows x S slices, mB: of tile.w / 2 rows x S slices.
 template <int S, int FMT>
 cudaError_t launch_tc_pair(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs_dev,
@@ -745,7 +749,7 @@ cudaError_t launch_tc_pair(const CUtensorMap* mA, const CUtensorMap* mB, const T
 
 // One product with float64 output: p.out[n][m] (pitch ldo) = scale 2^14 units of
 // the class sums of segment p.seg[0], and / or its largest magnitude in *amax
-// (p.out NULL: only that).  Tile from pair_tile(S, N, 128).
+// (p.out NULL: only that).  Tile from pair_tile_f64.
 template <int S, int FMT>
 cudaError_t launch_tc_pair_f64(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb& p,
                                int M, int N, int ldo, double scale, int* flag,
