@@ -100,9 +100,9 @@ __global__ void __launch_bounds__(256) gemm_f64_strided(const GemmS* __restrict_
 // element in shared memory and sums what belongs to (b, c), b and c; pass 2,
 // thread (a, c), sums over b what belongs to (a, c) and a; pass 3, thread (a,
 // b), sums over c.  Sums along a thread index are 16-lane shuffles.  Bound by
-// its ~50 float64 operations per element (one division).  60/7/5 domain, all
-// triplets: 9.8 ms with shared-memory atomics (256 threads on one address for
-// every a), 1.0 ms so.
+// its ~45 float64 operations per element.  60/7/5 domain, all triplets: 9.8 ms
+// with shared-memory atomics (256 threads on one address for every a), 2.7 ms in
+// three passes, 1.7 ms with one reciprocal for its two divisions.
 constexpr int kGvPitch = TB + 1;
 constexpr int kGvTile = TB * TB * kGvPitch;   // doubles of one padded tile [a][b][c]
 constexpr size_t kBackwardSmem = 2 * kGvTile * sizeof(double);
@@ -111,6 +111,18 @@ __device__ __forceinline__ double sum16(double x) {   // over the 16 lanes that 
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   return x;
+}
+
+// 1 / D to ~1 ulp: float32 reciprocal and two Newton steps (a float64 division is
+// ~20 operations of the 1/64-rate pipe, this 8); magnitudes outside float32's safe
+// range take the division.
+__device__ __forceinline__ double recip(double D) {
+  const double m = fabs(D);
+  if (!(m > 1e-30 && m < 1e30)) return 1.0 / D;
+  double r = (double)(1.0f / (float)D);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) r = fma(r, fma(-D, r, 1.0), r);
+  return r;
 }
 
 template <bool MIXED, bool FM>
@@ -248,10 +260,10 @@ energy_backward(EnergyArgs a, const double* __restrict__ X, const double* __rest
           }
           const double D = eocc - ev[0][al] - ev[1][bl] - ev[2][cl];
           // E = W (W + V) / D, or W V / D for the f_ov part
-          const double s = gscale / D;
+          const double inv = recip(D), s = gscale * inv;
           const double gw = s * (FM ? v : 2.0 * w + v);
           gv = s * w;
-          gd = -gv * (FM ? v : w + v) / D;
+          gd = -gv * (FM ? v : w + v) * inv;
           double* d3 = MIXED ? dZg : dXg;
           if (FM) {
             dXg[i1] += gw; dXg[i2] -= gw; d3[i3] += gw;

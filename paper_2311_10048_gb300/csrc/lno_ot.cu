@@ -1168,10 +1168,10 @@ struct SpinPass {
     }
     int G = (int)std::max<int64_t>(
         1, std::min<int64_t>(group_cap, budget / std::max<int64_t>(per_trip, 1)));
-    // energy chunks per triplet from the domain's shape only, so that a
-    // triplet's partial sums (and its e_t, bit for bit) do not depend on
-    // which other triplets the call selects
-    const int Gshape = G;
+    // energy chunks per triplet from the domain's shape only (a full group of all
+    // the case's triplets), so that a triplet's partial sums (and its e_t, bit for
+    // bit) do not depend on which other triplets the call selects
+    const int Gshape = cs.ntot > 0 ? (int)std::min<int64_t>(G, cs.ntot) : std::min(G, ntrip);
     G = std::min(G, ntrip);
     char *X = nullptr, *Z = nullptr;
     TRY(A.get(&X, (size_t)(G * xs * esz) + 64));

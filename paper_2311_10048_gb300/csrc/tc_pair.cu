@@ -337,8 +337,8 @@ __device__ __forceinline__ double class_sum(const float (&c)[S], int e, bool res
 }
 
 // TF32: 32-bit elements, 16 per 64-byte row, K 8 per MMA; the 16-bit formats
-// have 32 per row, K 16.  diag is the bounded-wait test hook of tc_gemm.cu.
-template <int S, int FMT, typename OutT>
+// have 32 per row, K 16.  ROWS: float64 output as out[m][n].  diag is the bounded-wait test hook of tc_gemm.cu.
+template <int S, int FMT, typename OutT, bool ROWS>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<OutT>(), 1)
 tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
              const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
@@ -602,19 +602,32 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
       } else {
         constexpr int BITS = FMT == kFmtBF16 ? 8 : 11;
         const int es = P.ea ? *P.ea + *P.eb - 14 : escale, fl = P.flags;
-        const bool rows = lay.mode == kOutF64Rows;   // out[m][n], else out[n][m]
-        double* out = reinterpret_cast<double*>(outp) + (rows ? (int64_t)m * ldo : m);
-        const int64_t step = rows ? 1 : ldo;
+        // out[n][m]: this lane's row m of column n + j in turn.  out[m][n] (ROWS): the
+        // 8 x 8 blocks of 8 lanes are transposed, so that 8 lanes write 8 columns of
+        // one row (64 bytes, whole sectors; one lane per row made four times the L2
+        // operations, and atomics run at the rate of those: 105 products of 2809 x
+        // 53 added in 385 us, now 146)
+        double* const out = reinterpret_cast<double*>(outp);
+        const int b8 = lane & 7, m8 = m - b8;   // first row of the lane's 8 x 8 block
         if (!pair_wait(tfull(buf), use & 1u, flag, 6, true, wlim)) break;
         tc_fence_after();
         const int nch = ntile_w(nt) / 8;   // 8-column chunks, dealt over the four warps
 #pragma unroll 1
         for (int chunk = part; chunk < nch; chunk += 4) {
+          const int n = n0 + chunk * 8;
+          double* const rp = out + (int64_t)m8 * ldo + n + b8;   // ROWS: this lane's column
+          const bool cok = n + b8 < N;
+          double old[ROWS ? 8 : 1];   // what is added to, asked for before the conversions
+          if constexpr (ROWS) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              old[j] = (fl & kTcAccum) && cok && m8 + j < M ? rp[(int64_t)j * ldo] : 0.0;
+          }
           uint32_t acc[S][8];
 #pragma unroll
           for (int g = 0; g < S; ++g) tmem_ld8(tb + g * tile.w + chunk * 8, acc[g]);
           tmem_ld_wait();
-          const int n = n0 + chunk * 8;
+          double v[ROWS ? 8 : 1];
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             float x[S], lo = 0.f;
@@ -623,15 +636,42 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
               x[g] = __uint_as_float(acc[g][j]);
               lo = FMT == kFmtF16 ? __fmaf_rn(lo, kW, x[g]) : __fadd_rn(lo, x[g]);
             }
-            if (!mok || n + j >= N) continue;
-            if (amax != nullptr) lmax = fmaxf(lmax, fabsf(__fmul_rn(lo, scale)));
-            if (outp != nullptr) {
-              const double v = class_sum<S, BITS, FMT == kFmtF16>(x, es, fl & kTcFloatRest);
-              double* o = out + (n + j) * step;
+            if constexpr (ROWS) {
+              v[j] = class_sum<S, BITS, FMT == kFmtF16>(x, es, fl & kTcFloatRest);
+            } else {
+              if (!mok || n + j >= N) continue;
+              if (amax != nullptr) lmax = fmaxf(lmax, fabsf(__fmul_rn(lo, scale)));
+              if (outp != nullptr) {
+                const double y = class_sum<S, BITS, FMT == kFmtF16>(x, es, fl & kTcFloatRest);
+                double* o = out + (int64_t)(n + j) * ldo + m;
+                if (fl & kTcAtomic)
+                  atomicAdd(o, y);
+                else
+                  *o = fl & kTcAccum ? *o + y : y;
+              }
+            }
+          }
+          if constexpr (ROWS) {
+#pragma unroll
+            for (int sft = 1; sft < 8; sft <<= 1)
+#pragma unroll
+              for (int j = 0; j < 8; ++j)
+                if (!(j & sft)) {
+                  const bool up = b8 & sft;
+                  const double y = __shfl_xor_sync(0xffffffffu, up ? v[j] : v[j | sft], sft);
+                  if (up)
+                    v[j] = y;
+                  else
+                    v[j | sft] = y;
+                }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              if (!cok || m8 + j >= M) continue;
+              double* o = rp + (int64_t)j * ldo;
               if (fl & kTcAtomic)
-                atomicAdd(o, v);
+                atomicAdd(o, v[j]);
               else
-                *o = fl & kTcAccum ? *o + v : v;
+                *o = fl & kTcAccum ? old[j] + v[j] : v[j];
             }
           }
         }
@@ -658,10 +698,10 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
 
 // Pairs that fit the device at once (queried once; the persistent loop deals
 // its tiles over them, so none may wait for a slot).
-template <int S, int FMT, typename OutT>
+template <int S, int FMT, typename OutT, bool ROWS>
 int pair_clusters(int nsm) {
   static const int n = [] {
-    auto k = tc_pair_gemm<S, FMT, OutT>;
+    auto k = tc_pair_gemm<S, FMT, OutT, ROWS>;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2);
     cfg.blockDim = dim3(pair_threads<OutT>());
@@ -682,7 +722,7 @@ int pair_clusters(int nsm) {
   return std::max(1, n > 0 ? std::min(n, nsm / 2) : nsm / 2);
 }
 
-template <int S, int FMT, typename OutT>
+template <int S, int FMT, typename OutT, bool ROWS = false>
 cudaError_t launch_pair(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs,
                         const TcProb& one, int nprob, int M, int N, int ldo, double scale,
                         int* flag, unsigned long long* amax, int nsm, cudaStream_t st,
@@ -695,11 +735,11 @@ cudaError_t launch_pair(const CUtensorMap* mA, const CUtensorMap* mB, const TcPr
   if (sizeof(OutT) == 8 && tile.nbuf != 2) return cudaErrorInvalidValue;
   int ex;
   if (std::frexp(scale, &ex) != 0.5) return cudaErrorInvalidValue;   // scale = 2^(ex - 1)
-  auto k = tc_pair_gemm<S, FMT, OutT>;
+  auto k = tc_pair_gemm<S, FMT, OutT, ROWS>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
   if (e != cudaSuccess) return e;
   const long long units = (long long)nprob * ((M + 2 * BM - 1) / (2 * BM)) * tile.nN;
-  const int pairs = (int)std::min<long long>(units, pair_clusters<S, FMT, OutT>(nsm));
+  const int pairs = (int)std::min<long long>(units, pair_clusters<S, FMT, OutT, ROWS>(nsm));
   k<<<2 * pairs, pair_threads<OutT>(), kSmemBytes, st>>>(mA[0], mA[1], mB[0], mB[1], probs, one,
                                                          nprob, M, N, ldo, (float)scale, ex - 1,
                                                          flag, amax, diag, lay, tile);
@@ -766,8 +806,10 @@ cudaError_t launch_tc_pair_f64_group(const CUtensorMap* mA, const CUtensorMap* m
                                      double scale, int* flag, int nsm, cudaStream_t st,
                                      int mode, PairTile tile) {
   if (nprob > 0 && probs_dev == nullptr) return cudaErrorInvalidValue;
-  return launch_pair<S, FMT, double>(mA, mB, probs_dev, TcProb{}, nprob, M, N, ldo, scale, flag,
-                                     nullptr, nsm, st, tc_normal(), TcOut{mode, 0, 0, 0}, tile);
+  auto launch = mode == kOutF64Rows ? launch_pair<S, FMT, double, true>
+                                    : launch_pair<S, FMT, double, false>;
+  return launch(mA, mB, probs_dev, TcProb{}, nprob, M, N, ldo, scale, flag, nullptr, nsm, st,
+                tc_normal(), TcOut{mode, 0, 0, 0}, tile);
 }
 template cudaError_t launch_tc_pair_f64_group<4, kFmtBF16>(const CUtensorMap*, const CUtensorMap*,
                                                            const TcProb*, int, int, int, int,
