@@ -102,6 +102,32 @@ __device__ __forceinline__ int64_t ovts_idx(const EnergyArgs& a, int K, int C, i
   return (((int64_t)a.oslot_t[K] * a.nvt + C) * a.ns_c + a.oslot_s[p]) * a.nvs + x;
 }
 
+// Case sums of one call (case_sums in energy.cu): out[c] = sum of e[c][0..n[c]), copied
+// to copy[c] where given.
+struct CaseSums {
+  const double* e[4];
+  int64_t n[4];
+  double* copy[4];
+  double* out;
+};
+
+// Arrays measured by one launch of absmax: *out[q] = max |x[q]| (bits of a double).
+struct AbsmaxList {
+  static constexpr int kMax = 5;
+  const double* x[kMax];
+  int64_t n[kMax];
+  unsigned long long* out[kMax];
+  int count;
+};
+
+// The DF factor blocks of one spin in one layout launch (transpose_blocks).
+template <class St>
+struct BlockList {
+  static constexpr int kMax = 3;
+  int p0[kMax], np[kMax], q0[kMax], nq[kMax], Qp[kMax];
+  St st[kMax];
+};
+
 // Inputs of the orbital partition: per-case triplets and contributions.
 struct OrbPartArgs {
   const double* e[4];   // per-triplet contributions of cases aaa, aab, abb, bbb

@@ -960,14 +960,20 @@ __global__ void __launch_bounds__(256) orbital_partition(OrbPartArgs A) {
   if (threadIdx.x == 0 && out) out[p] = v.s + v.c;
 }
 
-// out[0] = Neumaier sum of e[0..n): one CTA of 256 threads, fixed order.  (Adding
-// the 256 threads' pairs one after the other took 73 us, this 4.)
-__global__ void __launch_bounds__(256)
-neumaier_sum(const double* __restrict__ e, int64_t n, double* out) {
+// Per-case Neumaier sums (fixed order) and the caller's copies of the per-triplet
+// values: one CTA per case, one launch per call.  (Adding the 256 threads' pairs
+// one after the other took 73 us a case, this 7 for all.)
+__global__ void __launch_bounds__(256) case_sums(CaseSums A) {
+  const int c = blockIdx.x;
+  const double* e = A.e[c];
   Nsum v{0.0, 0.0};
-  for (int64_t q = threadIdx.x; q < n; q += 256) v.add(e[q]);
+  for (int64_t q = threadIdx.x; q < A.n[c]; q += 256) {
+    const double x = e[q];
+    v.add(x);
+    if (A.copy[c]) A.copy[c][q] = x;
+  }
   v = block_sum(v);
-  if (threadIdx.x == 0) out[0] = v.s + v.c;
+  if (threadIdx.x == 0) A.out[c] = v.s + v.c;
 }
 
 }  // namespace
@@ -1177,8 +1183,8 @@ cudaError_t energy_timeout_selftest(long long wait_cycles, int nsm, int* code, c
   return finish(cudaSuccess);
 }
 
-cudaError_t launch_neumaier_sum(const double* e, int64_t n, double* out, cudaStream_t st) {
-  neumaier_sum<<<1, 256, 0, st>>>(e, n, out);
+cudaError_t launch_case_sums(const CaseSums& A, cudaStream_t st) {
+  case_sums<<<4, 256, 0, st>>>(A);
   return cudaGetLastError();
 }
 

@@ -43,12 +43,11 @@ cudaError_t launch_energy_f32_fused(const EnergyArgs& a, const float* X, const f
 cudaError_t launch_reduce_partials(const double* partial, int np, const double* partial2,
                                    int ntrip, double* e_trip, cudaStream_t st);
 cudaError_t launch_orbital_partition(const OrbPartArgs& A, cudaStream_t st);
-cudaError_t launch_neumaier_sum(const double* e, int64_t n, double* out, cudaStream_t st);
+cudaError_t launch_case_sums(const CaseSums& A, cudaStream_t st);
 cudaError_t energy_timeout_selftest(long long wait_cycles, int nsm, int* code, cudaStream_t st);
 // pack.cu
 template <class St>
-cudaError_t launch_transpose_block(const double*, int, int, int, int, int, int, int, St,
-                                   cudaStream_t);
+cudaError_t launch_transpose_blocks(const double*, int, int, const BlockList<St>&, cudaStream_t);
 template <class St>
 cudaError_t launch_pack_at_same(const int2*, int, int, int, int, int, const double*, const double*,
                                 St, cudaStream_t);
@@ -69,6 +68,7 @@ cudaError_t launch_pack_at2(const int2*, int, int, int, int, int, int, int, cons
                             const double*, St, cudaStream_t);
 cudaError_t launch_transpose_t2ab(const double*, int, int, int, int, double*, cudaStream_t);
 cudaError_t launch_absmax(const double*, int64_t, unsigned long long*, cudaStream_t);
+cudaError_t launch_absmax_list(const AbsmaxList& L, cudaStream_t s);
 cudaError_t launch_row_norm2(const void* p, int64_t rows, int Kp, unsigned long long* out,
                              cudaStream_t s);
 cudaError_t launch_view_absmax(const double* in, int64_t rs, int64_t ks, int rows, int K,
@@ -525,24 +525,25 @@ struct Run {
       if (noi[s] < 0 || noi[s] > no[s]) noi[s] = no[s];
     }
     if (!f64) {  // global scales of B and T2
-      CU(cudaMemsetAsync(ctx->d_amax, 0, sizeof(unsigned long long), st));
-      for (int s = 0; s < 2; ++s)
-        CU(launch_absmax(dom->B[s], (int64_t)naux * nbs[s] * nbs[s], ctx->d_amax, st));
-      unsigned long long h;
-      CU(cudaMemcpyAsync(&h, ctx->d_amax, sizeof h, cudaMemcpyDeviceToHost, st));
-      CU(cudaMemsetAsync(ctx->d_amax, 0, sizeof(unsigned long long), st));
-      CU(launch_absmax(dom->t2aa, (int64_t)no[0] * no[0] * nv[0] * nv[0], ctx->d_amax, st));
-      CU(launch_absmax(dom->t2bb, (int64_t)no[1] * no[1] * nv[1] * nv[1], ctx->d_amax, st));
-      CU(launch_absmax(dom->t2ab, (int64_t)no[0] * no[1] * nv[0] * nv[1], ctx->d_amax, st));
-      unsigned long long ht;
-      CU(cudaMemcpyAsync(&ht, ctx->d_amax, sizeof ht, cudaMemcpyDeviceToHost, st));
+      CU(cudaMemsetAsync(ctx->d_amax, 0, 2 * sizeof(unsigned long long), st));
+      AbsmaxList L{};
+      auto measure = [&](const double* x, int64_t n, int slot) {
+        if (n == 0) return;
+        L.x[L.count] = x;
+        L.n[L.count] = n;
+        L.out[L.count++] = ctx->d_amax + slot;
+      };
+      for (int s = 0; s < 2; ++s) measure(dom->B[s], (int64_t)naux * nbs[s] * nbs[s], 0);
+      measure(dom->t2aa, (int64_t)no[0] * no[0] * nv[0] * nv[0], 1);
+      measure(dom->t2bb, (int64_t)no[1] * no[1] * nv[1] * nv[1], 1);
+      measure(dom->t2ab, (int64_t)no[0] * no[1] * nv[0] * nv[1], 1);
+      CU(launch_absmax_list(L, st));
+      double h[2];
+      CU(cudaMemcpyAsync(h, ctx->d_amax, sizeof h, cudaMemcpyDeviceToHost, st));
       CU(cudaStreamSynchronize(st));
-      double mb, mt;
-      std::memcpy(&mb, &h, 8);
-      std::memcpy(&mt, &ht, 8);
-      sigB = pow2_scale(mb);
-      sigT = pow2_scale(mt);
-      stats->other_launches += 5;
+      sigB = pow2_scale(h[0]);
+      sigT = pow2_scale(h[1]);
+      stats->other_launches++;
     }
     if (dom->fov[0] || dom->fov[1]) {  // a missing spin block is zero
       for (int s = 0; s < 2; ++s) {
@@ -562,30 +563,37 @@ struct Run {
       TRY(alloc_operand(Boo[s], 1, (int64_t)oi * o, naux, Sdf));
       TRY(alloc_operand(Bov[s], 1, (int64_t)o * v, naux, Sdf));
       TRY(alloc_operand(Bvv[s], 1, (int64_t)v * v, naux, Sdf));
-      struct Blk {
-        Operand* op;
-        int p0, np, q0, nq;
-      } blks[3] = {{&Boo[s], 0, oi, 0, o}, {&Bov[s], 0, o, o, v}, {&Bvv[s], o, v, o, v}};
+      Operand* ops[3] = {&Boo[s], &Bov[s], &Bvv[s]};
+      const int p0[3] = {0, 0, o}, np[3] = {oi, o, v}, q0[3] = {0, o, o}, nq[3] = {o, v, v};
       const int eB = 7 - std::ilogb(sigB);
-      for (auto& b : blks) {
-        stats->other_launches++;
-        if (f64)
-          CU(launch_transpose_block(dom->B[s], naux, nbs[s], b.p0, b.np, b.q0, b.nq, b.op->Kp,
-                                    StoreF64{b.op->f64}, st));
-        else if (f16)
-          CU(launch_transpose_block(
-              dom->B[s], naux, nbs[s], b.p0, b.np, b.q0, b.nq, b.op->Kp,
-              StoreSlices<3, __half>{reinterpret_cast<__half*>(b.op->bf), b.op->slice_stride,
-                                     eB + 3, eB + 3}, st));
-        else if (Sdf == 5)
-          CU(launch_transpose_block(
-              dom->B[s], naux, nbs[s], b.p0, b.np, b.q0, b.nq, b.op->Kp,
-              StoreSlices<5>{b.op->bf, b.op->slice_stride, eB, eB}, st));
-        else
-          CU(launch_transpose_block(
-              dom->B[s], naux, nbs[s], b.p0, b.np, b.q0, b.nq, b.op->Kp,
-              StoreSlices<4>{b.op->bf, b.op->slice_stride, eB, eB}, st));
-      }
+      auto layout = [&](auto&& store) {
+        BlockList<std::decay_t<decltype(store(Boo[s]))>> L{};
+        for (int k = 0; k < 3; ++k) {
+          L.p0[k] = p0[k];
+          L.np[k] = np[k];
+          L.q0[k] = q0[k];
+          L.nq[k] = nq[k];
+          L.Qp[k] = ops[k]->Kp;
+          L.st[k] = store(*ops[k]);
+        }
+        return launch_transpose_blocks(dom->B[s], naux, nbs[s], L, st);
+      };
+      stats->other_launches++;
+      if (f64)
+        CU(layout([&](const Operand& op) { return StoreF64{op.f64}; }));
+      else if (f16)
+        CU(layout([&](const Operand& op) {
+          return StoreSlices<3, __half>{reinterpret_cast<__half*>(op.bf), op.slice_stride, eB + 3,
+                                        eB + 3};
+        }));
+      else if (Sdf == 5)
+        CU(layout([&](const Operand& op) {
+          return StoreSlices<5>{op.bf, op.slice_stride, eB, eB};
+        }));
+      else
+        CU(layout([&](const Operand& op) {
+          return StoreSlices<4>{op.bf, op.slice_stride, eB, eB};
+        }));
       if (f16) {
         CU(cudaMemsetAsync(ctx->d_amax + kNormB + s, 0, sizeof(unsigned long long), st));
         for (const Operand* op : {&Boo[s], &Bov[s], &Bvv[s]}) TRY(row_norm2(*op, kNormB + s));
@@ -693,6 +701,29 @@ void add_chunks(std::vector<TcProb>& out, int a_row, int b_row, int K, bool neg,
   }
 }
 
+// Several host arrays in one device buffer and one copy.
+struct Upload {
+  std::vector<char> blob;
+  std::vector<std::pair<const void**, size_t>> dst;
+  template <typename T>
+  void add(const std::vector<T>& h, const T** d) {
+    *d = nullptr;
+    const size_t off = (blob.size() + 63) / 64 * 64;
+    if (h.empty()) return;
+    blob.resize(off + h.size() * sizeof(T));
+    std::memcpy(blob.data() + off, h.data(), h.size() * sizeof(T));
+    dst.push_back({reinterpret_cast<const void**>(d), off});
+  }
+  int send(Run& R, Arena& A) {
+    if (blob.empty()) return LNO_OT_OK;
+    char* p;
+    TRY(A.get(&p, blob.size()));
+    CU(R.ctx->h2d(p, blob.data(), blob.size()));
+    for (auto& d : dst) *d.first = p + d.second;
+    return LNO_OT_OK;
+  }
+};
+
 // Spin-case triplet selection.
 struct CaseSel {
   std::vector<Trip> trips;   // triplets to compute, in output order
@@ -799,10 +830,11 @@ struct SpinPass {
   Operand BsS, BsT;          // Bov rows of the slots, [slot][vir] x naux
   double* ovss = nullptr;    // (ia|jb) as [nS][vs][nS][vs]
   double* ovts = nullptr;    // (jb|KC) as [nT][vt][nS][vs]
-  int* d_slot_s = nullptr;   // occupied index -> slot (-1 absent), spin s [os]
-  int* d_slot_t = nullptr;   // spin t [ot]
-  int* d_list_s = nullptr;   // slot -> occupied index
-  int* d_list_t = nullptr;
+  const int* d_slot_s = nullptr;   // occupied index -> slot (-1 absent), spin s [os]
+  const int* d_slot_t = nullptr;   // spin t [ot]
+  const int* d_list_s = nullptr;   // slot -> occupied index
+  const int* d_list_t = nullptr;
+  const int2 *d_AT = nullptr, *d_A1 = nullptr, *d_AT2 = nullptr;   // pair lists
 
   Arena own;  // operands and temporaries of this spin pass
 
@@ -905,12 +937,6 @@ struct SpinPass {
       if (p) A.drop(p);
     };
     // pair operands: one DF block, one layout launch
-    auto upload_pairs = [&](const std::vector<int2>& l, int2** dl) -> int {
-      TRY(A.get(dl, l.size()));
-      CU(R.ctx->h2d(*dl, l.data(), l.size() * sizeof(int2)));
-      R.stats->other_launches++;
-      return LNO_OT_OK;
-    };
     // per-orbital operands: the blocks (L rows x [x][r_rows]) of a run at a time
     auto per_orbital = [&](const std::vector<int>& list, const Operand& L, int64_t l_rows,
                            const Operand& Ro, int r_rows, auto&& pack) -> int {
@@ -957,9 +983,8 @@ struct SpinPass {
       TRY(block(&oovoT, (int64_t)o * v * oi * o));
       TRY(R.df(R.Boo[s], 0, oi * o, R.Bov[s], 0, o * v, oovoT, oi * o));
       if (!meas) {
-        int2* dl;
-        TRY(upload_pairs(listAT, &dl));
-        CU(launch_pack_at_same(dl, (int)listAT.size(), o, oi, v, AT.Kp, t2ss, oovoT, stAT, st));
+        R.stats->other_launches++;
+        CU(launch_pack_at_same(d_AT, (int)listAT.size(), o, oi, v, AT.Kp, t2ss, oovoT, stAT, st));
       }
       drop(oovoT);
     }
@@ -974,9 +999,8 @@ struct SpinPass {
       TRY(block(&jT, (int64_t)o * v * oti * ot));
       TRY(R.df(R.Bov[s], 0, o * v, R.Boo[t], 0, oti * ot, jT, o * v));
       if (!meas) {
-        int2* dl;
-        TRY(upload_pairs(listA1, &dl));
-        CU(launch_pack_a1(dl, (int)listA1.size(), o, v, ot, oti, vt, A1.Kp, t2st, jT, stA1, st));
+        R.stats->other_launches++;
+        CU(launch_pack_a1(d_A1, (int)listA1.size(), o, v, ot, oti, vt, A1.Kp, t2st, jT, stA1, st));
       }
       drop(jT);
     }
@@ -995,9 +1019,8 @@ struct SpinPass {
       TRY(block(&lT, (int64_t)ot * vt * oi * o));
       TRY(R.df(R.Boo[s], 0, oi * o, R.Bov[t], 0, ot * vt, lT, oi * o));
       if (!meas) {
-        int2* dl;
-        TRY(upload_pairs(listAT2, &dl));
-        CU(launch_pack_at2(dl, (int)listAT2.size(), o, oi, v, ot, vt, AT2.Kp, t2st, lT, stAT2,
+        R.stats->other_launches++;
+        CU(launch_pack_at2(d_AT2, (int)listAT2.size(), o, oi, v, ot, vt, AT2.Kp, t2st, lT, stAT2,
                            st));
       }
       drop(lT);
@@ -1006,19 +1029,17 @@ struct SpinPass {
     return LNO_OT_OK;
   }
 
-  int upload_ints(const std::vector<int>& h, int** d) {
-    TRY(own.get(d, std::max<size_t>(h.size(), 1)));
-    if (!h.empty())
-      CU(R.ctx->h2d(*d, h.data(), h.size() * sizeof(int)));
-    return LNO_OT_OK;
-  }
-
   int build_v_blocks() {
     const int nS = (int)listBT.size(), nT = (int)listBF.size();
-    TRY(upload_ints(slotBT, &d_slot_s));
-    TRY(upload_ints(slotBF, &d_slot_t));
-    TRY(upload_ints(listBT, &d_list_s));
-    TRY(upload_ints(listBF, &d_list_t));
+    Upload up;
+    up.add(slotBT, &d_slot_s);
+    up.add(slotBF, &d_slot_t);
+    up.add(listBT, &d_list_s);
+    up.add(listBF, &d_list_t);
+    up.add(listAT, &d_AT);
+    up.add(listA1, &d_A1);
+    up.add(listAT2, &d_AT2);
+    TRY(up.send(R, own));
     const int64_t ns = (int64_t)nS * v;
     TRY(R.gather_operand(own, R.Bov[s], d_list_s, nS, v, BsS));
     TRY(own.get(&ovss, (size_t)std::max<int64_t>(ns * ns, 1)));
@@ -1115,14 +1136,6 @@ struct SpinPass {
     return LNO_OT_OK;
   }
 
-  template <typename T>
-  int upload(Arena& A, const std::vector<T>& h, T** d) {
-    if (h.empty()) return LNO_OT_OK;
-    TRY(A.get(d, h.size()));
-    CU(R.ctx->h2d(*d, h.data(), h.size() * sizeof(T)));
-    return LNO_OT_OK;
-  }
-
   void seg_f64(SegF64& sg, const Operand& A, int64_t arow, const Operand& B, int64_t brow,
                double sign) {
     sg = SegF64{A.f64 + arow * A.Kp, B.f64 + brow * B.Kp, A.K, A.Kp, B.Kp, sign};
@@ -1193,12 +1206,6 @@ struct SpinPass {
       CU(cudaMemsetAsync(is_mixed ? e_mixed : e_same, 0, (size_t)ntrip * sizeof(double), R.st));
       return LNO_OT_OK;
     }
-    int3* dblocks;
-    TRY(A.get(&dblocks, blocks.size()));
-    CU(R.ctx->h2d(dblocks, blocks.data(), blocks.size() * sizeof(int3)));
-    Trip* dtrips;
-    TRY(A.get(&dtrips, (size_t)ntrip));
-    CU(R.ctx->h2d(dtrips, cs.trips.data(), ntrip * sizeof(Trip)));
     // float64 path: P chunks per triplet, one CTA each.  Float32 path: P
     // items per triplet on a persistent grid, about 32 items per resident CTA
     // in a full group (so the last round of items is a small fraction), one
@@ -1231,7 +1238,6 @@ struct SpinPass {
     ea.t1s = R.dom->t1[s];
     ea.t1t = R.dom->t1[is_mixed ? t : s];
     set_v_args(ea, is_mixed);
-    ea.blocks = dblocks;
     ea.nblocks = (int)blocks.size();
     ea.pitch_x = P1;
     ea.pitch_z = P2;
@@ -1330,12 +1336,19 @@ struct SpinPass {
         }
       }
     }
-    ProbF64 *dpf = nullptr, *dpf2 = nullptr;
-    TcProb *dpt = nullptr, *dpt2 = nullptr;
-    TRY(upload(A, pf, &dpf));
-    TRY(upload(A, pf2, &dpf2));
-    TRY(upload(A, pt, &dpt));
-    TRY(upload(A, pt2, &dpt2));
+    const int3* dblocks = nullptr;
+    const Trip* dtrips = nullptr;
+    const ProbF64 *dpf = nullptr, *dpf2 = nullptr;
+    const TcProb *dpt = nullptr, *dpt2 = nullptr;
+    Upload up;
+    up.add(blocks, &dblocks);
+    up.add(cs.trips, &dtrips);
+    up.add(pf, &dpf);
+    up.add(pf2, &dpf2);
+    up.add(pt, &dpt);
+    up.add(pt2, &dpt2);
+    TRY(up.send(R, A));
+    ea.blocks = dblocks;
 
     for (int g0 = 0; g0 < ntrip; g0 += G) {
       const int ng = std::min(G, ntrip - g0);
@@ -1480,18 +1493,16 @@ bool scale_too_small(const Run& R, unsigned long long built) {
 int finish_call(lno_ot_ctx* ctx, Run& R, Arena& A, const lno_ot_domain* dom, const CaseSel* cs,
                 double* const* e_int, bool thirds, bool kept, cudaEvent_t t0, cudaEvent_t t1,
                 cudaEvent_t t2, lno_ot_result* out) {
-  // per-case sums
+  // per-case sums and the caller's per-triplet values
+  CaseSums sums{};
   for (int c = 0; c < 4; ++c) {
-    if (cs[c].trips.empty()) {
-      CU(cudaMemsetAsync(ctx->d_sums + c, 0, sizeof(double), R.st));
-    } else {
-      CU(launch_neumaier_sum(e_int[c], (int64_t)cs[c].trips.size(), ctx->d_sums + c, R.st));
-      R.stats->other_launches++;
-      if (dom->e_trip[c])
-        CU(cudaMemcpyAsync(dom->e_trip[c], e_int[c], cs[c].trips.size() * sizeof(double),
-                           cudaMemcpyDeviceToDevice, R.st));
-    }
+    sums.e[c] = e_int[c];
+    sums.n[c] = (int64_t)cs[c].trips.size();
+    sums.copy[c] = dom->e_trip[c];
   }
+  sums.out = ctx->d_sums;
+  CU(launch_case_sums(sums, R.st));
+  R.stats->other_launches++;
   // orbital contributions (eq cim_pt_energy) of the computed triplets
   if (dom->e_orb[0] || dom->e_orb[1]) {
     OrbPartArgs oa{};

@@ -36,13 +36,22 @@ namespace lno {
 
 namespace {
 
-// B[s] [naux][nbas][nbas] -> out[p'][q'][Q] = B[Q][p0+p'][q0+q'] (p' < np, q' < nq)
+// B[s] [naux][nbas][nbas] -> out[p'][q'][Q] = B[Q][p0+p'][q0+q'] (p' < np, q' < nq),
+// for the blocks of a list: blockIdx.x runs over the 32-row tiles of all of them
 template <class St>
-__global__ void transpose_block(const double* __restrict__ B, int naux, int nbas, int p0, int np,
-                                int q0, int nq, int Qp, St st) {
+__global__ void transpose_blocks(const double* __restrict__ B, int naux, int nbas,
+                                 BlockList<St> L) {
   __shared__ double tile[32][33];
+  int k = 0;
+  int64_t t = blockIdx.x;
+  for (; k < BlockList<St>::kMax - 1; ++k) {
+    const int64_t nt = ((int64_t)L.np[k] * L.nq[k] + 31) / 32;
+    if (t < nt) break;
+    t -= nt;
+  }
+  const int p0 = L.p0[k], np = L.np[k], q0 = L.q0[k], nq = L.nq[k], Qp = L.Qp[k];
   const int64_t nrows = (int64_t)np * nq;
-  const int64_t r0 = (int64_t)blockIdx.x * 32;
+  const int64_t r0 = t * 32;
   const int Q0 = blockIdx.y * 32;
   for (int yy = threadIdx.y; yy < 32; yy += blockDim.y) {
     const int Q = Q0 + yy;
@@ -58,7 +67,7 @@ __global__ void transpose_block(const double* __restrict__ B, int naux, int nbas
   for (int yy = threadIdx.y; yy < 32; yy += blockDim.y) {
     const int64_t r = r0 + yy;
     const int Q = Q0 + threadIdx.x;
-    if (r < nrows && Q < Qp) st(r * Qp + Q, Q < naux ? tile[threadIdx.x][yy] : 0.0, 1);
+    if (r < nrows && Q < Qp) L.st[k](r * Qp + Q, Q < naux ? tile[threadIdx.x][yy] : 0.0, 1);
   }
 }
 
@@ -418,15 +427,18 @@ __global__ void sum_partials(const double* __restrict__ part, int nsp, int M, in
   }
 }
 
-// max |x| over n doubles, as the bits of a non-negative double in *out (atomicMax).
-__global__ void absmax_kernel(const double* __restrict__ x, int64_t n,
-                              unsigned long long* __restrict__ out) {
+// max |x| over the arrays of a list, as the bits of a non-negative double in their
+// *out (atomicMax); blockIdx.y is the array.
+__global__ void absmax_kernel(AbsmaxList L) {
+  const double* __restrict__ x = L.x[blockIdx.y];
+  const int64_t n = L.n[blockIdx.y];
   double m = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     m = fmax(m, fabs(x[i]));
   for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
+  if ((threadIdx.x & 31) == 0 && m > 0.0)
+    atomicMax(L.out[blockIdx.y], (unsigned long long)__double_as_longlong(m));
 }
 
 // Row-block gather: dst slot q <- src slot list[q], each slot `row16` 16-byte
@@ -511,12 +523,17 @@ inline int grid_for(int64_t n) {
 // Host launchers (templated store: F64 or slices)
 // ---------------------------------------------------------------------------
 template <class St>
-cudaError_t launch_transpose_block(const double* B, int naux, int nbas, int p0, int np, int q0,
-                                   int nq, int Qp, St st, cudaStream_t s) {
-  int64_t rows = (int64_t)np * nq;
-  if (rows == 0) return cudaSuccess;
-  dim3 grid(ceil_div(rows, 32), ceil_div(Qp, 32));
-  transpose_block<<<grid, dim3(32, 8), 0, s>>>(B, naux, nbas, p0, np, q0, nq, Qp, st);
+cudaError_t launch_transpose_blocks(const double* B, int naux, int nbas, const BlockList<St>& L,
+                                    cudaStream_t s) {
+  int64_t tiles = 0;
+  int Qp = 0;
+  for (int k = 0; k < BlockList<St>::kMax; ++k) {
+    tiles += ((int64_t)L.np[k] * L.nq[k] + 31) / 32;
+    Qp = std::max(Qp, L.Qp[k]);
+  }
+  if (tiles == 0) return cudaSuccess;
+  transpose_blocks<<<dim3((unsigned)tiles, ceil_div(Qp, 32)), dim3(32, 8), 0, s>>>(B, naux, nbas,
+                                                                                 L);
   return cudaGetLastError();
 }
 
@@ -622,10 +639,21 @@ cudaError_t launch_row_norm2(const void* p, int64_t rows, int Kp, unsigned long 
   return cudaGetLastError();
 }
 
-cudaError_t launch_absmax(const double* x, int64_t n, unsigned long long* out, cudaStream_t s) {
+cudaError_t launch_absmax_list(const AbsmaxList& L, cudaStream_t s) {
+  int64_t n = 0;
+  for (int q = 0; q < L.count; ++q) n = std::max(n, L.n[q]);
   if (n == 0) return cudaSuccess;
-  absmax_kernel<<<grid_for(n), 256, 0, s>>>(x, n, out);
+  absmax_kernel<<<dim3(std::min(grid_for(n), 152 * 8), L.count), 256, 0, s>>>(L);
   return cudaGetLastError();
+}
+
+cudaError_t launch_absmax(const double* x, int64_t n, unsigned long long* out, cudaStream_t s) {
+  AbsmaxList L{};
+  L.x[0] = x;
+  L.n[0] = n;
+  L.out[0] = out;
+  L.count = 1;
+  return launch_absmax_list(L, s);
 }
 
 cudaError_t launch_sum_partials(const double* part, int nsp, int M, int N, double* C,
@@ -681,8 +709,8 @@ template cudaError_t launch_view_slices<5>(const double*, int64_t, int64_t, int,
                                            __nv_bfloat16*, int64_t, double, cudaStream_t);
 
 #define LNO_INST(St)                                                                           \
-  template cudaError_t launch_transpose_block<St>(const double*, int, int, int, int, int, int,  \
-                                                  int, St, cudaStream_t);                       \
+  template cudaError_t launch_transpose_blocks<St>(const double*, int, int,                      \
+                                                   const BlockList<St>&, cudaStream_t);         \
   template cudaError_t launch_pack_at_same<St>(const int2*, int, int, int, int, int,           \
                                                const double*, const double*, St, cudaStream_t); \
   template cudaError_t launch_pack_bt_same<St>(int, int, int, int, int, int, int,               \
