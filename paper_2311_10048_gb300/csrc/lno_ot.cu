@@ -188,6 +188,7 @@ struct lno_ot_ctx {
   }
   bool exact_measure = false;          // integral scale from every slice (measure_sigI)
   bool no_f16 = false;                 // BF16X10 on its BF16 slices only (kNoF16)
+  bool frugal = false;                 // the call runs again after the device ran out of memory
   // prepared operands of the last domain (options.keep_operands)
   bool keep = false;
   struct DomainCache* cache = nullptr;
@@ -246,33 +247,41 @@ constexpr double kExactSum = 16777216.0 * 0.999;
 struct Arena {
   cudaStream_t st;
   size_t limit, used = 0;
-  std::vector<void*> ptrs;
+  struct Block {
+    void* p;
+    size_t charge;
+  };
+  std::vector<Block> ptrs;
   Arena(cudaStream_t s, size_t lim) : st(s), limit(lim) {}
   ~Arena() { release(); }
   void release() {
-    for (void* p : ptrs) cudaFreeAsync(p, st);
+    for (const Block& b : ptrs) cudaFreeAsync(b.p, st);
     ptrs.clear();
     used = 0;
   }
+  // `charged` < n elements count against the limit: the caller's bound covers the
+  // data, not what rows are padded with for the loads' sake (the pitch of a sliced
+  // row adds up to 31 elements), so a finer pitch refuses no call.
   template <typename T>
-  int get(T** out, size_t n) {
-    size_t bytes = std::max<size_t>(n * sizeof(T), 256);
-    bytes = (bytes + 255) / 256 * 256;
-    if (limit && used + bytes > limit) return LNO_OT_ENOMEM;
+  int get(T** out, size_t n, size_t charged = SIZE_MAX) {
+    auto whole = [](size_t k) { return (std::max<size_t>(k * sizeof(T), 256) + 255) / 256 * 256; };
+    const size_t bytes = whole(n), charge = whole(std::min(n, charged));
+    if (limit && used + charge > limit) return LNO_OT_ENOMEM;
     void* p = nullptr;
     if (cudaMallocAsync(&p, bytes, st) != cudaSuccess) {
       cudaGetLastError();
       return LNO_OT_ENOMEM;
     }
-    ptrs.push_back(p);
-    used += bytes;
+    ptrs.push_back({p, charge});
+    used += charge;
     *out = static_cast<T*>(p);
     return LNO_OT_OK;
   }
   void drop(void* p) {
     for (auto& q : ptrs)
-      if (q == p) {
-        cudaFreeAsync(q, st);
+      if (q.p == p) {
+        cudaFreeAsync(p, st);
+        used -= q.charge;
         q = ptrs.back();
         ptrs.pop_back();
         return;
@@ -427,16 +436,18 @@ struct Run {
     op.Kp = (int)round_up(std::max(K, 1), f64 || tf ? 16 : 32);
     op.S = f64 ? 0 : S_;
     const int64_t n = std::max<int64_t>((int64_t)nslot * rows * op.Kp, 8);
+    const int64_t data =
+        std::max<int64_t>((int64_t)nslot * rows * round_up(std::max(K, 1), 8), 8);
     if (f64) {
-      TRY(ar.get(&op.f64, (size_t)n));
+      TRY(ar.get(&op.f64, (size_t)n, (size_t)data));
     } else {
       op.slice_stride = round_up(n, 8);
       if (tf) {
         op.esz = 4;
-        TRY(ar.get(&op.f32, (size_t)(op.slice_stride * op.S)));
+        TRY(ar.get(&op.f32, (size_t)(op.slice_stride * op.S), (size_t)(data * op.S)));
       } else {
         op.esz = 2;
-        TRY(ar.get(&op.bf, (size_t)(op.slice_stride * op.S)));
+        TRY(ar.get(&op.bf, (size_t)(op.slice_stride * op.S), (size_t)(data * op.S)));
       }
     }
     return LNO_OT_OK;
@@ -803,6 +814,10 @@ double kpad16(double k) { return std::ceil(k / 16.0) * 16.0; }
 // one or two tiles (their number per triplet falls as the group grows) cost 20%:
 // 121/14/11 domain 28.8 ms at 64, 24.6 at 256, 23.4 at 1024.
 constexpr int kGroupCap = 1024;
+// After an allocation failed (the device is shared, or nearly full) a call runs
+// again in small pieces: groups of at most 64 triplets, DF blocks of one orbital,
+// the adjoint's products one by one.
+constexpr int kFrugalGroup = 64;
 
 // ----------------------------------------------------------------------------
 // Per spin s: same-spin case (sss) and the mixed case with two s orbitals.
@@ -905,9 +920,12 @@ struct SpinPass {
     int q, x, n;
   };
   static constexpr int64_t kRunBytes = (int64_t)512 << 20;
-  static std::vector<OrbRun> orb_runs(const std::vector<int>& list, int64_t block_elems) {
-    const int cap = (int)std::max<int64_t>(
-        1, std::min<int64_t>(65535, kRunBytes / 8 / std::max<int64_t>(block_elems, 1)));
+  static std::vector<OrbRun> orb_runs(const std::vector<int>& list, int64_t block_elems,
+                                      bool frugal) {
+    const int cap =
+        frugal ? 1
+               : (int)std::max<int64_t>(1, std::min<int64_t>(65535, kRunBytes / 8 /
+                                                  std::max<int64_t>(block_elems, 1)));
     std::vector<OrbRun> runs;
     for (size_t q = 0; q < list.size(); ++q) {
       if (!runs.empty() && runs.back().n < cap && runs.back().x + runs.back().n == list[q])
@@ -940,7 +958,7 @@ struct SpinPass {
     // per-orbital operands: the blocks (L rows x [x][r_rows]) of a run at a time
     auto per_orbital = [&](const std::vector<int>& list, const Operand& L, int64_t l_rows,
                            const Operand& Ro, int r_rows, auto&& pack) -> int {
-      const auto runs = orb_runs(list, l_rows * r_rows);
+      const auto runs = orb_runs(list, l_rows * r_rows, R.ctx->frugal);
       double* buf;
       TRY(block(&buf, l_rows * r_rows * longest(runs)));
       // adjoint on the tensor cores: one launch per run as well, each orbital's rows
@@ -1179,6 +1197,7 @@ struct SpinPass {
       bn = row->bn;
       group_cap = std::max(1, row->group_cap);
     }
+    if (R.ctx->frugal) group_cap = std::min(group_cap, kFrugalGroup);
     int G = (int)std::max<int64_t>(
         1, std::min<int64_t>(group_cap, budget / std::max<int64_t>(per_trip, 1)));
     // energy chunks per triplet from the domain's shape only (a full group of all
@@ -1828,11 +1847,14 @@ int energy_once(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
 int energy_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
                 const PassSpec* spec = nullptr) {
   int rc = energy_once(ctx, dom, out, spec);
-  for (int tries = 0; rc > 0 && tries < 2; ++tries) {
-    (rc == kRescale ? ctx->exact_measure : ctx->no_f16) = true;
+  for (int tries = 0; tries < 3; ++tries) {
+    if (rc == kRescale) ctx->exact_measure = true;
+    else if (rc == kNoF16) ctx->no_f16 = true;
+    else if (rc == LNO_OT_ENOMEM && !ctx->frugal) ctx->frugal = true;
+    else break;
     rc = energy_once(ctx, dom, out, spec);
   }
-  ctx->exact_measure = ctx->no_f16 = false;
+  ctx->exact_measure = ctx->no_f16 = ctx->frugal = false;
   return rc > 0 ? LNO_OT_EINVAL : rc;   // not reached: neither can come twice
 }
 
@@ -1880,6 +1902,7 @@ int naf_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, double eps, double* cons
   CU(launch_get_diag(W, n, d, st));
   std::vector<double> lam(n);
   unsigned int hasym = 1;
+  for (double* q : {W, W2, norms}) A.drop(q);   // before the factors' copies
   CU(cudaMemcpyAsync(lam.data(), d, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, st));
   CU(cudaMemcpyAsync(&hasym, asym, sizeof hasym, cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));
@@ -2239,7 +2262,7 @@ int backward_spin(SpinPass& P, GradAcc& G, double gE) {
   // slices of all operand slots (batched form)
   const Operand* ops[6] = {&P.AT, &P.BT, &P.A1, &P.BG, &P.BF, &P.AT2};
   SlicedBatch sl[6];
-  bool batched = R.tc_adjoint;
+  bool batched = R.tc_adjoint && !R.ctx->frugal;
   if (batched) {
     int64_t bytes = 0;
     for (const Operand* op : ops) {
@@ -2559,7 +2582,7 @@ int backward_spin(SpinPass& P, GradAcc& G, double gE) {
   auto per_orbital = [&](const std::vector<int>& list, const Operand& L, Operand& dL,
                          int64_t l_rows, const Operand& Ro, Operand& dR, int r_rows,
                          auto&& layout) -> int {
-    const auto runs = SpinPass::orb_runs(list, l_rows * r_rows);
+    const auto runs = SpinPass::orb_runs(list, l_rows * r_rows, R.ctx->frugal);
     const int nmax = SpinPass::longest(runs);
     if (nmax == 0 || l_rows == 0 || r_rows == 0) return LNO_OT_OK;
     const int64_t blk = l_rows * r_rows;
@@ -2695,7 +2718,7 @@ int backward_spin(SpinPass& P, GradAcc& G, double gE) {
   return LNO_OT_OK;
 }
 
-int backward_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, double gE, lno_ot_grad* g) {
+int backward_once(lno_ot_ctx* ctx, const lno_ot_domain* dom, double gE, lno_ot_grad* g) {
   TRY(validate(ctx, dom));
   const int nbas = dom->nbas, naux = dom->naux;
   const int na = dom->nocc[0], nb = dom->nocc[1];
@@ -2820,6 +2843,18 @@ int backward_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, double gE, lno_ot_g
     if (cudaEventElapsedTime(&ms, p.first, p.second) == cudaSuccess) acc += ms;
   ctx->stats.ms_energy = acc;
   return LNO_OT_OK;
+}
+
+// Every gradient buffer is cleared or written by the call itself, so a second run
+// leaves what a first one would.
+int backward_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, double gE, lno_ot_grad* g) {
+  int rc = backward_once(ctx, dom, gE, g);
+  if (rc == LNO_OT_ENOMEM) {
+    ctx->frugal = true;
+    rc = backward_once(ctx, dom, gE, g);
+    ctx->frugal = false;
+  }
+  return rc;
 }
 
 }  // namespace

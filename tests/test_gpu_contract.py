@@ -118,3 +118,28 @@ def test_fp16_slices_and_their_fallback(kind):
         got = np.concatenate([e[:x.size].cpu().numpy() for e, x in zip(et, sel)])
         assert np.abs(got - ref).max() <= TOL["bf16x10"] * np.abs(ref).max()
     ctx.close()
+
+
+@pytest.mark.parametrize("prec,nbas,na,nb,naux,limit", [
+    ("bf16x10", 33, 5, 3, 67, 1139968), ("bf16x15", 33, 5, 3, 67, 1420800),
+    ("tf32", 40, 6, 4, 120, 2758912), ("fp64", 40, 6, 4, 120, 2749696)])
+def test_workspace_bound_counts_the_data_not_the_pitch(prec, nbas, na, nb, naux, limit):
+    """workspace_bytes that held a domain when its rows were padded to 16 bytes holds
+    it with 64-byte rows (the smallest accepted bounds of that layout)."""
+    dd = lno_ot.to_device(make_domain(nbas, (na, nb), naux=naux, L=15.0, seed=5))
+    e = []
+    for bound in (limit, 0):
+        ctx = lno_ot.Context(0, prec, workspace_bytes=bound)
+        e.append(ctx.energy(dd)["total"])
+        ctx.close()
+    assert e[0] == e[1]
+
+
+def test_naf_workspace_bound():
+    dd = lno_ot.to_device(make_domain(24, (4, 3), naux=100, L=15.0, seed=5))
+    lam = []
+    for bound in (1160704, 0):
+        ctx = lno_ot.Context(0, "fp64", workspace_bytes=bound)
+        lam.append(ctx.naf(dd)[1])
+        ctx.close()
+    assert np.array_equal(lam[0], lam[1])
