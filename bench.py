@@ -848,7 +848,7 @@ def run_domain(args):
         "energy_Eh": e_case,
         "accuracy": accuracy,
         "parity": parity,
-        "roofline": {"kernel": "tc_gemm_sliced (W contraction)", "bound": "tensor",
+        "roofline": {"kernel": "tc_pair (W contraction)", "bound": "tensor",
                      "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "traffic_unit": "GB per launch (ncu DRAM bytes per tensor flop, scaled)",
