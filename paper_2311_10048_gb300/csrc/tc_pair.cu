@@ -34,6 +34,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "class_sum.cuh"
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -291,49 +292,6 @@ template <int S, typename OutT>
 constexpr int pair_max_width() {
   return sizeof(OutT) == 4 ? std::min(256, 512 / S / 16 * 16)
                            : std::min(kF64Width, 256 / S / 16 * 16);
-}
-
-// I 2^e as a float64, |I| < 2^53 and the result a normal number (integer
-// operations only: a float64 add or conversion of every element would cost
-// more than the tile's MMAs, at 1/64 of the float32 rate).
-__device__ __forceinline__ double fixed_to_double(int64_t I, int e) {
-  const uint64_t a = (uint64_t)(I < 0 ? -I : I);
-  if (a == 0) return 0.0;
-  const int lz = __clzll((long long)a);
-  const uint64_t m = (a << (lz - 11)) & ((1ull << 52) - 1);
-  const uint64_t bits = ((uint64_t)(I < 0) << 63) | ((uint64_t)(1023 + 63 - lz + e) << 52) | m;
-  return __longlong_as_double((long long)bits);
-}
-
-// Float64 value of one element's class sums: the exact sum of the classes times
-// 2^e.  Class g is an integer multiple of 2^(-BITS g), or (INTS) that integer.  A
-// class 0 too large for the integers or not finite becomes NaN (a NaN operand has
-// it in its leading slice, so in class 0).  rest: class 0 plus the float32 sum of
-// the others (BF16, kTcFloatRest).
-template <int S, int BITS, bool INTS>
-__device__ __forceinline__ double class_sum(const float (&c)[S], int e, bool rest) {
-  if (!(fabsf(c[0]) < 1073741824.0f)) return __longlong_as_double(0x7ff8000000000000ll);
-  int64_t I = __float2int_rn(c[0]);
-  if (!INTS && S > 1 && rest) {
-    float lo = 0.f;
-#pragma unroll
-    for (int g = S - 1; g >= 1; --g) lo = __fadd_rn(lo, c[g]);
-    constexpr int sh = BITS * (S - 1);      // <= 32
-    const float l1 = rintf(lo);             // lo = l1 + l0, both exact
-    const float l0 = __fmul_rn(__fsub_rn(lo, l1), (float)(1ll << (sh < 24 ? sh : 24)));
-    I = ((I + __float2int_rn(l1)) << sh) +
-        ((int64_t)__float2int_rn(l0) << (sh < 24 ? 0 : sh - 24));
-  } else {
-    float w = 1.0f;
-#pragma unroll
-    for (int g = 1; g < S; ++g) {
-      w *= (float)(1 << BITS);
-      I = (I << BITS) + __float2int_rn(INTS ? c[g] : c[g] * w);   // exact: a power of two
-    }
-  }
-  e -= BITS * (S - 1);
-  if (e < -960 || e > 960) return ldexp((double)I, e);   // extreme scales only
-  return fixed_to_double(I, e);
 }
 
 // TF32: 32-bit elements, 16 per 64-byte row, K 8 per MMA; the 16-bit formats
