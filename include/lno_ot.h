@@ -330,8 +330,8 @@ LNO_OT_API int lno_ot_selftest_gemm(int device, int S, int M, int N, int K, cons
                                     const double* B, double* C, void* stream);
 
 /* Diagnostic (no counterpart in the paper): checks the bounded device waits
- * of the contraction kernel.  Runs one 128 x 256 tile with the kernel's test
- * hook that issues no copy, so its first wait for operand data can only end
+ * of the contraction kernels.  Runs one 128 x 256 product on each of them with
+ * their test hook that issues no copy, so the first wait for operand data can only end
  * by the time limit `wait_cycles` (1000 .. the library's normal limit of
  * 4e9 cycles); the kernel then records which wait gave up, releases its TMEM
  * and returns, and the context stays usable.  Returns LNO_OT_ETIMEOUT when

@@ -246,7 +246,7 @@ template <int S, int FMT>
 cudaError_t launch_tc_pair_f64_group(const CUtensorMap* mA, const CUtensorMap* mB,
                                      const TcProb* probs_dev, int nprob, int M, int N, int ldo,
                                      double scale, int* flag, int nsm, cudaStream_t st,
-                                     int mode, PairTile tile);
+                                     int mode, PairTile tile, TcDiag diag = tc_normal());
 int sliced_product_bn(int S);
 cudaError_t launch_sliced_product(int S, const CUtensorMap* mA, const CUtensorMap* mB,
                                   const TcProb* dp, int M, int N, double scale, int* flag,

@@ -3108,20 +3108,20 @@ int lno_ot_selftest_timeout(int device, long long wait_cycles, int* code, void* 
   if (!(prop.major == 10 && prop.minor == 3)) return LNO_OT_EUNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // one 128 x 256 tile of a 2-slice product, K = 64: grid of one CTA
-  constexpr int S = 2, M = 128, N = 256, K = 64;
+  constexpr int S = 2, SD = 4, M = 128, N = 256, K = 64;
   Arena ar(st, 0);
   int* flag;
   __nv_bfloat16 *a16, *b16;
   double* out;
   TcProb* dp;
   TRY(ar.get(&flag, 1));
-  TRY(ar.get(&a16, (size_t)S * M * K));
-  TRY(ar.get(&b16, (size_t)S * N * K));
+  TRY(ar.get(&a16, (size_t)SD * M * K));
+  TRY(ar.get(&b16, (size_t)SD * N * K));
   TRY(ar.get(&out, (size_t)M * N));
   TRY(ar.get(&dp, 1));
   CU(cudaMemsetAsync(flag, 0, 4, st));
-  CU(cudaMemsetAsync(a16, 0, (size_t)S * M * K * 2, st));
-  CU(cudaMemsetAsync(b16, 0, (size_t)S * N * K * 2, st));
+  CU(cudaMemsetAsync(a16, 0, (size_t)SD * M * K * 2, st));
+  CU(cudaMemsetAsync(b16, 0, (size_t)SD * N * K * 2, st));
   CUtensorMap mA[2], mB[2];
   TRY(make_operand_map(&mA[0], a16, K, M, S, (int64_t)M * K, 128));
   TRY(make_operand_map(&mB[0], b16, K, N, S, (int64_t)N * K, sliced_product_bn(S)));
@@ -3145,6 +3145,19 @@ int lno_ot_selftest_timeout(int device, long long wait_cycles, int* code, void* 
     CU(cudaMemsetAsync(flag, 0, 4, st));
     CU((launch_tc_pair<S, kFmtBF16>(mA, mB, dp, 1, M, N, N, 1.0, flag, 2, st,
                                     TcDiag{wait_cycles, 1}, TcOut{kOutRows, 0, 0, 0}, t)));
+    CU(cudaMemcpyAsync(&hflag, flag, 4, cudaMemcpyDeviceToHost, st));
+    CU(cudaStreamSynchronize(st));
+  }
+  for (int mode : {kOutRows, kOutF64Rows}) {   // and of its float64 outputs
+    if (!hflag) break;
+    const PairTile t = pair_tile_f64(SD, 1, M, N);
+    TRY(make_operand_map(&mA[0], a16, K, M, SD, (int64_t)M * K, 128, 2, SD));
+    TRY(make_operand_map(&mB[0], b16, K, N, SD, (int64_t)N * K, t.w / 2, 2, SD));
+    mA[1] = mA[0];
+    mB[1] = mB[0];
+    CU(cudaMemsetAsync(flag, 0, 4, st));
+    CU((launch_tc_pair_f64_group<SD, kFmtBF16>(mA, mB, dp, 1, M, N, mode == kOutRows ? M : N, 1.0,
+                                               flag, 2, st, mode, t, TcDiag{wait_cycles, 1})));
     CU(cudaMemcpyAsync(&hflag, flag, 4, cudaMemcpyDeviceToHost, st));
     CU(cudaStreamSynchronize(st));
   }

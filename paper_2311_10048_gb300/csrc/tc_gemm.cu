@@ -387,7 +387,8 @@ tc_gemm_sliced(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
       long long pr;
       decode(u, mt, nt, pr);
       const TcProb& P = probs[pr];
-      if (!mbar_wait(tfull, tile_it & 1u, flag, 6, true, wlim)) break;
+      // the warp agrees: after an abort no lane runs a warp-wide tcgen05.ld alone
+      if (!__all_sync(0xffffffffu, mbar_wait(tfull, tile_it & 1u, flag, 6, true, wlim))) break;
       tc_fence_after();
       const int m = mt * BM + row;
       OutT* out = reinterpret_cast<OutT*>(P.out);

@@ -76,7 +76,8 @@ __device__ __noinline__ bool pair_wait(uint32_t bar, uint32_t parity, int* flag,
   }
 }
 
-// The same for a whole warp (all lanes return the same).
+// The same for a whole warp: all lanes return the same, so that none runs a
+// warp-wide instruction (tcgen05.ld, shuffles) without the others after an abort.
 __device__ __noinline__ bool pair_wait_warp_slow(uint32_t bar, uint32_t parity, int* flag,
                                                  int code, long long limit) {
   const long long t0 = clock64();
@@ -519,7 +520,7 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
         constexpr int CH = (pair_max_width<S, OutT>() / 16 + 1) / 2;   // chunks of one warp
         const RowOut ro = mok ? row_out(reinterpret_cast<float*>(outp), lay, ldo, m)
                               : RowOut{nullptr, 0, 0};
-        if (!pair_wait(tfull(buf), use & 1u, flag, 6, true, wlim)) break;
+        if (!pair_wait_warp(tfull(buf), use & 1u, flag, 6, wlim)) break;
         tc_fence_after();
         const int nch = ntile_w(nt) / 16;
         float v[CH * 16];
@@ -567,7 +568,7 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
         // 53 added in 385 us, now 146)
         double* const out = reinterpret_cast<double*>(outp);
         const int b8 = lane & 7, m8 = m - b8;   // first row of the lane's 8 x 8 block
-        if (!pair_wait(tfull(buf), use & 1u, flag, 6, true, wlim)) break;
+        if (!pair_wait_warp(tfull(buf), use & 1u, flag, 6, wlim)) break;
         tc_fence_after();
         const int nch = ntile_w(nt) / 8;   // 8-column chunks, dealt over the four warps
 #pragma unroll 1
@@ -762,17 +763,17 @@ template <int S, int FMT>
 cudaError_t launch_tc_pair_f64_group(const CUtensorMap* mA, const CUtensorMap* mB,
                                      const TcProb* probs_dev, int nprob, int M, int N, int ldo,
                                      double scale, int* flag, int nsm, cudaStream_t st,
-                                     int mode, PairTile tile) {
+                                     int mode, PairTile tile, TcDiag diag) {
   if (nprob > 0 && probs_dev == nullptr) return cudaErrorInvalidValue;
   auto launch = mode == kOutF64Rows ? launch_pair<S, FMT, double, true>
                                     : launch_pair<S, FMT, double, false>;
   return launch(mA, mB, probs_dev, TcProb{}, nprob, M, N, ldo, scale, flag, nullptr, nsm, st,
-                tc_normal(), TcOut{mode, 0, 0, 0}, tile);
+                diag, TcOut{mode, 0, 0, 0}, tile);
 }
 template cudaError_t launch_tc_pair_f64_group<4, kFmtBF16>(const CUtensorMap*, const CUtensorMap*,
                                                            const TcProb*, int, int, int, int,
                                                            double, int*, int, cudaStream_t, int,
-                                                           PairTile);
+                                                           PairTile, TcDiag);
 
 #define LNO_PAIR_INST(S, F)                                                                   \
   template cudaError_t launch_tc_pair<S, F>(const CUtensorMap*, const CUtensorMap*,            \
