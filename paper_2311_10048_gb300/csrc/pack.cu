@@ -330,19 +330,21 @@ struct StoreSlicesInt {
 // ld), sliced in both layouts for the adjoint's grouped products: n [z][r][Kd] (k
 // = column) and t [z][c][Nd] (k = row), Kd and Nd multiples of 32, zero in the
 // pads.  Each matrix has its own scale 2^e[z] (slice_exponents).
-__global__ void batch_absmax(const double* __restrict__ src, int64_t src_stride, int rows,
-                             int cols, int ld, unsigned long long* __restrict__ amax) {
-  const double* p = src + (int64_t)blockIdx.y * src_stride;
+__global__ void batch_absmax(const double* __restrict__ src, int64_t src_stride, int count,
+                             int rows, int cols, int ld, unsigned long long* __restrict__ amax) {
   const int64_t n = (int64_t)rows * cols;
-  double m = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / cols;
-    m = fmax(m, fabs(p[r * ld + (i - r * cols)]));
+  for (int z = blockIdx.y; z < count; z += gridDim.y) {
+    const double* p = src + (int64_t)z * src_stride;
+    double m = 0.0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+      const int64_t r = i / cols;
+      m = fmax(m, fabs(p[r * ld + (i - r * cols)]));
+    }
+    for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
+    if ((threadIdx.x & 31) == 0 && m > 0.0)
+      atomicMax(amax + z, (unsigned long long)__double_as_longlong(m));
   }
-  for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
-  if ((threadIdx.x & 31) == 0 && m > 0.0)
-    atomicMax(amax + blockIdx.y, (unsigned long long)__double_as_longlong(m));
 }
 
 // e = smallest exponent with 2^e >= max (0 for a zero matrix); an infinite
@@ -362,30 +364,37 @@ __global__ void slice_exponents(const unsigned long long* __restrict__ amax, int
   }
 }
 
+// Row tiles and matrices beyond the grid's limits (65535 each) are taken in strides.
 template <int S>
-__global__ void batch_slices(const double* __restrict__ src, int64_t src_stride, int rows,
-                             int cols, int ld, const int* __restrict__ e,
+__global__ void batch_slices(const double* __restrict__ src, int64_t src_stride, int count,
+                             int rows, int cols, int ld, const int* __restrict__ e,
                              __nv_bfloat16* __restrict__ dn, int Kd, int64_t stride_n,
                              __nv_bfloat16* __restrict__ dt, int Nd, int64_t stride_t) {
   __shared__ double t[32][33];   // [r][c]
-  const int tx = threadIdx.x, ty = threadIdx.y, z = blockIdx.z;
-  const double* p = src + (int64_t)z * src_stride;
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int i = ty; i < 32; i += 8) {
-    const int r = r0 + i, c = c0 + tx;
-    t[i][tx] = r < rows && c < cols ? p[(int64_t)r * ld + c] : 0.0;
-  }
-  __syncthreads();
-  const int e2 = 7 - e[z] + 8 * (S - 1);
-  if (dn != nullptr) {
-    const StoreSlicesInt<S> st{dn, stride_n, e2};
-    for (int i = ty; i < 32; i += 8)
-      if (r0 + i < rows) st(((int64_t)z * rows + r0 + i) * Kd + c0 + tx, t[i][tx]);
-  }
-  if (dt != nullptr) {
-    const StoreSlicesInt<S> st{dt, stride_t, e2};
-    for (int i = ty; i < 32; i += 8)
-      if (c0 + i < cols) st(((int64_t)z * cols + c0 + i) * Nd + r0 + tx, t[tx][i]);
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int c0 = blockIdx.x * 32;
+  for (int z = blockIdx.z; z < count; z += gridDim.z) {
+    const double* p = src + (int64_t)z * src_stride;
+    const int e2 = 7 - e[z] + 8 * (S - 1);
+    for (int64_t r0 = (int64_t)blockIdx.y * 32; r0 < Nd; r0 += (int64_t)gridDim.y * 32) {
+      for (int i = ty; i < 32; i += 8) {
+        const int64_t r = r0 + i;
+        const int c = c0 + tx;
+        t[i][tx] = r < rows && c < cols ? p[r * ld + c] : 0.0;
+      }
+      __syncthreads();
+      if (dn != nullptr) {
+        const StoreSlicesInt<S> st{dn, stride_n, e2};
+        for (int i = ty; i < 32; i += 8)
+          if (r0 + i < rows) st(((int64_t)z * rows + r0 + i) * Kd + c0 + tx, t[i][tx]);
+      }
+      if (dt != nullptr) {
+        const StoreSlicesInt<S> st{dt, stride_t, e2};
+        for (int i = ty; i < 32; i += 8)
+          if (c0 + i < cols) st(((int64_t)z * cols + c0 + i) * Nd + r0 + tx, t[tx][i]);
+      }
+      __syncthreads();
+    }
   }
 }
 
@@ -677,15 +686,16 @@ cudaError_t launch_batch_slices(const double* src, int64_t src_stride, int count
                                 __nv_bfloat16* dn, int Kd, int64_t stride_n, __nv_bfloat16* dt,
                                 int Nd, int64_t stride_t, cudaStream_t s) {
   if (count <= 0 || rows <= 0 || cols <= 0) return cudaSuccess;
-  if (count > 65535 || Kd % 32 || Nd % 32) return cudaErrorInvalidValue;
+  if (Kd % 32 || Nd % 32) return cudaErrorInvalidValue;
   cudaError_t rc = cudaMemsetAsync(amax, 0, (size_t)count * sizeof(unsigned long long), s);
   if (rc != cudaSuccess) return rc;
+  constexpr int kMaxGrid = 65535;   // y and z
   const int bx = (int)std::min<int64_t>(((int64_t)rows * cols + 1023) / 1024, 512);
-  batch_absmax<<<dim3(bx, count), 256, 0, s>>>(src, src_stride, rows, cols, ld, amax);
+  batch_absmax<<<dim3(bx, std::min(count, kMaxGrid)), 256, 0, s>>>(src, src_stride, count, rows,
+                                                                  cols, ld, amax);
   slice_exponents<<<ceil_div(count, 256), 256, 0, s>>>(amax, count, e, flag);
-  const dim3 grid(Kd / 32, Nd / 32, count);
-  if (grid.y > 65535) return cudaErrorInvalidValue;
-  batch_slices<4><<<grid, dim3(32, 8), 0, s>>>(src, src_stride, rows, cols, ld, e, dn, Kd,
+  const dim3 grid(Kd / 32, std::min(Nd / 32, kMaxGrid), std::min(count, kMaxGrid));
+  batch_slices<4><<<grid, dim3(32, 8), 0, s>>>(src, src_stride, count, rows, cols, ld, e, dn, Kd,
                                                stride_n, dt, Nd, stride_t);
   return cudaGetLastError();
 }

@@ -44,3 +44,26 @@ def test_flat_factors(naux, prec, tol):
     dd = lno_ot.to_device(d)
     ref = e_trips("fp64", dd)
     assert np.abs(e_trips(prec, dd) - ref).max() <= tol * np.abs(ref).max()
+
+
+def test_gradient_of_a_domain_whose_slicing_exceeds_one_grid(lib):
+    """1449 virtuals: the v^2 rows of a DF block are more than 65535 32-row tiles.  One
+    aaa triplet; E is homogeneous of degree -1 in the orbital energies, 4 in the DF
+    factors and 2 in (T1, T2) together, so sum x dE/dx is -E, 4 E and 2 E: float32 in
+    the forward's elements leaves ~1e-9 of E, the adjoint's 32-bit operands less."""
+    v = 1449
+    d = make_domain(v + 3, (3, 0), naux=8, L=6.0, seed=13, t1_sd=0.02)
+    dd = lno_ot.to_device(d)
+    torch.cuda.empty_cache()
+    ctx = lno_ot.Context(0, "bf16x10")
+    E = ctx.energy(dd)["total"]
+    z = torch.zeros_like
+    g = dict(dB=[z(dd["B"][0]), None], deps=[z(dd["eps"][0]), None], dt1=[z(dd["t1"][0]), None],
+             dt2aa=z(dd["t2aa"]))
+    ctx.backward(dd, 1.0, g)
+    ctx.close()
+    dot = lambda x, y: float((x * y).sum())
+    assert abs(dot(dd["eps"][0], g["deps"][0]) + E) <= 1e-6 * abs(E)
+    assert abs(dot(dd["B"][0], g["dB"][0]) - 4 * E) <= 1e-6 * abs(E)
+    amp = dot(dd["t1"][0], g["dt1"][0]) + dot(dd["t2aa"], g["dt2aa"])
+    assert abs(amp - 2 * E) <= 1e-6 * abs(E)
