@@ -95,7 +95,15 @@ typedef struct {
   int precision;          /* lno_ot_precision */
   void* stream;           /* cudaStream_t to order all work on; NULL = the
                              legacy default stream */
-  size_t workspace_bytes; /* upper bound on device workspace; 0 = no bound */
+  size_t workspace_bytes; /* 0 = no bound; else an upper bound, in bytes
+                             allocated, on what a call stages of its input: the
+                             DF factor blocks of both spins, the per-triplet
+                             results, the augmented arrays of the central
+                             orbitals, everything of lno_ot_naf.  A call that
+                             needs more returns LNO_OT_ENOMEM.  The contraction
+                             operands and intermediates of one spin at a time
+                             are not part of it.  With a bound the DF blocks
+                             are packed more tightly (a little slower). */
   const char* tune_cache; /* NULL, or a tuning table written by the autotuner
                              (paper_2311_10048_gb300/tune.py): text lines
                              "vmax bn group_cap" giving, per bucket of

@@ -249,7 +249,7 @@ struct Arena {
   size_t limit, used = 0;
   struct Block {
     void* p;
-    size_t charge;
+    size_t bytes;
   };
   std::vector<Block> ptrs;
   Arena(cudaStream_t s, size_t lim) : st(s), limit(lim) {}
@@ -259,21 +259,17 @@ struct Arena {
     ptrs.clear();
     used = 0;
   }
-  // `charged` < n elements count against the limit: the caller's bound covers the
-  // data, not what rows are padded with for the loads' sake (the pitch of a sliced
-  // row adds up to 31 elements), so a finer pitch refuses no call.
   template <typename T>
-  int get(T** out, size_t n, size_t charged = SIZE_MAX) {
-    auto whole = [](size_t k) { return (std::max<size_t>(k * sizeof(T), 256) + 255) / 256 * 256; };
-    const size_t bytes = whole(n), charge = whole(std::min(n, charged));
-    if (limit && used + charge > limit) return LNO_OT_ENOMEM;
+  int get(T** out, size_t n) {
+    const size_t bytes = (std::max<size_t>(n * sizeof(T), 256) + 255) / 256 * 256;
+    if (limit && used + bytes > limit) return LNO_OT_ENOMEM;
     void* p = nullptr;
     if (cudaMallocAsync(&p, bytes, st) != cudaSuccess) {
       cudaGetLastError();
       return LNO_OT_ENOMEM;
     }
-    ptrs.push_back({p, charge});
-    used += charge;
+    ptrs.push_back({p, bytes});
+    used += bytes;
     *out = static_cast<T*>(p);
     return LNO_OT_OK;
   }
@@ -281,7 +277,7 @@ struct Arena {
     for (auto& q : ptrs)
       if (q.p == p) {
         cudaFreeAsync(p, st);
-        used -= q.charge;
+        used -= q.bytes;
         q = ptrs.back();
         ptrs.pop_back();
         return;
@@ -425,29 +421,31 @@ struct Run {
   int alloc_operand(Operand& op, int nslot, int64_t rows, int K, int S_) {
     return alloc_operand(arena, op, nslot, rows, K, S_);
   }
-  // tf: TF32 slices (the W operands of precision TF32); DF blocks are BF16
+  // tf: TF32 slices (the W operands of precision TF32); DF blocks are BF16.
+  // pitch: multiple of the row pitch in elements (0: the widest useful one).
   int alloc_operand(Arena& ar, Operand& op, int nslot, int64_t rows, int K, int S_,
-                    bool tf = false) {
+                    bool tf = false, int pitch = 0) {
     op.nslot = nslot;
     op.rows = rows;
     op.K = K;
     // sliced rows start on 64-byte boundaries: the contractions' 64-byte box
-    // rows then are two sectors of L2 (1.3x fewer bytes than at 16-byte pitches)
-    op.Kp = (int)round_up(std::max(K, 1), f64 || tf ? 16 : 32);
+    // rows then are two sectors of L2 (1.3x fewer bytes than at 16-byte pitches).
+    // Where a bound holds (workspace_bytes: the DF blocks), rows take the 8
+    // elements the loads need, so that the bound admits as large a domain as it can.
+    if (pitch == 0) pitch = ar.limit ? 8 : f64 || tf ? 16 : 32;
+    op.Kp = (int)round_up(std::max(K, 1), pitch);
     op.S = f64 ? 0 : S_;
     const int64_t n = std::max<int64_t>((int64_t)nslot * rows * op.Kp, 8);
-    const int64_t data =
-        std::max<int64_t>((int64_t)nslot * rows * round_up(std::max(K, 1), 8), 8);
     if (f64) {
-      TRY(ar.get(&op.f64, (size_t)n, (size_t)data));
+      TRY(ar.get(&op.f64, (size_t)n));
     } else {
       op.slice_stride = round_up(n, 8);
       if (tf) {
         op.esz = 4;
-        TRY(ar.get(&op.f32, (size_t)(op.slice_stride * op.S), (size_t)(data * op.S)));
+        TRY(ar.get(&op.f32, (size_t)(op.slice_stride * op.S)));
       } else {
         op.esz = 2;
-        TRY(ar.get(&op.bf, (size_t)(op.slice_stride * op.S), (size_t)(data * op.S)));
+        TRY(ar.get(&op.bf, (size_t)(op.slice_stride * op.S)));
       }
     }
     return LNO_OT_OK;
@@ -617,7 +615,7 @@ struct Run {
   // restricted to some occupied orbitals (same slicing and scales as src)
   int gather_operand(Arena& ar, const Operand& src, const int* dlist, int nlist, int64_t rows,
                      Operand& dst) {
-    TRY(alloc_operand(ar, dst, nlist, rows, src.K, Sdf));
+    TRY(alloc_operand(ar, dst, nlist, rows, src.K, Sdf, false, src.Kp));
     if (nlist == 0 || rows == 0) return LNO_OT_OK;
     stats->other_launches++;
     if (f64)

@@ -1,6 +1,8 @@
 """Inputs at the edges of what the entry points accept: factors whose sums over the
 auxiliary index are large in every slice, sizes at a launch's limits, bounded and
 nearly full memory."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -67,3 +69,58 @@ def test_gradient_of_a_domain_whose_slicing_exceeds_one_grid(lib):
     assert abs(dot(dd["B"][0], g["dB"][0]) - 4 * E) <= 1e-6 * abs(E)
     amp = dot(dd["t1"][0], g["dt1"][0]) + dot(dd["t2aa"], g["dt2aa"])
     assert abs(amp - 2 * E) <= 1e-6 * abs(E)
+
+
+class PoolHigh:
+    """Most bytes in use in the device's default pool (what cudaMallocAsync takes)."""
+    USED, HIGH = 7, 8   # CU_MEMPOOL_ATTR_USED_MEM_CURRENT, _HIGH
+
+    def __init__(self):
+        self.cu = ctypes.CDLL("libcuda.so.1")
+        self.pool = ctypes.c_void_p()
+        assert self.cu.cuDeviceGetDefaultMemPool(ctypes.byref(self.pool), 0) == 0
+
+    def _get(self, attr):
+        x = ctypes.c_uint64()
+        assert self.cu.cuMemPoolGetAttribute(self.pool, attr, ctypes.byref(x)) == 0
+        return x.value
+
+    def reset(self):
+        torch.cuda.synchronize()
+        x = ctypes.c_uint64(0)
+        assert self.cu.cuMemPoolSetAttribute(self.pool, self.HIGH, ctypes.byref(x)) == 0
+        self.base = self._get(self.USED)
+
+    def high(self):
+        torch.cuda.synchronize()
+        return self._get(self.HIGH) - self.base
+
+
+@pytest.mark.parametrize("prec", ["bf16x10", "bf16x15", "tf32", "fp64"])
+@pytest.mark.parametrize("naux", [8, 33])
+def test_workspace_bound_holds_for_what_is_allocated(prec, naux):
+    """A domain without triplets only stages its DF blocks: at the smallest bound that
+    is accepted, no more than that is allocated (rows of few auxiliary functions were
+    charged at a quarter of what they took)."""
+    dd = lno_ot.to_device(make_domain(150, (1, 0), naux=naux, L=15.0, seed=5))
+    pool = PoolHigh()
+
+    def run(bound):
+        ctx = lno_ot.Context(0, prec, workspace_bytes=bound)
+        pool.reset()
+        rc = ctx.energy(dd, raise_on_error=False)["status"]
+        high = pool.high()
+        ctx.close()
+        assert rc in (lno_ot.OK, lno_ot.ENOMEM)
+        return rc == lno_ot.OK, high
+
+    lo, hi = 256, 256 << 20
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        ok, high = run(mid)
+        if ok:
+            hi = mid
+            assert high <= mid + 4096   # the pool's own rounding of a dozen blocks
+        else:
+            lo = mid
+    assert run(hi)[0]
