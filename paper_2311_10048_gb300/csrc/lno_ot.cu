@@ -209,7 +209,8 @@ struct CallState {
 };
 
 // Internal codes, the call has to run again: with the integral scale measured in
-// full (scale_too_small), or without FP16 slices (class 0 not provably exact).
+// full (scale_too_small), or without FP16 slices (class 0 of the DF products not
+// provably exact; known before any contraction).
 constexpr int kRescale = 1, kNoF16 = 2;
 
 // Precision BF16X10 runs on three FP16 slices of 11 bits (6 slice products
@@ -381,7 +382,7 @@ struct Run {
   Arena arena;
   bool f64;
   bool tf32 = false;  // W contraction operands as TF32 slices (precision TF32)
-  bool f16 = false;   // precision BF16X10 on three FP16 slices (choose_f16)
+  bool f16 = false;   // precision BF16X10 on three FP16 slices (set_precision)
   bool tc_adjoint = false;  // adjoint: its contractions on the tensor cores (tc_matmul)
   int S = 0;          // slices of the W contraction operands
   int Sdf = 4;        // slices of the DF factors
@@ -463,7 +464,6 @@ struct Run {
     return StoreSlices<3, __half>{reinterpret_cast<__half*>(op.bf), op.slice_stride,
                                   9 - std::ilogb(sigT), 10 - std::ilogb(sigI)};
   }
-  int fmt() const { return tf32 ? kFmtTF32 : f16 ? kFmtF16 : kFmtBF16; }
 
   // Largest squared row norm of the leading (integer) slice of an FP16 operand.
   int row_norm2(const Operand& op, int slot) {
@@ -829,6 +829,8 @@ struct SpinPass {
   double* e_same;  // per-triplet outputs (device)
   double* e_mixed;
 
+  bool f16;                  // W operands as FP16 slices (prepare may refuse them)
+  int S;                     // slices of the W operands
   Operand AT, BT, A1, BG, BF, AT2;
   std::vector<int> slotAT, slotBT, slotA1, slotBG, slotBF, slotAT2;  // -1 = unused
   std::vector<int2> listAT, listA1, listAT2;
@@ -852,8 +854,8 @@ struct SpinPass {
   Arena own;  // operands and temporaries of this spin pass
 
   SpinPass(Run& r, int s_, CaseSel& sm, CaseSel& mx, double* es, double* em)
-      : R(r), s(s_), t(1 - s_), same(sm), mixed(mx), e_same(es), e_mixed(em),
-        own(r.st, 0) {
+      : R(r), s(s_), t(1 - s_), same(sm), mixed(mx), e_same(es), e_mixed(em), f16(r.f16),
+        S(r.S), own(r.st, 0) {
     o = R.no[s];
     v = R.nv[s];
     ot = R.no[t];
@@ -1106,27 +1108,27 @@ struct SpinPass {
 
   int build() {
     const bool tf = R.tf32;
-    TRY(R.alloc_operand(own, AT, (int)listAT.size(), v, v + oi, R.S, tf));
-    TRY(R.alloc_operand(own, BT, (int)listBT.size(), npairs(v), v + oi, R.S, tf));
-    TRY(R.alloc_operand(own, A1, (int)listA1.size(), v, vt + oti, R.S, tf));
-    TRY(R.alloc_operand(own, BG, (int)listBG.size(), (int64_t)v * vt, vt + oti, R.S, tf));
-    TRY(R.alloc_operand(own, BF, (int)listBF.size(), (int64_t)v * vt, v + oi, R.S, tf));
-    TRY(R.alloc_operand(own, AT2, (int)listAT2.size(), vt, v + oi, R.S, tf));
+    TRY(R.alloc_operand(own, AT, (int)listAT.size(), v, v + oi, S, tf));
+    TRY(R.alloc_operand(own, BT, (int)listBT.size(), npairs(v), v + oi, S, tf));
+    TRY(R.alloc_operand(own, A1, (int)listA1.size(), v, vt + oti, S, tf));
+    TRY(R.alloc_operand(own, BG, (int)listBG.size(), (int64_t)v * vt, vt + oti, S, tf));
+    TRY(R.alloc_operand(own, BF, (int)listBF.size(), (int64_t)v * vt, v + oi, S, tf));
+    TRY(R.alloc_operand(own, AT2, (int)listAT2.size(), vt, v + oi, S, tf));
     if (R.f64) return pack_all(StoreF64{AT.f64}, StoreF64{BT.f64}, StoreF64{A1.f64},
                                StoreF64{BG.f64}, StoreF64{BF.f64}, StoreF64{AT2.f64});
     if (tf)
       return pack_all(R.tf32_slices(AT), R.tf32_slices(BT), R.tf32_slices(A1),
                       R.tf32_slices(BG), R.tf32_slices(BF), R.tf32_slices(AT2));
-    if (R.f16)
+    if (f16)
       return pack_all(R.f16_slices(AT), R.f16_slices(BT), R.f16_slices(A1), R.f16_slices(BG),
                       R.f16_slices(BF), R.f16_slices(AT2));
-    if (R.S == 2)
+    if (S == 2)
       return pack_all(R.slices<2>(AT), R.slices<2>(BT), R.slices<2>(A1), R.slices<2>(BG),
                       R.slices<2>(BF), R.slices<2>(AT2));
-    if (R.S == 4)
+    if (S == 4)
       return pack_all(R.slices<4>(AT), R.slices<4>(BT), R.slices<4>(A1), R.slices<4>(BG),
                       R.slices<4>(BF), R.slices<4>(AT2));
-    if (R.S == 5)
+    if (S == 5)
       return pack_all(R.slices<5>(AT), R.slices<5>(BT), R.slices<5>(A1), R.slices<5>(BG),
                       R.slices<5>(BF), R.slices<5>(AT2));
     return pack_all(R.slices<3>(AT), R.slices<3>(BT), R.slices<3>(A1), R.slices<3>(BG),
@@ -1142,8 +1144,9 @@ struct SpinPass {
     if (R.f64) {
       CU(launch_gemm_f64(dpf, nprob, M, N, ldo, R.st));
     } else {
-      const double scale = R.sigT * R.sigI * std::ldexp(1.0, R.f16 ? -19 : R.tf32 ? -20 : -14);
-      CU(launch_contract(R.S, R.fmt(), bn, opA0, opA1, opB0, opB1, dpt, nprob, M, N, ldo, scale,
+      const double scale = R.sigT * R.sigI * std::ldexp(1.0, f16 ? -19 : R.tf32 ? -20 : -14);
+      const int fmt = R.tf32 ? kFmtTF32 : f16 ? kFmtF16 : kFmtBF16;
+      CU(launch_contract(S, fmt, bn, opA0, opA1, opB0, opB1, dpt, nprob, M, N, ldo, scale,
                          R.ctx->d_flag, R.ctx->nsm, R.st, lay));
     }
     if (e1) cudaEventRecord(e1, R.st);
@@ -1279,7 +1282,7 @@ struct SpinPass {
                                  : 2.0 * dv * (double)npairs(v) * 3 * kpad16(dv + doi);
     R.stats->flops_algorithmic += alg * ntrip;
     R.stats->flops_executed += exe * ntrip;
-    if (!f64) R.stats->tensor_flops += tens * ntrip * (R.S * (R.S + 1) / 2);
+    if (!f64) R.stats->tensor_flops += tens * ntrip * (S * (S + 1) / 2);
     R.stats->triplets += ntrip;
     R.stats->elements += (int64_t)ntrip *
                          (is_mixed ? npairs(v) * vt : (int64_t)v * (v - 1) * (v - 2) / 6);
@@ -1429,10 +1432,19 @@ struct SpinPass {
     TRY(prepare_inputs());
     TRY(build_v_blocks());
     TRY(build());
-    return R.f16 ? check_exact() : LNO_OT_OK;
+    if (!f16) return LNO_OT_OK;
+    bool exact;
+    TRY(check_exact(&exact));
+    if (exact) return LNO_OT_OK;
+    // this spin's operands once more, on the BF16 slices; what the other spin has
+    // computed stands, and the DF blocks stay as they are
+    for (Operand* op : {&AT, &BT, &A1, &BG, &BF, &AT2}) own.drop(op->bf);
+    f16 = false;
+    S = 4;
+    return build();
   }
-  // FP16 slices: the class-0 sums of every contraction are exact (kExactSum)
-  int check_exact() {
+  // FP16 slices: whether the class-0 sums of every contraction are exact (kExactSum)
+  int check_exact(bool* exact) {
     unsigned long long* slot = R.ctx->d_amax + kNormW;
     CU(cudaMemsetAsync(slot, 0, 6 * sizeof(unsigned long long), R.st));
     const Operand* ops[6] = {&AT, &BT, &A1, &BG, &BF, &AT2};
@@ -1444,7 +1456,8 @@ struct SpinPass {
     std::memcpy(n, h, sizeof h);
     for (double& x : n) x = std::sqrt(x);
     const double x = 3 * n[0] * n[1], y = 2 * n[2] * n[3] + n[0] * n[4], z = 2 * n[5] * n[1];
-    return std::max({x, y, z}) <= kExactSum ? LNO_OT_OK : kNoF16;
+    *exact = std::max({x, y, z}) <= kExactSum;
+    return LNO_OT_OK;
   }
   int compute() {
     TRY(run_case(false));

@@ -124,3 +124,38 @@ def test_workspace_bound_holds_for_what_is_allocated(prec, naux):
         else:
             lo = mid
     assert run(hi)[0]
+
+
+@pytest.mark.parametrize("flat", [False, True])
+def test_fp16_slices_refused_by_the_second_spin_only(flat):
+    """Doubles of the second spin near the largest magnitude throughout: its leading FP16
+    sums are not provably exact, so its operands are laid out again on the BF16 slices.
+    What the first spin has computed is not computed again (triplets and products of the
+    call), at any point of the quadrature."""
+    v, n = 256, 3
+    d = make_domain(v + n, (n, n), naux=150, L=50.0, seed=77, t1_sd=0.02)
+    if flat:
+        top = max(np.abs(d[k]).max() for k in ("t2aa", "t2bb", "t2ab"))
+        d["t2bb"] = np.sign(d["t2bb"]) * 0.99 * 2.0 ** np.ceil(np.log2(top))
+    dd = lno_ot.to_device(d)
+    ref = e_trips("fp64", dd)
+    got = e_trips("bf16x10", dd)
+    assert np.abs(got - ref).max() <= 2e-8 * np.abs(ref).max()
+    U = torch.eye(n, dtype=torch.float64, device="cuda")[:1].contiguous()
+    s, w = [0.05, 0.4], [0.2, 0.5]
+    dE = []
+    for prec in ("fp64", "bf16x10"):
+        ctx = lno_ot.Context(0, prec)
+        dE.append(ctx.energy_central(dd, 0, U, s, w)[0])
+        st = ctx.stats()
+        ctx.close()
+    assert abs(dE[0] - dE[1]) <= 2e-8 * abs(dE[0])
+    # holding the central orbital: C(3,2) aaa and 3 x 3 aab triplets in the first spin's
+    # pass, C(3,2) abb ones in the second's
+    assert st["triplets"] == len(s) * 15
+    k16 = lambda k: (k + 15) // 16 * 16
+    pairs, K = v * (v - 1) // 2, k16(v + n)
+    same = 2.0 * v * pairs * 3 * K
+    mixed = 2.0 * v * v * v * 3 * K + 2.0 * v * pairs * 2 * K
+    want = 6 * (3 * same + 9 * mixed) + (10 if flat else 6) * 3 * mixed
+    assert abs(st["tensor_flops"] - len(s) * want) <= 1e-9 * want
