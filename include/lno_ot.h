@@ -361,6 +361,12 @@ LNO_OT_API int lno_ot_selftest_timeout(int device, long long wait_cycles, int* c
 LNO_OT_API int lno_ot_selftest_energy_timeout(int device, long long wait_cycles, int* code,
                                               void* stream);
 
+/* Diagnostic (no counterpart in the paper): on != 0 makes the energy and
+ * gradient calls of this context run in small pieces, as they do by themselves
+ * after the device ran out of memory (groups of at most 64 triplets, DF blocks
+ * one orbital at a time, the adjoint's products one by one); 0 ends that. */
+LNO_OT_API int lno_ot_selftest_small_pieces(lno_ot_ctx* ctx, int on);
+
 /* The same product as lno_ot_selftest_gemm (same slicing, same kernel, same
  * result) for callers that must not allocate device memory: programs whose
  * HBM is owned by their own pool or arena, or code paths where a cudaMalloc

@@ -189,6 +189,7 @@ struct lno_ot_ctx {
   bool exact_measure = false;          // integral scale from every slice (measure_sigI)
   bool no_f16 = false;                 // BF16X10 on its BF16 slices only (kNoF16)
   bool frugal = false;                 // the call runs again after the device ran out of memory
+  bool small_pieces = false;           // every call does (lno_ot_selftest_small_pieces)
   // prepared operands of the last domain (options.keep_operands)
   bool keep = false;
   struct DomainCache* cache = nullptr;
@@ -814,7 +815,8 @@ double kpad16(double k) { return std::ceil(k / 16.0) * 16.0; }
 constexpr int kGroupCap = 1024;
 // After an allocation failed (the device is shared, or nearly full) a call runs
 // again in small pieces: groups of at most 64 triplets, DF blocks of one orbital,
-// the adjoint's products one by one.
+// the adjoint's recompute and adjoint products one by one.  (Its DF assembly keeps
+// the slices of a whole factor block: a single product would need them as well.)
 constexpr int kFrugalGroup = 64;
 
 // ----------------------------------------------------------------------------
@@ -1198,13 +1200,14 @@ struct SpinPass {
       bn = row->bn;
       group_cap = std::max(1, row->group_cap);
     }
-    if (R.ctx->frugal) group_cap = std::min(group_cap, kFrugalGroup);
     int G = (int)std::max<int64_t>(
         1, std::min<int64_t>(group_cap, budget / std::max<int64_t>(per_trip, 1)));
     // energy chunks per triplet from the domain's shape only (a full group of all
     // the case's triplets), so that a triplet's partial sums (and its e_t, bit for
-    // bit) do not depend on which other triplets the call selects
+    // bit) do not depend on which other triplets the call selects, nor on whether
+    // it has to run in small pieces
     const int Gshape = cs.ntot > 0 ? (int)std::min<int64_t>(G, cs.ntot) : std::min(G, ntrip);
+    if (R.ctx->frugal) G = std::min(G, kFrugalGroup);
     G = std::min(G, ntrip);
     char *X = nullptr, *Z = nullptr;
     TRY(A.get(&X, (size_t)(G * xs * esz) + 64));
@@ -1857,6 +1860,7 @@ int energy_once(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
 
 int energy_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
                 const PassSpec* spec = nullptr) {
+  ctx->frugal = ctx->small_pieces;
   int rc = energy_once(ctx, dom, out, spec);
   for (int tries = 0; tries < 3; ++tries) {
     if (rc == kRescale) ctx->exact_measure = true;
@@ -2859,12 +2863,13 @@ int backward_once(lno_ot_ctx* ctx, const lno_ot_domain* dom, double gE, lno_ot_g
 // Every gradient buffer is cleared or written by the call itself, so a second run
 // leaves what a first one would.
 int backward_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, double gE, lno_ot_grad* g) {
+  ctx->frugal = ctx->small_pieces;
   int rc = backward_once(ctx, dom, gE, g);
-  if (rc == LNO_OT_ENOMEM) {
+  if (rc == LNO_OT_ENOMEM && !ctx->frugal) {
     ctx->frugal = true;
     rc = backward_once(ctx, dom, gE, g);
-    ctx->frugal = false;
   }
+  ctx->frugal = false;
   return rc;
 }
 
@@ -3174,6 +3179,12 @@ int lno_ot_selftest_timeout(int device, long long wait_cycles, int* code, void* 
   }
   if (code) *code = hflag;
   return hflag ? LNO_OT_ETIMEOUT : LNO_OT_OK;
+}
+
+int lno_ot_selftest_small_pieces(lno_ot_ctx* ctx, int on) {
+  if (!ctx) return LNO_OT_EINVAL;
+  ctx->small_pieces = on != 0;
+  return LNO_OT_OK;
 }
 
 int lno_ot_selftest_energy_timeout(int device, long long wait_cycles, int* code, void* stream) {

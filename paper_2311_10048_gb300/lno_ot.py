@@ -121,6 +121,8 @@ def load_library(build_if_missing=False):
     lib.lno_ot_selftest_energy_timeout.argtypes = [C.c_int, C.c_longlong, C.POINTER(C.c_int),
                                                    C.c_void_p]
     lib.lno_ot_selftest_energy_timeout.restype = C.c_int
+    lib.lno_ot_selftest_small_pieces.argtypes = [C.c_void_p, C.c_int]
+    lib.lno_ot_selftest_small_pieces.restype = C.c_int
     _lib = lib
     return lib
 

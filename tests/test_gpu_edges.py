@@ -159,3 +159,31 @@ def test_fp16_slices_refused_by_the_second_spin_only(flat):
     mixed = 2.0 * v * v * v * 3 * K + 2.0 * v * pairs * 2 * K
     want = 6 * (3 * same + 9 * mixed) + (10 if flat else 6) * 3 * mixed
     assert abs(st["tensor_flops"] - len(s) * want) <= 1e-9 * want
+
+
+@pytest.mark.parametrize("prec", ["bf16x10", "bf16x6", "fp64"])
+def test_small_pieces_give_the_same_triplets_and_gradients(lib, prec):
+    """What a call does after it ran out of device memory: the triplets' energies are
+    the same bit for bit (a triplet is cut into chunks by the domain's shape alone), and
+    the gradients agree within the 32-bit operands of their products."""
+    dd = lno_ot.to_device(make_domain(100, (8, 6), naux=120, L=40.0, seed=3, t1_sd=0.02))
+    n = all_trips(8, 6)
+    z = torch.zeros_like
+    e, grads = [], []
+    for on in (0, 1):
+        ctx = lno_ot.Context(0, prec)
+        assert lib.lno_ot_selftest_small_pieces(ctx.h, on) == 0
+        et = [torch.zeros(x, dtype=torch.float64, device="cuda") for x in n]
+        out = ctx.energy(dd, e_trip=et)
+        e.append([out["total"]] + [x.cpu().numpy() for x in et])
+        g = dict(dB=[z(x) for x in dd["B"]], deps=[z(x) for x in dd["eps"]],
+                 dt1=[z(x) for x in dd["t1"]], dt2aa=z(dd["t2aa"]), dt2bb=z(dd["t2bb"]),
+                 dt2ab=z(dd["t2ab"]))
+        ctx.backward(dd, 1.0, g)
+        ctx.close()
+        grads.append(g["dB"] + g["deps"] + g["dt1"] + [g["dt2aa"], g["dt2bb"], g["dt2ab"]])
+    assert e[0][0] == e[1][0]
+    for x, y in zip(e[0][1:], e[1][1:]):
+        assert np.array_equal(x, y)
+    for x, y in zip(*grads):
+        assert float((x - y).abs().max()) <= 1e-7 * float(x.abs().max())
