@@ -107,11 +107,10 @@ typedef struct {
   const char* tune_cache; /* NULL, or a tuning table written by the autotuner
                              (paper_2311_10048_gb300/tune.py): text lines
                              "vmax bn group_cap" giving, per bucket of
-                             virtual-space size, the tile width of the W
-                             contraction (64, 96, 128 or 256 where the
-                             precision has that variant; 0 = its default) and
-                             the cap
-                             on triplets per contraction launch.  Lines
+                             virtual-space size, a cap on the tile width of the
+                             W contraction (columns, rounded down to a multiple
+                             of 16; 0 = none) and the cap on triplets per
+                             contraction launch (1024 without a table).  Lines
                              starting with '#' are comments.  Unreadable
                              file: lno_ot_init returns LNO_OT_EINVAL. */
   int keep_operands;      /* 0: every lno_ot_energy call builds and frees its

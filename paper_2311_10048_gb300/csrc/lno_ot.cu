@@ -162,8 +162,8 @@ struct lno_ot_ctx {
   size_t ws_limit = 0;
   int nsm = 152;
   // tuning table: per virtual-space size bucket (rows of the contraction,
-  // ascending vmax) the contraction tile width (0 = the precision's default)
-  // and the triplet-group cap
+  // ascending vmax) a cap on the contraction tile's width (0 = none) and the
+  // triplet-group cap
   struct TuneRow {
     int vmax, bn, group_cap;
   };
