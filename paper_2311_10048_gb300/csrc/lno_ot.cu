@@ -715,6 +715,7 @@ void add_chunks(std::vector<TcProb>& out, int a_row, int b_row, int K, bool neg,
 struct Upload {
   std::vector<char> blob;
   std::vector<std::pair<const void**, size_t>> dst;
+  char* base = nullptr;   // the device buffer
   template <typename T>
   void add(const std::vector<T>& h, const T** d) {
     *d = nullptr;
@@ -726,10 +727,9 @@ struct Upload {
   }
   int send(Run& R, Arena& A) {
     if (blob.empty()) return LNO_OT_OK;
-    char* p;
-    TRY(A.get(&p, blob.size()));
-    CU(R.ctx->h2d(p, blob.data(), blob.size()));
-    for (auto& d : dst) *d.first = p + d.second;
+    TRY(A.get(&base, blob.size()));
+    CU(R.ctx->h2d(base, blob.data(), blob.size()));
+    for (auto& d : dst) *d.first = base + d.second;
     return LNO_OT_OK;
   }
 };
@@ -818,6 +818,8 @@ constexpr int kGroupCap = 1024;
 // the adjoint's recompute and adjoint products one by one.  (Its DF assembly keeps
 // the slices of a whole factor block: a single product would need them as well.)
 constexpr int kFrugalGroup = 64;
+// Triplets whose contraction problems are on the device at once (17 MB).
+constexpr int kWindow = 65536;
 
 // ----------------------------------------------------------------------------
 // Per spin s: same-spin case (sss) and the mixed case with two s orbitals.
@@ -1290,141 +1292,148 @@ struct SpinPass {
     R.stats->elements += (int64_t)ntrip *
                          (is_mixed ? npairs(v) * vt : (int64_t)v * (v - 1) * (v - 2) / 6);
 
-    // Contraction problems of every triplet, uploaded once: a copy from pageable
+    // Contraction problems, uploaded kWindow triplets at a time: a copy from pageable
     // memory waits for the stream, so one per group kept the launches from running
-    // ahead of the device
-    std::vector<ProbF64> pf(f64 ? ntrip : 0), pf2(f64 && is_mixed ? ntrip : 0);
-    std::vector<TcProb> pt(f64 ? 0 : ntrip), pt2(!f64 && is_mixed ? ntrip : 0);
-    for (int q = 0; q < ntrip; ++q) {
-      const Trip tr = cs.trips[q];
-      const int g = q % G;   // its place in its group
-      const int i = tr.i, j = tr.j, k = tr.k;
-      char* Xg = X + (size_t)g * xs * esz;
-      if (!is_mixed) {
-        const int64_t r_jk = (int64_t)slotAT[(size_t)j * o + k] * v;
-        const int64_t r_ki = (int64_t)slotAT[(size_t)k * o + i] * v;
-        const int64_t r_ij = (int64_t)slotAT[(size_t)i * o + j] * v;
-        const int64_t b_i = slotBT[i] * npairs(v), b_j = slotBT[j] * npairs(v),
-                      b_k = slotBT[k] * npairs(v);
-        if (f64) {
-          ProbF64& p = pf[q];
-          p.nseg = 3;
-          seg_f64(p.seg[0], AT, r_jk, BT, b_i, 1.0);
-          seg_f64(p.seg[1], AT, r_ki, BT, b_j, 1.0);
-          seg_f64(p.seg[2], AT, r_ij, BT, b_k, 1.0);
-          p.XT = reinterpret_cast<double*>(Xg);
-        } else {
-          TcProb& p = pt[q];
-          p.nseg = 3;
-          seg_tc(p.seg[0], 0, AT, r_jk, 0, BT, b_i, 0);
-          seg_tc(p.seg[1], 0, AT, r_ki, 0, BT, b_j, 0);
-          seg_tc(p.seg[2], 0, AT, r_ij, 0, BT, b_k, 0);
-          p.out = Xg;
-        }
-      } else {
-        const int K = k;
-        const int64_t a1_jK = (int64_t)slotA1[(size_t)j * ot + K] * v;
-        const int64_t a1_iK = (int64_t)slotA1[(size_t)i * ot + K] * v;
-        const int64_t at_ij = (int64_t)slotAT[(size_t)i * o + j] * v;
-        const int64_t bg_i = (int64_t)slotBG[i] * v * vt, bg_j = (int64_t)slotBG[j] * v * vt;
-        const int64_t bf_K = (int64_t)slotBF[K] * v * vt;
-        const int64_t a2_jK = (int64_t)slotAT2[(size_t)j * ot + K] * vt;
-        const int64_t a2_iK = (int64_t)slotAT2[(size_t)i * ot + K] * vt;
-        const int64_t bt_i = slotBT[i] * npairs(v), bt_j = slotBT[j] * npairs(v);
-        char* Zg = Z + (size_t)g * zs * esz;
-        if (f64) {
-          ProbF64& p = pf[q];
-          p.nseg = 3;
-          seg_f64(p.seg[0], A1, a1_jK, BG, bg_i, 1.0);
-          seg_f64(p.seg[1], A1, a1_iK, BG, bg_j, -1.0);
-          seg_f64(p.seg[2], AT, at_ij, BF, bf_K, 1.0);
-          p.XT = reinterpret_cast<double*>(Xg);
-          ProbF64& p2 = pf2[q];
-          p2.nseg = 2;
-          seg_f64(p2.seg[0], AT2, a2_jK, BT, bt_i, -1.0);
-          seg_f64(p2.seg[1], AT2, a2_iK, BT, bt_j, 1.0);
-          p2.XT = reinterpret_cast<double*>(Zg);
-        } else {
-          TcProb& p = pt[q];
-          p.nseg = 3;
-          seg_tc(p.seg[0], 0, A1, a1_jK, 0, BG, bg_i, 0);
-          seg_tc(p.seg[1], 0, A1, a1_iK, 0, BG, bg_j, 1);
-          seg_tc(p.seg[2], 1, AT, at_ij, 1, BF, bf_K, 0);
-          p.out = Xg;
-          TcProb& p2 = pt2[q];
-          p2.nseg = 2;
-          seg_tc(p2.seg[0], 0, AT2, a2_jK, 0, BT, bt_i, 1);
-          seg_tc(p2.seg[1], 0, AT2, a2_iK, 0, BT, bt_j, 0);
-          p2.out = Zg;
-        }
-      }
-    }
+    // ahead of the device, and one for all triplets took 250 bytes of each.
+    const int W = std::max(G, kWindow / G * G);
     const int3* dblocks = nullptr;
     const Trip* dtrips = nullptr;
-    const ProbF64 *dpf = nullptr, *dpf2 = nullptr;
-    const TcProb *dpt = nullptr, *dpt2 = nullptr;
-    Upload up;
-    up.add(blocks, &dblocks);
-    up.add(cs.trips, &dtrips);
-    up.add(pf, &dpf);
-    up.add(pf2, &dpf2);
-    up.add(pt, &dpt);
-    up.add(pt2, &dpt2);
-    TRY(up.send(R, A));
-    ea.blocks = dblocks;
-
-    for (int g0 = 0; g0 < ntrip; g0 += G) {
-      const int ng = std::min(G, ntrip - g0);
-      TRY(contract(ng, M1, (int)N1, P1, is_mixed ? A1 : AT, AT, is_mixed ? BG : BT,
-                   is_mixed ? BF : BT, f64 ? dpf + g0 : nullptr, f64 ? nullptr : dpt + g0, lay1));
-      if (is_mixed)
-        TRY(contract(ng, M2, (int)N2, P2, AT2, AT2, BT, BT, f64 ? dpf2 + g0 : nullptr,
-                     f64 ? nullptr : dpt2 + g0, lay2));
-      // energy
-      ea.trips = dtrips + g0;
-      ea.partial = partial;
-      cudaEvent_t e0 = R.event(), e1 = R.event();
-      if (e0) cudaEventRecord(e0, R.st);
-      if (f64) {
-        CU(launch_energy(ea, X, Z, f64, ng, P, R.st));
-      } else if (fuse) {
-        EnergyArgs ef = ea;
-        ef.fs = R.fov[s];
-        ef.ft = R.fov[t];
-        ef.t2ss = t2ss;
-        ef.t2st = t2st;
-        CU(launch_energy_f32_fused(ef, reinterpret_cast<const float*>(X),
-                                   reinterpret_cast<const float*>(Z), vtab, vt_stride, pv, pvt,
-                                   ng, P, R.st));
-        R.stats->energy_launches += 1;
-      } else {
-        CU(launch_energy_f32(ea, reinterpret_cast<const float*>(X),
-                             reinterpret_cast<const float*>(Z), vtab, vt_stride, pv, pvt, ng, P,
-                             R.st));
+    for (int w0 = 0; w0 < ntrip; w0 += W) {
+      const int nw = std::min(W, ntrip - w0);
+      std::vector<ProbF64> pf(f64 ? nw : 0), pf2(f64 && is_mixed ? nw : 0);
+      std::vector<TcProb> pt(f64 ? 0 : nw), pt2(!f64 && is_mixed ? nw : 0);
+      for (int q = 0; q < nw; ++q) {
+        const Trip tr = cs.trips[w0 + q];
+        const int g = q % G;   // its place in its group
+        const int i = tr.i, j = tr.j, k = tr.k;
+        char* Xg = X + (size_t)g * xs * esz;
+        if (!is_mixed) {
+          const int64_t r_jk = (int64_t)slotAT[(size_t)j * o + k] * v;
+          const int64_t r_ki = (int64_t)slotAT[(size_t)k * o + i] * v;
+          const int64_t r_ij = (int64_t)slotAT[(size_t)i * o + j] * v;
+          const int64_t b_i = slotBT[i] * npairs(v), b_j = slotBT[j] * npairs(v),
+                        b_k = slotBT[k] * npairs(v);
+          if (f64) {
+            ProbF64& p = pf[q];
+            p.nseg = 3;
+            seg_f64(p.seg[0], AT, r_jk, BT, b_i, 1.0);
+            seg_f64(p.seg[1], AT, r_ki, BT, b_j, 1.0);
+            seg_f64(p.seg[2], AT, r_ij, BT, b_k, 1.0);
+            p.XT = reinterpret_cast<double*>(Xg);
+          } else {
+            TcProb& p = pt[q];
+            p.nseg = 3;
+            seg_tc(p.seg[0], 0, AT, r_jk, 0, BT, b_i, 0);
+            seg_tc(p.seg[1], 0, AT, r_ki, 0, BT, b_j, 0);
+            seg_tc(p.seg[2], 0, AT, r_ij, 0, BT, b_k, 0);
+            p.out = Xg;
+          }
+        } else {
+          const int K = k;
+          const int64_t a1_jK = (int64_t)slotA1[(size_t)j * ot + K] * v;
+          const int64_t a1_iK = (int64_t)slotA1[(size_t)i * ot + K] * v;
+          const int64_t at_ij = (int64_t)slotAT[(size_t)i * o + j] * v;
+          const int64_t bg_i = (int64_t)slotBG[i] * v * vt, bg_j = (int64_t)slotBG[j] * v * vt;
+          const int64_t bf_K = (int64_t)slotBF[K] * v * vt;
+          const int64_t a2_jK = (int64_t)slotAT2[(size_t)j * ot + K] * vt;
+          const int64_t a2_iK = (int64_t)slotAT2[(size_t)i * ot + K] * vt;
+          const int64_t bt_i = slotBT[i] * npairs(v), bt_j = slotBT[j] * npairs(v);
+          char* Zg = Z + (size_t)g * zs * esz;
+          if (f64) {
+            ProbF64& p = pf[q];
+            p.nseg = 3;
+            seg_f64(p.seg[0], A1, a1_jK, BG, bg_i, 1.0);
+            seg_f64(p.seg[1], A1, a1_iK, BG, bg_j, -1.0);
+            seg_f64(p.seg[2], AT, at_ij, BF, bf_K, 1.0);
+            p.XT = reinterpret_cast<double*>(Xg);
+            ProbF64& p2 = pf2[q];
+            p2.nseg = 2;
+            seg_f64(p2.seg[0], AT2, a2_jK, BT, bt_i, -1.0);
+            seg_f64(p2.seg[1], AT2, a2_iK, BT, bt_j, 1.0);
+            p2.XT = reinterpret_cast<double*>(Zg);
+          } else {
+            TcProb& p = pt[q];
+            p.nseg = 3;
+            seg_tc(p.seg[0], 0, A1, a1_jK, 0, BG, bg_i, 0);
+            seg_tc(p.seg[1], 0, A1, a1_iK, 0, BG, bg_j, 1);
+            seg_tc(p.seg[2], 1, AT, at_ij, 1, BF, bf_K, 0);
+            p.out = Xg;
+            TcProb& p2 = pt2[q];
+            p2.nseg = 2;
+            seg_tc(p2.seg[0], 0, AT2, a2_jK, 0, BT, bt_i, 1);
+            seg_tc(p2.seg[1], 0, AT2, a2_iK, 0, BT, bt_j, 0);
+            p2.out = Zg;
+          }
+        }
       }
-      double* partial2 = nullptr;
-      if (fov && !fuse) {
-        // the f_ov part of V in a second pass over the same X (and Z'):
-        // sum W V_f / D with V_f built like the T1 term from f_ov and T2
-        EnergyArgs ef = ea;
-        ef.vmode = 1;
-        ef.t1s = R.fov[s];
-        ef.t1t = R.fov[is_mixed ? t : s];
-        ef.t2ss = t2ss;
-        ef.t2st = t2st;
-        ef.partial = partial2 = partial + (size_t)G * npart;
-        if (f64)
-          CU(launch_energy(ef, X, Z, f64, ng, P, R.st));
-        else
-          CU(launch_energy_f32(ef, reinterpret_cast<const float*>(X),
-                               reinterpret_cast<const float*>(Z), vtab, vt_stride, pv, pvt, ng,
-                               P, R.st));
+      const ProbF64 *dpf = nullptr, *dpf2 = nullptr;
+      const TcProb *dpt = nullptr, *dpt2 = nullptr;
+      Upload up;
+      if (w0 == 0) {
+        up.add(blocks, &dblocks);
+        up.add(cs.trips, &dtrips);
+      }
+      up.add(pf, &dpf);
+      up.add(pf2, &dpf2);
+      up.add(pt, &dpt);
+      up.add(pt2, &dpt2);
+      TRY(up.send(R, A));
+      ea.blocks = dblocks;
+
+      for (int g0 = w0; g0 < w0 + nw; g0 += G) {
+        const int ng = std::min(G, w0 + nw - g0), gw = g0 - w0;
+        TRY(contract(ng, M1, (int)N1, P1, is_mixed ? A1 : AT, AT, is_mixed ? BG : BT,
+                     is_mixed ? BF : BT, f64 ? dpf + gw : nullptr, f64 ? nullptr : dpt + gw, lay1));
+        if (is_mixed)
+          TRY(contract(ng, M2, (int)N2, P2, AT2, AT2, BT, BT, f64 ? dpf2 + gw : nullptr,
+                       f64 ? nullptr : dpt2 + gw, lay2));
+        // energy
+        ea.trips = dtrips + g0;
+        ea.partial = partial;
+        cudaEvent_t e0 = R.event(), e1 = R.event();
+        if (e0) cudaEventRecord(e0, R.st);
+        if (f64) {
+          CU(launch_energy(ea, X, Z, f64, ng, P, R.st));
+        } else if (fuse) {
+          EnergyArgs ef = ea;
+          ef.fs = R.fov[s];
+          ef.ft = R.fov[t];
+          ef.t2ss = t2ss;
+          ef.t2st = t2st;
+          CU(launch_energy_f32_fused(ef, reinterpret_cast<const float*>(X),
+                                     reinterpret_cast<const float*>(Z), vtab, vt_stride, pv, pvt,
+                                     ng, P, R.st));
+          R.stats->energy_launches += 1;
+        } else {
+          CU(launch_energy_f32(ea, reinterpret_cast<const float*>(X),
+                               reinterpret_cast<const float*>(Z), vtab, vt_stride, pv, pvt, ng, P,
+                               R.st));
+        }
+        double* partial2 = nullptr;
+        if (fov && !fuse) {
+          // the f_ov part of V in a second pass over the same X (and Z'):
+          // sum W V_f / D with V_f built like the T1 term from f_ov and T2
+          EnergyArgs ef = ea;
+          ef.vmode = 1;
+          ef.t1s = R.fov[s];
+          ef.t1t = R.fov[is_mixed ? t : s];
+          ef.t2ss = t2ss;
+          ef.t2st = t2st;
+          ef.partial = partial2 = partial + (size_t)G * npart;
+          if (f64)
+            CU(launch_energy(ef, X, Z, f64, ng, P, R.st));
+          else
+            CU(launch_energy_f32(ef, reinterpret_cast<const float*>(X),
+                                 reinterpret_cast<const float*>(Z), vtab, vt_stride, pv, pvt, ng,
+                                 P, R.st));
+          R.stats->energy_launches += 2;
+        }
+        CU(launch_reduce_partials(partial, npart, partial2, ng, eout + g0, R.st));
+        if (e1) cudaEventRecord(e1, R.st);
+        if (e0 && e1) R.energy_ev.push_back({e0, e1});
         R.stats->energy_launches += 2;
       }
-      CU(launch_reduce_partials(partial, npart, partial2, ng, eout + g0, R.st));
-      if (e1) cudaEventRecord(e1, R.st);
-      if (e0 && e1) R.energy_ev.push_back({e0, e1});
-      R.stats->energy_launches += 2;
+      if (w0 > 0) A.drop(up.base);
     }
     return LNO_OT_OK;
   }

@@ -187,3 +187,36 @@ def test_small_pieces_give_the_same_triplets_and_gradients(lib, prec):
         assert np.array_equal(x, y)
     for x, y in zip(*grads):
         assert float((x - y).abs().max()) <= 1e-7 * float(x.abs().max())
+
+
+def test_many_triplets_take_little_memory_each(lib):
+    """1.27 million triplets of a few virtuals: the contraction problems are on the device a
+    window at a time, so a triplet costs its index and its energy (20 bytes, and as much
+    again for slack), and those beyond the first window are what they are alone, bit for
+    bit and against the float64 path."""
+    na, nb = 100, 98
+    dd = lno_ot.to_device(make_domain(103, (na, nb), naux=20, L=10.0, seed=4, t1_sd=0.02))
+    n = all_trips(na, nb)
+    rng = np.random.default_rng(0)
+    part = [np.sort(rng.choice(x, x // 5, replace=False)) for x in n]
+    pool = PoolHigh()
+
+    def run(prec, sel):
+        ctx = lno_ot.Context(0, prec)
+        m = n if sel is None else [len(x) for x in sel]
+        et = [torch.zeros(x, dtype=torch.float64, device="cuda") for x in m]
+        pool.reset()
+        ctx.energy(dd, e_trip=et, trip_sel=sel)
+        high = pool.high()
+        ctx.close()
+        return [e.cpu().numpy() for e in et], high
+
+    full, hi_full = run("bf16x10", None)
+    some, hi_some = run("bf16x10", part)
+    assert hi_full - hi_some <= 40 * (sum(n) - sum(len(x) for x in part))
+    for f, s, x in zip(full, some, part):
+        assert np.array_equal(f[x], s)
+    few = [x[::997] for x in part]
+    ref, _ = run("fp64", few)
+    for f, r, x in zip(full, ref, few):
+        assert np.abs(f[x] - r).max() <= 1e-7 * np.abs(r).max()
