@@ -208,13 +208,7 @@ struct TcDiag {
   int starve;
 };
 
-// tc_gemm.cu: grouped sliced contraction.  mA: maps with 128-row boxes,
-// mB: maps with BN-row boxes; transposed output out[n][m].  The instances
-// (S, BN, OutT, TF) are listed there.
-template <int S, int BN, typename OutT, bool TF = false>
-cudaError_t launch_tc_gemm(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs_dev,
-                           int nprob, int M, int N, int ldo, double scale, int* flag,
-                           unsigned long long* amax, int nsm, cudaStream_t st, TcDiag diag);
+// tc_gemm.cu
 long long tc_default_wait_cycles();
 inline TcDiag tc_normal() { return TcDiag{tc_default_wait_cycles(), 0}; }
 int make_operand_map(CUtensorMap* map, const void* base, int64_t Kp, int64_t rows, int S,

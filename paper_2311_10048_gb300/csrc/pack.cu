@@ -715,8 +715,6 @@ cudaError_t launch_view_slices(const double* in, int64_t rs, int64_t ks, int row
 }
 template cudaError_t launch_view_slices<4>(const double*, int64_t, int64_t, int, int, int,
                                            __nv_bfloat16*, int64_t, double, cudaStream_t);
-template cudaError_t launch_view_slices<5>(const double*, int64_t, int64_t, int, int, int,
-                                           __nv_bfloat16*, int64_t, double, cudaStream_t);
 
 #define LNO_INST(St)                                                                           \
   template cudaError_t launch_transpose_blocks<St>(const double*, int, int,                      \

@@ -1,5 +1,7 @@
-// Tensor-core contraction for sm_103a: tcgen05.mma (BF16 x BF16 -> FP32 in
-// TMEM) fed by TMA, on exactly sliced float64 operands.
+// Tensor-core contraction for sm_103a, one CTA per tile: tcgen05.mma (BF16 x
+// BF16 -> FP32 in TMEM) fed by TMA, on exactly sliced float64 operands, with
+// float64 output.  The single-product diagnostics run it (the library's own
+// contractions run on CTA pairs, tc_pair.cu).
 //
 // Each float64 operand value is stored as S BF16 slices with a power-of-two
 // scale sigma (StoreSlices in common.cuh):
@@ -10,32 +12,21 @@
 // class g = p + q in its own TMEM accumulator.  Every term of class g is an
 // integer multiple of 2^(-8g) no larger than 2^(14-8g), so each class sum is
 // exact (no rounding at all) while it needs at most 24 significant bits:
-// always for k <= 1024, and for random-sign data far beyond.  (Measured on sm_103a: a single FP32
-// accumulator shared by classes of different weight drifts by ~2^-17 of its
-// value over a few hundred MMAs, because each MMA rounds the running sum at
-// its own magnitude.)  The epilogue adds the classes from the smallest up in
-// float32 (the lower classes are ~2^-8 of the next, so this is one rounding
-// of the final sum) and scales by the power of two sigma_A sigma_B 2^-14.
-// Float64 output (the DF assembly) adds the exact class sums in float64.  No float64
-// arithmetic runs per element: this GPU's FP64 rate is ~1/64 of FP32.  No
-// systematic bias enters the sum of ~1e12 positive-definite energy terms.
+// always for k <= 1024 / (g + 1), and for random-sign data far beyond.  (Measured on
+// sm_103a: a single FP32 accumulator shared by classes of different weight drifts by
+// ~2^-17 of its value over a few hundred MMAs, because each MMA rounds the running
+// sum at its own magnitude.)  The epilogue adds the class sums in float64.
 //
 // A problem is XT[n][m] = sum_seg (+/-) A_seg[m][:] . B_seg[n][:]: up to 3
-// K-segments from different operand tensors (the three occupied
-// permutations of P(i/jk), or the mixed-spin terms); the sign is applied with
-// the instruction descriptor's negate-A bit.  Operand tensors are 3-D TMA
-// maps (k, row, slice); k beyond the tensor and rows beyond the last row
-// arrive as zeros.
+// K-segments; the sign is applied with the instruction descriptor's negate-A bit.
+// Operand tensors are 3-D TMA maps (k, row, slice); k beyond the tensor and rows
+// beyond the last row arrive as zeros.
 //
 // Kernel structure (one CTA per SM, persistent over tiles of 128 x BN):
 //   warp 0      TMA producer (one thread), STAGES-deep smem ring
 //   warp 1      TMEM allocator and MMA issuer (one thread); S accumulators
-//               of 128 x BN FP32 (S * BN <= 512 TMEM columns: BN = 256 or 128
-//               for S = 2, 128 or 64 for S = 3, 128, 96 or 64 for S = 4, and 64
-//               for S = 5)
-//   warps 2..5  epilogue: tcgen05.ld -> scale -> coalesced stores along m; when
-//               TMEM has room ((S + 1) BN <= 512) the combined tile is parked in
-//               spare columns so the next tile's MMAs overlap the stores
+//               of 128 x BN FP32 (S * BN <= 512 TMEM columns)
+//   warps 2..5  epilogue: tcgen05.ld -> float64 sum -> coalesced stores along m
 // Tiles are visited m fastest: the CTAs that run at the same time share the
 // B tile of one n-tile (read from HBM once, the other m-tiles hit L2), and the
 // small A operand of a problem stays resident in L2.
@@ -90,52 +81,31 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint6
       : "memory");
 }
 
-__device__ __forceinline__ void umma_tf32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                          uint32_t idesc, uint32_t accum) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
-      : "memory");
-}
-
 // The same MMAs with a collector-buffer usage for A: consecutive MMAs that
 // share one A operand (slice pa against the slices pb of B) read it from shared
 // memory once (fill), then from the collector (use, lastuse).
-#define LNO_UMMA_C(NAME, KIND, COLL)                                                        \
+#define LNO_UMMA_C(NAME, COLL)                                                              \
   __device__ __forceinline__ void NAME(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,     \
                                        uint32_t idesc, uint32_t accum) {                    \
     asm volatile("{\n\t.reg .pred p;\n\t"                                                   \
                  "setp.ne.b32 p, %4, 0;\n\t"                                               \
-                 "tcgen05.mma.cta_group::1.kind::" KIND ".collector::a::" COLL                \
+                 "tcgen05.mma.cta_group::1.kind::f16.collector::a::" COLL                     \
                  " [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),                                 \
                  "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)                             \
                  : "memory");                                                               \
   }
-LNO_UMMA_C(umma_bf16_fill, "f16", "fill")
-LNO_UMMA_C(umma_bf16_use, "f16", "use")
-LNO_UMMA_C(umma_bf16_last, "f16", "lastuse")
-LNO_UMMA_C(umma_tf32_fill, "tf32", "fill")
-LNO_UMMA_C(umma_tf32_use, "tf32", "use")
-LNO_UMMA_C(umma_tf32_last, "tf32", "lastuse")
+LNO_UMMA_C(umma_bf16_fill, "fill")
+LNO_UMMA_C(umma_bf16_use, "use")
+LNO_UMMA_C(umma_bf16_last, "lastuse")
 #undef LNO_UMMA_C
 
 // mode 0: no collector, 1: fill, 2: use, 3: last use
-template <bool TF>
 __device__ __forceinline__ void umma_any(int mode, uint32_t d, uint64_t a, uint64_t b,
                                          uint32_t id, uint32_t acc) {
-  if constexpr (TF) {
-    if (mode == 1) umma_tf32_fill(d, a, b, id, acc);
-    else if (mode == 2) umma_tf32_use(d, a, b, id, acc);
-    else if (mode == 3) umma_tf32_last(d, a, b, id, acc);
-    else umma_tf32(d, a, b, id, acc);
-  } else {
-    if (mode == 1) umma_bf16_fill(d, a, b, id, acc);
-    else if (mode == 2) umma_bf16_use(d, a, b, id, acc);
-    else if (mode == 3) umma_bf16_last(d, a, b, id, acc);
-    else umma_bf16(d, a, b, id, acc);
-  }
+  if (mode == 1) umma_bf16_fill(d, a, b, id, acc);
+  else if (mode == 2) umma_bf16_use(d, a, b, id, acc);
+  else if (mode == 3) umma_bf16_last(d, a, b, id, acc);
+  else umma_bf16(d, a, b, id, acc);
 }
 
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
@@ -153,17 +123,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32"
-      " [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
-      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-      "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-      : "memory");
-}
-__device__ __forceinline__ void tmem_st_wait() {
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -179,12 +138,10 @@ __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t saddr) {
   return d;
 }
 
-// Instruction descriptor: D FP32, A/B K-major of format 1 (BF16, kind::f16)
-// or 2 (TF32, kind::tf32), M=128, N=n (a multiple of 16, 16..256).
-template <bool TF>
+// Instruction descriptor: D FP32, A/B K-major BF16, M=128, N=n (a multiple of
+// 16, 16..256).
 __device__ __forceinline__ uint32_t idesc_mma(int neg, int n) {
-  constexpr uint32_t fmt = TF ? 2u : 1u;
-  return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)neg << 13) |
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)neg << 13) |
          ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 }
 
@@ -205,20 +162,16 @@ struct Cfg {
 // at all, so the MMA thread's first wait (on a full barrier nothing will
 // complete) runs out after wait_cycles and the kernel takes its error exit
 // with nothing in flight.  Library calls always pass {kWaitCycles, 0}.
-// TF: TF32 slices (32-bit elements, 16 per 64-byte row, K 8 per MMA) instead
-// of BF16 ones (32 per row, K 16 per MMA); the shared-memory layout, the
-// descriptors and the MMAs per row are the same in bytes.
 // Transposed output out[n][m], m-tiles fastest.  The last n-tile's MMAs are only
 // as wide as its columns (rounded up to 16), so a narrow n costs little.
-template <int S, int BN, typename OutT, bool TF>
+template <int S, int BN>
 __global__ void __launch_bounds__(192, 1)
 tc_gemm_sliced(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
                const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
                const TcProb* __restrict__ probs, int nprob, int M, int N, int ldo, double scale,
-               int* __restrict__ flag, unsigned long long* __restrict__ amax, TcDiag diag) {
+               int* __restrict__ flag, TcDiag diag) {
   using C = Cfg<S, BN>;
-  constexpr int BKE = TF ? BK / 2 : BK;   // elements per 64-byte row
-  constexpr int KM = TF ? 8 : 16;         // K of one MMA
+  constexpr int KM = 16;   // K of one MMA
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -288,7 +241,7 @@ tc_gemm_sliced(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
           const TcSeg seg = P.seg[sg];
           const CUtensorMap* ma = seg.amap ? &mapA1 : &mapA0;
           const CUtensorMap* mb = seg.bmap ? &mapB1 : &mapB0;
-          for (int k0 = 0; k0 < seg.K; k0 += BKE) {
+          for (int k0 = 0; k0 < seg.K; k0 += BK) {
             if (!mbar_wait(empty_bar(stage), phase ^ 1u, flag, 1, true, wlim)) {
               ok = false;
               break;
@@ -333,8 +286,8 @@ tc_gemm_sliced(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
         const int nw = ntile_w(nt);
         for (int sg = 0; sg < P.nseg && ok; ++sg) {
           const TcSeg seg = P.seg[sg];
-          const uint32_t idesc = idesc_mma<TF>(seg.neg, nw);
-          for (int k0 = 0; k0 < seg.K; k0 += BKE) {
+          const uint32_t idesc = idesc_mma(seg.neg, nw);
+          for (int k0 = 0; k0 < seg.K; k0 += BK) {
             if (!mbar_wait(full_bar(stage), phase, flag, 3, true, wlim)) {
               ok = false;
               break;
@@ -353,7 +306,7 @@ tc_gemm_sliced(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                     // A slice pa meets S - pa slices of B in a row: read it once
                     const int last = S - 1 - pa;
                     const int mode = last == 0 ? 0 : pb == 0 ? 1 : pb == last ? 3 : 2;
-                    umma_any<TF>(mode, tmem + g * BN, ad, bd, idesc, (cls_on >> g) & 1u);
+                    umma_any(mode, tmem + g * BN, ad, bd, idesc, (cls_on >> g) & 1u);
                     cls_on |= 1u << g;
                     any = true;
                   }
@@ -379,9 +332,6 @@ tc_gemm_sliced(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     const int q = warp & 3;
     const int row = q * 32 + lane;
     uint32_t tile_it = 0;
-    float lmax = 0.f;
-    // scale = sigma_A sigma_B 2^-14 is a power of two: exact in float
-    const float fscale = (float)scale;
     for (long long u = blockIdx.x; u < nunits; u += gridDim.x, ++tile_it) {
       int mt, nt;
       long long pr;
@@ -391,95 +341,29 @@ tc_gemm_sliced(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
       if (!__all_sync(0xffffffffu, mbar_wait(tfull, tile_it & 1u, flag, 6, true, wlim))) break;
       tc_fence_after();
       const int m = mt * BM + row;
-      OutT* out = reinterpret_cast<OutT*>(P.out);
-      const bool mok = m < M && out != nullptr;
+      double* out = reinterpret_cast<double*>(P.out);
       const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16);
-      if constexpr ((S + 1) * BN <= 512 && sizeof(OutT) == 4) {
-        // combine the classes into the spare TMEM columns, free the class
-        // accumulators for the next tile's MMAs, then store from the spare copy
-        const uint32_t spare = tbase + S * BN;
-        const int nch = ntile_w(nt) / 16;
+      const int nch = ntile_w(nt) / 16;
 #pragma unroll 1
-        for (int c = 0; c < nch; ++c) {
-          uint32_t acc[S][16];
+      for (int c = 0; c < nch; ++c) {
+        uint32_t acc[S][16];
 #pragma unroll
-          for (int g = 0; g < S; ++g) tmem_ld16(tbase + g * BN + c * 16, acc[g]);
-          tmem_ld_wait();
-          uint32_t v[16];
+        for (int g = 0; g < S; ++g) tmem_ld16(tbase + g * BN + c * 16, acc[g]);
+        tmem_ld_wait();
+        const int n0 = nt * BN + c * 16;
+        double* op = out + (int64_t)n0 * ldo + m;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            float lo = 0.f;
+        for (int j = 0; j < 16; ++j) {
+          if (m >= M || n0 + j >= N) continue;
+          double v = 0.0;   // the exact class sums, smallest first
 #pragma unroll
-            for (int g = S - 1; g >= 1; --g) lo = __fadd_rn(lo, __uint_as_float(acc[g][j]));
-            v[j] = __float_as_uint(__fmul_rn(__fadd_rn(__uint_as_float(acc[0][j]), lo), fscale));
-          }
-          tmem_st16(spare + c * 16, v);
+          for (int g = S - 1; g >= 0; --g) v += (double)__uint_as_float(acc[g][j]);
+          op[(int64_t)j * ldo] = v * scale;
         }
-        tmem_st_wait();
-        tc_fence_before();
-        mbar_arrive(tempty);
-#pragma unroll 1
-        for (int c = 0; c < nch; ++c) {
-          uint32_t v[16];
-          tmem_ld16(spare + c * 16, v);
-          tmem_ld_wait();
-          const int n0 = nt * BN + c * 16;
-          OutT* op = out + (int64_t)n0 * ldo + m;
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const float x = __uint_as_float(v[j]);
-            if (mok && n0 + j < N) op[(int64_t)j * ldo] = x;
-            if (amax != nullptr && m < M && n0 + j < N) lmax = fmaxf(lmax, fabsf(x));
-          }
-        }
-      } else {
-        const int nch = ntile_w(nt) / 16;
-#pragma unroll 1
-        for (int c = 0; c < nch; ++c) {
-          uint32_t acc[S][16];
-#pragma unroll
-          for (int g = 0; g < S; ++g) tmem_ld16(tbase + g * BN + c * 16, acc[g]);
-          tmem_ld_wait();
-          const int n0 = nt * BN + c * 16;
-          OutT* op = out + (int64_t)n0 * ldo + m;
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            // lower classes first (each exact), then one rounding against HI
-            float lo = 0.f;
-#pragma unroll
-            for (int g = S - 1; g >= 1; --g) lo = __fadd_rn(lo, __uint_as_float(acc[g][j]));
-            const float hi = __uint_as_float(acc[0][j]);
-            if constexpr (sizeof(OutT) == 4) {
-              const float v = __fmul_rn(__fadd_rn(hi, lo), fscale);
-              if (mok && n0 + j < N) op[(int64_t)j * ldo] = v;
-              if (amax != nullptr && m < M && n0 + j < N) lmax = fmaxf(lmax, fabsf(v));
-            } else {
-              // float64 output: the exact class sums added in float64 (smallest
-              // first), so the output keeps ~53 bits instead of HI + a float32 rest
-              if (mok && n0 + j < N) {
-                double r;
-                if (P.flags & kTcFloatRest) {
-                  r = (double)__fmul_rn(hi, fscale) + (double)__fmul_rn(lo, fscale);
-                } else {
-                  double v = 0.0;
-#pragma unroll
-                  for (int g = S - 1; g >= 1; --g) v += (double)__uint_as_float(acc[g][j]);
-                  r = ((double)hi + v) * scale;
-                }
-                double* o = &op[(int64_t)j * ldo];
-                *o = (P.flags & kTcAccum) ? *o + r : r;
-              }
-              if (amax != nullptr && m < M && n0 + j < N)
-                lmax = fmaxf(lmax, fabsf(__fmul_rn(__fadd_rn(hi, lo), fscale)));
-            }
-          }
-        }
-        tc_fence_before();
-        mbar_arrive(tempty);
       }
+      tc_fence_before();
+      mbar_arrive(tempty);
     }
-    if (amax != nullptr)
-      atomicMax(amax, (unsigned long long)__double_as_longlong((double)lmax));
   }
   tc_fence_before();
   __syncthreads();
@@ -533,23 +417,21 @@ int make_operand_map(CUtensorMap* map, const void* base, int64_t Kp, int64_t row
 }
 
 // mB must be maps with boxes of BN rows; mA boxes of 128 rows.
-template <int S, int BN, typename OutT, bool TF>
-cudaError_t launch_tc_gemm(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs_dev,
-                           int nprob, int M, int N, int ldo, double scale, int* flag,
-                           unsigned long long* amax, int nsm, cudaStream_t st, TcDiag diag) {
+template <int S, int BN>
+static cudaError_t launch_tc_gemm(const CUtensorMap* mA, const CUtensorMap* mB,
+                                  const TcProb* probs_dev, int nprob, int M, int N, int ldo,
+                                  double scale, int* flag, int nsm, cudaStream_t st, TcDiag diag) {
   using C = Cfg<S, BN>;
   if (nprob <= 0 || M <= 0 || N <= 0) return cudaSuccess;
-  auto k = tc_gemm_sliced<S, BN, OutT, TF>;
+  auto k = tc_gemm_sliced<S, BN>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
   if (e != cudaSuccess) return e;
   const long long ntiles = (long long)nprob * ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
   const int grid = (int)(ntiles < nsm ? ntiles : nsm);
   k<<<grid, 192, C::kSmem, st>>>(mA[0], mA[1], mB[0], mB[1], probs_dev, nprob, M, N, ldo, scale,
-                                 flag, amax, diag);
+                                 flag, diag);
   return cudaGetLastError();
 }
-
-int tc_products(int S) { return S * (S + 1) / 2; }
 
 // Tile width of the single-product diagnostics for S slices.
 int sliced_product_bn(int S) { return S <= 2 ? 256 : S <= 4 ? 128 : 64; }
@@ -560,26 +442,14 @@ cudaError_t launch_sliced_product(int S, const CUtensorMap* mA, const CUtensorMa
                                   const TcProb* dp, int M, int N, double scale, int* flag,
                                   int nsm, cudaStream_t st, TcDiag dg) {
   switch (S) {
-    case 1: return launch_tc_gemm<1, 256, double, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
-    case 2: return launch_tc_gemm<2, 256, double, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
-    case 3: return launch_tc_gemm<3, 128, double, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
-    case 4: return launch_tc_gemm<4, 128, double, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
-    case 5: return launch_tc_gemm<5, 64, double, false>(mA, mB, dp, 1, M, N, M, scale, flag, nullptr, nsm, st, dg);
+    case 1: return launch_tc_gemm<1, 256>(mA, mB, dp, 1, M, N, M, scale, flag, nsm, st, dg);
+    case 2: return launch_tc_gemm<2, 256>(mA, mB, dp, 1, M, N, M, scale, flag, nsm, st, dg);
+    case 3: return launch_tc_gemm<3, 128>(mA, mB, dp, 1, M, N, M, scale, flag, nsm, st, dg);
+    case 4: return launch_tc_gemm<4, 128>(mA, mB, dp, 1, M, N, M, scale, flag, nsm, st, dg);
+    case 5: return launch_tc_gemm<5, 64>(mA, mB, dp, 1, M, N, M, scale, flag, nsm, st, dg);
     default: return cudaErrorInvalidValue;
   }
 }
 long long tc_default_wait_cycles() { return kWaitCycles; }
-
-#define LNO_TC_INST(S, BN, T, TF)                                                            \
-  template cudaError_t launch_tc_gemm<S, BN, T, TF>(                                         \
-      const CUtensorMap*, const CUtensorMap*, const TcProb*, int, int, int, int, double, int*, \
-      unsigned long long*, int, cudaStream_t, TcDiag);
-// DF assembly and the diagnostics (float64 transposed output)
-LNO_TC_INST(1, 256, double, false)
-LNO_TC_INST(2, 256, double, false)
-LNO_TC_INST(3, 128, double, false)
-LNO_TC_INST(4, 128, double, false)
-LNO_TC_INST(5, 64, double, false)
-#undef LNO_TC_INST
 
 }  // namespace lno
