@@ -9,6 +9,7 @@
 
 #include <cstdio>
 
+#include "class_sum.cuh"
 #include "lno_ot.h"
 
 namespace lno {

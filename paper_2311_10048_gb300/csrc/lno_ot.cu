@@ -968,7 +968,8 @@ struct SpinPass {
       // adjoint on the tensor cores: one launch per run as well, each orbital's rows
       // with their own scale
       SlicedBatch sL, sR;
-      const bool sliced = R.tc_adjoint && !runs.empty() && l_rows > 0 && r_rows > 0;
+      const bool sliced = R.tc_adjoint && R.naux <= kWideBF16 && !runs.empty() && l_rows > 0 &&
+                          r_rows > 0;
       if (sliced) {
         const int norb = (int)(Ro.total_rows() / r_rows);
         TRY(sL.alloc(A, 1, (int)l_rows, R.naux, true, false));
@@ -2135,6 +2136,7 @@ int tc_matmul(Run& R, Arena& A, int M, int N, int K, View a, View b, double* C, 
   if (tiles < 2 * R.ctx->nsm && K >= 4096)
     nsp = (int)std::max<int64_t>(1, std::min<int64_t>({ceil_div(4 * R.ctx->nsm, tiles),
                                                        K / 2048, kMaxSplit}));
+  nsp = std::max(nsp, ceil_div(K, kWideBF16));   // class sums within class_sum's range
   const int Kc = (int)round_up(ceil_div(K, nsp), 32);
   nsp = ceil_div(K, Kc);
   const int64_t Kp = round_up(Kc, 32);

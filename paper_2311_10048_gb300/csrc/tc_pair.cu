@@ -296,8 +296,9 @@ constexpr int pair_max_width() {
 }
 
 // TF32: 32-bit elements, 16 per 64-byte row, K 8 per MMA; the 16-bit formats
-// have 32 per row, K 16.  ROWS: float64 output as out[m][n].  diag is the bounded-wait test hook of tc_gemm.cu.
-template <int S, int FMT, typename OutT, bool ROWS>
+// have 32 per row, K 16.  ROWS: float64 output as out[m][n]; WIDE: its
+// K may pass what class_sum needs no checks for.  diag is the bounded-wait test hook of tc_gemm.cu.
+template <int S, int FMT, typename OutT, bool ROWS, bool WIDE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<OutT>(), 1)
 tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
              const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
@@ -596,12 +597,12 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
               lo = FMT == kFmtF16 ? __fmaf_rn(lo, kW, x[g]) : __fadd_rn(lo, x[g]);
             }
             if constexpr (ROWS) {
-              v[j] = class_sum<S, BITS, FMT == kFmtF16>(x, es, fl & kTcFloatRest);
+              v[j] = class_sum<S, BITS, FMT == kFmtF16, WIDE>(x, es, fl & kTcFloatRest);
             } else {
               if (!mok || n + j >= N) continue;
               if (amax != nullptr) lmax = fmaxf(lmax, fabsf(__fmul_rn(lo, scale)));
               if (outp != nullptr) {
-                const double y = class_sum<S, BITS, FMT == kFmtF16>(x, es, fl & kTcFloatRest);
+                const double y = class_sum<S, BITS, FMT == kFmtF16, WIDE>(x, es, fl & kTcFloatRest);
                 double* o = out + (int64_t)(n + j) * ldo + m;
                 if (fl & kTcAtomic)
                   atomicAdd(o, y);
@@ -657,10 +658,10 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
 
 // Pairs that fit the device at once (queried once; the persistent loop deals
 // its tiles over them, so none may wait for a slot).
-template <int S, int FMT, typename OutT, bool ROWS>
+template <int S, int FMT, typename OutT, bool ROWS, bool WIDE>
 int pair_clusters(int nsm) {
   static const int n = [] {
-    auto k = tc_pair_gemm<S, FMT, OutT, ROWS>;
+    auto k = tc_pair_gemm<S, FMT, OutT, ROWS, WIDE>;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2);
     cfg.blockDim = dim3(pair_threads<OutT>());
@@ -681,7 +682,7 @@ int pair_clusters(int nsm) {
   return std::max(1, n > 0 ? std::min(n, nsm / 2) : nsm / 2);
 }
 
-template <int S, int FMT, typename OutT, bool ROWS = false>
+template <int S, int FMT, typename OutT, bool ROWS = false, bool WIDE = false>
 cudaError_t launch_pair(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb* probs,
                         const TcProb& one, int nprob, int M, int N, int ldo, double scale,
                         int* flag, unsigned long long* amax, int nsm, cudaStream_t st,
@@ -694,11 +695,11 @@ cudaError_t launch_pair(const CUtensorMap* mA, const CUtensorMap* mB, const TcPr
   if (sizeof(OutT) == 8 && tile.nbuf != 2) return cudaErrorInvalidValue;
   int ex;
   if (std::frexp(scale, &ex) != 0.5) return cudaErrorInvalidValue;   // scale = 2^(ex - 1)
-  auto k = tc_pair_gemm<S, FMT, OutT, ROWS>;
+  auto k = tc_pair_gemm<S, FMT, OutT, ROWS, WIDE>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
   if (e != cudaSuccess) return e;
   const long long units = (long long)nprob * ((M + 2 * BM - 1) / (2 * BM)) * tile.nN;
-  const int pairs = (int)std::min<long long>(units, pair_clusters<S, FMT, OutT, ROWS>(nsm));
+  const int pairs = (int)std::min<long long>(units, pair_clusters<S, FMT, OutT, ROWS, WIDE>(nsm));
   k<<<2 * pairs, pair_threads<OutT>(), kSmemBytes, st>>>(mA[0], mA[1], mB[0], mB[1], probs, one,
                                                          nprob, M, N, ldo, (float)scale, ex - 1,
                                                          flag, amax, diag, lay, tile);
@@ -753,12 +754,16 @@ template <int S, int FMT>
 cudaError_t launch_tc_pair_f64(const CUtensorMap* mA, const CUtensorMap* mB, const TcProb& p,
                                int M, int N, int ldo, double scale, int* flag,
                                unsigned long long* amax, int nsm, cudaStream_t st, PairTile tile) {
-  return launch_pair<S, FMT, double>(mA, mB, nullptr, p, 1, M, N, ldo, scale, flag, amax, nsm, st,
-                                     tc_normal(), TcOut{kOutRows, 0, 0, 0}, tile);
+  auto launch = launch_pair<S, FMT, double>;
+  if constexpr (S > 2)   // two slices: the measuring pass only
+    if (p.seg[0].K > (FMT == kFmtF16 ? kWideFP16 : kWideBF16))
+      launch = launch_pair<S, FMT, double, false, true>;
+  return launch(mA, mB, nullptr, p, 1, M, N, ldo, scale, flag, amax, nsm, st, tc_normal(),
+                TcOut{kOutRows, 0, 0, 0}, tile);
 }
 
 // A group of such products, each with its own flags and, where TcProb.ea and eb
-// are given, its own scale.
+// are given, its own scale; K at most kWideBF16.
 template <int S, int FMT>
 cudaError_t launch_tc_pair_f64_group(const CUtensorMap* mA, const CUtensorMap* mB,
                                      const TcProb* probs_dev, int nprob, int M, int N, int ldo,

@@ -1,7 +1,7 @@
 """Float64 value of an element's weight-class sums (csrc/class_sum.cuh), compiled for
 the host: correctly rounded from the exact sum of the classes while all of them stay
 below 2^30 in units of their last digit (sums around and beyond 2^53 for four and five
-slices among them); beyond that within 2^-51 of the sum of their
+slices among them), with or without the checks of long contractions; beyond that within 2^-51 of the sum of their
 magnitudes (S roundings of a float64 sum)."""
 import os
 import subprocess
@@ -37,10 +37,12 @@ def test_class_sum_ranges(tmp_path):
               c[g] = INTS ? f : std::ldexp(f, -BITS * g);
             }
             const int e = (int)(rng() % 1800) - 900;
-            const double got = lno::class_sum<S, BITS, INTS>(c, e, false);
+            const double got = lno::class_sum<S, BITS, INTS, true>(c, e, false);
             const double want = std::ldexp((double)exact, e - BITS * (S - 1));
             const double tol = std::ldexp((double)mag, e - BITS * (S - 1) - 51);
             if (fits ? got != want : !(std::fabs(got - want) <= tol)) ++bad;
+            if (top0 <= 28 && top <= 30 &&
+                lno::class_sum<S, BITS, INTS, false>(c, e, false) != want) ++bad;
           }
         }
         int main() {
@@ -52,10 +54,10 @@ def test_class_sum_ranges(tmp_path):
               run<3, 11, true>(t0, t);
             }
           const float nan4[4] = {NAN, 1.f, 0.f, 0.f}, inf4[4] = {INFINITY, 0.f, 0.f, 0.f};
-          if (!std::isnan(lno::class_sum<4, 8, false>(nan4, 0, false))) ++bad;
-          if (!std::isnan(lno::class_sum<4, 8, false>(inf4, 0, true))) ++bad;
+          if (!std::isnan(lno::class_sum<4, 8, false, true>(nan4, 0, false))) ++bad;
+          if (!std::isnan(lno::class_sum<4, 8, false, false>(inf4, 0, true))) ++bad;
           const float flat[5] = {4194304.f, 0.f, 0.f, 0.f, 0.f};   // 2^22 2^32 = 2^54
-          if (lno::class_sum<5, 8, false>(flat, -14, false) != 256.0) ++bad;
+          if (lno::class_sum<5, 8, false, false>(flat, -14, false) != 256.0) ++bad;
           std::printf("%d\\n", bad);
           return 0;
         }

@@ -220,3 +220,31 @@ def test_many_triplets_take_little_memory_each(lib):
     ref, _ = run("fp64", few)
     for f, r, x in zip(full, ref, few):
         assert np.abs(f[x] - r).max() <= 1e-7 * np.abs(r).max()
+
+
+@pytest.mark.parametrize("prec,v,n,short", [("bf16x10", 256, (3, 3), 1536),
+                                            ("bf16x10", 24, (4, 3), 16384),
+                                            ("bf16x15", 24, (4, 3), 16384)])
+def test_long_auxiliary_index(prec, v, n, short):
+    """Auxiliary bases beyond the lengths whose class sums need no checks (1536 on FP16
+    slices, 16384 on BF16 ones): with zero factors there they give the shorter basis's
+    energies bit for bit.  Beyond 16384 the adjoint splits its products; its gradients
+    agree with the float64 path's within the 32-bit operands."""
+    d = make_domain(v + n[0], n, naux=short, L=short / 3, seed=6, t1_sd=0.02)
+    e = [e_trips(prec, lno_ot.to_device(d))]
+    d["naux"] = short + 40
+    d["B"] = [np.concatenate([b, np.zeros((40,) + b.shape[1:])]) for b in d["B"]]
+    dd = lno_ot.to_device(d)
+    e.append(e_trips(prec, dd))
+    assert np.array_equal(e[0], e[1])
+    if v > 100:
+        return
+    g = []
+    for p in ("fp64", prec):
+        ctx = lno_ot.Context(0, p)
+        x = dict(dB=[torch.zeros_like(b) for b in dd["B"]], dt2ab=torch.zeros_like(dd["t2ab"]))
+        ctx.backward(dd, 1.0, x)
+        ctx.close()
+        g.append(x["dB"] + [x["dt2ab"]])
+    for x, y in zip(*g):
+        assert float((x - y).abs().max()) <= 1e-7 * float(x.abs().max())
