@@ -568,6 +568,11 @@ struct Run {
         }
       }
     }
+    return stage_blocks();
+  }
+
+  // the DF factor blocks in the present slice format
+  int stage_blocks() {
     for (int s = 0; s < 2; ++s) {
       const int o = no[s], oi = noi[s], v = nv[s];
       TRY(alloc_operand(Boo[s], 1, (int64_t)oi * o, naux, Sdf));
@@ -610,6 +615,15 @@ struct Run {
       }
     }
     return LNO_OT_OK;
+  }
+
+  // From here on without FP16 slices: the DF blocks are laid out again.
+  int leave_f16() {
+    f16 = false;
+    S = Sdf = 4;
+    for (int s = 0; s < 2; ++s)
+      for (Operand* op : {&Boo[s], &Bov[s], &Bvv[s]}) arena.drop(op->bf);
+    return stage_blocks();
   }
 
   // dst slot q = src rows [dlist[q] * rows, (dlist[q] + 1) * rows): a DF block
@@ -1441,6 +1455,8 @@ struct SpinPass {
 
   // operands for the current selections (the whole domain when cached)
   int prepare() {
+    f16 = R.f16;
+    S = R.S;
     plan();
     TRY(prepare_inputs());
     TRY(build_v_blocks());
@@ -1449,12 +1465,13 @@ struct SpinPass {
     bool exact;
     TRY(check_exact(&exact));
     if (exact) return LNO_OT_OK;
-    // this spin's operands once more, on the BF16 slices; what the other spin has
-    // computed stands, and the DF blocks stay as they are
-    for (Operand* op : {&AT, &BT, &A1, &BG, &BF, &AT2}) own.drop(op->bf);
-    f16 = false;
-    S = 4;
-    return build();
+    // Not provably exact: this spin again, DF blocks and operands on the BF16 slices
+    // (as a whole call on them computes it).  What the other spin has computed on FP16
+    // slices stands.
+    own.release();
+    t2st = nullptr;
+    TRY(R.leave_f16());
+    return prepare();
   }
   // FP16 slices: whether the class-0 sums of every contraction are exact (kExactSum)
   int check_exact(bool* exact) {
@@ -1872,15 +1889,16 @@ int energy_impl(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
                 const PassSpec* spec = nullptr) {
   ctx->frugal = ctx->small_pieces;
   int rc = energy_once(ctx, dom, out, spec);
-  for (int tries = 0; tries < 3; ++tries) {
-    if (rc == kRescale) ctx->exact_measure = true;
+  for (int tries = 0; tries < 4; ++tries) {
+    if (rc == kRescale && ctx->exact_measure) ctx->no_f16 = true;   // measured and built alike
+    else if (rc == kRescale) ctx->exact_measure = true;
     else if (rc == kNoF16) ctx->no_f16 = true;
     else if (rc == LNO_OT_ENOMEM && !ctx->frugal) ctx->frugal = true;
     else break;
     rc = energy_once(ctx, dom, out, spec);
   }
   ctx->exact_measure = ctx->no_f16 = ctx->frugal = false;
-  return rc > 0 ? LNO_OT_EINVAL : rc;   // not reached: neither can come twice
+  return rc > 0 ? LNO_OT_EINVAL : rc;   // not reached: none comes again
 }
 
 // ---------------------------------------------------------------------------
