@@ -63,10 +63,9 @@ def peaks():
 # DRAM bytes (read + write) per tensor-core flop of the contraction kernel as
 # it is now, from one ncu capture per precision on a c1-sized group; the
 # per-launch traffic scales with the launch's tensor flops at a fixed virtual
-# space.  None is listed while the kernel has changed since its last capture
-# (profiles/tc_gemm_sliced_bf16x10_c1shape.md holds the last one, 1.3239e-3
-# B/flop, before the register-staged epilogue and the tiled Y/Z' stores), and
-# the bench line then reports traffic as null.
+# space.  None is listed: the captures of the present kernel are of small groups
+# (profiles/tc_pair_w_fp16.md), whose operands are read for few triplets, so the
+# bench line reports traffic as null.
 DRAM_BYTES_PER_TENSOR_FLOP = {}
 
 # FP32 operations per restricted (abc) element in the float32 energy kernel
@@ -823,7 +822,7 @@ def run_domain(args):
         "steps": K, "warmup": args.warmup, "ms_per_step": ms_step,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": "bf16", "data": "synthetic",
-        "precision": (f"{args.precision.upper()}: exact BF16 slices of float64 operands on "
+        "precision": (f"{args.precision.upper()}: 16-bit slices of float64 operands on "
                       f"tcgen05 (FP32 TMEM accumulators per weight class), float64 "
                       f"denominators and compensated sums"),
         "config": {"workload": (f"single LNO domain E(T): nbas={nbas} nocc={nocc[0]}/{nocc[1]} "

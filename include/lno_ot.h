@@ -66,6 +66,11 @@ typedef enum {
  *  BF16X10 4 slices per operand and 10 slice products (8 bits more again):
  *          the accurate mode for large domains, where the BF16X6 truncation
  *          adds up over ~1e5 triplets; about 1.7x the contraction time.
+ *          Domains of at least 256 virtuals, or 160 and 8 occupied orbitals
+ *          per spin, run on 3 FP16 slices of 11 bits and 6 products instead
+ *          (32 to 33 bits of each operand either way) where the row norms show
+ *          that the leading products add up without rounding; a spin whose
+ *          data do not allow it runs on the BF16 slices.
  *  BF16X15 5 slices per operand and 15 slice products, with the DF assembly
  *          on 5 slices too: 8 bits more again than BF16X10 in both steps, at
  *          about 1.5x its contraction time.  The reference mode against which
@@ -253,8 +258,8 @@ LNO_OT_API int lno_ot_energy_batched(lno_ot_ctx* ctx, int ndom, const lno_ot_dom
  * per triplet (never stored).  Operands, energy adjoint and layout adjoints
  * run in float64; the contractions (the DF assembly, the X recompute, the
  * contraction and DF adjoints) run in float64 in an LNO_OT_FP64 context and on
- * the tensor cores otherwise (4 exact BF16 slices of each float64 operand with
- * a power-of-two scale, float64 output of the exact class sums).  Stats of the
+ * the tensor cores otherwise (4 BF16 slices of each float64 operand with a
+ * power-of-two scale, float64 output).  Stats of the
  * call (lno_ot_last_stats): ms_total wall clock, ms_stage staging and operand
  * builds, ms_contract the contraction kernels (tensor-core context), ms_energy
  * the energy adjoint kernels. */
@@ -316,8 +321,7 @@ LNO_OT_API int lno_ot_laplace_quadrature(double xmin, double xmax, double tol, i
  * DEVICE [naux][nbas][nbas] caller-owned (the first *naux_out blocks are
  * written; may be dom->B[s] itself).  eigenvalues: HOST [naux] (all
  * eigenvalues of W, descending) or NULL.  Runs in float64 on the CUDA cores
- * (pair-packed contraction, cyclic Jacobi rotations replayed as a CUDA
- * graph, contraction), whatever the context's precision; synchronous. */
+ * (pair-packed contraction, cyclic Jacobi rotations, contraction), whatever the context's precision; synchronous. */
 LNO_OT_API int lno_ot_naf(lno_ot_ctx* ctx, const lno_ot_domain* dom, double eps_naf,
                           double* B_out[2], int* naux_out, double* eigenvalues);
 

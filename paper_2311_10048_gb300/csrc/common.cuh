@@ -165,7 +165,7 @@ struct TcSeg {
 
 // TcProb.flags: kTcAccum adds the result to out instead of storing it;
 // kTcFloatRest forms the float64 result as HI + the float32 sum of the lower
-// weight classes instead of the exact sum of all (the adjoint's products)
+// weight classes instead of the sum of all in integers (the adjoint's products)
 // kTcAtomic (tc_pair.cu) adds with atomics: problems of one launch share an output
 constexpr int kTcAccum = 1, kTcFloatRest = 2, kTcAtomic = 4;
 

@@ -10,9 +10,9 @@
 //     spin) or Y and Z' (mixed) per triplet, one energy launch assembles W,
 //     V and sums W (W + V) / D per triplet (energy.cu);
 //  4. per-triplet sums -> per-case compensated sums -> host.
-// Precision FP64 runs every contraction on the CUDA cores in float64; the
-// BF16X3 / BF16X6 precisions run them on the tensor cores on exact BF16
-// slices (tc_gemm.cu), with float64 kept for orbital energies and sums.
+// Precision FP64 runs every contraction on the CUDA cores in float64; the others
+// run them on the tensor cores on 16-bit or TF32 slices of the float64 operands
+// (tc_pair.cu), with float64 kept for orbital energies and sums.
 #include <algorithm>
 #include <cstdlib>
 #include <chrono>
@@ -235,8 +235,15 @@ bool f16_sizes(const int* nvir, const int* nocc) {
          (v >= kF16MinVirtuals && std::min(nocc[0], nocc[1]) >= kF16MinOccupied);
 }
 // FP32 sums of integers are exact while no partial sum exceeds 2^24: by
-// Cauchy-Schwarz the product of the row norms bounds every one (the BF16 slices
-// are exact for any data only to K = 1024).  0.999: the norms' own rounding.
+// Cauchy-Schwarz the product of the leading slices' row norms bounds every sum of
+// class 0 (on the BF16 slices class g is exact for any data to K = 1024 / (g + 1)).
+// Classes 1 and 2 are not checked: their digits run over +-1024 whatever the data,
+// so a sum may pass 2^24 and lose its last bits there, 2^-11 or 2^-22 of class 0's
+// unit each.  By estimate that is 1/20 of what the dropped products leave for K =
+// 1200 factors of mixed signs, and about as much as those for factors of one sign
+// and size throughout; per-triplet errors against float64 are those of the BF16
+// slices (sd 4e-11 to 9e-11 Eh, worst 2e-10 to 4e-10, at 160 to 290 virtuals).
+// 0.999: the norms' own rounding.
 constexpr double kExactSum = 16777216.0 * 0.999;
 
 #define TRY(expr)                       \
@@ -709,8 +716,10 @@ int grouped_products(Run& R, Arena& A, const std::vector<TcProb>& pr, const Slic
   return LNO_OT_OK;
 }
 
-// Problems of one product, its k range in chunks of at most `chunk` (enough
-// problems for the device, and class sums within what FP32 holds exactly).
+// Problems of one product, its k range in chunks of at most `chunk`: enough
+// problems for the device.  (Class 0 of a chunk is exact for any data to K = 1024
+// and for random signs far beyond; a longer sum of one sign rounds at 2^-24 of
+// itself, as the single products of tc_matmul do.)
 void add_chunks(std::vector<TcProb>& out, int a_row, int b_row, int K, bool neg, double* dst,
                 int flags, const int* ea, const int* eb, int chunk = 4096) {
   for (int k = 0; k < K; k += chunk) {
@@ -2135,8 +2144,9 @@ int zero_operand_like(Arena& A, const Operand& src, Operand& d, cudaStream_t st)
 }
 
 // C[m ldc + n] (+)= alpha sum_k a(m, k) b(n, k) on the tensor cores: both views
-// are cut into 4 exact BF16 slices with power-of-two scales (the DF assembly's
-// representation, 10 slice products, float64 output of the exact class sums).
+// are cut into 4 BF16 slices with power-of-two scales (the DF assembly's
+// representation, 10 slice products, float64 output: class 0 plus the float32 sum of
+// the others).
 // Used by the adjoint of the tensor-core precisions.
 int tc_matmul(Run& R, Arena& A, int M, int N, int K, View a, View b, double* C, int64_t ldc,
               double alpha, bool accum, bool b_const) {

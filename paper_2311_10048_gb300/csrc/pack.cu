@@ -16,17 +16,18 @@
 //   AT2[p][K][C][kk] = t^{eC}_{pK}  (kk=e),     (mp|CK) (kk = vs+m)
 //   Y[a,(bC)]   = A1[j][K].BG[i] - A1[i][K].BG[j] + AT[i][j].BF[K]
 //   Z'[C,(a<b)] = -AT2[j][K].BT[i] + AT2[i][K].BT[j]
-// Rows are padded with zeros to a pitch Kp (multiple of 8).
+// Rows are padded with zeros to a pitch Kp (a multiple of 32 elements on 16-bit
+// slices, of 16 otherwise; of 8 for the DF blocks of a call with a memory bound).
 // Occupied indices come in two ranges: the summed (internal) m, M run over the
 // first oi (oti) orbitals, the external ones over all o (ot) the arrays hold.
 // The two differ only when pseudo-orbitals (the central LMOs of the Laplace
 // form, Sec. 3.7) are appended after the real occupied orbitals; the DF
 // blocks with one internal occupied index are laid out [internal][external].
 //
-// Every pack kernel is templated on its store: float64, or the exact
-// BF16 slices of the tensor-core path (value = scale 2^-7 (s1 + s2 + s3),
-// s1 an integer in [-128, 128], s2 a multiple of 2^-8 in [-1/2, 1/2], ...,
-// each step rounded to nearest).
+// Every pack kernel is templated on its store: float64, or the slices of the
+// tensor-core path (BF16: value = scale 2^-7 (s1 + s2 + s3), s1 an integer in
+// [-128, 128], s2 a multiple of 2^-8 in [-1/2, 1/2], ..., each digit the nearest;
+// FP16 and TF32 in common.cuh).
 #include <algorithm>
 #include <cmath>
 

@@ -1,15 +1,19 @@
 // Tensor-core contraction on CTA pairs for sm_103a: tcgen05.mma.cta_group::2
-// (256 x w tiles, FP32 accumulators in TMEM) fed by TMA, on exactly sliced
-// float64 operands.  Runs the W contractions (float32 row-major output) and the
-// DF assembly (float64 output out[n][m], or only its largest magnitude).  The slicing, the weight-class
-// accumulators and the segment sums are those of tc_gemm.cu: one TMEM
-// accumulator per weight class g = p + q of the slice products, so every class
-// sum is exact, added smallest class first in float32.
+// (256 x w tiles, FP32 accumulators in TMEM) fed by TMA, on sliced float64
+// operands.  Runs the W contractions (float32 row-major output), the DF assembly
+// (float64 output out[n][m], or only its largest magnitude) and the adjoint's
+// products.  One TMEM accumulator per weight class g = p + q of the slice products,
+// so that none is rounded at the magnitude of a larger one; the classes are added
+// smallest first (float32 output) or as integers (class_sum.cuh).  A class is exact
+// while it stays below 2^24 of its unit: on BF16 slices for any data to K = 1024 / (g +
+// 1) and for random signs far beyond; on FP16 slices class 0 is shown to be (row norms,
+// lno_ot.cu), classes 1 and 2 may round at 2^-24 of themselves; TF32 rounds.
 //
 // What bounds it: the feed from L2 into shared memory.  A tile that one CTA
 // computes alone loads S (128 + w) 64-byte rows per k block; measured on five
-// shapes every launch of that form moved 8.0-9.2 TB/s from L2 whatever its
-// tensor rate (21-60%).  So
+// shapes every launch of that form moved 8.0-9.2 TB/s of operand rows whatever its
+// tensor rate (21-60%); this form moves 11.4 TB/s at 182 virtuals (tensor pipe 63%
+// active) and at 360 (87%).  So
 //  * the two CTAs of a pair share one 256 x w tile: each loads its 128 rows of
 //    the long (pair) operand and half of the w rows of the short one, and the
 //    tensor cores of both read both halves: S (128 + w / 2) rows per k block;
@@ -297,7 +301,7 @@ constexpr int pair_max_width() {
 
 // TF32: 32-bit elements, 16 per 64-byte row, K 8 per MMA; the 16-bit formats
 // have 32 per row, K 16.  ROWS: float64 output as out[m][n]; WIDE: its
-// K may pass what class_sum needs no checks for.  diag is the bounded-wait test hook of tc_gemm.cu.
+// K may pass what class_sum needs no checks for.  diag is the bounded-wait test hook (TcDiag).
 template <int S, int FMT, typename OutT, bool ROWS, bool WIDE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<OutT>(), 1)
 tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
@@ -535,7 +539,7 @@ tc_pair_gemm(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ 
             tmem_ld_wait();
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-              // lower classes first (each exact), then one rounding against class 0
+              // lower classes first, then one rounding against class 0
               float lo = 0.f;
 #pragma unroll
               for (int g = S - 1; g >= 1; --g)
