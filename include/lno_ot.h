@@ -107,8 +107,9 @@ typedef struct {
                              orbitals, everything of lno_ot_naf.  A call that
                              needs more returns LNO_OT_ENOMEM.  The contraction
                              operands and intermediates of one spin at a time
-                             are not part of it.  With a bound the DF blocks
-                             are packed more tightly (a little slower). */
+                             are not part of it.  The DF blocks are packed more
+                             tightly (up to 7% slower) where the bound asks
+                             for it. */
   const char* tune_cache; /* NULL, or a tuning table written by the autotuner
                              (paper_2311_10048_gb300/tune.py): text lines
                              "vmax bn group_cap" giving, per bucket of

@@ -269,8 +269,12 @@ struct Arena {
     used = 0;
   }
   template <typename T>
+  static size_t bytes_of(size_t n) {
+    return (std::max<size_t>(n * sizeof(T), 256) + 255) / 256 * 256;
+  }
+  template <typename T>
   int get(T** out, size_t n) {
-    const size_t bytes = (std::max<size_t>(n * sizeof(T), 256) + 255) / 256 * 256;
+    const size_t bytes = bytes_of<T>(n);
     if (limit && used + bytes > limit) return LNO_OT_ENOMEM;
     void* p = nullptr;
     if (cudaMallocAsync(&p, bytes, st) != cudaSuccess) {
@@ -388,6 +392,7 @@ struct Run {
   const lno_ot_domain* dom;
   cudaStream_t st;
   Arena arena;
+  size_t held_back = 0;   // bytes that a bounded call takes of the arena after stage()
   bool f64;
   bool tf32 = false;  // W contraction operands as TF32 slices (precision TF32)
   bool f16 = false;   // precision BF16X10 on three FP16 slices (set_precision)
@@ -427,9 +432,6 @@ struct Run {
   }
 
   // ---- operand allocation -------------------------------------------------
-  int alloc_operand(Operand& op, int nslot, int64_t rows, int K, int S_) {
-    return alloc_operand(arena, op, nslot, rows, K, S_);
-  }
   // tf: TF32 slices (the W operands of precision TF32); DF blocks are BF16.
   // pitch: multiple of the row pitch in elements (0: the widest useful one).
   int alloc_operand(Arena& ar, Operand& op, int nslot, int64_t rows, int K, int S_,
@@ -438,10 +440,8 @@ struct Run {
     op.rows = rows;
     op.K = K;
     // sliced rows start on 64-byte boundaries: the contractions' 64-byte box
-    // rows then are two sectors of L2 (1.3x fewer bytes than at 16-byte pitches).
-    // Where a bound holds (workspace_bytes: the DF blocks), rows take the 8
-    // elements the loads need, so that the bound admits as large a domain as it can.
-    if (pitch == 0) pitch = ar.limit ? 8 : f64 || tf ? 16 : 32;
+    // rows then are two sectors of L2 (1.3x fewer bytes than at 16-byte pitches)
+    if (pitch == 0) pitch = f64 || tf ? 16 : 32;
     op.Kp = (int)round_up(std::max(K, 1), pitch);
     op.S = f64 ? 0 : S_;
     const int64_t n = std::max<int64_t>((int64_t)nslot * rows * op.Kp, 8);
@@ -580,11 +580,23 @@ struct Run {
 
   // the DF factor blocks in the present slice format
   int stage_blocks() {
+    // Under a bound (workspace_bytes) rows have the 8-element pitch that the loads need
+    // unless everything fits with the wide one, so that the bound admits as large a
+    // domain as it can (366/8/6, naux 1000: whole call 245 ms wide, 263 ms at 8).
+    int pitch = 0;
+    if (arena.limit) {
+      size_t wide = arena.used + held_back;
+      for (int s = 0; s < 2; ++s)
+        for (int64_t rows : {(int64_t)noi[s] * no[s], (int64_t)no[s] * nv[s],
+                             (int64_t)nv[s] * nv[s]})
+          wide += round_up(std::max<int64_t>(rows * round_up(naux, 32), 8) * Sdf * 2, 256);
+      pitch = f64 || wide > arena.limit ? 8 : 0;
+    }
     for (int s = 0; s < 2; ++s) {
       const int o = no[s], oi = noi[s], v = nv[s];
-      TRY(alloc_operand(Boo[s], 1, (int64_t)oi * o, naux, Sdf));
-      TRY(alloc_operand(Bov[s], 1, (int64_t)o * v, naux, Sdf));
-      TRY(alloc_operand(Bvv[s], 1, (int64_t)v * v, naux, Sdf));
+      TRY(alloc_operand(arena, Boo[s], 1, (int64_t)oi * o, naux, Sdf, false, pitch));
+      TRY(alloc_operand(arena, Bov[s], 1, (int64_t)o * v, naux, Sdf, false, pitch));
+      TRY(alloc_operand(arena, Bvv[s], 1, (int64_t)v * v, naux, Sdf, false, pitch));
       Operand* ops[3] = {&Boo[s], &Bov[s], &Bvv[s]};
       const int p0[3] = {0, 0, o}, np[3] = {oi, o, v}, q0[3] = {0, o, o}, nq[3] = {o, v, v};
       const int eB = 7 - std::ilogb(sigB);
@@ -1846,6 +1858,9 @@ int energy_once(lno_ot_ctx* ctx, const lno_ot_domain* dom, lno_ot_result* out,
   double* e_int[4];
   for (int c = 0; c < 4; ++c)
     TRY(R.arena.get(&e_int[c], std::max<size_t>(cs[c].trips.size(), 1)));
+  if (dom->e_orb[0] || dom->e_orb[1])   // the triplet lists of finish_call
+    for (int c = 0; c < 4; ++c)
+      R.held_back += Arena::bytes_of<Trip>(std::max<size_t>(cs[c].trips.size(), 1));
   // Closed-shell domain (both spins given by the same arrays, spin-flip
   // symmetric mixed amplitudes): bbb and abb are the spin-flip images of aaa
   // and aab, with identical values, so only the spin-up pass runs.

@@ -17,7 +17,7 @@
 //   Y[a,(bC)]   = A1[j][K].BG[i] - A1[i][K].BG[j] + AT[i][j].BF[K]
 //   Z'[C,(a<b)] = -AT2[j][K].BT[i] + AT2[i][K].BT[j]
 // Rows are padded with zeros to a pitch Kp (a multiple of 32 elements on 16-bit
-// slices, of 16 otherwise; of 8 for the DF blocks of a call with a memory bound).
+// slices, of 16 otherwise; of 8 for the DF blocks where a memory bound asks for it).
 // Occupied indices come in two ranges: the summed (internal) m, M run over the
 // first oi (oti) orbitals, the external ones over all o (ot) the arrays hold.
 // The two differ only when pseudo-orbitals (the central LMOs of the Laplace

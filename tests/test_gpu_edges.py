@@ -248,3 +248,26 @@ def test_long_auxiliary_index(prec, v, n, short):
         g.append(x["dB"] + [x["dt2ab"]])
     for x, y in zip(*g):
         assert float((x - y).abs().max()) <= 1e-7 * float(x.abs().max())
+
+
+@pytest.mark.parametrize("prec", ["bf16x10", "fp64"])
+def test_every_bound_above_the_smallest_is_accepted(prec):
+    """Rows are packed tightly only where the wide ones (and the lists that the orbital
+    contributions take afterwards) do not fit: no bound in between is refused, and the
+    results are the same bit for bit."""
+    dd = lno_ot.to_device(make_domain(40, (12, 10), naux=41, L=15.0, seed=5))
+
+    def run(bound):
+        ctx = lno_ot.Context(0, prec, workspace_bytes=bound)
+        orb = [torch.zeros(n, dtype=torch.float64, device="cuda") for n in (12, 10)]
+        out = ctx.energy(dd, raise_on_error=False, e_orb=orb)
+        ctx.close()
+        return out["total"] if out["status"] == lno_ot.OK else None
+
+    want = run(0)
+    lo, hi = 256, 64 << 20
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if run(mid) is not None else (mid, hi)
+    for bound in np.linspace(hi, 2.2 * hi, 60).astype(int):
+        assert run(int(bound)) == want, bound
