@@ -242,7 +242,7 @@ bool f16_sizes(const int* nvir, const int* nocc) {
 // unit each.  By estimate that is 1/20 of what the dropped products leave for K =
 // 1200 factors of mixed signs, and about as much as those for factors of one sign
 // and size throughout; per-triplet errors against float64 are those of the BF16
-// slices (sd 4e-11 to 9e-11 Eh, worst 2e-10 to 4e-10, at 160 to 290 virtuals).
+// slices (sd 4e-11 to 9e-11 Eh at 160 to 290 virtuals, worst 2e-10 to 5e-10 up to 360).
 // 0.999: the norms' own rounding.
 constexpr double kExactSum = 16777216.0 * 0.999;
 
